@@ -334,20 +334,21 @@ int zolo_dgemm_noalloc(int transA, int transB, int64_t m, int64_t n, int64_t k, 
    then on, every zolo_pd / zolo_svd / zolo_dgemm call on h that meets a
    contraction shape (M, N, K, batch, transposes, triangular-structure flags,
    slice count) for the first time runs it once with each candidate kernel
-   (FP64 tiles 64x64, 32x128, 32x64; split-K in 2, 4 or 8 slices with a
-   deterministic reduction; the split tensor-core path when opts.prec asks for
+   (the built-in FP64 rule's tile and K split, FP64 tiles 32x128 and 32x64,
+   64x64 tiles with K split in 2, 4 or 8 over a thread-block cluster; the split tensor-core path when opts.prec asks for
    it) into a scratch output, timed with CUDA events, and keeps the fastest
    for that shape; the call's own outputs are written once, by the kept
    kernel.  To bound the cost of measuring, a shape whose built-in kernel takes
    over 50 ms keeps it, and the split path (or FP64) is not timed where the
    cost model puts it 4x behind the other.  zolo_autotune(h, 0) stops measuring; choices already made stay in
    use.  Without choices the built-in rules apply (the split path where its
-   cost model predicts a gain, else the 64x64 FP64 tile, 32x128 for M <= 32).
+   cost model predicts a gain, else the FP64 tile and K split of least estimated
+   time).
    zolo_pd_batched uses the handle's choices too: with tuning on, it first
    decomposes one matrix of every distinct configuration of the batch (sizes,
    r, iteration forms, options) on the caller's stream, outside any capture,
    while the shapes met are timed; its concurrent lanes then replay the
-   choices, each with its own split-K scratch.  There the split-or-FP64 choice
+   choices.  There the split-or-FP64 choice
    stays with the batch's throughput cost model (many calls in flight hide
    each call's latency), and only the FP64 kernels of the products it leaves
    on the FP64 pipe are measured.  A tuned kernel may sum in

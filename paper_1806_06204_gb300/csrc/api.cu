@@ -63,8 +63,7 @@ struct BatchSlot {
   int* exps = nullptr;
   size_t exp_elems = 0;
   int* err = nullptr;
-  // the handle's kernel choices as this lane replays them, with the lane's own
-  // scratch for split-K partial sums (lanes run concurrently)
+  // the handle's kernel choices as this lane replays them
   std::unique_ptr<GemmTuner> tuner;
   uint64_t tuner_gen = ~0ull;
 };
@@ -199,8 +198,6 @@ size_t layout(void* base, int64_t m, int64_t n, int r, bool svd, PdBufs* b) {
     t.qr.Tb = q.take<double>(r * t.qr.strideTb);
     t.qr.strideG = kQrBlock * kQrBlock;
     t.qr.G = q.take<double>(r * t.qr.strideG);
-    t.qr.elemsP = qr_partial_elems(m, r);
-    t.qr.P = q.take<double>(t.qr.elemsP);
     t.qr.strideW1 = kQrBlock * n;
     t.qr.W1 = q.take<double>(r * t.qr.strideW1);
     t.qr.strideW2 = kQrBlock * n;
@@ -1654,7 +1651,7 @@ int zolo_pd_batched(zolo_handle_t h, int count, const double* const* A, const in
   // distinct configuration (sizes, r, iteration forms, options) is decomposed
   // first on the caller's stream, outside any capture, in lane 0's workspace,
   // while the handle's tuner times the contraction shapes it meets; the lanes
-  // then replay the handle's choices, each with its own split-K scratch.
+  // then replay the handle's choices.
   if (h->tuner.tuning) {
     TunerScope ts(&h->tuner);
     std::map<std::vector<int64_t>, int> seen;
@@ -1689,16 +1686,6 @@ int zolo_pd_batched(zolo_handle_t h, int count, const double* const* A, const in
       sl.tuner_gen = h->tuner.gen;
     }
     sl.tuner->tuning = false;
-    if (sl.tuner->scratch_elems < h->tuner.scratch_elems) {
-      if (sl.tuner->scratch) cudaFree(sl.tuner->scratch);
-      sl.tuner->scratch = nullptr;
-      sl.tuner->scratch_elems = 0;
-      if (cudaMalloc(&sl.tuner->scratch, h->tuner.scratch_elems * sizeof(double)) != cudaSuccess) {
-        cudaGetLastError();
-        return ZOLO_ENOMEM;
-      }
-      sl.tuner->scratch_elems = h->tuner.scratch_elems;
-    }
   }
   if (!h->cap && cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking) != cudaSuccess)
     return ZOLO_ECUDA;

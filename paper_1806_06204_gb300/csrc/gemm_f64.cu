@@ -1,31 +1,55 @@
 // FP64 GEMM on the FP64 FMA pipe (DFMA), batched or batch-reduced.
 //
-// On GB300 the FP64 rate is ~1.2 TFLOP/s (about 2 DFMA per clock per SM) while
-// HBM delivers ~6.7 TB/s, so every FP64 contraction here is bound by the FMA
-// pipe, not by memory: a 64x64 output tile per CTA with 4x4 outputs per thread
-// reaches the pipe's rate with plain shared-memory staging.  tcgen05 has no
-// FP64 kind, and the FP64 mma.sync path measured slower than DFMA on this part.
+// On GB300 the FP64 rate is ~1.2 TFLOP/s (2 DFMA per clock per SM: a warp's DFMA
+// holds its sub-partition's unit for 64 clocks) while HBM delivers ~6.7 TB/s, so
+// every FP64 contraction here is bound by the FMA pipe, not by memory, and what
+// decides a product's time is how evenly its outputs spread over the 152 SMs: a
+// 64 x 64 x 256 tile holds one SM for 250 us.  The issue slots between two DFMAs
+// are nearly free, so small tiles cost little, and the tile and a K split over a
+// thread-block cluster are chosen per shape (gemm_f64_rule).  tcgen05 has no FP64
+// kind, and the FP64 mma.sync path measured slower than DFMA on this part.
+#include <cooperative_groups.h>
+
 #include <algorithm>
+#include <cmath>
 
 #include "zolo_internal.h"
 
 namespace zolo {
 namespace {
 
-// ksplit > 1: blockIdx.z = batch entry * ksplit + K slice; the slice's raw sum
-// goes to P (ld M, one M x N plane per (slice, entry)) for splitk_reduce_kernel.
-template <int BM, int BN, int BK, int TM, int TN>
+constexpr int kBK = 16;
+
+// One BM x BN output tile per cluster of `ks` CTAs (ks = 1: no cluster), each on
+// one slice of K (whole kBK steps, so every step lies in exactly one slice); the
+// ranks' partial tiles meet in distributed shared memory and are added in rank
+// order (deterministic, no scratch).  The next step's operands are fetched into
+// registers while the current one is multiplied from shared memory (two buffers,
+// one barrier per step).  alpha scales op(A) as it is staged (one FP64 multiply
+// per staged element, 1/BN of the FMAs) except for +-1, which cost nothing: the
+// sign is applied to the result.
+template <int BM, int BN, int TM, int TN>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN))
-gemm_f64_kernel(const GemmArgs g, int ksplit, double* __restrict__ P) {
+gemm_f64_kernel(const GemmArgs g, int ks) {
   constexpr int RT = BM / TM;           // threads along rows
   constexpr int CT = BN / TN;           // threads along columns
   constexpr int NT = RT * CT;
-  __shared__ double As[BK][BM + 1];
-  __shared__ double Bs[BK][BN + 1];
+  constexpr int NA = BM * kBK / NT, NB = BN * kBK / NT;   // staged elements per thread
+  static_assert(NA * NT == BM * kBK && NB * NT == BN * kBK, "whole staging rounds");
+  constexpr int kStage = kBK * (BM + 1) + kBK * (BN + 1);
+  constexpr int kSmem = 2 * kStage > BM * BN ? 2 * kStage : BM * BN;
+  __shared__ double sm[kSmem];
 
-  const int m0 = blockIdx.y * BM;
-  const int n0 = blockIdx.x * BN;
-  if (g.c_upper && m0 > n0 + BN - 1) return;   // tile strictly below the diagonal
+  const int rank = blockIdx.x % ks;            // K slice (the cluster's CTAs are x-neighbours)
+  int tm = blockIdx.y, tn = blockIdx.x / ks;
+  if (g.b_lower) {
+    // a tile's inner length is K - n0: the longest tiles start first
+    const int lin = blockIdx.y * (gridDim.x / ks) + tn;
+    tm = lin % gridDim.y;
+    tn = lin / gridDim.y;
+  }
+  const int m0 = tm * BM, n0 = tn * BN;
+  if (g.c_upper && m0 > n0 + BN - 1) return;   // tile strictly below the diagonal (all ranks)
   const int tid = threadIdx.x;
   const int tr = tid % RT;
   const int tc = tid / RT;
@@ -36,112 +60,124 @@ gemm_f64_kernel(const GemmArgs g, int ksplit, double* __restrict__ P) {
 #pragma unroll
     for (int j = 0; j < TN; ++j) acc[i][j] = 0.0;
 
-  const int zs = blockIdx.z % ksplit;          // K slice
-  const int zb = blockIdx.z / ksplit;          // batch entry (output plane)
-  const int bbeg = g.reduce ? 0 : zb;
-  const int bend = g.reduce ? g.batch : zb + 1;
-  int kbeg = g.b_lower ? (n0 / BK) * BK : 0;
+  const int zb = blockIdx.z;                   // batch entry (output plane)
+  const int zo = g.reduce ? 0 : zb / g.inner, zi = g.reduce ? 0 : zb % g.inner;
+  const int bbeg = zo;
+  const int nb = g.reduce ? g.batch : 1;
+  int kbeg = g.b_lower ? (n0 / kBK) * kBK : 0;
   int kend = g.K;
-  if (ksplit > 1) {
-    // slices of whole BK steps, so every step lies in exactly one slice
-    const int kc = ((g.K + ksplit - 1) / ksplit + BK - 1) / BK * BK;
-    kbeg = max(kbeg, zs * kc);
-    kend = min(g.K, (zs + 1) * kc);
+  if (ks > 1) {
+    const int kc = ((g.K + ks - 1) / ks + kBK - 1) / kBK * kBK;
+    kbeg = max(kbeg, rank * kc);
+    kend = min(g.K, (rank + 1) * kc);
+  }
+  const int per = kend > kbeg ? (kend - kbeg + kBK - 1) / kBK : 0;   // steps per batch entry
+  const int steps = per * nb;
+
+  const bool unit = !g.reduce && fabs(g.alpha[zo]) == 1.0;
+  double ra[NA], rb[NB];
+  auto fetch = [&](int step) {
+    const int b = bbeg + step / per;
+    const int k0 = kbeg + (step % per) * kBK;
+    const double* A = g.A + (int64_t)b * g.strideA + zi * g.innerA;
+    const double* B = g.B + (int64_t)b * g.strideB + zi * g.innerB;
+#pragma unroll
+    for (int u = 0; u < NA; ++u) {
+      const int e = tid + u * NT;
+      const int i = g.transA ? e / kBK : e % BM, kk = g.transA ? e % kBK : e / BM;
+      const int gi = m0 + i, gk = k0 + kk;
+      double v = 0.0;
+      if (gi < g.M && gk < g.K)
+        v = g.transA ? A[gk + (int64_t)gi * g.lda] : A[gi + (int64_t)gk * g.lda];
+      ra[u] = v;
+    }
+#pragma unroll
+    for (int u = 0; u < NB; ++u) {
+      const int e = tid + u * NT;
+      const int j = g.transB ? e % BN : e / kBK, kk = g.transB ? e / BN : e % kBK;
+      const int gk = k0 + kk, gj = n0 + j;
+      double v = 0.0;
+      if (gk < g.K && gj < g.N)
+        v = g.transB ? B[gj + (int64_t)gk * g.ldb] : B[gk + (int64_t)gj * g.ldb];
+      rb[u] = v;
+    }
+  };
+  auto stage = [&](int step, int buf) {
+    double* As = sm + buf * kStage;
+    double* Bs = As + kBK * (BM + 1);
+    const double al = unit ? 1.0 : g.alpha[bbeg + step / per];
+#pragma unroll
+    for (int u = 0; u < NA; ++u) {
+      const int e = tid + u * NT;
+      const int i = g.transA ? e / kBK : e % BM, kk = g.transA ? e % kBK : e / BM;
+      As[kk * (BM + 1) + i] = unit ? ra[u] : al * ra[u];
+    }
+#pragma unroll
+    for (int u = 0; u < NB; ++u) {
+      const int e = tid + u * NT;
+      const int j = g.transB ? e % BN : e / kBK, kk = g.transB ? e / BN : e % kBK;
+      Bs[kk * (BN + 1) + j] = rb[u];
+    }
+  };
+  if (steps > 0) {
+    fetch(0);
+    stage(0, 0);
+  }
+  __syncthreads();
+  for (int step = 0; step < steps; ++step) {
+    if (step + 1 < steps) fetch(step + 1);
+    const double* As = sm + (step & 1) * kStage;
+    const double* Bs = As + kBK * (BM + 1);
+#pragma unroll
+    for (int kk = 0; kk < kBK; ++kk) {
+      double a[TM], bv[TN];
+#pragma unroll
+      for (int i = 0; i < TM; ++i) a[i] = As[kk * (BM + 1) + tr + i * RT];
+#pragma unroll
+      for (int j = 0; j < TN; ++j) bv[j] = Bs[kk * (BN + 1) + tc + j * CT];
+#pragma unroll
+      for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int j = 0; j < TN; ++j) acc[i][j] = fma(a[i], bv[j], acc[i][j]);
+    }
+    if (step + 1 < steps) stage(step + 1, (step + 1) & 1);
+    __syncthreads();
   }
 
-  for (int b = bbeg; b < bend; ++b) {
-    const double* A = g.A + (int64_t)b * g.strideA;
-    const double* B = g.B + (int64_t)b * g.strideB;
-    const double alpha = g.alpha[b];
-    for (int k0 = kbeg; k0 < kend; k0 += BK) {
-      for (int e = tid; e < BM * BK; e += NT) {
-        int i, kk;
-        if (!g.transA) { i = e % BM; kk = e / BM; } else { kk = e % BK; i = e / BK; }
-        const int gi = m0 + i, gk = k0 + kk;
-        double v = 0.0;
-        if (gi < g.M && gk < g.K)
-          v = g.transA ? A[gk + (int64_t)gi * g.lda] : A[gi + (int64_t)gk * g.lda];
-        As[kk][i] = alpha * v;
-      }
-      for (int e = tid; e < BK * BN; e += NT) {
-        int kk, j;
-        if (!g.transB) { kk = e % BK; j = e / BK; } else { j = e % BN; kk = e / BN; }
-        const int gk = k0 + kk, gj = n0 + j;
-        double v = 0.0;
-        if (gk < g.K && gj < g.N)
-          v = g.transB ? B[gj + (int64_t)gk * g.ldb] : B[gk + (int64_t)gj * g.ldb];
-        Bs[kk][j] = v;
-      }
-      __syncthreads();
+  double* C = g.Cout + (int64_t)zo * g.strideCout + zi * g.innerC;
+  const double* Cin = g.Cin ? g.Cin + (int64_t)zo * g.strideCin + zi * g.innerC : nullptr;
+  const bool use_in = Cin != nullptr && g.beta != 0.0;
+  const bool minus = unit && g.alpha[zo] < 0.0;
+  auto put = [&](int i, int j, double v) {
+    const int gi = m0 + i, gj = n0 + j;
+    if (gi >= g.M || gj >= g.N) return;
+    if (minus) v = -v;
+    if (use_in) v = fma(g.beta, Cin[gi + (int64_t)gj * g.ldcin], v);
+    C[gi + (int64_t)gj * g.ldcout] = v;
+  };
+  if (ks == 1) {
 #pragma unroll
-      for (int kk = 0; kk < BK; ++kk) {
-        double a[TM], bv[TN];
+    for (int j = 0; j < TN; ++j)
 #pragma unroll
-        for (int i = 0; i < TM; ++i) a[i] = As[kk][tr + i * RT];
-#pragma unroll
-        for (int j = 0; j < TN; ++j) bv[j] = Bs[kk][tc + j * CT];
-#pragma unroll
-        for (int i = 0; i < TM; ++i)
-#pragma unroll
-          for (int j = 0; j < TN; ++j) acc[i][j] = fma(a[i], bv[j], acc[i][j]);
-      }
-      __syncthreads();
-    }
-  }
-
-  const int z = g.reduce ? 0 : zb;
-  if (ksplit > 1) {
-    const int nz = g.reduce ? 1 : g.batch;
-    double* Pz = P + ((int64_t)zs * nz + z) * (int64_t)g.M * g.N;
-#pragma unroll
-    for (int j = 0; j < TN; ++j) {
-      const int gj = n0 + tc + j * CT;
-      if (gj >= g.N) continue;
-#pragma unroll
-      for (int i = 0; i < TM; ++i) {
-        const int gi = m0 + tr + i * RT;
-        if (gi < g.M) Pz[gi + (int64_t)gj * g.M] = acc[i][j];
-      }
-    }
+      for (int i = 0; i < TM; ++i) put(tr + i * RT, tc + j * CT, acc[i][j]);
     return;
   }
-  double* C = g.Cout + (int64_t)z * g.strideCout;
-  const double* Cin = g.Cin ? g.Cin + (int64_t)z * g.strideCin : nullptr;
-  const bool use_in = Cin != nullptr && g.beta != 0.0;
+  // every rank has read its operands before any rank writes C (the barrier), so
+  // a product whose one row tile covers M may be formed in place
+  namespace cgrp = cooperative_groups;
+  cgrp::cluster_group cluster = cgrp::this_cluster();
 #pragma unroll
-  for (int j = 0; j < TN; ++j) {
-    const int gj = n0 + tc + j * CT;
-    if (gj >= g.N) continue;
+  for (int j = 0; j < TN; ++j)
 #pragma unroll
-    for (int i = 0; i < TM; ++i) {
-      const int gi = m0 + tr + i * RT;
-      if (gi >= g.M) continue;
-      double v = acc[i][j];
-      if (use_in) v = fma(g.beta, Cin[gi + (int64_t)gj * g.ldcin], v);
-      C[gi + (int64_t)gj * g.ldcout] = v;
-    }
-  }
-}
-
-// C_z = sum_s P[s][z] (+ beta Cin_z), written only where the one-pass kernel with
-// BM x BN tiles writes (c_upper: tiles on or above the diagonal).
-template <int BM, int BN>
-__global__ void splitk_reduce_kernel(const GemmArgs g, int ksplit, const double* __restrict__ P) {
-  const int nz = g.reduce ? 1 : g.batch;
-  const int64_t mn = (int64_t)g.M * g.N;
-  const int z = blockIdx.y;
-  double* C = g.Cout + (int64_t)(g.reduce ? 0 : z) * g.strideCout;
-  const double* Cin = g.Cin ? g.Cin + (int64_t)(g.reduce ? 0 : z) * g.strideCin : nullptr;
-  const bool use_in = Cin != nullptr && g.beta != 0.0;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < mn;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = e % g.M, j = e / g.M;
-    if (g.c_upper && (i / BM) * BM > (j / BN) * BN + BN - 1) continue;
+    for (int i = 0; i < TM; ++i) sm[(tr + i * RT) + (tc + j * CT) * BM] = acc[i][j];
+  cluster.sync();
+  const int share = BM * BN / ks;
+  for (int e = rank * share + tid; e < (rank + 1) * share; e += NT) {
     double v = 0.0;
-    for (int s = 0; s < ksplit; ++s) v += P[((int64_t)s * nz + z) * mn + e];
-    if (use_in) v = fma(g.beta, Cin[i + j * g.ldcin], v);
-    C[i + j * g.ldcout] = v;
+    for (int q = 0; q < ks; ++q) v += cluster.map_shared_rank(sm, q)[e];
+    put(e % BM, e / BM, v);
   }
+  cluster.sync();   // no rank leaves while another reads its partial tile
 }
 
 __global__ void gemm_beta_only(const GemmArgs g) {
@@ -154,27 +190,31 @@ __global__ void gemm_beta_only(const GemmArgs g) {
   C[i + j * g.ldcout] = (Cin && g.beta != 0.0) ? g.beta * Cin[i + j * g.ldcin] : 0.0;
 }
 
-template <int BM, int BN>
-cudaError_t launch(const GemmArgs& g, int ksplit, double* P, cudaStream_t st) {
-  const int nz = g.reduce ? 1 : g.batch;
-  dim3 grid((g.N + BN - 1) / BN, (g.M + BM - 1) / BM, nz * ksplit);
+template <int BM, int BN, int TM, int TN>
+cudaError_t launch(const GemmArgs& g, int ks, cudaStream_t st) {
+  const int nz = g.reduce ? 1 : g.batch * g.inner;
+  constexpr int NT = (BM / TM) * (BN / TN);
+  dim3 grid((g.N + BN - 1) / BN * ks, (g.M + BM - 1) / BM, nz);
   const double bytes = 8.0 * g.batch * ((double)g.M * g.K + (double)g.K * g.N) +
                        8.0 * nz * (double)g.M * g.N * (g.beta != 0.0 ? 2 : 1);
-  {
-    ProfScope ps(kProfGemm, st, gemm_flops(g), bytes);
-    ps.blocks((const void*)gemm_f64_kernel<BM, BN, 16, 4, 4>, dim3((BM / 4) * (BN / 4)), 0,
-              dim3(grid));
-    gemm_f64_kernel<BM, BN, 16, 4, 4><<<grid, (BM / 4) * (BN / 4), 0, st>>>(g, ksplit, P);
+  ProfScope ps(kProfGemm, st, gemm_flops(g), bytes);
+  ps.blocks((const void*)gemm_f64_kernel<BM, BN, TM, TN>, dim3(NT), 0, grid);
+  if (ks == 1) {
+    gemm_f64_kernel<BM, BN, TM, TN><<<grid, NT, 0, st>>>(g, 1);
+    return cudaGetLastError();
   }
-  if (ksplit > 1) {
-    if (cudaError_t e = cudaGetLastError()) return e;
-    const int64_t mn = (int64_t)g.M * g.N;
-    const unsigned bx = (unsigned)std::min<int64_t>((mn + 255) / 256, 2048);
-    ProfScope ps(kProfOther, st, 0.0, 8.0 * nz * mn * (ksplit + 1));
-    ps.blocks((const void*)splitk_reduce_kernel<BM, BN>, dim3(256), 0, dim3(bx, nz));
-    splitk_reduce_kernel<BM, BN><<<dim3(bx, nz), 256, 0, st>>>(g, ksplit, P);
-  }
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(NT);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = ks;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, gemm_f64_kernel<BM, BN, TM, TN>, g, ks);
 }
 
 }  // namespace
@@ -184,22 +224,74 @@ double gemm_flops(const GemmArgs& g) {
   double per = 2.0 * g.M * (double)g.N * g.K;
   if (g.c_upper) per = (double)g.K * g.N * (g.N + 1.0);
   else if (g.b_lower) per = 2.0 * g.M * ((double)g.N * g.K - 0.5 * (double)g.N * (g.N - 1.0));
-  return per * g.batch;
+  return per * g.batch * g.inner;
 }
 
-int gemm_f64_default_variant(const GemmArgs& g) {
-  return g.M <= 32 ? kGemmV32x128 : kGemmV64x64;
+int gemm_f64_default_variant(const GemmArgs&) { return kGemmVRule; }
+
+// The tile and K split the rule takes: the least estimated time, in clocks, of
+//   c (BM BN K / ks) / 2 / eff(c) + a cluster's fixed cost,   c = ceil(CTAs / SMs)
+// (2 DFMA per clock per SM; the c CTAs that share an SM share its FP64 units, so a
+// wave that is not full costs as much as a full one, and a single small CTA leaves
+// them waiting at its barriers).  Measured at 2.0 GHz: 1024^3 takes 2.09 / 1.88 /
+// 1.88 ms with one 64 / 32 / 16 tile per CTA (c = 2 / 7 / 27); 256^3 takes 271 / 88
+// / 44 us unsplit and 39 us as 16 x 16 tiles cut in four; 32 x 96 x 8224 in a batch
+// of six takes 980 / 494 / 338 / 297 us as 16 x 16 tiles cut in 1 / 2 / 4 / 8 (c = 1
+// / 1 / 2 / 4); 144 CTAs in clusters of eight found two to an SM.
+F64Tile gemm_f64_rule(const GemmArgs& g) {
+  struct Cand { int id, bm, bn; double eff[4]; };   // eff at c = 1, 2, 3, >= 4
+  static const Cand all[] = {{0, 64, 64, {0.95, 0.99, 1.0, 1.0}},
+                             {1, 32, 32, {0.73, 0.92, 0.96, 0.98}},
+                             {2, 16, 16, {0.54, 0.78, 0.86, 0.93}}};
+  static const Cand inplace[] = {{3, 64, 16, {0.73, 0.92, 0.96, 0.97}},
+                                 {0, 64, 64, {0.95, 0.99, 1.0, 1.0}}};
+  // C over A or B: only tiles that hold all of a column's rows (M <= 64)
+  const bool alias = gemm_output_aliases_input(g);
+  const Cand* c = alias ? inplace : all;
+  const int nc = alias ? 2 : 3;
+  F64Tile best{0, 1};
+  // with many lanes in flight (the split forms' batch) large clusters wait for
+  // room: 48 matrices take 201.5 / 199.2 / 197.2 / 198.1 ms with up to 8 / 4 / 2 / 1
+  const bool crowded = get_split_engine() && get_split_engine()->throughput;
+  const int ks_max = g.b_lower || crowded ? 2 : 8;
+  double best_t = 1e300;
+  for (int q = 0; q < nc; ++q) {
+    const double tm = (g.M + c[q].bm - 1) / c[q].bm, tn = (g.N + c[q].bn - 1) / c[q].bn;
+    if (tm > 65535.0) continue;   // grid.y
+    double tiles = tm * tn * (g.reduce ? 1 : g.batch * g.inner);
+    if (g.c_upper) tiles *= 0.5 * (1.0 + 1.0 / tn);
+    const double kfrac = g.b_lower ? 0.5 * (1.0 + (double)c[q].bn / std::max(g.K, c[q].bn)) : 1.0;
+    for (int ks = 1; ks <= ks_max; ks *= 2) {
+      if (ks > 1 && g.K < 2 * kBK * ks) break;
+      const double kc = ((g.K + ks - 1) / ks + kBK - 1) / kBK * kBK;
+      const double cta = 0.5 * c[q].bm * c[q].bn * kc * (g.reduce ? g.batch : 1);
+      double per_sm = std::ceil(tiles * ks / 152.0);
+      if (ks == 8 && tiles * ks > 128.0) per_sm = std::max(per_sm, 2.0);
+      const double eff = c[q].eff[per_sm > 4.0 ? 3 : (int)per_sm - 1];
+      // triangular op(B): the CTAs' lengths differ, so an SM that holds few of them
+      // ends with the longest one alone, and K slices are uneven (1024^3, r = 6
+      // reduced: 8.98 / 7.11 / 5.70 ms with 64 / 32 / 16 tiles, 8.45 as 16 cut in two)
+      const double uneven = g.b_lower ? (1.0 + 2.0 / per_sm) * (ks > 1 ? 1.5 : 1.0) : 1.0;
+      const double t = std::max(per_sm * kfrac, 1.0) * cta * uneven / eff + (ks > 1 ? 3000.0 + 300.0 * ks : 0.0);
+      if (t < best_t) {
+        best_t = t;
+        best = {c[q].id, ks};
+      }
+    }
+  }
+  return best;
 }
 
-size_t gemm_f64_scratch_elems(const GemmArgs& g, int variant) {
-  const int ks = variant == kGemmVSplitK2 ? 2 : variant == kGemmVSplitK4 ? 4 :
-                 variant == kGemmVSplitK8 ? 8 : 1;
-  if (ks == 1) return 0;
-  return (size_t)ks * (g.reduce ? 1 : g.batch) * (size_t)g.M * (size_t)g.N;
+cudaError_t gemm_f64_tile(const GemmArgs& g, F64Tile t, cudaStream_t st) {
+  switch (t.tile) {
+    case 1: return launch<32, 32, 4, 2>(g, t.ks, st);
+    case 2: return launch<16, 16, 1, 2>(g, t.ks, st);
+    case 3: return launch<64, 16, 4, 2>(g, t.ks, st);
+    default: return launch<64, 64, 4, 4>(g, t.ks, st);
+  }
 }
 
-cudaError_t gemm_f64_variant(const GemmArgs& g, int variant, double* scratch,
-                             size_t scratch_elems, cudaStream_t st) {
+cudaError_t gemm_f64_variant(const GemmArgs& g, int variant, cudaStream_t st) {
   if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return cudaSuccess;
   if (g.batch > kGemmMaxBatch) return cudaErrorInvalidValue;
   if (g.K <= 0) {
@@ -211,15 +303,13 @@ cudaError_t gemm_f64_variant(const GemmArgs& g, int variant, double* scratch,
     gemm_beta_only<<<grid, 256, 0, st>>>(g);
     return cudaGetLastError();
   }
-  const size_t need = gemm_f64_scratch_elems(g, variant);
-  if (need > 0 && (scratch == nullptr || need > scratch_elems)) variant = kGemmV64x64;
   switch (variant) {
-    case kGemmV32x128: return launch<32, 128>(g, 1, nullptr, st);
-    case kGemmV32x64: return launch<32, 64>(g, 1, nullptr, st);
-    case kGemmVSplitK2: return launch<64, 64>(g, 2, scratch, st);
-    case kGemmVSplitK4: return launch<64, 64>(g, 4, scratch, st);
-    case kGemmVSplitK8: return launch<64, 64>(g, 8, scratch, st);
-    default: return launch<64, 64>(g, 1, nullptr, st);
+    case kGemmV32x128: return launch<32, 128, 4, 4>(g, 1, st);
+    case kGemmV32x64: return launch<32, 64, 4, 4>(g, 1, st);
+    case kGemmVSplitK2: return launch<64, 64, 4, 4>(g, 2, st);
+    case kGemmVSplitK4: return launch<64, 64, 4, 4>(g, 4, st);
+    case kGemmVSplitK8: return launch<64, 64, 4, 4>(g, 8, st);
+    default: return gemm_f64_tile(g, gemm_f64_rule(g), st);
   }
 }
 

@@ -4,13 +4,13 @@
 // Gram matrices, the triangular-solve updates, the eigensolver's products) goes
 // through gemm_any (FP64 or split tensor-core path) or gemm_f64 (FP64 only).
 // Without a tuner both follow fixed rules: the split path where its cost model
-// says it is faster, else the 64 x 64 FP64 tile (32 x 128 for M <= 32).  With
-// a handle's tuner current and tuning on, the first call of a shape runs every
-// candidate (three FP64 tile shapes, split-K in 2 / 4 / 8 slices when K holds
-// at least two 16-deep steps per slice, and the split path when it is on) into
-// a scratch output, times each with CUDA events on the call's stream, keeps
-// the fastest in the handle's cache, and then runs it for real.  The real
-// output is written once, by the chosen variant.
+// says it is faster, else the FP64 tile and K split of gemm_f64_rule.  With a
+// handle's tuner current and tuning on, the first call of a shape runs every
+// candidate (the rule's choice, two wide tiles, 64 x 64 tiles with K split in 2 /
+// 4 / 8 when K holds at least two 16-deep steps per slice, and the split path
+// when it is on) into a scratch output, times each with CUDA events on the call's
+// stream, keeps the fastest in the handle's cache, and then runs it for real.
+// The real output is written once, by the chosen variant.
 #include <algorithm>
 #include <cfloat>
 #include <vector>
@@ -36,8 +36,9 @@ struct Extent {
   const double* lo;
   const double* hi;
 };
-Extent extent(const double* p, int64_t ld, int64_t rows, int64_t cols, int64_t stride, int count) {
-  return {p, p + (int64_t)(count - 1) * stride + (cols - 1) * ld + rows};
+Extent extent(const double* p, int64_t ld, int64_t rows, int64_t cols, int64_t stride, int count,
+              int64_t inner_stride, int inner) {
+  return {p, p + (int64_t)(count - 1) * stride + (inner - 1) * inner_stride + (cols - 1) * ld + rows};
 }
 bool overlap(Extent a, Extent b) { return a.lo < b.hi && b.lo < a.hi; }
 
@@ -45,13 +46,12 @@ int ksplit_of(int v) {
   return v == kGemmVSplitK2 ? 2 : v == kGemmVSplitK4 ? 4 : v == kGemmVSplitK8 ? 8 : 1;
 }
 
-cudaError_t run_variant(const GemmArgs& g, int v, SplitWork* split, double* scratch,
-                        size_t scratch_elems, cudaStream_t st) {
+cudaError_t run_variant(const GemmArgs& g, int v, SplitWork* split, cudaStream_t st) {
   if (v == kGemmVSplit) {
     if (split) return gemm_split(g, *split, st);
     v = gemm_f64_default_variant(g);
   }
-  return gemm_f64_variant(g, v, scratch, scratch_elems, st);
+  return gemm_f64_variant(g, v, st);
 }
 
 bool ensure_scratch(GemmTuner& t, size_t elems, cudaStream_t st) {
@@ -78,8 +78,8 @@ bool ensure_scratch(GemmTuner& t, size_t elems, cudaStream_t st) {
 // written for, and the variants that read all of A and B before writing C
 // (split-K, split).
 int tune(GemmTuner& t, const GemmArgs& g, SplitWork* split, cudaStream_t st) {
-  const size_t out = (size_t)(g.reduce ? 1 : g.batch) * (size_t)g.M * (size_t)g.N;
-  std::vector<int> cand = {kGemmV64x64, kGemmV32x128, kGemmV32x64};
+  const size_t out = (size_t)(g.reduce ? 1 : g.batch * g.inner) * (size_t)g.M * (size_t)g.N;
+  std::vector<int> cand = {kGemmVRule, kGemmV32x128, kGemmV32x64};
   if (gemm_output_aliases_input(g)) cand = {gemm_f64_default_variant(g)};
   for (int v : {kGemmVSplitK2, kGemmVSplitK4, kGemmVSplitK8})
     if (g.K >= 2 * 16 * ksplit_of(v)) cand.push_back(v);
@@ -90,23 +90,14 @@ int tune(GemmTuner& t, const GemmArgs& g, SplitWork* split, cudaStream_t st) {
     if (ratio < 0.25) return kGemmVSplit;
     if (ratio <= 4.0) cand.push_back(kGemmVSplit);
   }
-  size_t part = 0;
-  for (int v : cand) part = std::max(part, gemm_f64_scratch_elems(g, v));
-  if (!ensure_scratch(t, out + part, st)) {
-    // without split-K partials, if at least the output fits
-    cand.erase(std::remove_if(cand.begin(), cand.end(),
-                              [&](int v) { return gemm_f64_scratch_elems(g, v) > 0; }),
-               cand.end());
-    part = 0;
-    if (!ensure_scratch(t, out, st)) return -1;
-  }
+  if (!ensure_scratch(t, out, st)) return -1;
   if (!t.t0 && (cudaEventCreate(&t.t0) != cudaSuccess || cudaEventCreate(&t.t1) != cudaSuccess))
     return -1;
   GemmArgs h = g;   // same inputs (Cin is only read), output to the scratch
   h.Cout = t.scratch;
   h.ldcout = g.M;
-  h.strideCout = (int64_t)g.M * g.N;
-  double* partials = t.scratch + out;
+  h.innerC = (int64_t)g.M * g.N;
+  h.strideCout = h.innerC * g.inner;
   // the built-in choice first: a shape that takes it over 50 ms keeps it (large
   // products already fill the GPU, and timing every candidate there would cost
   // seconds per shape)
@@ -119,7 +110,7 @@ int tune(GemmTuner& t, const GemmArgs& g, SplitWork* split, cudaStream_t st) {
     float ms = FLT_MAX;
     for (int rep = 0; rep < 3; ++rep) {
       if (cudaEventRecord(t.t0, st) != cudaSuccess) return -1;
-      if (run_variant(h, v, split, partials, part, st) != cudaSuccess) return -1;
+      if (run_variant(h, v, split, st) != cudaSuccess) return -1;
       float x = 0.f;
       if (cudaEventRecord(t.t1, st) != cudaSuccess || cudaEventSynchronize(t.t1) != cudaSuccess ||
           cudaEventElapsedTime(&x, t.t0, t.t1) != cudaSuccess)
@@ -150,13 +141,7 @@ int choose(const GemmArgs& g, SplitWork* split_engine, cudaStream_t st) {
     // FP8 211)
     const auto key = gemm_key(g, split ? split->slices_s + 100 * split->form : 0);
     const auto hit = t->choice.find(key);
-    if (hit != t->choice.end() && gemm_variant_allowed(key, hit->second)) {
-      // a split-K choice (e.g. loaded from a file) needs its partial sums' scratch
-      const size_t need = gemm_f64_scratch_elems(g, hit->second);
-      if (need <= t->scratch_elems || (!stream_capturing(st) && ensure_scratch(*t, need, st)))
-        return hit->second;
-      return gemm_f64_default_variant(g);
-    }
+    if (hit != t->choice.end() && gemm_variant_allowed(key, hit->second)) return hit->second;
     if (t->tuning && !stream_capturing(st)) {
       t->busy = true;
       const int v = tune(*t, g, split, st);
@@ -182,11 +167,12 @@ GemmTuner::~GemmTuner() {
 }
 
 bool gemm_output_aliases_input(const GemmArgs& g) {
-  const Extent c = extent(g.Cout, g.ldcout, g.M, g.N, g.strideCout, g.reduce ? 1 : g.batch);
+  const Extent c = extent(g.Cout, g.ldcout, g.M, g.N, g.strideCout, g.reduce ? 1 : g.batch,
+                          g.innerC, g.inner);
   const Extent a = extent(g.A, g.lda, g.transA ? g.K : g.M, g.transA ? g.M : g.K, g.strideA,
-                          g.batch);
+                          g.batch, g.innerA, g.inner);
   const Extent b = extent(g.B, g.ldb, g.transB ? g.N : g.K, g.transB ? g.K : g.N, g.strideB,
-                          g.batch);
+                          g.batch, g.innerB, g.inner);
   return overlap(c, a) || overlap(c, b);
 }
 
@@ -200,12 +186,12 @@ std::array<int, 7> gemm_key(const GemmArgs& g, int split_slices) {
 
 bool gemm_variant_allowed(const std::array<int, 7>& key, int v) {
   const bool split_k = v == kGemmVSplitK2 || v == kGemmVSplitK4 || v == kGemmVSplitK8;
-  const bool tiles = v == kGemmV64x64 || v == kGemmV32x128 || v == kGemmV32x64;
+  const bool tiles = v == kGemmVRule || v == kGemmV32x128 || v == kGemmV32x64;
   if (v == kGemmVSplit) return key[5] != 0;
   if (!split_k && !tiles) return false;
   if (!(key[4] & 128) || split_k) return true;
-  // in place: only the built-in tile for this M
-  return v == (key[0] <= 32 ? kGemmV32x128 : kGemmV64x64);
+  // in place: only the built-in rule (which then takes a tile of 64 rows)
+  return v == kGemmVRule || (key[0] <= 32 && v == kGemmV32x128);
 }
 
 void set_gemm_tuner(GemmTuner* t) { t_tuner = t; }
@@ -213,19 +199,15 @@ GemmTuner* get_gemm_tuner() { return t_tuner; }
 
 cudaError_t gemm_f64(const GemmArgs& g, cudaStream_t st) {
   if (g.M <= 0 || g.N <= 0 || g.K <= 0 || g.batch <= 0 || g.batch > kGemmMaxBatch)
-    return gemm_f64_variant(g, kGemmV64x64, nullptr, 0, st);
-  const int v = choose(g, nullptr, st);
-  GemmTuner* t = t_tuner;
-  return gemm_f64_variant(g, v, t ? t->scratch : nullptr, t ? t->scratch_elems : 0, st);
+    return gemm_f64_variant(g, kGemmVRule, st);
+  return gemm_f64_variant(g, choose(g, nullptr, st), st);
 }
 
 cudaError_t gemm_any(const GemmArgs& g, cudaStream_t st) {
   SplitWork* split = get_split_engine();
   if (!split || g.M <= 0 || g.N <= 0 || g.K <= 0 || g.batch > kGemmMaxBatch)
     return gemm_f64(g, st);
-  const int v = choose(g, split, st);
-  GemmTuner* t = t_tuner;
-  return run_variant(g, v, split, t ? t->scratch : nullptr, t ? t->scratch_elems : 0, st);
+  return run_variant(g, choose(g, split, st), split, st);
 }
 
 }  // namespace zolo

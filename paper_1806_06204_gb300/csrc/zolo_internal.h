@@ -104,6 +104,10 @@ struct GemmArgs {
   double beta = 0.0;
   double alpha[kGemmMaxBatch] = {};
   int batch = 1;
+  // FP64 path only (not with reduce): each batch entry is `inner` products, the
+  // inner ones at these strides (batch x inner output planes, alpha per entry)
+  int inner = 1;
+  int64_t innerA = 0, innerB = 0, innerC = 0;
   int reduce = 0;
   int b_lower = 0;
   int c_upper = 0;
@@ -114,21 +118,25 @@ struct GemmArgs {
   // the small rows their precision.
   int k_equilibrate = 0;
 };
-// Kernel variants of the FP64 contraction: output tile shape, and split-K
-// (K cut into 2 / 4 / 8 slices of whole BK steps whose raw sums go to a scratch
-// of ksplit * (reduce ? 1 : batch) * M * N doubles, then one deterministic
-// reduction kernel).  kGemmVSplit names the split tensor-core path.
+// Kernel variants of the FP64 contraction: the built-in rule (gemm_f64_rule picks
+// the tile and the K split per shape), or one tile shape, or 64 x 64 tiles with
+// K cut into 2 / 4 / 8 slices of whole steps over a thread-block cluster.
+// kGemmVSplit names the split tensor-core path.
 enum GemmVariant {
-  kGemmV64x64 = 0, kGemmV32x128 = 1, kGemmV32x64 = 2,
+  kGemmVRule = 0, kGemmV32x128 = 1, kGemmV32x64 = 2,
   kGemmVSplitK2 = 3, kGemmVSplitK4 = 4, kGemmVSplitK8 = 5,
   kGemmVSplit = 8
 };
-// one FP64 launch of the given variant (a split-K variant without enough
-// scratch runs as kGemmV64x64)
-cudaError_t gemm_f64_variant(const GemmArgs& g, int variant, double* scratch,
-                             size_t scratch_elems, cudaStream_t st);
-size_t gemm_f64_scratch_elems(const GemmArgs& g, int variant);
+// one FP64 launch of the given variant
+cudaError_t gemm_f64_variant(const GemmArgs& g, int variant, cudaStream_t st);
 int gemm_f64_default_variant(const GemmArgs& g);
+// the rule's choice: tile 0 = 64 x 64, 1 = 32 x 32, 2 = 16 x 16, 3 = 64 x 16; ks CTAs
+// of one cluster share the tile's K
+struct F64Tile {
+  int tile, ks;
+};
+F64Tile gemm_f64_rule(const GemmArgs& g);
+cudaError_t gemm_f64_tile(const GemmArgs& g, F64Tile t, cudaStream_t st);
 // FP64 contraction: the variant the current thread's tuner chose for this
 // shape, else the default one.
 cudaError_t gemm_f64(const GemmArgs& g, cudaStream_t st);
@@ -273,12 +281,9 @@ struct QrBuffers {
   double* T;   int64_t strideT;   // nb x nb triangular factor per panel
   double* Tb;  int64_t strideTb;  // NBb x NBb triangular factor per block
   double* G;   int64_t strideG;   // NBb x NBb Gram V_b^T V_b scratch
-  double* P;   int64_t elemsP;    // split-K partial products of the skinny products
   double* W1;  int64_t strideW1;  // NBb x n scratch
   double* W2;  int64_t strideW2;  // NBb x n scratch
 };
-// Doubles of QrBuffers::P for an m-row problem with r shifts.
-int64_t qr_partial_elems(int64_t m, int r);
 // Factor [X; sqrt(c_j) I] for j < r and overwrite W_j with the thin Q_j
 // (explicit_q = false: leave R on and above the diagonal of W_j's top block).
 // narrow_panels: many problems are in flight on other streams; the panel kernel
