@@ -334,17 +334,17 @@ def run_reference(args, w, rank):
 # Builder's DFMA microbenchmark on this GPU (a register-resident FMA chain on all
 # SMs, CUDA events): the FP64 pipe's measured ceiling beside the derived peak.
 FP64_DFMA_MEASURED_TFLOPS = 1.20
-# Tensor-core products issued per FP64-equivalent flop on the split path: nine
-# BF16 slices per operand, slice pairs (s, t) with s + t <= 11: 53; eight FP16
-# slices, s + t <= 9: 36; eleven FP8 (E4M3) slices, s + t <= 13: 76.  The FP8
-# products run at twice the 16-bit rate (nominal 4.5 against 2.25 PFLOP/s), so
-# their peak is the measured BF16 peak times 2.
-SPLIT_PAIRS = 53
-SPLIT_PAIRS_OF = {"bf16": 53, "fp16": 36, "fp8": 76}
+# Tensor-core products issued per FP64-equivalent flop on the split path: seven
+# 8-bit BF16 slices per operand, slice pairs (s, t) with s + t <= 9: 34; seven
+# 8-bit FP16 slices, s + t <= 8: 28; eleven 5-bit FP8 (E4M3) slices, s + t <= 13:
+# 76.  The FP8 products run at twice the 16-bit rate (nominal 4.5 against 2.25
+# PFLOP/s), so their peak is the measured BF16 peak times 2.
+SPLIT_PAIRS_OF = {"bf16": 34, "fp16": 28, "fp8": 76}
+SPLIT_PAIRS = 53   # roofline()'s default: nine six-bit slices
 SLICE_PEAK_RATIO = {"bf16": 1.0, "fp16": 1.0, "fp8": 2.0}
-SLICE_DTYPE = {"bf16": "bf16x9-slices->f64", "fp16": "fp16x8-slices->f64",
+SLICE_DTYPE = {"bf16": "bf16x7-slices->f64", "fp16": "fp16x7-slices->f64",
                "fp8": "e4m3x11-slices->f64"}
-SLICE_DESC = {"bf16": "nine BF16 slices", "fp16": "eight FP16 slices",
+SLICE_DESC = {"bf16": "seven 8-bit BF16 slices", "fp16": "seven 8-bit FP16 slices",
               "fp8": "eleven FP8 (E4M3) slices"}
 
 
@@ -696,8 +696,8 @@ def main():
                          "both (batch only): split timed, FP64 beside it; auto: both for the "
                          "batch, fp64 otherwise")
     ap.add_argument("--slices", default="bf16", choices=sorted(SLICE_DTYPE),
-                    help="split precision's slices: nine BF16 six-bit slices (53 slice-pair "
-                         "products), eight FP16 seven-bit slices (36) or eleven FP8 "
+                    help="split precision's slices: seven BF16 8-bit slices (34 slice-pair "
+                         "products), seven FP16 8-bit slices (28) or eleven FP8 "
                          "five-bit slices (76 at twice the rate)")
     ap.add_argument("--no-graph", action="store_true",
                     help="batch workload: queue the lanes directly every step instead of replaying "

@@ -51,17 +51,17 @@ enum {
 
 /* Arithmetic of the contractions.  ZOLO_FP64: plain FP64 on the FP64 FMA pipe.
    ZOLO_SPLIT_BF16: the iterations' products on the BF16 tensor cores, each FP64
-   operand cut into 9 power-of-two-scaled 6-bit slices (Ozaki scheme, product
-   error a few times sqrt(k) 2^-54 of max|row| max|column|); panel
-   factorisations, diagonal blocks and coefficients stay FP64.
-   ZOLO_SPLIT_FP16: the same on the FP16 tensor cores with 8 slices of 7-bit
-   integer digits and 36 slice-pair products instead of 53 (the same error
-   grade).
+   operand cut into power-of-two-scaled slices of integer digits (Ozaki scheme,
+   product error a few times sqrt(k) 2^-54 of max|row| max|column|): 7 slices of 8
+   bits, which hold what 9 six-bit ones would and more, 34 slice-pair products;
+   panel factorisations, diagonal blocks and coefficients stay FP64.
+   ZOLO_SPLIT_FP16: the same on the FP16 tensor cores with 28 slice-pair products
+   (the same error grade).
    ZOLO_SPLIT_FP8: the same on the FP8 (E4M3) tensor cores with 11 slices of
    5-bit integer digits and 76 slice-pair products at twice the BF16 rate
    (the same error grade).  A product whose inner dimension is longer than
-   the int64 of its exact level sums can hold at the digit bounds (114688 for
-   BF16 and FP8, 61440 for FP16) runs as consecutive products added in FP64. */
+   the int64 of its exact level sums can hold at the digit bounds (114688) runs
+   as consecutive products added in FP64. */
 enum { ZOLO_FP64 = 0, ZOLO_SPLIT_BF16 = 1, ZOLO_SPLIT_FP16 = 2, ZOLO_SPLIT_FP8 = 3 };
 
 typedef struct {
@@ -285,9 +285,10 @@ int zolo_svd_host(zolo_handle_t handle, const double* A, int64_t m, int64_t n, i
 /* C = alpha op(A) op(B) + beta C for device FP64 matrices (column-major,
    op = identity or transpose: trans = 0 / 1), the contraction the iterations
    run on.  prec = ZOLO_FP64 (DFMA), ZOLO_SPLIT_BF16 with `slices` = 8 or 9
-   (0 = 8) six-bit slices per operand on the tensor cores, ZOLO_SPLIT_FP16
-   (`slices` 0 or 8: eight seven-bit slices) or ZOLO_SPLIT_FP8 (`slices` 0 or
-   11: eleven five-bit slices).  On the split path an Inf or NaN in a row of
+   (0 = 8): the accuracy of that many six-bit slices per operand (held as six or
+   seven 8-bit ones) on the tensor cores, ZOLO_SPLIT_FP16 (`slices` 0 or 8: the
+   accuracy of eight seven-bit slices, held as seven 8-bit ones) or ZOLO_SPLIT_FP8
+   (`slices` 0 or 11: eleven five-bit slices).  On the split path an Inf or NaN in a row of
    op(A) or a column of op(B) makes that row or column of the product NaN.
    Not in the paper as
    an interface; it exposes the building block for testing and reuse.
@@ -335,8 +336,8 @@ int zolo_dgemm_noalloc(int transA, int transB, int64_t m, int64_t n, int64_t k, 
    contraction shape (M, N, K, batch, transposes, triangular-structure flags,
    slice count) for the first time runs it once with each candidate kernel
    (the built-in FP64 rule's tile and K split, FP64 tiles 32x128 and 32x64,
-   64x64 tiles with K split in 2, 4 or 8 over a thread-block cluster; the split tensor-core path when opts.prec asks for
-   it) into a scratch output, timed with CUDA events, and keeps the fastest
+   64x64 tiles with K split in 2, 4 or 8 over a thread-block cluster; the split
+   tensor-core path when opts.prec asks for it) into a scratch output, timed with CUDA events, and keeps the fastest
    for that shape; the call's own outputs are written once, by the kept
    kernel.  To bound the cost of measuring, a shape whose built-in kernel takes
    over 50 ms keeps it, and the split path (or FP64) is not timed where the

@@ -1,50 +1,37 @@
-// Split-precision FP64 GEMM on the BF16 tensor cores (tcgen05 + TMEM + TMA),
-// the Ozaki scheme: every FP64 operand row (of op(A)) / column (of op(B)) is
-// scaled by a power of two 2^e so that its entries lie in (-1/2, 1/2), rounded
-// to the fixed-point integer N = round(x 2^(6S - e)) and written in S balanced
-// base-64 digits,
-//     x 2^-e = sum_{s=1..S} d_s 2^{-6s} (+ rounding below 2^{-6S-1}),   |d_s| <= 32,
-// each stored pre-scaled (d_s 2^{-6s}) as BF16, which holds it exactly.  A
-// product is the sum over digit pairs (s, t) with s + t <= S + 2 of BF16 x BF16
-// GEMMs (53 for S = 9: the pairs at level S + 2 dominate the error of the ones
-// left out, so keeping them cuts it by about twenty).  Balanced digits make the dropped pairs and the rounding zero-mean
-// (truncated digits bias every term of a Gram diagonal the same way) and keep
-// |d_s d_t| <= 2^10, so a level (fixed s + t) of p pairs summed over k terms
-// stays below p k 2^10 units of its last place: exact in FP32 while that is
-// <= 2^24.  Levels 2..8 (p <= 7) therefore accumulate exactly in their own TMEM
-// accumulator over K-chunks of 2048; the levels >= 9 share one FP32
-// accumulator, whose rounding lies 2^-42 below the leading level.  After every
-// chunk the epilogue adds the exact levels to an int64 counting units of 2^-48
-// and the merged one to a float; at the end it joins them with one FMA and
-// applies 2^(e_i + f_j) through the exponent field, alpha and beta in FP64.
-// Accuracy: |C - AB| <~ 8 sqrt(K) 2^-6S max|A_i.| max|B_.j|, dominated by the
-// rounding of N against a row maximum in [1/4, 1/2) (S = 9: FP64 grade).
+// Split-precision FP64 GEMM on the tensor cores (tcgen05 + TMEM + TMA), the Ozaki
+// scheme: every FP64 operand row (of op(A)) / column (of op(B)) is scaled by a
+// power of two 2^e so that its entries lie in (-1/2, 1/2), rounded to the
+// fixed-point integer N = round(x 2^(bS - e)) and written in S balanced base-2^b
+// digits,
+//     x 2^-e = sum_{s=1..S} d_s 2^{-bs} (+ rounding below 2^{-bS-1}),
+//     |d_s| <= 2^(b-1),
+// each stored as the integer it is, which the slice type holds exactly (BF16 up
+// to 256, FP16 up to 2048, E4M3 up to 16).  A product is the sum over digit pairs
+// (s, t) with s + t <= top of tensor-core GEMMs, one TMEM accumulator per level
+// s + t, whose sums of integers are exact in FP32 while p k 2^(2b-2) <= 2^24 (p
+// pairs in the level, k terms).  Balanced digits make the dropped pairs and the
+// rounding zero-mean (truncated digits bias every term of a Gram diagonal the
+// same way).
 //
-// FP16 form: FP16 has three more significand bits than BF16 but
-// cannot hold a digit pre-scaled by 2^-7s (its range ends at 2^-24), so its
-// slices are the raw balanced base-128 digits, |d_s| <= 64 (exact in FP16).
-// S = 8 slices (56 bits) and the pairs with s + t <= S + 1 = 9: 36 slice-pair
-// products instead of 53.  Every level L = 2..9 keeps its own accumulator of
-// raw integer products, |d_s d_t| <= 2^12, exact in FP32 over K-chunks of 512
-// (8 pairs x 512 x 2^12 = 2^24); the epilogue adds levels 2..7 to an int64 of
-// 2^-49 units (shifted by 49 - 7L) and levels 8 and 9 to one float in 2^-56
-// units, joined as iacc + f 2^-7 before the scale 2^(e_i + f_j - 49).  The
-// error is the BF16 form's (CPU model: 1.43e-15 against 1.40e-15 of the row and
-// column maxima on the same operands).
+//   BF16 form  b = 8, S = 7 (56 bits), levels 2..9: 34 pairs (zolo_dgemm's
+//              slices = 9); S = 6 (48 bits), levels 2..8: 26 pairs (slices = 8)
+//   FP16 form  b = 8, S = 7, levels 2..8: 28 pairs
+//   FP8 form   b = 5, S = 11 (55 bits), levels 2..13: 76 pairs at the doubled rate
 //
-// FP8 form (E4M3, tcgen05 kind::f8f6f4): E4M3 holds every integer |d| <= 16
-// exactly but nothing pre-scaled below 2^-9, so its slices are raw balanced
-// base-32 digits, |d_s| <= 16: S = 11 slices (55 bits) and the pairs with
-// s + t <= S + 2 = 13 (76 slice pairs, 38 16-bit-product equivalents at FP8's
-// doubled rate; dropping level 13 would multiply the error by five).
-// |d_s d_t| <= 2^8, so a level of p <= 11 pairs stays exact in FP32 over
-// K-chunks of 4096.  Each of the 12 levels keeps its own accumulator of BN = 32
-// columns (384 of TMEM's 512); the epilogue adds levels 2..9 to an int64 of
-// 2^-48 units and levels 10..13 to one float in 2^-65 units, joined as
-// iacc + f 2^-17.  A K block is 128 one-byte elements, the same 128-byte
-// swizzled rows as the 16-bit forms, and one MMA takes K = 32 (32 bytes), so
-// the shared-memory layout and descriptors are the 16-bit forms' byte for byte.
-// The slice planes take 11 bytes per element against 18.
+// The leading levels (2..6 of the 8-bit digits, 2..9 of the 5-bit ones) are exact
+// over a K-chunk of 192 (4096) terms and are added to an int64 in units of 2^-48
+// after every chunk; the levels below go to one float (units of 2^-56 or 2^-65:
+// their FP32 rounding lies 2^-64 below the leading level).  At the end the two
+// are joined by one FP64 add, or in integers when one chunk held all of K, and
+// scaled by 2^(e_i + f_j) through the exponent field.  The digit width was
+// measured on the CPU against exact products (rms error over row and column
+// maxima, K = 512, N(0,1) / Gram / operands graded over eight decades): 34 pairs
+// of 8-bit digits 0.7 / 0.8 / 0.4 e-16, the 53 pairs of nine 6-bit digits they
+// replace 4.2 / 4.6 / 1.5 e-16; 28 pairs 4.2 / 4.6 / 4.1 e-16, the 36 pairs of
+// eight 7-bit digits they replace 4.7 / 8.1 / 4.5 e-16.  A K block of the FP8 form
+// is 128 one-byte elements, the same 128-byte swizzled rows as the 16-bit forms,
+// and one MMA takes K = 32 (32 bytes), so the shared-memory layout and
+// descriptors are the same byte for byte.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -57,37 +44,36 @@
 #include <algorithm>
 #include <mutex>
 
+#include <cooperative_groups.h>
+
 #include "tc_ptx.cuh"
 #include "zolo_internal.h"
 
 namespace zolo {
 namespace {
 
-constexpr int kBeta = 6;          // BF16 form: base-64 digits
 constexpr int kTileM = 128;
 constexpr int kRowBytes = 128;     // one 128-byte swizzle row of K per tile row
-// The slice forms: digit width, element bytes (K elements per 128-byte row),
-// exact-accumulation span of a level's sums, TMEM accumulators, tile width BN
-// and the largest 0-based level s + t kept (1-based S + 2 for BF16 and FP8,
-// S + 1 for FP16).  BF16: levels 2..8 exact, >= 9 merged in the last
-// accumulator; FP16 and FP8: one accumulator per level.
+// The slice forms: digit width, element bytes (K elements per 128-byte row), the
+// chunk of K whose leading level sums are exact, tile width BN, the last level
+// (1-based) that goes to the int64, and the largest 0-based s + t kept.
 template <int FORM> struct Form;
 template <> struct Form<kFormBF16> {
-  static constexpr int kBits = 6, kElem = 2, kChunkK = 2048, kAcc = 8, kBN = 64;
+  static constexpr int kBits = 8, kElem = 2, kChunkK = 192, kIntTop = 6, kFloatUnit = 56;
   __host__ __device__ static constexpr int top(int S) { return S; }
 };
 template <> struct Form<kFormFP16> {
-  static constexpr int kBits = 7, kElem = 2, kChunkK = 512, kAcc = 8, kBN = 64;
+  static constexpr int kBits = 8, kElem = 2, kChunkK = 192, kIntTop = 6, kFloatUnit = 56;
   __host__ __device__ static constexpr int top(int S) { return S - 1; }
 };
 template <> struct Form<kFormFP8> {
-  static constexpr int kBits = 5, kElem = 1, kChunkK = 4096, kAcc = 12, kBN = 32;
+  static constexpr int kBits = 5, kElem = 1, kChunkK = 4096, kBN = 32, kIntTop = 9, kFloatUnit = 65;
   __host__ __device__ static constexpr int top(int S) { return S; }
 };
 template <int FORM> __host__ __device__ constexpr int form_bk() { return kRowBytes / Form<FORM>::kElem; }
-constexpr int kARing = 4;
+constexpr int kARing = 7;
 constexpr int kFusedSliceK = 2048;  // slicing in one launch per product up to this padded K
-constexpr int kGroupM = 8;         // tile rows per CTA group (L2 reuse of the A slices)
+constexpr int kGroupM = 8;         // tile rows per group of tiles (L2 reuse of the A slices)
 constexpr int kEpiWarps = 16;      // four per TMEM lane quarter, each owning a quarter of the columns
 constexpr int kThreads = 64 + 32 * kEpiWarps;   // warp 0 TMA, warp 1 MMA, the rest epilogue
 
@@ -204,8 +190,8 @@ __global__ void col_exp_kernel(const double* __restrict__ X, int64_t ldx, int64_
 }
 
 // N = round(x 2^(bS - e)) from the bit pattern (|x| < 2^(e-1), so |N| <= 2^(bS-1));
-// ties round away from zero.  b = the digit width (6, or 7 for FP16).
-template <int S, int B = kBeta>
+// ties round away from zero.  b = the digit width.
+template <int S, int B>
 __device__ __forceinline__ long long fixed_point(double x, int e) {
   const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
   const unsigned long long mag = bits & 0x7FFFFFFFFFFFFFFFull;
@@ -220,25 +206,21 @@ __device__ __forceinline__ long long fixed_point(double x, int e) {
   return (bits >> 63) ? -(long long)F : (long long)F;
 }
 
-// The S slice values d_s 2^-6s of x against the row bound 2^(ee - 1): balanced
-// digits from the least significant one up; the leading digit takes what is
-// left, |d_1| <= 32 because |N| <= 2^(6S-1).  Each is exact in FP32 and BF16
-// (at most six significant bits).
+// The S digits of x against the row bound 2^(ee - 1), from the least significant
+// one up; the leading digit takes what is left, |d_1| <= 2^(b-1) because |N| <=
+// 2^(bS-1).  Each is exact in FP32 and in the slice type.
 template <int S, int FORM>
 __device__ __forceinline__ void slice_values(double x, int ee, float* v) {
   constexpr int B = Form<FORM>::kBits;
-  constexpr bool raw = FORM != kFormBF16;
   long long N = fixed_point<S, B>(x, ee);
 #pragma unroll
   for (int s = S; s >= 2; --s) {
     int d = (int)(N & ((1 << B) - 1));
     d = d >= (1 << (B - 1)) ? d - (1 << B) : d;
-    // BF16: the digit pre-scaled by 2^-Bs; FP16 and FP8: the raw digit (scaled
-    // in the epilogue)
-    v[s - 1] = raw ? (float)d : (float)d * __int_as_float((127 - B * s) << 23);
+    v[s - 1] = (float)d;
     N = (N - d) >> B;
   }
-  v[0] = raw ? (float)N : (float)N * __int_as_float((127 - B) << 23);
+  v[0] = (float)N;
 }
 
 // S slices of op(X), each rows_pad x K_pad elements of the form's type (BF16,
@@ -409,6 +391,18 @@ slice_fused_kernel(const SliceOp a, const SliceOp b, int nblk_a, int K, int K_pa
 // scarce ones on this part, and the epilogue of a product with a short K does
 // as much FP64 work per output as its MMAs do tensor work.
 
+// d 2^k for results outside the normal range: powers of two applied in steps that
+// are exact until the last one rounds (inline: a call to ldexp would have every
+// live register of the epilogue saved around it).
+__device__ __forceinline__ double scale_steps(double d, int k) {
+  for (int i = 0; i < 3 && k != 0; ++i) {
+    const int s = k < -1000 ? -1000 : (k > 1000 ? 1000 : k);
+    d *= __longlong_as_double((long long)(1023 + s) << 52);
+    k -= s;
+  }
+  return d;
+}
+
 // x 2^k for an int64 x, rounded to nearest (ties to even) like (double)x, then
 // scaled exactly: the leading one found by a count of leading zeros, 53 bits
 // kept, the exponent assembled; a result outside the normal range takes the
@@ -434,7 +428,7 @@ __device__ __forceinline__ double i64_scaled(long long x, int k) {
     }
   }
   const int be = msb + k + 1023;
-  if (be <= 0 || be >= 2047) return ldexp((double)x, k);
+  if (be <= 0 || be >= 2047) return scale_steps((double)x, k);
   return __longlong_as_double((long long)(sgn | ((unsigned long long)be << 52) | (m & 0xFFFFFFFFFFFFFull)));
 }
 
@@ -447,7 +441,7 @@ __device__ __forceinline__ double f32_scaled(float f, int k) {
   if ((u & 0x7FFFFFFFu) == 0) return __longlong_as_double((long long)sgn);
   const int ef = (int)((u >> 23) & 0xFFu);
   const int be = ef - 127 + k + 1023;
-  if (ef == 0 || ef == 255 || be <= 0 || be >= 2047) return ldexp((double)f, k);
+  if (ef == 0 || ef == 255 || be <= 0 || be >= 2047) return scale_steps((double)f, k);
   return __longlong_as_double(
       (long long)(sgn | ((unsigned long long)be << 52) | ((unsigned long long)(u & 0x7FFFFFu) << 29)));
 }
@@ -463,6 +457,10 @@ struct SplitEpi {
   const int* eb;            // column exponents (batch x Npad)
   int M, N, K, Mpad, Npad;
   int batch, reduce, swap;  // swap: the tile computes C^T (rows of the tile are columns of C)
+  int c_upper;              // only tiles that touch the upper triangle (square, no swap)
+  int b_lower;              // op(B)[k][j] = 0 for k < j: a tile starts at K block n0 / BK (no swap)
+  int ks;                   // CTAs (one cluster) that share a tile's K; 1: none
+  int tiles_z, tiles;       // tiles of one batch entry (of the reduced product), in all
   int* err;
   int stall;                // test hook: the MMA issuer first waits on a barrier nothing completes
   long long stall_ns;
@@ -471,28 +469,115 @@ struct SplitEpi {
                             // exponents may exceed it)
 };
 
-template <int BN, int S>
+template <int BN, int S, int FORM>
 struct SmemLayout {
+  static constexpr int kAcc = Form<FORM>::top(S) + 1;   // level accumulators
   static constexpr int kBTile = BN * 128;          // bytes of one B slice tile (BN rows of 128 bytes)
   static constexpr int kBStage = S * kBTile;
   static constexpr int kATile = kTileM * 128;      // 16 KB
   static constexpr int kOffB = 0;
   static constexpr int kOffA = 2 * kBStage;
   static constexpr int kOffBar = kOffA + kARing * kATile;
-  static constexpr int kBars = 2 + 2 + 2 * kARing + 3 + 1;   // the last: never completed
+  // B full / empty, A full / empty, level full / empty, done, never completed
+  static constexpr int kBars = 4 + 2 * kARing + 2 * kAcc + 2;
   static constexpr int kBytes = kOffBar + kBars * 8 + 16;
   static constexpr int kAlloc = kBytes + 1024;     // slack for 1024-byte alignment
+  static_assert(kAlloc <= 232448, "shared memory of one CTA");
+  static_assert(kOffBar >= kTileM * BN * 12, "the K split's partial tile reuses the operand stages");
 };
 
+// Tiles of one batch entry, in groups of kGroupM tile rows (their A slices stay
+// in L2 while B streams); with c_upper a group starts at the first tile column
+// its first row needs.  Host and device count alike.
+template <int BN>
+__host__ __device__ inline int split_tiles_z(int num_m, int num_n, int c_upper) {
+  if (!c_upper) return num_m * num_n;
+  int total = 0;
+  for (int first = 0; first < num_m; first += kGroupM) {
+    const int gm = num_m - first < kGroupM ? num_m - first : kGroupM;
+    total += gm * (num_n - first * (kTileM / BN));
+  }
+  return total;
+}
+
+struct TilePos {
+  int z, tm, tn;
+  bool valid;               // false: a tile below the diagonal inside a group
+};
+template <int BN>
+__device__ __forceinline__ TilePos split_tile(const SplitEpi& p, int idx) {
+  constexpr int R = kTileM / BN;
+  const int num_m = p.Mpad / kTileM, num_n = p.Npad / BN;
+  TilePos t;
+  t.z = idx / p.tiles_z;
+  idx -= t.z * p.tiles_z;
+  int first = 0, n_first = 0;
+  if (!p.c_upper) {
+    first = idx / (kGroupM * num_n) * kGroupM;
+    idx -= first * num_n;
+  } else {
+    for (;; first += kGroupM) {
+      const int gm = num_m - first < kGroupM ? num_m - first : kGroupM;
+      const int cnt = gm * (num_n - first * R);
+      if (idx < cnt) break;
+      idx -= cnt;
+    }
+    n_first = first * R;
+  }
+  const int gm = num_m - first < kGroupM ? num_m - first : kGroupM;
+  t.tm = first + idx % gm;
+  t.tn = n_first + idx / gm;
+  t.valid = !p.c_upper || t.tn >= t.tm * R;
+  return t;
+}
+
+// The output of one entry from its exact level sums (iacc, units of 2^-48) and
+// its float part: scaled by 2^(e_i + f_j), then alpha.  one_chunk: both fit one
+// int64 in units of 2^-56, so no FP64 instruction is needed (the FP64 units give
+// 2 lanes a clock, and a short product's epilogue would wait for them).
+template <int FORM>
+__device__ __forceinline__ double split_value(const SplitEpi& p, long long iacc, float fm, int ei,
+                                              int ej, double al, bool one_chunk) {
+  using F = Form<FORM>;
+  const int e = ei + ej;
+  double v;
+  if (F::kFloatUnit == 56 && one_chunk)
+    v = i64_scaled((iacc << 8) + __float2ll_rn(fm), e - 56);
+  else
+    v = i64_scaled(iacc, e - 48) + f32_scaled(fm, e - F::kFloatUnit);
+  // an Inf or NaN in the row of op(A) or the column of op(B): the digits carry no
+  // value, so the output is NaN (as the FP64 product gives NaN or Inf there)
+  if (p.nan_rows && (ei >= 1026 || ej >= 1026)) v = __longlong_as_double(0x7FF8000000000000ll);
+  if (al == -1.0) v = __longlong_as_double(__double_as_longlong(v) ^ (long long)0x8000000000000000ull);
+  else if (al != 1.0) v *= al;
+  return v;
+}
+
+// Persistent: CTA b takes the tiles b, b + gridDim.x, ... (with a K split, cluster
+// b one tile).  Warp 0 streams slice tiles by TMA (two B stages of S tiles, a ring
+// of A tiles), warp 1 issues the MMAs, sixteen warps drain the level accumulators;
+// the three run ahead of one another across K blocks, chunks and tiles, so a
+// tile's loads, its epilogue and the next tile's MMAs overlap.
+//
+// An MMA of M = 128, N = 64 reads 6 KB of operands in 32 clocks, more than shared
+// memory's 128 B a clock.  The levels are neighbours in TMEM and the B slices
+// neighbours in shared memory, so A slice s times the B slices t .. t+3 is one MMA
+// of N = 256 that adds to the levels s+t .. s+t+3: A is read once for four pairs.
+//
+// With the slices taken in order s = 1..S, level L is complete when s = L - 1 has
+// met t = 1: each level has its own full / empty barriers, so its drain runs under
+// the pairs that follow and only the last levels of a chunk are waited for.
 template <int BN, int S, int FORM>
 __global__ void __launch_bounds__(kThreads, 1)
 split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                   const SplitEpi p) {
-  using L = SmemLayout<BN, S>;
+  using L = SmemLayout<BN, S, FORM>;
   using F = Form<FORM>;
-  constexpr int kChunkK = F::kChunkK;
   constexpr int kBK = form_bk<FORM>();
-  constexpr int kAcc = F::kAcc;
+  constexpr int kChunkB = F::kChunkK / kBK;      // K blocks per chunk
+  constexpr int kAcc = L::kAcc;
+  constexpr int kTop = F::top(S);                // largest s + t (0-based) kept
+  constexpr int kG = 256 / BN;                   // B slices per MMA
   static_assert(kAcc * BN <= 512, "the level accumulators must fit in TMEM");
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sm = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -503,31 +588,26 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   uint64_t* bempty = bar + 2;
   uint64_t* afull = bar + 4;
   uint64_t* aempty = afull + kARing;
-  uint64_t* tfull = aempty + kARing;
-  uint64_t* tempty = tfull + 1;
-  uint64_t* tdone = tfull + 2;
-  uint64_t* never = tfull + 3;         // initialised, never arrived at (test hook)
+  uint64_t* lfull = aempty + kARing;
+  uint64_t* lempty = lfull + kAcc;
+  uint64_t* tdone = lempty + kAcc;
+  uint64_t* never = tdone + 1;         // initialised, never arrived at (test hook)
   uint32_t* tslot = (uint32_t*)(bar + L::kBars);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // CTAs in groups of kGroupM tile rows: one wave covers kGroupM rows of A
-  // tiles (kept in L2) while B streams, instead of all of B for two rows
-  int tm, tn;
-  {
-    const int num_n = gridDim.x, num_m = gridDim.y;
-    const int pid = blockIdx.y * num_n + blockIdx.x;
-    const int first_m = pid / (kGroupM * num_n) * kGroupM;
-    const int gm = num_m - first_m < kGroupM ? num_m - first_m : kGroupM;
-    const int idx = pid - first_m * num_n;
-    tm = first_m + idx % gm;
-    tn = idx / gm;
-  }
-  const int m0 = tm * kTileM, n0 = tn * BN;
-  const int nkb = (p.K + kBK - 1) / kBK;
-  const int nchunk_k = (nkb + (kChunkK / kBK) - 1) / (kChunkK / kBK);
-  const int b_first = p.reduce ? 0 : blockIdx.z;
-  const int b_last = p.reduce ? p.batch : blockIdx.z + 1;
-  const int nchunks = nchunk_k * (b_last - b_first);
+  const int rank = blockIdx.x % p.ks;
+  const int tile0 = blockIdx.x / p.ks, tile_step = gridDim.x / p.ks;
+  const int nkb_all = (p.K + kBK - 1) / kBK;
+  // this rank's K blocks of a tile: [lo, hi), the structurally zero ones skipped
+  auto k_range = [&](int tn, int* lo, int* hi) {
+    *lo = p.b_lower ? tn * BN / kBK : 0;
+    *hi = nkb_all;
+    if (p.ks > 1) {
+      const int per = (nkb_all - *lo + p.ks - 1) / p.ks;
+      *lo += rank * per;
+      *hi = min(*hi, *lo + per);
+    }
+  };
   int* err = p.err;
 
   if (threadIdx.x == 0) {
@@ -535,8 +615,10 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     tc::prefetch_tmap(&tmB);
     for (int i = 0; i < 2; ++i) { tc::mbar_init(&bfull[i], 1); tc::mbar_init(&bempty[i], 1); }
     for (int i = 0; i < kARing; ++i) { tc::mbar_init(&afull[i], 1); tc::mbar_init(&aempty[i], 1); }
-    tc::mbar_init(tfull, 1);
-    tc::mbar_init(tempty, kEpiWarps);
+    for (int i = 0; i < kAcc; ++i) {
+      tc::mbar_init(&lfull[i], 1);
+      tc::mbar_init(&lempty[i], kEpiWarps);
+    }
     tc::mbar_init(tdone, 1);
     tc::mbar_init(never, 1);
     tc::fence_barrier_init();
@@ -546,27 +628,47 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   tc::tc_fence_after();
   const uint32_t tmem = *tslot;
 
+  // the K split's partial tile: exact sums, then float parts (column-major, 128 rows)
+  long long* part_i = reinterpret_cast<long long*>(sm);
+  float* part_f = reinterpret_cast<float*>(sm + (size_t)kTileM * BN * 8);
+
   if (warp == 0 && lane == 0) {
     // ---------------- TMA producer
     int kbg = 0, ia = 0;
     bool ok = true;
     int kbg_armed = 0, ia_armed = 0;   // loads issued (for the error-path drain)
-    for (int b = b_first; b < b_last && ok; ++b) {
-      const int arow = b * S * p.Mpad + m0, brow = b * S * p.Npad + n0;
-      for (int kb = 0; kb < nkb && ok; ++kb, ++kbg) {
-        const int sb = kbg & 1;
-        if (kbg >= 2 && !(ok = tc::mbar_wait(&bempty[sb], ((kbg >> 1) & 1) ^ 1, err))) break;
-        tc::mbar_arrive_expect_tx(&bfull[sb], L::kBStage);
-        kbg_armed = kbg + 1;
-        for (int t = 0; t < S; ++t)
-          tc::tma_load_2d(sB + sb * L::kBStage + t * L::kBTile, &tmB, &bfull[sb], kb * kBK,
-                          brow + t * p.Npad);
-        for (int s = 0; s < S; ++s, ++ia) {
-          const int sa = ia % kARing;
-          if (ia >= kARing && !(ok = tc::mbar_wait(&aempty[sa], ((ia / kARing) & 1) ^ 1, err))) break;
-          tc::mbar_arrive_expect_tx(&afull[sa], L::kATile);
-          ia_armed = ia + 1;
-          tc::tma_load_2d(sA + sa * L::kATile, &tmA, &afull[sa], kb * kBK, arow + s * p.Mpad);
+    for (int idx = tile0; idx < p.tiles && ok; idx += tile_step) {
+      const TilePos t = split_tile<BN>(p, idx);
+      if (!t.valid) continue;
+      int kb_lo, kb_hi;
+      k_range(t.tn, &kb_lo, &kb_hi);
+      const int b_first = p.reduce ? 0 : t.z, b_last = p.reduce ? p.batch : t.z + 1;
+      for (int b = b_first; b < b_last && ok; ++b) {
+        const int arow = b * S * p.Mpad + t.tm * kTileM, brow = b * S * p.Npad + t.tn * BN;
+        for (int kb = kb_lo; kb < kb_hi && ok; ++kb, ++kbg) {
+          const int sb = kbg & 1;
+          if (kbg >= 2 && !(ok = tc::mbar_wait(&bempty[sb], ((kbg >> 1) & 1) ^ 1, err))) break;
+          tc::mbar_arrive_expect_tx(&bfull[sb], L::kBStage);
+          kbg_armed = kbg + 1;
+          for (int s = 0; s < S; ++s, ++ia) {
+            // the first A tile ahead of the B stage's: the MMAs start with both
+            const int sa = ia % kARing;
+            if (ia >= kARing && !(ok = tc::mbar_wait(&aempty[sa], ((ia / kARing) & 1) ^ 1, err))) {
+              // the armed B stage still gets the tiles it expects
+              if (s == 0)
+                for (int u = 0; u < S; ++u)
+                  tc::tma_load_2d(sB + sb * L::kBStage + u * L::kBTile, &tmB, &bfull[sb], kb * kBK,
+                                  brow + u * p.Npad);
+              break;
+            }
+            tc::mbar_arrive_expect_tx(&afull[sa], L::kATile);
+            ia_armed = ia + 1;
+            tc::tma_load_2d(sA + sa * L::kATile, &tmA, &afull[sa], kb * kBK, arow + s * p.Mpad);
+            if (s == 0)
+              for (int u = 0; u < S; ++u)
+                tc::tma_load_2d(sB + sb * L::kBStage + u * L::kBTile, &tmB, &bfull[sb], kb * kBK,
+                                brow + u * p.Npad);
+          }
         }
       }
     }
@@ -579,78 +681,111 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     }
   } else if (warp == 1 && lane == 0) {
     // ---------------- MMA issuer
-    // One thread issues 4 MMAs per slice pair and K block (32 bytes of K each):
-    // the descriptors are formed once and advanced by adding to their
+    // One thread issues 4 MMAs (32 bytes of K each) per A slice and group of B
+    // slices: the descriptors are formed once and advanced by adding to their
     // start-address field (address >> 4, 14 bits; shared addresses stay below
-    // 256 KB so no carry leaves the field), and the slice-pair loops are unrolled.
-    const uint32_t idesc = FORM == kFormFP8    ? tc::idesc_e4m3_f32(kTileM, BN)
-                           : FORM == kFormFP16 ? tc::idesc_f16_f32(kTileM, BN)
-                                               : tc::idesc_bf16_f32(kTileM, BN);
+    // 256 KB so no carry leaves the field).
+    const uint32_t idesc0 = FORM == kFormFP8    ? tc::idesc_e4m3_f32(kTileM, 0)
+                            : FORM == kFormFP16 ? tc::idesc_f16_f32(kTileM, 0)
+                                                : tc::idesc_bf16_f32(kTileM, 0);
     const uint64_t adesc0 = tc::sdesc_k128(tc::smem_u32(sA));
     const uint64_t bdesc0 = tc::sdesc_k128(tc::smem_u32(sB));
-    int kbg = 0, ia = 0;
+    int kbg = 0, ia = 0, cg = 0;       // K blocks, A tiles and chunks so far
     bool ok = true;
     if (p.stall) {
       tc::mbar_stall(never, err, p.stall_ns);
       ok = false;
     }
-    for (int c = 0; c < nchunks && ok; ++c) {
-      if (c > 0 && !(ok = tc::mbar_wait(tempty, (c - 1) & 1, err))) break;
-      tc::tc_fence_after();
-      uint32_t fresh = (1u << kAcc) - 1;   // accumulator a starts (accumulate = 0) at its first MMA
-      const int kc = c % nchunk_k;
-      const int kb_end = min(nkb, (kc + 1) * (kChunkK / kBK));
-      for (int kb = kc * (kChunkK / kBK); kb < kb_end && ok; ++kb, ++kbg) {
-        const int sb = kbg & 1;
-        if (!(ok = tc::mbar_wait(&bfull[sb], (kbg >> 1) & 1, err))) break;
-        tc::tc_fence_after();
-        const uint64_t bd = bdesc0 + (uint64_t)((sb * L::kBStage) >> 4);
+    for (int idx = tile0; idx < p.tiles && ok; idx += tile_step) {
+      const TilePos t = split_tile<BN>(p, idx);
+      if (!t.valid) continue;
+      int kb_lo, kb_hi;
+      k_range(t.tn, &kb_lo, &kb_hi);
+      const int entries = p.reduce ? p.batch : 1;
+      for (int b = 0; b < entries && ok; ++b) {
+        for (int kb = kb_lo; kb < kb_hi && ok; ++kb, ++kbg) {
+          const int in_chunk = (kb - kb_lo) % kChunkB;
+          const bool first = in_chunk == 0;                       // the levels start anew
+          const bool last = in_chunk == kChunkB - 1 || kb == kb_hi - 1;   // and are complete
+          const int sb = kbg & 1;
+          if (!(ok = tc::mbar_wait(&bfull[sb], (kbg >> 1) & 1, err))) break;
+          const uint64_t bd = bdesc0 + (uint64_t)((sb * L::kBStage) >> 4);
+          // level l drained by the epilogue after the previous chunk
+          auto drained = [&](int l) {
+            if (first && cg > 0 && ok) ok = tc::mbar_wait(&lempty[l], (cg - 1) & 1, err);
+          };
 #pragma unroll
-        for (int s = 0; s < S; ++s) {
-          const int sa = ia % kARing;
-          if (!(ok = tc::mbar_wait(&afull[sa], (ia / kARing) & 1, err))) break;
-          ++ia;
-          tc::tc_fence_after();
-          const uint64_t ad = adesc0 + (uint64_t)((sa * L::kATile) >> 4);
-          constexpr int kTop = F::top(S);   // largest s + t (0-based) kept
+          for (int s = 0; s < S; ++s) {
+            const int sa = ia % kARing;
+            if (!ok || !(ok = tc::mbar_wait(&afull[sa], (ia / kARing) & 1, err))) break;
+            ++ia;
+            tc::tc_fence_after();
+            const uint64_t ad = adesc0 + (uint64_t)((sa * L::kATile) >> 4);
+            // B slices [t0, t0 + nt) in one MMA per 32 bytes of K, levels s + t0 ..
+            auto group = [&](int t0, int nt, bool fresh) {
+              const uint32_t d = tmem + (s + t0) * BN;
+              const uint64_t bt = bd + (uint64_t)((t0 * L::kBTile) >> 4);
+              const uint32_t idesc = idesc0 | ((uint32_t)(nt * BN >> 3) << 17);
 #pragma unroll
-          for (int t = 0; t < (kTop - s + 1 < S ? kTop - s + 1 : S); ++t) {
-            const int lvl = s + t;                 // 0 -> level 2
-            // FP16 and FP8: one accumulator per level (raw digits of different
-            // scales must not share one); BF16: levels >= 9 share the last
-            const int acc = FORM != kFormBF16 ? lvl : (lvl < kAcc - 1 ? lvl : kAcc - 1);
-            const uint32_t d = tmem + acc * BN;
-            const uint64_t bt = bd + (uint64_t)((t * L::kBTile) >> 4);
-            const uint32_t first = (fresh >> acc) & 1u;
+              for (int kk = 0; kk < kRowBytes / 32; ++kk) {
+                const uint32_t accum = (fresh && kk == 0) ? 0u : 1u;
+                if (FORM == kFormFP8) tc::mma_f8(d, ad + 2 * kk, bt + 2 * kk, idesc, accum);
+                else tc::mma_bf16(d, ad + 2 * kk, bt + 2 * kk, idesc, accum);
+              }
+            };
+            constexpr int kTs0 = S;              // t of s = 0
+            const int ts = kTop - s + 1 < S ? kTop - s + 1 : S;
+            if (s == 0) {
+              // every level up to S - 1 is first touched here
 #pragma unroll
-            for (int kk = 0; kk < kRowBytes / 32; ++kk) {
-              const uint32_t accum = (first && kk == 0) ? 0u : 1u;
-              if (FORM == kFormFP8) tc::mma_f8(d, ad + 2 * kk, bt + 2 * kk, idesc, accum);
-              else tc::mma_bf16(d, ad + 2 * kk, bt + 2 * kk, idesc, accum);
+              for (int t0 = 0; t0 < kTs0; t0 += kG) {
+                const int nt = kTs0 - t0 < kG ? kTs0 - t0 : kG;
+                if (first) {
+#pragma unroll
+                  for (int u = 0; u < nt; ++u) drained(t0 + u);
+                  tc::tc_fence_after();
+                }
+                if (ok) group(t0, nt, first);
+              }
+            } else if (s == 1 && kTop == S) {
+              // the pair (1, S - 1) opens level S: alone in a chunk's first block
+              const int te = first ? ts - 1 : ts;
+              for (int t0 = 0; t0 < te; t0 += kG) group(t0, te - t0 < kG ? te - t0 : kG, false);
+              if (first) {
+                drained(S);
+                tc::tc_fence_after();
+                if (ok) group(ts - 1, 1, true);
+              }
+            } else {
+#pragma unroll
+              for (int t0 = 0; t0 < ts; t0 += kG) group(t0, ts - t0 < kG ? ts - t0 : kG, false);
             }
-            fresh &= ~(1u << acc);
+            // level s is complete once the slices 0..s have met t = 0 (the last
+            // slice also completes level S)
+            if (last) {
+              tc::mma_commit(&lfull[s]);
+              if (s == S - 1 && kTop == S) tc::mma_commit(&lfull[kTop]);
+            }
+            tc::mma_commit(&aempty[sa]);
           }
-          tc::mma_commit(&aempty[sa]);
+          if (!ok) break;
+          tc::mma_commit(&bempty[sb]);
+          if (last) ++cg;
         }
-        tc::mma_commit(&bempty[sb]);
       }
-      tc::mma_commit(tfull);
     }
     tc::mma_commit(tdone);   // arrives once every MMA issued above has completed
   } else if (warp >= 2) {
-    // ---------------- epilogue: drain chunks into integer accumulators
-    // Level L (2..8) of a chunk is an integer multiple of 2^-6L below 2^24 of
-    // those units, so it is added exactly to an int64 counting units of 2^-48
-    // (per chunk below 2^57.1: exact for 56 chunks, so gemm_split cuts a longer
-    // K into products of at most 56 x 2048).  The merged
-    // levels >= 9 go into a float, 2^-42 below the leading level.  FP64 is used
-    // only when a batch entry's result is written (two conversions, one FMA, the
-    // beta term; the power-of-two scale goes into the exponent field).
+    // ---------------- epilogue: drain the levels into an int64 and a float
+    // (level L of a chunk is an integer below 2^24 times 2^-bL; the int64 in units
+    // of 2^-48 has room for 600 chunks of 192, 28 of 4096, at the digit bounds, and
+    // gemm_split cuts a longer K into several products)
     constexpr int HALF = BN / (kEpiWarps / 4);     // columns of this warp
     const int q = warp & 3;
     const int half = (warp - 2) >> 2;              // which column slice
-    const int row = m0 + q * 32 + lane;            // tile row
     const uint32_t lane_off = (uint32_t)(q * 32) << 16;
+    int cg = 0;
+    bool ok = true;
     long long iacc[HALF];
     float fm[HALF];
 #pragma unroll
@@ -658,125 +793,132 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
       iacc[j] = 0;
       fm[j] = 0.f;
     }
-    bool ok = true;
-    const int z = p.reduce ? 0 : blockIdx.z;
-    double* C = p.C + (int64_t)z * p.strideC;
-    const double* Cin = p.Cin ? p.Cin + (int64_t)z * p.strideCin : nullptr;
-    for (int c = 0; c < nchunks; ++c) {
-      if (!(ok = tc::mbar_wait(tfull, c & 1, err))) break;
-      tc::tc_fence_after();
-      // one TMEM load (and one wait for it) per 16 columns where the warp has 16
-      constexpr int kLd = HALF % 16 == 0 ? 16 : 8;
+    for (int idx = tile0; idx < p.tiles && ok; idx += tile_step) {
+      const TilePos t = split_tile<BN>(p, idx);
+      if (!t.valid) continue;
+      int kb_lo, kb_hi;
+      k_range(t.tn, &kb_lo, &kb_hi);
+      const int nchunks = kb_hi > kb_lo ? (kb_hi - kb_lo + kChunkB - 1) / kChunkB : 0;
+      const int b_first = p.reduce ? 0 : t.z, b_last = p.reduce ? p.batch : t.z + 1;
+      const int row = t.tm * kTileM + q * 32 + lane;   // tile row
+      const int n0 = t.tn * BN;
+      double* C = p.C + (int64_t)(p.reduce ? 0 : t.z) * p.strideC;
+      const double* Cin = p.Cin ? p.Cin + (int64_t)(p.reduce ? 0 : t.z) * p.strideCin : nullptr;
+      for (int b = b_first; b < b_last && ok; ++b) {
+        for (int c = 0; c < nchunks && ok; ++c, ++cg) {
+          constexpr int kLd = HALF % 16 == 0 ? 16 : 8;
 #pragma unroll
-      for (int a = 0; a < kAcc; ++a) {
+          for (int a = 0; a < kAcc; ++a) {
+            if (!ok || !(ok = tc::mbar_wait(&lfull[a], cg & 1, err))) break;
+            tc::tc_fence_after();
+            const int lv = a + 2;
 #pragma unroll
-        for (int g = 0; g < HALF / kLd; ++g) {
-          float v[kLd];
-          if constexpr (kLd == 16) tc::tmem_ld16(tmem + lane_off + a * BN + half * HALF + g * kLd, v);
-          else tc::tmem_ld8(tmem + lane_off + a * BN + half * HALF + g * kLd, v);
-          if (FORM == kFormFP8) {
-            // raw integer level sums (|.| <= 2^24): levels 2..9 into 2^-48 units
-            // (level 2 of a 4096-chunk is below 2^20: 2^58 per chunk, so about
-            // 29 chunks fit); levels 10..13 into one float in units of 2^-65
-            // (times 2^(65 - 5L), exact)
-            const int L = a + 2;
+            for (int g = 0; g < HALF / kLd; ++g) {
+              float v[kLd];
+              if constexpr (kLd == 16) tc::tmem_ld16(tmem + lane_off + a * BN + half * HALF + g * kLd, v);
+              else tc::tmem_ld8(tmem + lane_off + a * BN + half * HALF + g * kLd, v);
 #pragma unroll
-            for (int i = 0; i < kLd; ++i) {
-              if (L <= 9) iacc[g * kLd + i] += (long long)__float2int_rn(v[i]) << (48 - 5 * L);
-              else fm[g * kLd + i] += v[i] * __int_as_float((127 + 65 - 5 * L) << 23);
+              for (int i = 0; i < kLd; ++i) {
+                if (lv <= F::kIntTop)
+                  iacc[g * kLd + i] += (long long)__float2int_rn(v[i]) << (48 - F::kBits * lv);
+                else
+                  fm[g * kLd + i] += v[i] * __int_as_float((127 + F::kFloatUnit - F::kBits * lv) << 23);
+              }
             }
-          } else if (FORM == kFormFP16) {
-            // raw integer level sums (|.| <= 2^24): levels 2..7 into 2^-49 units;
-            // levels 8 and 9 into one float in units of 2^-56 (level 9 times
-            // 2^-7, exact), whose rounding lies about 2^-56 below the leading level
-            const int L = a + 2;
-#pragma unroll
-            for (int i = 0; i < kLd; ++i) {
-              if (L <= 7) iacc[g * kLd + i] += (long long)__float2int_rn(v[i]) << (49 - 7 * L);
-              else if (L == 8) fm[g * kLd + i] += v[i];
-              else fm[g * kLd + i] += v[i] * 0x1p-7f;
-            }
-          } else if (a < kAcc - 1) {
-            const int L = a + 2;
-            // times 2^6L: an exact integer below 2^24
-            const float up = __int_as_float((127 + kBeta * L) << 23);
-#pragma unroll
-            for (int i = 0; i < kLd; ++i)
-              iacc[g * kLd + i] += (long long)__float2int_rn(v[i] * up) << (48 - kBeta * L);
-          } else {
-            // merged levels >= 9 stay in a float (2^-24 of a value 2^-30 below the
-            // leading level: rounding them to the int64's unit would cost 2^-49)
-#pragma unroll
-            for (int i = 0; i < kLd; ++i) fm[g * kLd + i] += v[i];
+            tc::tc_fence_before();
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&lempty[a]);
           }
         }
-      }
-      tc::tc_fence_before();
-      __syncwarp();
-      if (lane == 0) tc::mbar_arrive(tempty);
-      // end of a batch entry: scale, combine with beta C_in (first entry) or with
-      // the running sum already in C (reduce mode), write, reset
-      if ((c + 1) % nchunk_k == 0) {
-        const int b = b_first + c / nchunk_k;
-        const bool first = c / nchunk_k == 0;
+        if (!ok) break;
+        if (p.ks > 1) break;      // one entry per tile: joined over the cluster below
+        // end of a batch entry: scale, combine with beta C_in (first entry) or with
+        // the running sum already in C (reduce mode), write, reset
+        const bool first = b == b_first, one = nchunks == 1;
         const int ei = p.ea[b * p.Mpad + row];
         const int* ebb = p.eb + b * p.Npad + n0 + half * HALF;
         const double al = p.alpha[b];
-        // eight outputs at a time: their addends (beta C_in, or the running sum
-        // in reduce mode) loaded together first, then formed and stored (a load
-        // after a store to C could alias it, so a plain loop waits for each)
+        // four outputs at a time: their addends (beta C_in, or the running sum in
+        // reduce mode) loaded together first, then formed and stored (a load after
+        // a store to C could alias it, so a plain loop waits for each).  The strides
+        // are made opaque here: hoisted out of the loops, sixteen columns' addresses
+        // would spill the accumulators.
         const bool use_cin = Cin && p.beta != 0.0;
+        const int col0 = n0 + half * HALF;
+        int64_t st_c = p.swap ? 1 : p.ldc, st_i = first ? (p.swap ? 1 : p.ldcin) : st_c;
+        asm volatile("" : "+l"(st_c), "+l"(st_i));
+        double* cp = C + (p.swap ? col0 + row * p.ldc : row + col0 * p.ldc);
+        const double* ip = first ? Cin + (p.swap ? col0 + row * p.ldcin : row + col0 * p.ldcin) : cp;
+        const bool addend = !first || use_cin;
+        const double bt = first ? p.beta : 1.0;
+        const int jn = row < (p.swap ? p.N : p.M) ? (p.swap ? p.M : p.N) - col0 : 0;   // columns left
 #pragma unroll
-        for (int j0 = 0; j0 < HALF; j0 += 8) {
-          double add[8];
+        for (int j0 = 0; j0 < HALF; j0 += 4) {
+          double add[4];
 #pragma unroll
-          for (int jj = 0; jj < 8; ++jj) {
-            const int col = n0 + half * HALF + j0 + jj;
-            const int ci = p.swap ? col : row, cj = p.swap ? row : col;
-            add[jj] = 0.0;
-            if (row < (p.swap ? p.N : p.M) && col < (p.swap ? p.M : p.N)) {
-              if (!first) add[jj] = C[ci + (int64_t)cj * p.ldc];
-              else if (use_cin) add[jj] = Cin[ci + (int64_t)cj * p.ldcin];
-            }
+          for (int jj = 0; jj < 4; ++jj) {
+            add[jj] = addend && j0 + jj < jn ? *ip : 0.0;
+            ip += st_i;
           }
 #pragma unroll
-          for (int jj = 0; jj < 8; ++jj) {
+          for (int jj = 0; jj < 4; ++jj) {
             const int j = j0 + jj;
-            const int col = n0 + half * HALF + j;
-            const int ci = p.swap ? col : row, cj = p.swap ? row : col;
-            if (row < (p.swap ? p.N : p.M) && col < (p.swap ? p.M : p.N)) {
-              // the integer part and the float part, each scaled by the power of
-              // two 2^(e_i + f_j) in its exponent field, joined by one FP64 add
-              // (the same single rounding as converting the int64 and adding the
-              // float part at its weight)
-              const int ej = __ldg(ebb + j), e = ei + ej;
-              double v;
-              if (FORM == kFormFP8)
-                v = i64_scaled(iacc[j], e - 48) + f32_scaled(fm[j], e - 48 - 17);
-              else if (FORM == kFormFP16)
-                v = i64_scaled(iacc[j], e - 49) + f32_scaled(fm[j], e - 49 - 7);
-              else
-                v = i64_scaled(iacc[j], e - 48) + f32_scaled(fm[j], e);
-              // an Inf or NaN in the row of op(A) or the column of op(B): the
-              // digits carry no value, so the output is NaN (as the FP64 product
-              // gives NaN or Inf there)
-              if (p.nan_rows && (ei >= 1026 || ej >= 1026)) v = __longlong_as_double(0x7FF8000000000000ll);
-              if (al == -1.0) v = __longlong_as_double(__double_as_longlong(v) ^ (long long)0x8000000000000000ull);
-              else if (al != 1.0) v *= al;
-              if (first) {
-                if (use_cin) v = fma(p.beta, add[jj], v);
-              } else {
-                v += add[jj];
-              }
-              C[ci + (int64_t)cj * p.ldc] = v;
+            if (j < jn) {
+              double v = split_value<FORM>(p, iacc[j], fm[j], ei, __ldg(ebb + j), al, one);
+              if (addend) v = fma(bt, add[jj], v);
+              *cp = v;
             }
+            cp += st_c;
             iacc[j] = 0;
             fm[j] = 0.f;
           }
         }
       }
     }
-    (void)ok;
+    if (p.ks > 1) {
+      // the operand stages are free: every MMA of this CTA (the last levels'
+      // barrier) and every load it consumed are done
+#pragma unroll
+      for (int j = 0; j < HALF; ++j) {
+        part_i[(half * HALF + j) * kTileM + q * 32 + lane] = iacc[j];
+        part_f[(half * HALF + j) * kTileM + q * 32 + lane] = fm[j];
+      }
+    }
+  }
+  if (p.ks > 1) {
+    // K split: the ranks' exact sums are added as integers and their float parts in
+    // rank order; rank r writes the columns r BN / ks ..  Every thread of every rank
+    // reaches both barriers, on the error path too.
+    namespace cgrp = cooperative_groups;
+    cgrp::cluster_group cluster = cgrp::this_cluster();
+    __syncthreads();
+    cluster.sync();
+    if (warp >= 2 && tile0 < p.tiles) {
+      const TilePos t = split_tile<BN>(p, tile0);
+      if (t.valid && !*(volatile int*)err) {
+        const int e = threadIdx.x - 64, r = e % kTileM, row = t.tm * kTileM + r;
+        const int share = BN / p.ks;
+        double* C = p.C + (int64_t)t.z * p.strideC;
+        const double* Cin = p.Cin ? p.Cin + (int64_t)t.z * p.strideCin : nullptr;
+        const int ei = p.ea[t.z * p.Mpad + row];
+        for (int jc = e / kTileM; jc < share; jc += 32 * kEpiWarps / kTileM) {
+          const int j = rank * share + jc, col = t.tn * BN + j;
+          const int ci = p.swap ? col : row, cj = p.swap ? row : col;
+          if (row >= (p.swap ? p.N : p.M) || col >= (p.swap ? p.M : p.N)) continue;
+          long long si = 0;
+          float sf = 0.f;
+          for (int k = 0; k < p.ks; ++k) {
+            si += cluster.map_shared_rank(part_i, k)[j * kTileM + r];
+            sf += cluster.map_shared_rank(part_f, k)[j * kTileM + r];
+          }
+          double v = split_value<FORM>(p, si, sf, ei, __ldg(p.eb + t.z * p.Npad + col), p.alpha[t.z],
+                                       false);
+          if (Cin && p.beta != 0.0) v = fma(p.beta, Cin[ci + (int64_t)cj * p.ldcin], v);
+          C[ci + (int64_t)cj * p.ldc] = v;
+        }
+      }
+    }
+    cluster.sync();   // no rank leaves while another reads its partial tile
   }
   tc::tc_fence_before();
   __syncthreads();
@@ -854,6 +996,22 @@ cudaError_t slice_operand(const double* X, int64_t ldx, int64_t strideX, int tra
   return cudaGetLastError();
 }
 
+constexpr int kSplitSMs = 152;
+
+// CTAs per tile: with too few tiles for the SMs, K is cut over a cluster while
+// every rank keeps two chunks of K blocks (entries > 1: a reduced batch runs its
+// entries one after another into the same output and is not cut).  Clusters of
+// eight find room on about 128 SMs, of four on 144.
+int split_ks(int tiles, int entries, int nkb, int chunk) {
+  if (entries > 1) return 1;
+  int best = 1;
+  for (int ks = 2; ks <= 8; ks *= 2) {
+    if (tiles * ks > (ks == 8 ? 128 : ks == 4 ? 144 : kSplitSMs) || nkb < ks * std::min(2 * chunk, 8)) break;
+    best = ks;
+  }
+  return best;
+}
+
 template <int BN, int S, int FORM>
 cudaError_t run_split(const GemmArgs& g, SplitWork& w, cudaStream_t st) {
   constexpr int kE = Form<FORM>::kElem;
@@ -926,33 +1084,41 @@ cudaError_t run_split(const GemmArgs& g, SplitWork& w, cudaStream_t st) {
   p.ea = ea; p.eb = eb;
   p.M = g.M; p.N = g.N; p.K = K; p.Mpad = Mpad; p.Npad = Npad;
   p.batch = nb; p.reduce = g.reduce; p.swap = swap ? 1 : 0;
+  // structural zeros: c_upper is square (never swapped); b_lower's op(B) is the
+  // tile's B side unless swapped
+  p.c_upper = g.c_upper && !swap && g.M == g.N;
+  p.b_lower = g.b_lower && !swap;
+  const int nz = g.reduce ? 1 : nb;
+  p.tiles_z = split_tiles_z<BN>(Mpad / kTileM, Npad / BN, p.c_upper);
+  p.tiles = p.tiles_z * nz;
+  p.ks = split_ks(p.tiles, g.reduce ? nb : 1, Kpad / form_bk<FORM>(), Form<FORM>::kChunkK / form_bk<FORM>());
   p.err = w.err;
   p.stall = w.stall;
   p.stall_ns = w.stall_ns;
   p.nan_rows = keq ? 0 : 1;
-  using L = SmemLayout<BN, S>;
-  if ((err = smem_attr_once((const void*)split_gemm_kernel<BN, S, FORM>, L::kAlloc)) != cudaSuccess) {
-    if (std::getenv("ZOLO_DEBUG"))
-      std::fprintf(stderr, "zolo: cudaFuncSetAttribute(%d B): %s\n", L::kAlloc,
-                   cudaGetErrorString(err));
-    return err;
-  }
-  dim3 grid((unsigned)(Npad / BN), (unsigned)(Mpad / kTileM), g.reduce ? 1 : nb);
+  using L = SmemLayout<BN, S, FORM>;
+  const auto kernel = split_gemm_kernel<BN, S, FORM>;
+  if ((err = smem_attr_once((const void*)kernel, L::kAlloc)) != cudaSuccess) return err;
+  const dim3 grid((unsigned)(p.ks > 1 ? p.tiles * p.ks : std::min(p.tiles, kSplitSMs)));
   ProfScope ps(kProfSplitGemm, st, gemm_flops(g), 0.0);
-  ps.blocks((const void*)split_gemm_kernel<BN, S, FORM>, dim3(kThreads), L::kAlloc, dim3(grid));
-  split_gemm_kernel<BN, S, FORM><<<grid, kThreads, L::kAlloc, st>>>(mA, mB, p);
-  err = cudaGetLastError();
-  if (err != cudaSuccess && std::getenv("ZOLO_DEBUG")) {
-    cudaFuncAttributes fa{};
-    cudaFuncGetAttributes(&fa, split_gemm_kernel<BN, S, FORM>);
-    std::fprintf(stderr,
-                 "zolo: split_gemm_kernel<%d,%d> launch (grid %u x %u x %u, %d threads, %d B smem): %s"
-                 " [maxThreadsPerBlock %d, numRegs %d, localSizeBytes %zu, maxDynamicSmem %d]\n",
-                 BN, S, grid.x, grid.y, grid.z, kThreads, L::kAlloc, cudaGetErrorString(err),
-                 fa.maxThreadsPerBlock, fa.numRegs, fa.localSizeBytes,
-                 fa.maxDynamicSharedSizeBytes);
+  ps.blocks((const void*)kernel, dim3(kThreads), L::kAlloc, grid);
+  if (p.ks == 1) {
+    kernel<<<grid, kThreads, L::kAlloc, st>>>(mA, mB, p);
+    return cudaGetLastError();
   }
-  return err;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = L::kAlloc;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = p.ks;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, mA, mB, p);
 }
 
 }  // namespace
@@ -961,10 +1127,10 @@ cudaError_t gemm_split(const GemmArgs& g, SplitWork& w, cudaStream_t st) {
   if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return cudaSuccess;
   if (g.K <= 0 || g.batch > kGemmMaxBatch) return gemm_f64(g, st);
   // The int64 that holds an output's exact level sums has room for a bounded
-  // number of K-chunks at the digit bounds (BF16: 2^57.1 per 2048-chunk, FP16:
-  // 2^56.1 per 512-chunk, FP8: 2^58.1 per 4096-chunk); a longer K runs as
-  // consecutive products whose partial results are added in FP64.
-  const int64_t kmax = w.form == kFormFP16 ? 120 * 512 : w.form == kFormFP8 ? 28 * 4096 : 56 * 2048;
+  // number of K-chunks at the digit bounds (8-bit digits: 2^53.6 per 192-chunk,
+  // FP8: 2^58.1 per 4096-chunk); a longer K runs as consecutive products whose
+  // partial results are added in FP64.
+  const int64_t kmax = 28 * 4096;
   if (g.K > kmax) {
     for (int64_t k0 = 0; k0 < g.K; k0 += kmax) {
       GemmArgs h = g;
@@ -990,9 +1156,9 @@ cudaError_t gemm_split(const GemmArgs& g, SplitWork& w, cudaStream_t st) {
   if (gs < 1) return cudaErrorMemoryAllocation;
   auto run = [&](const GemmArgs& h) {
     if (w.form == kFormFP8) return run_split<Form<kFormFP8>::kBN, 11, kFormFP8>(h, w, st);
-    if (w.form == kFormFP16) return run_split<64, 8, kFormFP16>(h, w, st);
-    return w.slices_s == 9 ? run_split<64, 9, kFormBF16>(h, w, st)
-                           : run_split<64, 8, kFormBF16>(h, w, st);
+    if (w.form == kFormFP16) return run_split<64, 7, kFormFP16>(h, w, st);
+    return w.slices_s == 9 ? run_split<64, 7, kFormBF16>(h, w, st)
+                           : run_split<64, 6, kFormBF16>(h, w, st);
   };
   if (gs >= g.batch) return run(g);
   for (int b0 = 0; b0 < g.batch; b0 += gs) {
@@ -1013,12 +1179,16 @@ cudaError_t gemm_split(const GemmArgs& g, SplitWork& w, cudaStream_t st) {
   return cudaSuccess;
 }
 
+template <int BN, int S, int FORM>
+static void prepare_form() {
+  smem_attr_once((const void*)split_gemm_kernel<BN, S, FORM>, SmemLayout<BN, S, FORM>::kAlloc);
+}
+
 void split_prepare() {
-  smem_attr_once((const void*)split_gemm_kernel<64, 8, kFormBF16>, SmemLayout<64, 8>::kAlloc);
-  smem_attr_once((const void*)split_gemm_kernel<64, 9, kFormBF16>, SmemLayout<64, 9>::kAlloc);
-  smem_attr_once((const void*)split_gemm_kernel<64, 8, kFormFP16>, SmemLayout<64, 8>::kAlloc);
-  smem_attr_once((const void*)split_gemm_kernel<Form<kFormFP8>::kBN, 11, kFormFP8>,
-                 SmemLayout<Form<kFormFP8>::kBN, 11>::kAlloc);
+  prepare_form<64, 6, kFormBF16>();
+  prepare_form<64, 7, kFormBF16>();
+  prepare_form<64, 7, kFormFP16>();
+  prepare_form<Form<kFormFP8>::kBN, 11, kFormFP8>();
   encode_fn();
 }
 
@@ -1030,6 +1200,13 @@ SplitWork* get_split_engine() { return t_split; }
 // Estimated seconds on GB300 of one call on the FP64 pipe and on the split
 // tensor-core path (slicing traffic + output traffic + slice-pair products +
 // launch latency).
+// Slice planes of a form: zolo_dgemm's `slices` of 9 and 8 six-bit digits (54 and 48
+// bits) are held as 7 and 6 eight-bit ones, the FP16 form's 8 seven-bit ones as 7.
+int split_planes(int slices, int form) {
+  if (form == kFormFP8) return slices;
+  return form == kFormFP16 || slices == 9 ? 7 : 6;
+}
+
 bool split_preferred(const GemmArgs& g, const SplitWork& w) { return split_time_ratio(g, w) < 1.0; }
 
 namespace {
@@ -1041,14 +1218,14 @@ struct SplitShape {
 SplitShape split_shape(const GemmArgs& g, const SplitWork& w) {
   const bool swap = g.M < kTileM && g.N > g.M;
   const bool fp8 = w.form == kFormFP8;
-  const double S = w.slices_s;
   SplitShape sh;
   sh.ra = (double)round_up(swap ? g.N : g.M, kTileM);
   sh.rb = (double)round_up(swap ? g.M : g.N, fp8 ? Form<kFormFP8>::kBN : 64);
   sh.kp = (double)round_up(g.K, fp8 ? form_bk<kFormFP8>() : form_bk<kFormBF16>());
   sh.elem_bytes = fp8 ? 1.0 : 2.0;
-  // slice pairs: s + t <= S + 2 (BF16, FP8), s + t <= S + 1 (FP16)
-  const double pairs = w.form == kFormFP16 ? S * (S + 1) / 2 : S * (S + 1) / 2 + (S - 1);
+  const double P = split_planes(w.slices_s, w.form);
+  // slice pairs: s + t <= P + 2 (BF16, FP8), s + t <= P + 1 (FP16)
+  const double pairs = w.form == kFormFP16 ? P * (P + 1) / 2 : P * (P + 1) / 2 + (P - 1);
   sh.pairs = fp8 ? pairs / 2 : pairs;
   return sh;
 }
@@ -1056,7 +1233,7 @@ SplitShape split_shape(const GemmArgs& g, const SplitWork& w) {
 
 double split_time_ratio(const GemmArgs& g, const SplitWork& w) {
   const SplitShape sh = split_shape(g, w);
-  const double S = w.slices_s;
+  const double S = split_planes(w.slices_s, w.form);
   const double slice_bytes = g.batch * (8.0 + sh.elem_bytes * S) * (sh.ra + sh.rb) * sh.kp;
   const double out_bytes = (g.reduce ? 1 : g.batch) * 8.0 * g.M * (double)g.N * (g.beta != 0.0 ? 2 : 1);
   const double products = sh.pairs * 2.0 * sh.ra * sh.rb * sh.kp * g.batch;
@@ -1088,7 +1265,7 @@ size_t split_slice_elems(int64_t M, int64_t N, int64_t K, int batch, int S, int 
   const bool fp8 = form == kFormFP8;
   const int64_t rows = swap ? N : M, cols = swap ? M : N;
   const int64_t bk = fp8 ? form_bk<kFormFP8>() : form_bk<kFormBF16>();
-  const size_t elems = (size_t)batch * S *
+  const size_t elems = (size_t)batch * split_planes(S, form) *
                        (round_up(rows, kTileM) + round_up(cols, fp8 ? Form<kFormFP8>::kBN : 64)) *
                        round_up(K, bk);
   return fp8 ? (elems + 1) / 2 : elems;

@@ -175,12 +175,12 @@ struct TunerScope {
 double gemm_flops(const GemmArgs& g);
 
 // --------------------------------------------------- split-precision GEMM
-// Same contract as gemm_f64 (c_upper / b_lower are computed in full), on the
-// tensor cores with the operands cut into S slices of one of three forms.
+// Same contract as gemm_f64, on the tensor cores with the operands cut into
+// slices of one of three forms.
 enum : int {
-  kFormBF16 = 0,   // S = 8 or 9 pre-scaled base-64 digits in BF16
-  kFormFP16 = 1,   // S = 8 raw base-128 digits in FP16
-  kFormFP8 = 2     // S = 11 raw base-32 digits in E4M3
+  kFormBF16 = 0,   // 7 (slices = 9) or 6 (slices = 8) base-256 digits in BF16
+  kFormFP16 = 1,   // 7 base-256 digits in FP16
+  kFormFP8 = 2     // 11 base-32 digits in E4M3
 };
 struct SplitWork {
   void* slices;          // slice planes
@@ -188,7 +188,7 @@ struct SplitWork {
   int* exps;             // per-row / per-column power-of-two exponents
   size_t exp_elems;
   int* err;              // device error flag (bounded waits)
-  int slices_s;          // S
+  int slices_s;          // the caller's slice count (9, 8 or 11; see split_planes)
   int form = kFormBF16;
   // test hook of the failure path: with stall = 1 the MMA issuer first waits,
   // for stall_ns, on an mbarrier that nothing arrives at, then takes the
@@ -202,6 +202,8 @@ struct SplitWork {
   bool throughput = false;
 };
 cudaError_t gemm_split(const GemmArgs& g, SplitWork& w, cudaStream_t st);
+// slice planes the caller's slice count stands for
+int split_planes(int slices, int form);
 // slice planes (16-bit units) one call of the given shape needs in a form
 size_t split_slice_elems(int64_t M, int64_t N, int64_t K, int batch, int S, int form = kFormBF16);
 // exponent entries (ints) one call of the given shape needs

@@ -1,5 +1,5 @@
 """Time one building-block GEMM of libzolo: C = op(A) op(B) in FP64 (DFMA) or
-split precision (nine BF16, eight FP16 or eleven FP8 slices on the tensor cores),
+split precision (seven BF16, seven FP16 or eleven FP8 slices on the tensor cores),
 through zolo_dgemm.
 
     python -m paper_1806_06204_gb300.profile_gemm --m 4096 --n 4096 --k 4096 --prec split
@@ -9,7 +9,7 @@ CUDA events on the current stream.  `--tune-cache F`: the FP64 kernel comes
 from the tuning file F when it holds this shape; otherwise the warm-up call
 measures the candidates (zolo_autotune) and F is written with the choice.  Prints one JSON line: milliseconds per
 call, FP64-equivalent TFLOP/s (2MNK per call), and for the split path the BF16
-tensor TFLOP/s actually issued (53, 36 or 76 slice-pair products; FP8 at twice
+tensor TFLOP/s actually issued (34, 28 or 76 slice-pair products; FP8 at twice
 the rate).  Also the launch
 target for kernel profilers: each call is one row-exponent + slicing pass per
 operand and one GEMM kernel (split), or one GEMM kernel (FP64).
@@ -80,9 +80,9 @@ def main():
     out = {"m": args.m, "n": args.n, "k": args.k, "prec": args.prec, "ms_per_call": ms,
            "fp64_equiv_tflops": flops / ms / 1e9}
     if args.prec == "split":
-        # slice-pair products issued: 53 (nine BF16 slices), 36 (eight FP16
-        # slices), 76 (eleven FP8 slices, whose peak is twice the 16-bit one)
-        pairs = {"bf16": 53, "fp16": 36, "fp8": 76}[args.slices]
+        # slice-pair products issued: 34 (seven 8-bit BF16 slices), 28 (seven 8-bit
+        # FP16 slices), 76 (eleven FP8 slices, whose peak is twice the 16-bit one)
+        pairs = {"bf16": 34, "fp16": 28, "fp8": 76}[args.slices]
         out["slices"] = args.slices
         out["tensor_issued_tflops"] = pairs * flops / ms / 1e9
     if kernel:
