@@ -20,9 +20,9 @@
 //
 // The leading levels (2..6 of the 8-bit digits, 2..9 of the 5-bit ones) are exact
 // over a K-chunk of 192 (4096) terms and are added to an int64 in units of 2^-48
-// after every chunk; the levels below go to one float (units of 2^-56 or 2^-65:
-// their FP32 rounding lies 2^-64 below the leading level).  At the end the two
-// are joined by one FP64 add, or in integers when one chunk held all of K, and
+// after every chunk; the levels below go to one float in units of 2^-56, whose FP32
+// rounding lies 2^-64 below the leading level.  At the end the two are joined in
+// integers, rounded once to FP64 and
 // scaled by 2^(e_i + f_j) through the exponent field.  The digit width was
 // measured on the CPU against exact products (rms error over row and column
 // maxima, K = 512, N(0,1) / Gram / operands graded over eight decades): 34 pairs
@@ -59,15 +59,15 @@ constexpr int kRowBytes = 128;     // one 128-byte swizzle row of K per tile row
 // (1-based) that goes to the int64, and the largest 0-based s + t kept.
 template <int FORM> struct Form;
 template <> struct Form<kFormBF16> {
-  static constexpr int kBits = 8, kElem = 2, kChunkK = 192, kIntTop = 6, kFloatUnit = 56;
+  static constexpr int kBits = 8, kElem = 2, kChunkK = 192, kIntTop = 6;
   __host__ __device__ static constexpr int top(int S) { return S; }
 };
 template <> struct Form<kFormFP16> {
-  static constexpr int kBits = 8, kElem = 2, kChunkK = 192, kIntTop = 6, kFloatUnit = 56;
+  static constexpr int kBits = 8, kElem = 2, kChunkK = 192, kIntTop = 6;
   __host__ __device__ static constexpr int top(int S) { return S - 1; }
 };
 template <> struct Form<kFormFP8> {
-  static constexpr int kBits = 5, kElem = 1, kChunkK = 4096, kBN = 32, kIntTop = 9, kFloatUnit = 65;
+  static constexpr int kBits = 5, kElem = 1, kChunkK = 4096, kBN = 32, kIntTop = 9;
   __host__ __device__ static constexpr int top(int S) { return S; }
 };
 template <int FORM> __host__ __device__ constexpr int form_bk() { return kRowBytes / Form<FORM>::kElem; }
@@ -386,64 +386,62 @@ slice_fused_kernel(const SliceOp a, const SliceOp b, int nblk_a, int K, int K_pa
 }
 
 // ----------------------------------------------------------------- GEMM
-// The epilogue's conversions by integer operations: FP64 instructions, int64
-// and float conversions to FP64 among them, go through the FP64 units, the
-// scarce ones on this part, and the epilogue of a product with a short K does
-// as much FP64 work per output as its MMAs do tensor work.
+// The epilogue's conversions: FP64 instructions, and conversions of int64 or float
+// to or from FP64, go through the FP64 units (2 lanes a clock), conversions of 32
+// bits and leading-zero counts through a unit of 16, and the epilogue of a product
+// with a short K has as much work per output as its MMAs.  So an output takes one
+// FP64 conversion (and the addend's FMA), the rest is plain integer work: an
+// all-integer conversion measured slower (45 more instructions per output).
 
-// d 2^k for results outside the normal range: powers of two applied in steps that
-// are exact until the last one rounds (inline: a call to ldexp would have every
-// live register of the epilogue saved around it).
-__device__ __forceinline__ double scale_steps(double d, int k) {
+// An output's exact value from its level sums: iacc in units of 2^-48 and fm in
+// units of 2^-56, as x 2^k with |x| < 2^63: the eight bits below iacc's unit are
+// kept while they fit, else they only decide the rounding (the last bit is set
+// when any of them is).  WIDE: fm may exceed 2^30.
+struct Fixed {
+  long long x;
+  int k;
+};
+template <bool WIDE>
+__device__ __forceinline__ Fixed split_fixed(long long iacc, float fm) {
+  long long hi;
+  int lo;
+  if (WIDE) {
+    const int fh = __float2int_rn(fm * 0x1p-16f);
+    const long long f = (long long)fh * 65536 + __float2int_rn(fmaf(-65536.f, (float)fh, fm));
+    hi = iacc + (f >> 8);
+    lo = (int)f & 255;
+  } else {
+    const int f = __float2int_rn(fm);
+    hi = iacc + (f >> 8);
+    lo = f & 255;
+  }
+  const bool big = (unsigned)((int)(hi >> 32) + (1 << 22)) >> 23 != 0;   // outside [-2^54, 2^54)
+  Fixed r;
+  r.x = big ? (hi | (lo != 0)) : ((hi << 8) | lo);
+  r.k = big ? -48 : -56;
+  return r;
+}
+
+// x 2^k rounded to nearest (ties to even), with the sign bit of flip (its high word)
+// toggled; *rare when the result is outside the normal range (its value is then
+// scale_steps').
+__device__ __forceinline__ double fixed_to_double(long long x, int k, unsigned flip, bool* rare) {
+  const double d = (double)x;
+  const int h = __double2hiint(d);
+  *rare |= h != 0 && (unsigned)(((h >> 20) & 0x7FF) + k - 1) >= 2045u;
+  return __hiloint2double((int)((unsigned)(h + (h != 0 ? k << 20 : 0)) ^ flip), __double2loint(d));
+}
+
+// x 2^k outside the normal range: powers of two applied in steps that are exact
+// until the last one rounds.
+__device__ __forceinline__ double scale_steps(long long x, int k) {
+  double d = (double)x;
   for (int i = 0; i < 3 && k != 0; ++i) {
     const int s = k < -1000 ? -1000 : (k > 1000 ? 1000 : k);
     d *= __longlong_as_double((long long)(1023 + s) << 52);
     k -= s;
   }
   return d;
-}
-
-// x 2^k for an int64 x, rounded to nearest (ties to even) like (double)x, then
-// scaled exactly: the leading one found by a count of leading zeros, 53 bits
-// kept, the exponent assembled; a result outside the normal range takes the
-// FP64 route.
-__device__ __forceinline__ double i64_scaled(long long x, int k) {
-  if (x == 0) return 0.0;
-  const unsigned long long sgn = x < 0 ? 0x8000000000000000ull : 0ull;
-  const unsigned long long a = x < 0 ? 0ull - (unsigned long long)x : (unsigned long long)x;
-  int msb = 63 - __clzll((long long)a);
-  unsigned long long m;
-  if (msb <= 52) {
-    m = a << (52 - msb);
-  } else {
-    const int sh = msb - 52;
-    const unsigned long long rem = a & ((1ull << sh) - 1ull), half = 1ull << (sh - 1);
-    m = a >> sh;
-    if (rem > half || (rem == half && (m & 1ull))) {
-      ++m;
-      if (m >> 53) {
-        m >>= 1;
-        ++msb;
-      }
-    }
-  }
-  const int be = msb + k + 1023;
-  if (be <= 0 || be >= 2047) return scale_steps((double)x, k);
-  return __longlong_as_double((long long)(sgn | ((unsigned long long)be << 52) | (m & 0xFFFFFFFFFFFFFull)));
-}
-
-// f 2^k for a float f, exact: the float's fields moved into an FP64 pattern
-// (zero keeps its sign; subnormal floats and results outside the normal range
-// take the FP64 route).
-__device__ __forceinline__ double f32_scaled(float f, int k) {
-  const unsigned u = __float_as_uint(f);
-  const unsigned long long sgn = (unsigned long long)(u >> 31) << 63;
-  if ((u & 0x7FFFFFFFu) == 0) return __longlong_as_double((long long)sgn);
-  const int ef = (int)((u >> 23) & 0xFFu);
-  const int be = ef - 127 + k + 1023;
-  if (ef == 0 || ef == 255 || be <= 0 || be >= 2047) return scale_steps((double)f, k);
-  return __longlong_as_double(
-      (long long)(sgn | ((unsigned long long)be << 52) | ((unsigned long long)(u & 0x7FFFFFu) << 29)));
 }
 
 struct SplitEpi {
@@ -531,26 +529,17 @@ __device__ __forceinline__ TilePos split_tile(const SplitEpi& p, int idx) {
   return t;
 }
 
-// The output of one entry from its exact level sums (iacc, units of 2^-48) and
-// its float part: scaled by 2^(e_i + f_j), then alpha.  one_chunk: both fit one
-// int64 in units of 2^-56, so no FP64 instruction is needed (the FP64 units give
-// 2 lanes a clock, and a short product's epilogue would wait for them).
-template <int FORM>
+// The output of one entry, any alpha and range: an Inf or NaN in the row of op(A)
+// or the column of op(B) leaves digits that carry no value, so the output is NaN (as
+// the FP64 product gives NaN or Inf there).
 __device__ __forceinline__ double split_value(const SplitEpi& p, long long iacc, float fm, int ei,
-                                              int ej, double al, bool one_chunk) {
-  using F = Form<FORM>;
-  const int e = ei + ej;
-  double v;
-  if (F::kFloatUnit == 56 && one_chunk)
-    v = i64_scaled((iacc << 8) + __float2ll_rn(fm), e - 56);
-  else
-    v = i64_scaled(iacc, e - 48) + f32_scaled(fm, e - F::kFloatUnit);
-  // an Inf or NaN in the row of op(A) or the column of op(B): the digits carry no
-  // value, so the output is NaN (as the FP64 product gives NaN or Inf there)
+                                              int ej, double al) {
+  const Fixed q = split_fixed<true>(iacc, fm);
+  bool rare = false;
+  double v = fixed_to_double(q.x, q.k + ei + ej, 0u, &rare);
+  if (rare) v = scale_steps(q.x, q.k + ei + ej);
   if (p.nan_rows && (ei >= 1026 || ej >= 1026)) v = __longlong_as_double(0x7FF8000000000000ll);
-  if (al == -1.0) v = __longlong_as_double(__double_as_longlong(v) ^ (long long)0x8000000000000000ull);
-  else if (al != 1.0) v *= al;
-  return v;
+  return v * al;
 }
 
 // Persistent: CTA b takes the tiles b, b + gridDim.x, ... (with a K split, cluster
@@ -781,6 +770,7 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     // of 2^-48 has room for 600 chunks of 192, 28 of 4096, at the digit bounds, and
     // gemm_split cuts a longer K into several products)
     constexpr int HALF = BN / (kEpiWarps / 4);     // columns of this warp
+    constexpr int kLd = HALF % 16 == 0 ? 16 : 8;   // columns per TMEM load
     const int q = warp & 3;
     const int half = (warp - 2) >> 2;              // which column slice
     const uint32_t lane_off = (uint32_t)(q * 32) << 16;
@@ -805,8 +795,25 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
       double* C = p.C + (int64_t)(p.reduce ? 0 : t.z) * p.strideC;
       const double* Cin = p.Cin ? p.Cin + (int64_t)(p.reduce ? 0 : t.z) * p.strideCin : nullptr;
       for (int b = b_first; b < b_last && ok; ++b) {
+        // the addends (beta C_in for the first entry, the running sum in C for the
+        // later ones of a reduced batch): their lines are brought to L2 before the
+        // chunks are waited for.  The strides are made opaque here: hoisted out of
+        // the loops, the columns' addresses would spill the accumulators.
+        const bool first = b == b_first;
+        const bool addend = p.ks == 1 && (!first || (Cin && p.beta != 0.0));
+        const int col0 = n0 + half * HALF;
+        const int jn = row < (p.swap ? p.N : p.M) ? (p.swap ? p.M : p.N) - col0 : 0;   // columns left
+        const int64_t ldi = first ? p.ldcin : p.ldc;
+        const double* ip0 = (first ? Cin : C) + (p.swap ? col0 + row * ldi : row + col0 * ldi);
+        int64_t st_i = p.swap ? 1 : ldi;
+        asm volatile("" : "+l"(st_i));
+        if (addend && (lane & 15) == 0 && !p.swap) {
+          const double* ip = ip0;
+#pragma unroll 4
+          for (int j = 0; j < HALF; ++j, ip += st_i)
+            if (j < jn) asm volatile("prefetch.global.L2 [%0];" ::"l"(ip));
+        }
         for (int c = 0; c < nchunks && ok; ++c, ++cg) {
-          constexpr int kLd = HALF % 16 == 0 ? 16 : 8;
 #pragma unroll
           for (int a = 0; a < kAcc; ++a) {
             if (!ok || !(ok = tc::mbar_wait(&lfull[a], cg & 1, err))) break;
@@ -819,10 +826,14 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
               else tc::tmem_ld8(tmem + lane_off + a * BN + half * HALF + g * kLd, v);
 #pragma unroll
               for (int i = 0; i < kLd; ++i) {
-                if (lv <= F::kIntTop)
-                  iacc[g * kLd + i] += (long long)__float2int_rn(v[i]) << (48 - F::kBits * lv);
-                else
-                  fm[g * kLd + i] += v[i] * __int_as_float((127 + F::kFloatUnit - F::kBits * lv) << 23);
+                // one 32 x 32 + 64 bit multiply-add per element
+                if (lv <= F::kIntTop) {
+                  const int sh = 48 - F::kBits * lv;
+                  if (sh < 31) iacc[g * kLd + i] += (long long)__float2int_rn(v[i]) * (long long)(1 << (sh < 31 ? sh : 0));
+                  else iacc[g * kLd + i] += (long long)__float2int_rn(v[i]) << sh;
+                } else {
+                  fm[g * kLd + i] += v[i] * __int_as_float((127 + 56 - F::kBits * lv) << 23);
+                }
               }
             }
             tc::tc_fence_before();
@@ -832,43 +843,77 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         }
         if (!ok) break;
         if (p.ks > 1) break;      // one entry per tile: joined over the cluster below
-        // end of a batch entry: scale, combine with beta C_in (first entry) or with
-        // the running sum already in C (reduce mode), write, reset
-        const bool first = b == b_first, one = nchunks == 1;
+        // end of a batch entry: scale, combine with the addend, write, reset.  The
+        // fast loop's FP64 work is one conversion and the addend's FMA (the sign of
+        // alpha = +-1 is a bit); a result outside the normal range, an Inf or NaN operand or
+        // another alpha sends the warp through the general loop after it.
         const int ei = p.ea[b * p.Mpad + row];
-        const int* ebb = p.eb + b * p.Npad + n0 + half * HALF;
-        const double al = p.alpha[b];
-        // four outputs at a time: their addends (beta C_in, or the running sum in
-        // reduce mode) loaded together first, then formed and stored (a load after
-        // a store to C could alias it, so a plain loop waits for each).  The strides
-        // are made opaque here: hoisted out of the loops, sixteen columns' addresses
-        // would spill the accumulators.
-        const bool use_cin = Cin && p.beta != 0.0;
-        const int col0 = n0 + half * HALF;
-        int64_t st_c = p.swap ? 1 : p.ldc, st_i = first ? (p.swap ? 1 : p.ldcin) : st_c;
-        asm volatile("" : "+l"(st_c), "+l"(st_i));
+        const int* ebb = p.eb + b * p.Npad + col0;
+        const double al = p.alpha[b], bt = first ? p.beta : 1.0;
+        const unsigned flip = al < 0.0 ? 0x80000000u : 0u;
+        const bool wide = p.K > 8192;   // |fm| < 2^30 up to there
+        const int nan_at = p.nan_rows ? 1026 : INT_MAX;
+        bool rare = al != 1.0 && al != -1.0;
+        int64_t st_c = p.swap ? 1 : p.ldc;
+        asm volatile("" : "+l"(st_c));
         double* cp = C + (p.swap ? col0 + row * p.ldc : row + col0 * p.ldc);
-        const double* ip = first ? Cin + (p.swap ? col0 + row * p.ldcin : row + col0 * p.ldcin) : cp;
-        const bool addend = !first || use_cin;
-        const double bt = first ? p.beta : 1.0;
-        const int jn = row < (p.swap ? p.N : p.M) ? (p.swap ? p.M : p.N) - col0 : 0;   // columns left
+        const double* ip = ip0;
+        constexpr int kAdd = 8;
+        double add[HALF > kAdd ? HALF : kAdd];
 #pragma unroll
-        for (int j0 = 0; j0 < HALF; j0 += 4) {
-          double add[4];
+        for (int j0 = 0; j0 < HALF; j0 += kAdd) {
+          // the addends of eight outputs first (a load after a store to C could alias
+          // it, so a plain loop waits for each)
+          if (addend) {
 #pragma unroll
-          for (int jj = 0; jj < 4; ++jj) {
-            add[jj] = addend && j0 + jj < jn ? *ip : 0.0;
-            ip += st_i;
+            for (int j = j0; j < j0 + kAdd; ++j) {
+              add[j] = j < jn ? *ip : 0.0;
+              ip += st_i;
+            }
+          }
+          double* cq = cp;
+          double v[kAdd];
+#pragma unroll
+          for (int jj = 0; jj < kAdd; ++jj) {
+            const int j = j0 + jj, ej = __ldg(ebb + j);
+            const Fixed q = wide ? split_fixed<true>(iacc[j], fm[j]) : split_fixed<false>(iacc[j], fm[j]);
+            v[jj] = fixed_to_double(q.x, q.k + ei + ej, flip, &rare);
+            rare |= max(ei, ej) >= nan_at;
+          }
+          if (addend) {
+#pragma unroll
+            for (int jj = 0; jj < kAdd; ++jj) v[jj] = fma(bt, add[j0 + jj], v[jj]);
           }
 #pragma unroll
-          for (int jj = 0; jj < 4; ++jj) {
-            const int j = j0 + jj;
-            if (j < jn) {
-              double v = split_value<FORM>(p, iacc[j], fm[j], ei, __ldg(ebb + j), al, one);
-              if (addend) v = fma(bt, add[jj], v);
-              *cp = v;
+          for (int jj = 0; jj < kAdd; ++jj) {
+            if (j0 + jj < jn) *cq = v[jj];
+            cq += st_c;
+          }
+          if (__any_sync(0xffffffffu, rare)) {
+            cq = cp;
+#pragma unroll 1
+            for (int jj = 0; jj < kAdd; ++jj) {
+              long long xi = 0;
+              float xf = 0.f;
+              double xa = 0.0;
+#pragma unroll
+              for (int u = 0; u < kAdd; ++u)
+                if (u == jj) {
+                  xi = iacc[j0 + u];
+                  xf = fm[j0 + u];
+                  if (addend) xa = add[j0 + u];
+                }
+              if (j0 + jj < jn) {
+                double w = split_value(p, xi, xf, ei, __ldg(ebb + j0 + jj), al);
+                if (addend) w = fma(bt, xa, w);
+                *cq = w;
+              }
+              cq += st_c;
             }
-            cp += st_c;
+          }
+          cp = cq;
+#pragma unroll
+          for (int j = j0; j < j0 + kAdd; ++j) {
             iacc[j] = 0;
             fm[j] = 0.f;
           }
@@ -911,8 +956,7 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
             si += cluster.map_shared_rank(part_i, k)[j * kTileM + r];
             sf += cluster.map_shared_rank(part_f, k)[j * kTileM + r];
           }
-          double v = split_value<FORM>(p, si, sf, ei, __ldg(p.eb + t.z * p.Npad + col), p.alpha[t.z],
-                                       false);
+          double v = split_value(p, si, sf, ei, __ldg(p.eb + t.z * p.Npad + col), p.alpha[t.z]);
           if (Cin && p.beta != 0.0) v = fma(p.beta, Cin[ci + (int64_t)cj * p.ldcin], v);
           C[ci + (int64_t)cj * p.ldc] = v;
         }
