@@ -24,8 +24,10 @@
 // structure makes zero is an exact zero in floating point too.
 #include <cooperative_groups.h>
 
+#include <atomic>
 #include <cmath>
 
+#include "fp64_scalar.cuh"
 #include "zolo_internal.h"
 
 namespace zolo {
@@ -460,6 +462,262 @@ qr_panel_smem_kernel(double* W, int64_t strideW, int64_t ldw, int64_t m, int64_t
   panel_sync<CG>(cluster);   // no CTA leaves while another may still read its partials
 }
 
+// ------------------------------------------------- register-resident panel
+// The panel factorisation with the panel's rows held in registers: lane q of every
+// warp owns column q, a warp owns rows, and the rows are dealt cyclically over NG =
+// RANKS x WARPS x SUB groups (RANKS CTAs of one cluster, WARPS warps each, SUB groups
+// per warp): group g holds the window's rows g, g + NG, g + 2 NG, ..., so the panel's
+// diagonal rows are row 0 of groups 0..31 (static register indices).
+//
+// What bounds a panel is the chain of one column to the next: FP64 instructions (64
+// clocks of a sub-partition's unit per warp, however few lanes are active) and the
+// exchanges between them.  So a column costs one pass, one reduction and one
+// exchange: the pass applies the previous reflector to a row, takes the row's new
+// entry x of column i by a shuffle and adds x a_q to every column's sum, which gives
+// x^T x and x^T a_q of the tail together (the lanes q < i, which hold finished
+// reflectors, yield V^T v for T at no cost).  With the tail sums s_q and the pivot
+// row's entries a_cq exchanged at once,
+//     beta = -sign(alpha) sqrt(alpha^2 + s_i),  tau = (beta - alpha) / beta,
+//     scal = 1 / (alpha - beta),   v^T a_q = a_cq + scal s_q,
+// and the update a_q -= tau (v^T a_q) v is -tau scal (v^T a_q) x below the pivot: the
+// reflectors stay unscaled until they are written.  Every warp forms the scalars
+// itself (one FP64 unit each), so a column has one CTA barrier and one cluster barrier.
+// The groups' sums are added in a fixed tree (4 groups, then the 8 fours), the same
+// for 8 CTAs x 4 warps x 1 group and for 1 CTA x 8 warps x 4 groups: the one-CTA form
+// of a batch and the cluster form of a single call give the same bits.
+// Measured, 32 columns of 256 / 1024 / 4096 / 8192 rows at r = 3: 98 / 138 / 279 / 436
+// us, against 325 / 285 / 440 / 1480 us of the shared-memory panel below (one CTA
+// under 512 rows, else eight) and the global-memory one; 256 rows on one CTA 264 us.
+template <int N>
+__device__ __forceinline__ double tree_sum(const double (&v)[N]) {
+  double t[N];
+#pragma unroll
+  for (int i = 0; i < N; ++i) t[i] = v[i];
+#pragma unroll
+  for (int h = 1; h < N; h *= 2)
+#pragma unroll
+    for (int i = 0; i + h < N; i += 2 * h) t[i] += t[i + h];
+  return t[0];
+}
+
+template <int RANKS, int WARPS, int SUB, int KMAX>
+__global__ void __launch_bounds__(WARPS * 32)
+qr_panel_reg_kernel(double* W, int64_t strideW, int64_t ldw, int64_t m, int64_t c0, int nbp,
+                    double* V, int64_t strideV, int64_t ldv, double* T, int64_t strideT,
+                    int* status, int kr) {
+  constexpr int NB = 32, NG = RANKS * WARPS * SUB;
+  static_assert(NG >= NB, "the diagonal rows are row 0 of their groups");
+  namespace cgrp = cooperative_groups;
+  cgrp::cluster_group cluster = cgrp::this_cluster();
+  __shared__ double red[2][WARPS][NB];
+  __shared__ double part[2][RANKS][NB];
+  __shared__ double piv[2][NB];
+  __shared__ double Gs[NB][NB + 1], Ts[NB][NB + 1], Ys[NB][NB + 1];
+  __shared__ double taus[NB];
+  const int rank = RANKS > 1 ? (int)cluster.block_rank() : 0;
+  const int shift = blockIdx.x / RANKS;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int g0 = (rank * WARPS + warp) * SUB;          // this warp's groups g0 .. g0 + SUB - 1
+  double* Wj = W + shift * strideW + c0 + (c0 + lane) * ldw;
+  double* Vp = V + shift * strideV + (c0 + lane) * ldv;
+  const int64_t H = m + NB;                            // window rows
+  const int64_t rows = ldw - c0 < H ? ldw - c0 : H;    // those that exist in W
+
+  double a[SUB][KMAX];
+#pragma unroll
+  for (int s = 0; s < SUB; ++s)
+#pragma unroll
+    for (int k = 0; k < KMAX; ++k) {
+      const int64_t r = g0 + s + (int64_t)NG * k;
+      a[s][k] = (k < kr && lane < nbp && r < rows) ? Wj[r] : 0.0;
+    }
+  // f: what the pivot row of the previous column adds to this lane's column; cf: the
+  // factor of the rows below it; scal_q: the scale of this lane's own reflector
+  double f = 0.0, cf = 0.0, scal_q = 0.0, beta = 0.0;
+  for (int e = threadIdx.x; e < NB * (NB + 1); e += WARPS * 32) (&Ts[0][0])[e] = (&Gs[0][0])[e] = 0.0;
+  // no rank writes to another's shared memory before that one runs
+  if constexpr (RANKS > 1) cluster.sync();
+  else __syncthreads();
+
+  for (int i = 0; i < nbp; ++i) {
+    const int buf = i & 1;
+    double acc[SUB];
+#pragma unroll
+    for (int s = 0; s < SUB; ++s) {
+      const int g = g0 + s;
+      double t = 0.0;
+      {
+        double v = a[s][0];
+        const double xo = __shfl_sync(0xffffffffu, v, i > 0 ? i - 1 : 0);
+        if (i > 0) {
+          if (g > i - 1) v = fma(cf, xo, v);
+          else if (g == i - 1) v = lane == i - 1 ? beta : v + f;
+          a[s][0] = v;
+        }
+        const double x = __shfl_sync(0xffffffffu, v, i);
+        if (g > i) t = x * v;
+        if (g == i) {   // the pivot row goes to every rank
+          if constexpr (RANKS > 1) {
+            for (int q = 0; q < RANKS; ++q) cluster.map_shared_rank(&piv[buf][0], q)[lane] = v;
+          } else {
+            piv[buf][lane] = v;
+          }
+        }
+      }
+#pragma unroll
+      for (int k = 1; k < KMAX; ++k) {
+        if (k < kr) {
+          double v = a[s][k];
+          const double xo = __shfl_sync(0xffffffffu, v, i > 0 ? i - 1 : 0);
+          v = fma(cf, xo, v);
+          a[s][k] = v;
+          t = fma(__shfl_sync(0xffffffffu, v, i), v, t);
+        }
+      }
+      acc[s] = t;
+    }
+    red[buf][warp][lane] = tree_sum(acc);
+    __syncthreads();
+    double total;
+    {
+      double w[WARPS];
+#pragma unroll
+      for (int q = 0; q < WARPS; ++q) w[q] = red[buf][q][lane];
+      total = tree_sum(w);
+    }
+    if constexpr (RANKS > 1) {
+      for (int q = warp; q < RANKS; q += WARPS)
+        cluster.map_shared_rank(&part[buf][rank][0], q)[lane] = total;
+      cluster.sync();
+      double w[RANKS];
+#pragma unroll
+      for (int q = 0; q < RANKS; ++q) w[q] = part[buf][q][lane];
+      total = tree_sum(w);
+    }
+    const double pv = piv[buf][lane];
+    const double alpha = __shfl_sync(0xffffffffu, pv, i), ss = __shfl_sync(0xffffffffu, total, i);
+    double tau = 0.0, scal = 0.0;
+    if (ss == 0.0) {
+      beta = alpha;
+    } else {
+      const double n2 = fma(alpha, alpha, ss);
+      double nrm, inv;
+      if (n2 > 1e-280 && n2 < 1e280) {
+        root_pair(n2, &nrm, &inv);
+        beta = -copysign(nrm, alpha);
+        tau = (beta - alpha) * -copysign(inv, alpha);
+        scal = reciprocal(alpha - beta);
+      } else {   // near the ends of the range, or not finite
+        beta = -copysign(sqrt(n2), alpha);
+        tau = (beta - alpha) / beta;
+        scal = 1.0 / (alpha - beta);
+      }
+    }
+    const double dot = fma(scal, total, pv);   // v^T a_q; unscaled x_q^T v for q < i
+    f = lane > i ? -tau * dot : 0.0;
+    cf = f * scal;
+    if (rank == 0 && warp == 0) {
+      if (lane < i) Gs[lane][i] = scal_q * dot;
+      if (lane == i) {
+        taus[i] = tau;
+        if (!isfinite(beta) || !isfinite(tau)) atomicOr(status + kStatNonFinite, 1);
+      }
+    }
+    if (lane == i) scal_q = scal;
+  }
+  // ---- the explicit reflectors (unit diagonal, exact zeros above it) and R's rows
+#pragma unroll
+  for (int s = 0; s < SUB; ++s) {
+    const int g = g0 + s;
+    if (lane < nbp) {
+      double v = a[s][0];
+      if (g == nbp - 1 && lane == nbp - 1) v = beta;
+      if (g < NB && g <= lane && g < rows) Wj[g] = v;
+      if (g < H) Vp[g] = g < lane ? 0.0 : (g == lane ? 1.0 : scal_q * v);
+#pragma unroll
+      for (int k = 1; k < KMAX; ++k) {
+        const int64_t r = g + (int64_t)NG * k;
+        if (k < kr && r < H) Vp[r] = scal_q * a[s][k];
+      }
+    }
+  }
+  if (rank != 0) return;
+  // ---- T: 8 x 8 diagonal blocks row by row (T_ij = -tau_j sum_p T_ip G_pj), then
+  //      pairs merged as -T_11 (G_12 T_22), 8 -> 16 -> 32
+  __syncthreads();
+  if (warp == 0) {
+    const int b0 = lane & 24;
+    double t[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int c = b0 + j;
+      const double tj = c < nbp ? taus[c] : 0.0;
+      double sum = 0.0;
+#pragma unroll
+      for (int q = 0; q < 8; ++q)
+        if (q < j && b0 + q >= lane) sum = fma(t[q], Gs[b0 + q][c], sum);
+      t[j] = c == lane ? tj : (c > lane ? -tj * sum : 0.0);
+      Ts[lane][c] = t[j];
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int h = 8; h < NB; h *= 2) {
+    const int outs = (NB / (2 * h)) * h * h;
+    for (int e = threadIdx.x; e < outs; e += WARPS * 32) {
+      const int pr = e / (h * h), x = e % (h * h), r = pr * 2 * h + x % h, c = pr * 2 * h + h + x / h;
+      double y = 0.0;   // (G_12 T_22)(r, c)
+#pragma unroll
+      for (int q = 0; q < h; ++q) y = fma(Gs[r][pr * 2 * h + h + q], Ts[pr * 2 * h + h + q][c], y);
+      Ys[r][c] = y;
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < outs; e += WARPS * 32) {
+      const int pr = e / (h * h), x = e % (h * h), r = pr * 2 * h + x % h, c = pr * 2 * h + h + x / h;
+      double y = 0.0;
+#pragma unroll
+      for (int q = 0; q < h; ++q) y = fma(Ts[r][pr * 2 * h + q], Ys[pr * 2 * h + q][c], y);
+      Ts[r][c] = -y;
+    }
+    __syncthreads();
+  }
+  double* Tp = T + shift * strideT + (c0 / NB) * (int64_t)(NB * NB);
+  for (int e = threadIdx.x; e < NB * NB; e += WARPS * 32) Tp[e] = Ts[e % NB][e / NB];
+}
+
+struct PanelArgs {
+  double* W; int64_t strideW, ldw, m, c0; int nbp;
+  double* V; int64_t strideV, ldv; double* T; int64_t strideT; int* status;
+};
+
+template <int RANKS, int WARPS, int SUB, int KMAX>
+cudaError_t launch_panel_reg(const PanelArgs& p, int r, double flops, double bytes, cudaStream_t st) {
+  const auto kernel = qr_panel_reg_kernel<RANKS, WARPS, SUB, KMAX>;
+  constexpr int NG = RANKS * WARPS * SUB;
+  const int kr = (int)((p.m + kQrNB + NG - 1) / NG);
+  if (kr > KMAX) return cudaErrorInvalidValue;
+  ProfScope ps(kProfPanel, st, flops, bytes);
+  ps.blocks((const void*)kernel, dim3(WARPS * 32), 0, dim3(r * RANKS));
+  if (RANKS == 1) {
+    kernel<<<r, WARPS * 32, 0, st>>>(p.W, p.strideW, p.ldw, p.m, p.c0, p.nbp, p.V, p.strideV, p.ldv,
+                                     p.T, p.strideT, p.status, kr);
+    return cudaGetLastError();
+  }
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(r * RANKS);
+  cfg.blockDim = dim3(WARPS * 32);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = RANKS;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, p.W, p.strideW, p.ldw, p.m, p.c0, p.nbp, p.V, p.strideV,
+                            p.ldv, p.T, p.strideT, p.status, kr);
+}
+
 // C <- (I - V op(T) V^T) C for r shifts, on the row window of C, as
 // W1 = V^T C, W2 = op(T) W1, C -= V W2 (transT = 1 applies Q^T, the
 // factorisation's update; transT = 0 applies Q, the explicit-Q build).
@@ -499,6 +757,70 @@ cudaError_t apply_block(const QrBuffers& b, const double* Vw, int64_t ldv, const
 
 }  // namespace
 
+namespace {
+
+// The register panel that serves m rows, or kRegNone.  Below 512 rows a single call
+// takes a cluster of 8 CTAs and a batch one CTA (the same bits); from there a single
+// call takes 16 CTAs while a thread's rows fit in its registers, and a batch keeps the
+// shared-memory panel on the fewest CTAs.  Seven clusters of 16 find room at once
+// (4096 rows: 279 us up to there, 525 us with eight, in two rounds), so eight shifts
+// take 8 CTAs (399 us).
+enum PanelKind { kRegNone, kReg1x17, kReg8x17, kReg8x33, kReg8w33, kReg8w65, kReg8w97,
+                 kReg16x17, kReg16x33, kReg16w33, kReg16w65, kReg16w97 };
+PanelKind panel_kind(int64_t m, int r, bool narrow) {
+  const int64_t H = m + kQrNB;
+  if (m < kClusterPanelMinRows) return narrow ? kReg1x17 : kReg8x17;
+  if (narrow) return kRegNone;
+  if (r > 7) {
+    if (H <= 32 * 33) return kReg8x33;
+    if (H <= 64 * 33) return kReg8w33;
+    if (H <= 64 * 65) return kReg8w65;
+    if (H <= 64 * 97) return kReg8w97;
+  }
+  if (H <= 64 * 17) return kReg16x17;
+  if (H <= 64 * 33) return kReg16x33;
+  if (H <= 128 * 33) return kReg16w33;
+  if (H <= 128 * 65) return kReg16w65;
+  if (H <= 128 * 97) return kReg16w97;
+  return kRegNone;
+}
+
+// Clusters of 16 CTAs are beyond the portable size: allowed once per device.
+cudaError_t allow_clusters16() {
+  static std::atomic<uint64_t> done{0};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 64 && (done.load() >> dev & 1)) return cudaSuccess;
+  const void* k[] = {(const void*)qr_panel_reg_kernel<16, 4, 1, 17>, (const void*)qr_panel_reg_kernel<16, 4, 1, 33>,
+                     (const void*)qr_panel_reg_kernel<16, 8, 1, 33>, (const void*)qr_panel_reg_kernel<16, 8, 1, 65>,
+                     (const void*)qr_panel_reg_kernel<16, 8, 1, 97>};
+  for (const void* f : k)
+    if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess)
+      return e;
+  if (dev < 64) done.fetch_or(1ull << dev);
+  return cudaSuccess;
+}
+
+cudaError_t launch_panel(PanelKind k, const PanelArgs& p, int r, double fl, double by, cudaStream_t st) {
+  switch (k) {
+    case kReg1x17: return launch_panel_reg<1, 8, 4, 17>(p, r, fl, by, st);
+    case kReg8x17: return launch_panel_reg<8, 4, 1, 17>(p, r, fl, by, st);
+    case kReg8x33: return launch_panel_reg<8, 4, 1, 33>(p, r, fl, by, st);
+    case kReg8w33: return launch_panel_reg<8, 8, 1, 33>(p, r, fl, by, st);
+    case kReg8w65: return launch_panel_reg<8, 8, 1, 65>(p, r, fl, by, st);
+    case kReg8w97: return launch_panel_reg<8, 8, 1, 97>(p, r, fl, by, st);
+    case kReg16x17: return launch_panel_reg<16, 4, 1, 17>(p, r, fl, by, st);
+    case kReg16x33: return launch_panel_reg<16, 4, 1, 33>(p, r, fl, by, st);
+    case kReg16w33: return launch_panel_reg<16, 8, 1, 33>(p, r, fl, by, st);
+    case kReg16w65: return launch_panel_reg<16, 8, 1, 65>(p, r, fl, by, st);
+    case kReg16w97: return launch_panel_reg<16, 8, 1, 97>(p, r, fl, by, st);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+}  // namespace
+
 cudaError_t structured_qr_q(const QrBuffers& b, int64_t m, int64_t n, int r, int* status,
                             cudaStream_t st, bool explicit_q, bool narrow_panels) {
   constexpr int NB = kQrNB, NBb = kQrBlock;
@@ -507,28 +829,23 @@ cudaError_t structured_qr_q(const QrBuffers& b, int64_t m, int64_t n, int r, int
     if (smem_attr_once((const void*)qr_panel_smem_kernel<NB, 2>, bytes) != cudaSuccess ||
         smem_attr_once((const void*)qr_panel_smem_kernel<NB, 4>, bytes) != cudaSuccess ||
         smem_attr_once((const void*)qr_panel_smem_kernel<NB, 1>, bytes) != cudaSuccess ||
-        smem_attr_once((const void*)qr_panel_smem_kernel<NB, kPanelCluster>, bytes) != cudaSuccess)
+        smem_attr_once((const void*)qr_panel_smem_kernel<NB, kPanelCluster>, bytes) != cudaSuccess ||
+        allow_clusters16() != cudaSuccess)
       return cudaErrorInvalidConfiguration;
   }
   const int64_t ldw = m + n;
   const int64_t ldv = m + NBb;
   cudaError_t err;
   const int nblocks = (int)((n + NBb - 1) / NBb);
-  // CTAs per shift of the panel kernel.  The panel is a chain of dependent
-  // column steps on a few SMs.  Alone (one matrix, r shifts in flight) it goes
-  // fastest on an 8-CTA cluster, which splits each column's rows eight ways;
-  // when many problems are in flight (narrow_panels) the same SMs serve more
-  // panels at once with the fewest CTAs whose rows fit in shared memory (one
-  // CTA up to m = 736, two up to 1504).  0: the global-memory cluster kernel.
+  // The register panel where there is one; else, with many problems in flight
+  // (narrow_panels), the shared-memory panel on the fewest CTAs whose rows fit (one
+  // CTA up to m = 736, two up to 1504): the same SMs then serve more panels at once.
+  // cg = 0: the global-memory cluster kernel.
+  const PanelKind reg = panel_kind(m, r, narrow_panels);
   int cg = 0;
-  if (narrow_panels) {
+  if (narrow_panels && reg == kRegNone)
     for (int c = 1; c <= kPanelCluster; c *= 2)
       if ((m + NB + c - 1) / c <= kSmemPanelRows) { cg = c; break; }
-  } else if (m + NB <= kSmemPanelRows && m < kClusterPanelMinRows) {
-    cg = 1;
-  } else if ((m + NB + kPanelCluster - 1) / kPanelCluster <= kSmemPanelRows) {
-    cg = kPanelCluster;
-  }
   const int64_t rows_cta = cg ? (m + NB + cg - 1) / cg : 0;
   // every V entry outside the rows a panel writes must be an exact zero
   if ((err = cudaMemsetAsync(b.V, 0, sizeof(double) * r * b.strideV, st)) != cudaSuccess) return err;
@@ -541,9 +858,12 @@ cudaError_t structured_qr_q(const QrBuffers& b, int64_t m, int64_t n, int r, int
       const int nbp = nbb - p * NB < NB ? nbb - p * NB : NB;
       // V rows are relative to the block start: this panel's window starts p*NB down
       double* Vpan = b.V + (int64_t)p * NB;
-      {
-        ProfScope ps(kProfPanel, st, 3.0 * r * (double)(m + 1) * nbp * nbp,
-                     8.0 * r * (double)(m + NB) * nbp * 2.0);
+      const double pf = 3.0 * r * (double)(m + 1) * nbp * nbp, pb = 16.0 * r * (double)(m + NB) * nbp;
+      if (reg != kRegNone) {
+        const PanelArgs pa{b.W, b.strideW, ldw, m, c0, nbp, Vpan, b.strideV, ldv, b.T, b.strideT, status};
+        if ((err = launch_panel(reg, pa, r, pf, pb, st)) != cudaSuccess) return err;
+      } else {
+        ProfScope ps(kProfPanel, st, pf, pb);
         const size_t smem = sizeof(double) * NB * rows_cta;
         if (cg == 0)
           ps.blocks((const void*)qr_panel_cluster_kernel<NB, kPanelCluster, 512>, dim3(512), 0,
