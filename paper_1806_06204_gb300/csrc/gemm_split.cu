@@ -20,8 +20,8 @@
 //
 // The leading levels (2..6 of the 8-bit digits, 2..9 of the 5-bit ones) are exact
 // over a K-chunk of 192 (4096) terms and are added to an int64 in units of 2^-48
-// after every chunk; the levels below go to one float in units of 2^-56, whose FP32
-// rounding lies 2^-64 below the leading level.  At the end the two are joined in
+// after every chunk; the levels below go to one float in units of 2^-56 (2^-65),
+// whose FP32 rounding lies 2^-64 below the leading level.  At the end the two are joined in
 // integers, rounded once to FP64 and
 // scaled by 2^(e_i + f_j) through the exponent field.  The digit width was
 // measured on the CPU against exact products (rms error over row and column
@@ -59,15 +59,15 @@ constexpr int kRowBytes = 128;     // one 128-byte swizzle row of K per tile row
 // (1-based) that goes to the int64, and the largest 0-based s + t kept.
 template <int FORM> struct Form;
 template <> struct Form<kFormBF16> {
-  static constexpr int kBits = 8, kElem = 2, kChunkK = 192, kIntTop = 6;
+  static constexpr int kBits = 8, kElem = 2, kChunkK = 192, kIntTop = 6, kLo = 8;
   __host__ __device__ static constexpr int top(int S) { return S; }
 };
 template <> struct Form<kFormFP16> {
-  static constexpr int kBits = 8, kElem = 2, kChunkK = 192, kIntTop = 6;
+  static constexpr int kBits = 8, kElem = 2, kChunkK = 192, kIntTop = 6, kLo = 8;
   __host__ __device__ static constexpr int top(int S) { return S - 1; }
 };
 template <> struct Form<kFormFP8> {
-  static constexpr int kBits = 5, kElem = 1, kChunkK = 4096, kBN = 32, kIntTop = 9;
+  static constexpr int kBits = 5, kElem = 1, kChunkK = 4096, kBN = 32, kIntTop = 9, kLo = 17;
   __host__ __device__ static constexpr int top(int S) { return S; }
 };
 template <int FORM> __host__ __device__ constexpr int form_bk() { return kRowBytes / Form<FORM>::kElem; }
@@ -393,30 +393,41 @@ slice_fused_kernel(const SliceOp a, const SliceOp b, int nblk_a, int K, int K_pa
 // FP64 conversion (and the addend's FMA), the rest is plain integer work: an
 // all-integer conversion measured slower (45 more instructions per output).
 
-// An output's exact value from its level sums: iacc in units of 2^-48 and fm in
-// units of 2^-56, as x 2^k with |x| < 2^63: the eight bits below iacc's unit are
-// kept while they fit, else they only decide the rounding (the last bit is set
-// when any of them is).  WIDE: fm may exceed 2^30.
+// An output's value from its level sums, iacc in units of 2^-48 and fm in units of
+// 2^-(48 + LO), as x 2^k with |x| < 2^63: the LO bits below iacc's unit are kept while
+// they fit; where x has 53 bits and more without them, they only decide the rounding
+// (the last bit is set when any of them is).  WIDE: fm may exceed 2^30.
 struct Fixed {
   long long x;
   int k;
 };
-template <bool WIDE>
+// whether hi is outside [-2^b, 2^b)
+template <int B>
+__device__ __forceinline__ bool beyond(long long hi) {
+  return (unsigned)((int)(hi >> 32) + (1 << (B - 32))) >> (B - 31) != 0;
+}
+template <int LO, bool WIDE>
 __device__ __forceinline__ Fixed split_fixed(long long iacc, float fm) {
   long long hi;
   int lo;
   if (WIDE) {
     const int fh = __float2int_rn(fm * 0x1p-16f);
     const long long f = (long long)fh * 65536 + __float2int_rn(fmaf(-65536.f, (float)fh, fm));
-    hi = iacc + (f >> 8);
-    lo = (int)f & 255;
+    hi = iacc + (f >> LO);
+    lo = (int)f & ((1 << LO) - 1);
   } else {
     const int f = __float2int_rn(fm);
-    hi = iacc + (f >> 8);
-    lo = f & 255;
+    hi = iacc + (f >> LO);
+    lo = f & ((1 << LO) - 1);
   }
-  const bool big = (unsigned)((int)(hi >> 32) + (1 << 22)) >> 23 != 0;   // outside [-2^54, 2^54)
   Fixed r;
+  if (LO > 8 && !beyond<62 - LO>(hi)) {
+    r.x = (hi << LO) | lo;
+    r.k = -48 - LO;
+    return r;
+  }
+  if (LO > 8) lo = (lo >> (LO - 8)) | ((lo & ((1 << (LO - 8)) - 1)) != 0);
+  const bool big = beyond<54>(hi);
   r.x = big ? (hi | (lo != 0)) : ((hi << 8) | lo);
   r.k = big ? -48 : -56;
   return r;
@@ -532,9 +543,10 @@ __device__ __forceinline__ TilePos split_tile(const SplitEpi& p, int idx) {
 // The output of one entry, any alpha and range: an Inf or NaN in the row of op(A)
 // or the column of op(B) leaves digits that carry no value, so the output is NaN (as
 // the FP64 product gives NaN or Inf there).
+template <int FORM>
 __device__ __forceinline__ double split_value(const SplitEpi& p, long long iacc, float fm, int ei,
                                               int ej, double al) {
-  const Fixed q = split_fixed<true>(iacc, fm);
+  const Fixed q = split_fixed<Form<FORM>::kLo, true>(iacc, fm);
   bool rare = false;
   double v = fixed_to_double(q.x, q.k + ei + ej, 0u, &rare);
   if (rare) v = scale_steps(q.x, q.k + ei + ej);
@@ -832,7 +844,7 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
                   if (sh < 31) iacc[g * kLd + i] += (long long)__float2int_rn(v[i]) * (long long)(1 << (sh < 31 ? sh : 0));
                   else iacc[g * kLd + i] += (long long)__float2int_rn(v[i]) << sh;
                 } else {
-                  fm[g * kLd + i] += v[i] * __int_as_float((127 + 56 - F::kBits * lv) << 23);
+                  fm[g * kLd + i] += v[i] * __int_as_float((127 + 48 + F::kLo - F::kBits * lv) << 23);
                 }
               }
             }
@@ -851,7 +863,7 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         const int* ebb = p.eb + b * p.Npad + col0;
         const double al = p.alpha[b], bt = first ? p.beta : 1.0;
         const unsigned flip = al < 0.0 ? 0x80000000u : 0u;
-        const bool wide = p.K > 8192;   // |fm| < 2^30 up to there
+        const bool wide = F::kLo > 8 || p.K > 8192;   // |fm| < 2^30 up to there
         const int nan_at = p.nan_rows ? 1026 : INT_MAX;
         bool rare = al != 1.0 && al != -1.0;
         int64_t st_c = p.swap ? 1 : p.ldc;
@@ -876,7 +888,8 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
 #pragma unroll
           for (int jj = 0; jj < kAdd; ++jj) {
             const int j = j0 + jj, ej = __ldg(ebb + j);
-            const Fixed q = wide ? split_fixed<true>(iacc[j], fm[j]) : split_fixed<false>(iacc[j], fm[j]);
+            const Fixed q = wide ? split_fixed<F::kLo, true>(iacc[j], fm[j])
+                                 : split_fixed<F::kLo, false>(iacc[j], fm[j]);
             v[jj] = fixed_to_double(q.x, q.k + ei + ej, flip, &rare);
             rare |= max(ei, ej) >= nan_at;
           }
@@ -904,7 +917,7 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
                   if (addend) xa = add[j0 + u];
                 }
               if (j0 + jj < jn) {
-                double w = split_value(p, xi, xf, ei, __ldg(ebb + j0 + jj), al);
+                double w = split_value<FORM>(p, xi, xf, ei, __ldg(ebb + j0 + jj), al);
                 if (addend) w = fma(bt, xa, w);
                 *cq = w;
               }
@@ -956,7 +969,7 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
             si += cluster.map_shared_rank(part_i, k)[j * kTileM + r];
             sf += cluster.map_shared_rank(part_f, k)[j * kTileM + r];
           }
-          double v = split_value(p, si, sf, ei, __ldg(p.eb + t.z * p.Npad + col), p.alpha[t.z]);
+          double v = split_value<FORM>(p, si, sf, ei, __ldg(p.eb + t.z * p.Npad + col), p.alpha[t.z]);
           if (Cin && p.beta != 0.0) v = fma(p.beta, Cin[ci + (int64_t)cj * p.ldcin], v);
           C[ci + (int64_t)cj * p.ldc] = v;
         }
