@@ -718,6 +718,29 @@ cudaError_t launch_panel_reg(const PanelArgs& p, int r, double flops, double byt
                             p.ldv, p.T, p.strideT, p.status, kr);
 }
 
+// The products the block reflectors' T factors and a panel's own update hang on: in
+// FP64, or for the 16-bit forms on the tensor cores with the more accurate slices (the
+// BF16 form's 34 pairs), where the router expects a gain.  4096^2 at r = 8: 31.0 -> 4.2
+// ms of FP64 work for 5 ms of split products; backward errors of 256^2 .. 3000 x 500
+// matrices, kappa 1e2 .. 1e12: 1.3 .. 1.6e-15 (BF16) as with FP64 here.  The FP8 form's
+// own products are more accurate still (its errors grew by 2 to 9%): it keeps FP64.
+SplitWork fine_engine(const SplitWork& w) {
+  SplitWork f = w;
+  f.form = kFormBF16;
+  f.slices_s = 9;
+  return f;
+}
+bool gemm_fine_splits(const GemmArgs& g) {
+  const SplitWork* w = get_split_engine();
+  return w && w->form != kFormFP8 && split_preferred(g, fine_engine(*w));
+}
+cudaError_t gemm_fine(const GemmArgs& g, cudaStream_t st) {
+  SplitWork* w = get_split_engine();
+  if (!gemm_fine_splits(g)) return gemm_f64(g, st);
+  SplitWork f = fine_engine(*w);
+  return gemm_split(g, f, st);
+}
+
 // C <- (I - V op(T) V^T) C for r shifts, on the row window of C, as
 // W1 = V^T C, W2 = op(T) W1, C -= V W2 (transT = 1 applies Q^T, the
 // factorisation's update; transT = 0 applies Q, the explicit-Q build).
@@ -732,9 +755,7 @@ cudaError_t apply_block(const QrBuffers& b, const double* Vw, int64_t ldv, const
   g.Cout = b.W1; g.ldcout = kQrBlock; g.strideCout = b.strideW1;
   g.batch = r;
   for (int j = 0; j < r; ++j) g.alpha[j] = 1.0;
-  // a panel's own block: a skinny output over the whole window, in FP64 on every
-  // path (few outputs, split over K across the SMs)
-  err = w <= 32 && ncols <= 96 ? gemm_f64(g, st) : gemm_any(g, st);
+  err = w <= kQrNB ? gemm_fine(g, st) : gemm_any(g, st);
   if (err != cudaSuccess) return err;
   GemmArgs h = g;
   h.K = w; h.transA = transT;
@@ -910,28 +931,37 @@ cudaError_t structured_qr_q(const QrBuffers& b, int64_t m, int64_t n, int r, int
     }
     if ((err = cudaGetLastError()) != cudaSuccess) return err;
     if (nbb > NB) {
-      // the blocks of G = V_b^T V_b that the merges read: [0,32)x[32,64),
-      // [64,96)x[96,128) and [0,64)x[64,128) (clipped to the block), in FP64 on
-      // every path: they are small next to the columns' norms, and T_b carries
-      // their error into every update
+      // G = V_b^T V_b for the merges (they read the blocks [0,32)x[32,64),
+      // [64,96)x[96,128) and [0,64)x[64,128)): small next to the columns' norms, and
+      // T_b carries its error into every update.  On the FP64 pipe those three blocks
+      // alone; on the tensor cores one product.
       static_assert(kQrBlock == 4 * kQrNB, "the merge levels assume four panels per block");
-      auto gram = [&](int i0, int j0, int mt, int nt, int inner) {
-        GemmArgs g;
-        g.M = mt; g.N = nt; g.K = (int)(m + nbb); g.transA = 1;
-        g.A = Vb + i0 * ldv; g.lda = ldv; g.strideA = b.strideV;
-        g.B = Vb + j0 * ldv; g.ldb = ldv; g.strideB = b.strideV;
-        g.Cout = b.G + i0 + j0 * NBb; g.ldcout = NBb; g.strideCout = b.strideG;
-        g.batch = r;
-        g.inner = inner;
-        g.innerA = g.innerB = 2 * NB * ldv; g.innerC = 2 * NB + 2 * NB * NBb;
-        for (int j = 0; j < r; ++j) g.alpha[j] = 1.0;
-        return gemm_f64(g, st);
-      };
-      const int n01 = nbb - NB < NB ? nbb - NB : NB, n23 = nbb - 3 * NB;
-      // the two 32-wide pairs in one launch when both are whole
-      if ((err = gram(0, NB, NB, n01, n23 >= NB ? 2 : 1)) != cudaSuccess) return err;
-      if (n23 > 0 && n23 < NB && (err = gram(2 * NB, 3 * NB, NB, n23, 1)) != cudaSuccess) return err;
-      if (nbb > 2 * NB && (err = gram(0, 2 * NB, 2 * NB, nbb - 2 * NB, 1)) != cudaSuccess) return err;
+      GemmArgs g;
+      g.M = g.N = nbb; g.K = (int)(m + nbb); g.transA = 1;
+      g.A = g.B = Vb; g.lda = g.ldb = ldv; g.strideA = g.strideB = b.strideV;
+      g.Cout = b.G; g.ldcout = NBb; g.strideCout = b.strideG;
+      g.batch = r; g.c_upper = 1;
+      for (int j = 0; j < r; ++j) g.alpha[j] = 1.0;
+      if (gemm_fine_splits(g)) {
+        if ((err = gemm_fine(g, st)) != cudaSuccess) return err;
+      } else {
+        g.c_upper = 0;
+        auto gram = [&](int i0, int j0, int mt, int nt, int inner) {
+          GemmArgs q = g;
+          q.M = mt; q.N = nt;
+          q.A = Vb + i0 * ldv;
+          q.B = Vb + j0 * ldv;
+          q.Cout = b.G + i0 + j0 * NBb;
+          q.inner = inner;
+          q.innerA = q.innerB = 2 * NB * ldv; q.innerC = 2 * NB + 2 * NB * NBb;
+          return gemm_f64(q, st);
+        };
+        const int n01 = nbb - NB < NB ? nbb - NB : NB, n23 = nbb - 3 * NB;
+        // the two 32-wide pairs in one launch when both are whole
+        if ((err = gram(0, NB, NB, n01, n23 >= NB ? 2 : 1)) != cudaSuccess) return err;
+        if (n23 > 0 && n23 < NB && (err = gram(2 * NB, 3 * NB, NB, n23, 1)) != cudaSuccess) return err;
+        if (nbb > 2 * NB && (err = gram(0, 2 * NB, 2 * NB, nbb - 2 * NB, 1)) != cudaSuccess) return err;
+      }
       for (int h = NB; h < nbb; h *= 2) {
         const int pairs = (nbb + 2 * h - 1) / (2 * h);
         {
