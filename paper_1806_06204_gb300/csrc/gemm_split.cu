@@ -72,7 +72,6 @@ template <> struct Form<kFormFP8> {
 };
 template <int FORM> __host__ __device__ constexpr int form_bk() { return kRowBytes / Form<FORM>::kElem; }
 constexpr int kARing = 7;
-constexpr int kFusedSliceK = 2048;  // slicing in one launch per product up to this padded K
 constexpr int kGroupM = 8;         // tile rows per group of tiles (L2 reuse of the A slices)
 constexpr int kEpiWarps = 16;      // four per TMEM lane quarter, each owning a quarter of the columns
 constexpr int kThreads = 64 + 32 * kEpiWarps;   // warp 0 TMA, warp 1 MMA, the rest epilogue
@@ -89,54 +88,6 @@ __device__ __forceinline__ int exp_above(unsigned long long mag) {
   if (mag == 0) return 0;
   const int ef = (int)(mag >> 52);
   return ef ? ef - 1021 : -1021;   // normal: |x| < 2^(ef-1022); subnormal: < 2^-1022
-}
-
-// With ek != nullptr, element (i, k) counts as x 2^(esign ek[k]) (the inner-index
-// equilibration): e_i bounds the shifted row.
-__global__ void row_exp_kernel(const double* __restrict__ X, int64_t ldx, int64_t strideX, int trans,
-                               int rows, int K, int* __restrict__ e_out, int rows_pad,
-                               const int* __restrict__ ek, int esign, int K_pad) {
-  __shared__ long long red[8][33];
-  const double* Xb = X + blockIdx.z * strideX;
-  const int* ekb = ek ? ek + blockIdx.z * K_pad : nullptr;
-  const int tx = threadIdx.x, ty = threadIdx.y;   // 32 x 8
-  const unsigned long long kMag = 0x7FFFFFFFFFFFFFFFull;
-  // without shifts: the largest magnitude pattern; with shifts: the largest
-  // shifted exponent bound (both reduce with max)
-  long long mx = ek ? LLONG_MIN : 0;
-  auto take = [&](double x, int k) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(x) & kMag;
-    if (!ekb) {
-      mx = (long long)b > mx ? (long long)b : mx;
-    } else if (b != 0) {
-      const long long e = exp_above(b) + esign * ekb[k];
-      mx = e > mx ? e : mx;
-    }
-  };
-  auto finish = [&](long long v) -> int {
-    if (!ekb) return exp_above((unsigned long long)v);
-    return v == LLONG_MIN ? 0 : (int)v;
-  };
-  if (!trans) {   // 32 rows per block along tx, k split over ty
-    const int i = blockIdx.x * 32 + tx;
-    if (i < rows)
-      for (int k = ty; k < K; k += 8) take(Xb[i + (int64_t)k * ldx], k);
-    red[ty][tx] = mx;
-    __syncthreads();
-    if (ty == 0) {
-      for (int y = 1; y < 8; ++y) mx = red[y][tx] > mx ? red[y][tx] : mx;
-      if (i < rows_pad) e_out[blockIdx.z * rows_pad + i] = finish(mx);
-    }
-  } else {        // 8 rows per block, one warp per row, lanes along k
-    const int i = blockIdx.x * 8 + ty;
-    if (i < rows)
-      for (int k = tx; k < K; k += 32) take(Xb[k + (int64_t)i * ldx], k);
-    for (int o = 16; o > 0; o >>= 1) {
-      const long long t = __shfl_xor_sync(0xffffffffu, mx, o);
-      mx = t > mx ? t : mx;
-    }
-    if (tx == 0 && i < rows_pad) e_out[blockIdx.z * rows_pad + i] = finish(mx);
-  }
 }
 
 // ek[k] = the exponent bound of column k of the (rows x K) view of op(X)
@@ -190,123 +141,62 @@ __global__ void col_exp_kernel(const double* __restrict__ X, int64_t ldx, int64_
 }
 
 // N = round(x 2^(bS - e)) from the bit pattern (|x| < 2^(e-1), so |N| <= 2^(bS-1));
-// ties round away from zero.  b = the digit width.
-template <int S, int B>
+// ties round away from zero.
+template <int BITS>
 __device__ __forceinline__ long long fixed_point(double x, int e) {
   const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
-  const unsigned long long mag = bits & 0x7FFFFFFFFFFFFFFFull;
-  if (mag == 0) return 0;
-  const int ef = (int)(mag >> 52);
-  const unsigned long long M = (mag & ((1ull << 52) - 1)) | (ef ? (1ull << 52) : 0ull);
-  const int E = ef ? ef - 1075 : -1074;          // |x| = M 2^E
-  const int k = E - e + B * S;                   // |x| < 2^(e-1) keeps k <= bS - 54
+  const int ef = (int)(bits >> 52) & 0x7FF;
+  const unsigned long long M = (bits & ((1ull << 52) - 1)) | (ef ? (1ull << 52) : 0ull);
+  const int k = (ef ? ef - 1075 : -1074) - e + BITS;   // |x| = M 2^(k + e - BITS); k <= BITS - 54
   unsigned long long F;
   if (k >= 0) F = k < 11 ? M << k : 0;
-  else F = -k < 63 ? (M + (1ull << (-k - 1))) >> (-k) : 0;
-  return (bits >> 63) ? -(long long)F : (long long)F;
+  else F = k > -63 ? (M + (1ull << (-k - 1))) >> -k : 0;
+  return (long long)bits < 0 ? -(long long)F : (long long)F;
 }
 
-// The S digits of x against the row bound 2^(ee - 1), from the least significant
-// one up; the leading digit takes what is left, |d_1| <= 2^(b-1) because |N| <=
-// 2^(bS-1).  Each is exact in FP32 and in the slice type.
-template <int S, int FORM>
-__device__ __forceinline__ void slice_values(double x, int ee, float* v) {
+// The S balanced digits of two neighbouring entries, plane by plane, as one packed
+// pair of the slice type: o(s, pair).  Adding half a unit to every digit but the
+// leading one (a constant) turns the balanced digits into the plain ones plus that
+// half, so the digits of N are fields of one 64-bit word; an integer below 2^10
+// becomes FP16, and one below 2^23 FP32, by setting the exponent bits of 1024 (2^23)
+// over it and subtracting that: no conversion instruction (16 lanes a clock) per digit.
+template <int S, int FORM, class Put>
+__device__ __forceinline__ void slice_pair(double x0, double x1, int e0, int e1, Put put) {
   constexpr int B = Form<FORM>::kBits;
-  long long N = fixed_point<S, B>(x, ee);
+  constexpr long long half = 1ll << (B - 1);
+  constexpr long long bias = []() {
+    long long t = 0;
+    for (int s = 0; s < S - 1; ++s) t |= half << (B * s);
+    return t;
+  }();
+  const long long n0 = fixed_point<B * S>(x0, e0) + bias, n1 = fixed_point<B * S>(x1, e1) + bias;
+  // digit s (1-based, 1 leads) plus half
+  auto field = [&](long long n, int s) -> unsigned {
+    const int sh = B * (S - s);
+    return s == 1 ? (unsigned)((int)(n >> sh) + (int)half) : (unsigned)(n >> sh) & ((1u << B) - 1);
+  };
 #pragma unroll
-  for (int s = S; s >= 2; --s) {
-    int d = (int)(N & ((1 << B) - 1));
-    d = d >= (1 << (B - 1)) ? d - (1 << B) : d;
-    v[s - 1] = (float)d;
-    N = (N - d) >> B;
-  }
-  v[0] = (float)N;
-}
-
-// S slices of op(X), each rows_pad x K_pad elements of the form's type (BF16,
-// FP16 or E4M3), K contiguous; batch entry b at out + b * S * rows_pad * K_pad,
-// slice s (1-based) at + (s-1) * rows_pad * K_pad elements.  32 x 64 tiles
-// through shared memory: the read runs along X's contiguous dimension, and each
-// thread writes two neighbouring K entries per plane so that a warp stores whole
-// 128-byte (16-bit forms) or 64-byte (FP8) lines.  Xb, ob and ekb are the batch
-// entry's; er(r) gives the exponent of tile row r (rows i0 + r).
-template <int S, int FORM, class ExpOf>
-__device__ __forceinline__ void slice_tile(double (*tile)[65], const double* __restrict__ Xb,
-                                           int64_t ldx, int trans, int rows, int K, ExpOf er,
-                                           uint8_t* __restrict__ ob, int rows_pad, int K_pad,
-                                           const int* __restrict__ ekb, int esign, int i0, int k0) {
-  constexpr int kE = Form<FORM>::kElem;
-  const size_t plane = (size_t)rows_pad * K_pad;  // elements
-  const int tx = threadIdx.x, ty = threadIdx.y;   // 32 x 8
-  if (!trans) {     // rows contiguous: tx runs along i
-    const int i = i0 + tx;
-    for (int r = ty; r < 64; r += 8) {
-      const int k = k0 + r;
-      tile[tx][r] = (i < rows && k < K) ? Xb[i + (int64_t)k * ldx] : 0.0;
-    }
-  } else {          // K contiguous: tx runs along k
-    for (int r = ty; r < 32; r += 8) {
-      const int i = i0 + r;
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int k = k0 + h * 32 + tx;
-        tile[r][h * 32 + tx] = (i < rows && k < K) ? Xb[k + (int64_t)i * ldx] : 0.0;
+  for (int s = 1; s <= S; ++s) {
+    if (FORM == kFormBF16) {
+      const float f0 = __uint_as_float(0x4B000000u | field(n0, s)) - (8388608.f + (float)half);
+      const float f1 = __uint_as_float(0x4B000000u | field(n1, s)) - (8388608.f + (float)half);
+      // a digit has at most 8 significant bits: its BF16 is the float's upper half
+      put(s - 1, __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632));
+    } else {
+      const unsigned t = (field(n0, s) | field(n1, s) << 16) + 0x64006400u;
+      const __half2 h = __hsub2(*reinterpret_cast<const __half2*>(&t),
+                                __half2half2(__ushort_as_half((unsigned short)(0x6400 + half))));
+      if (FORM == kFormFP16) {
+        put(s - 1, *reinterpret_cast<const unsigned*>(&h));
+      } else {   // |d| <= 16: exact in E4M3
+        put(s - 1, (unsigned)__nv_cvt_halfraw2_to_fp8x2(*reinterpret_cast<const __half2_raw*>(&h),
+                                                        __NV_SATFINITE, __NV_E4M3));
       }
     }
   }
-  __syncthreads();
-  const int kl = 2 * tx, k = k0 + kl;             // this thread's two K entries
-  for (int r = ty; r < 32; r += 8) {
-    const int i = i0 + r;
-    if (i >= rows_pad) continue;
-    float va[S], vb[S];
-    if (i < rows) {
-      // element x 2^(esign ek[k]) against the row bound 2^(e_i - 1)
-      const int ei = er(r);
-      const int ea = ekb ? ei - esign * ekb[k] : ei;
-      const int eb2 = ekb ? ei - esign * ekb[k + 1] : ei;
-      slice_values<S, FORM>(tile[r][kl], ea, va);
-      slice_values<S, FORM>(tile[r][kl + 1], eb2, vb);
-    } else {
-#pragma unroll
-      for (int s = 0; s < S; ++s) va[s] = vb[s] = 0.f;
-    }
-    uint8_t* o = ob + ((size_t)i * K_pad + k) * kE;
-    if (FORM == kFormFP8) {   // two E4M3 bytes per plane (|d| <= 16: exact)
-#pragma unroll
-      for (int s = 0; s < S; ++s)
-        *reinterpret_cast<__nv_fp8x2_storage_t*>(o + s * plane) =
-            __nv_cvt_float2_to_fp8x2(make_float2(va[s], vb[s]), __NV_SATFINITE, __NV_E4M3);
-    } else if (FORM == kFormFP16) {
-#pragma unroll
-      for (int s = 0; s < S; ++s)
-        *reinterpret_cast<__half2*>(o + s * plane * 2) = __floats2half2_rn(va[s], vb[s]);
-    } else {
-#pragma unroll
-      for (int s = 0; s < S; ++s)
-        *reinterpret_cast<__nv_bfloat162*>(o + s * plane * 2) = __floats2bfloat162_rn(va[s], vb[s]);
-    }
-  }
 }
 
-// One 32 x 64 tile per block, with the row exponents row_exp_kernel wrote.
-template <int S, int FORM>
-__global__ void __launch_bounds__(256)
-slice_kernel(const double* __restrict__ X, int64_t ldx, int64_t strideX, int trans,
-             int rows, int K, const int* __restrict__ e_in,
-             uint8_t* __restrict__ out, int rows_pad, int K_pad,
-             const int* __restrict__ ek, int esign) {
-  __shared__ double tile[32][65];                 // [row][k]
-  const int* eb = e_in + blockIdx.z * rows_pad + blockIdx.y * 32;
-  const size_t plane = (size_t)rows_pad * K_pad;
-  slice_tile<S, FORM>(tile, X + blockIdx.z * strideX, ldx, trans, rows, K,
-                      [&](int r) { return eb[r]; },
-                      out + (size_t)blockIdx.z * S * plane * Form<FORM>::kElem, rows_pad, K_pad,
-                      ek ? ek + blockIdx.z * K_pad : nullptr, esign, blockIdx.y * 32,
-                      blockIdx.x * 64);
-}
-
-// One operand of a fused slicing launch.
+// One operand of a slicing launch.
 struct SliceOp {
   const double* X;
   int64_t ldx, strideX;
@@ -315,28 +205,43 @@ struct SliceOp {
   uint8_t* out;             // slice planes
 };
 
-// Row exponents and slices of both operands of a product in one launch: block
-// x < nblk_a takes 32 rows of op(A), the rest 32 rows of op(B)^T, blockIdx.z the
-// batch entry.  The block first finds its rows' exponents (the max over all K,
-// as row_exp_kernel), keeps them in shared memory, then slices its rows tile by
-// tile along K: one launch instead of four for the small products, whose K runs
-// are short (the caller uses it for K_pad <= 2048).
+// Row exponents and slices of both operands of a product in one launch.  A cluster of
+// `cl` CTAs takes 32 rows of op(A) (the first nblk_a clusters along x) or of op(B)^T,
+// blockIdx.z the batch entry; each CTA has its share of the 64-wide tiles of K.  It
+// finds its share's largest magnitudes, the ranks exchange them through distributed
+// shared memory, and then it slices its tiles, the next one loaded while the current
+// one is cut: S planes of rows_pad x K_pad elements, K contiguous, batch entry b at
+// out + b S rows_pad K_pad, plane s at + s rows_pad K_pad elements.  Reads run along
+// X's contiguous dimension, a warp writes a whole 128-byte line (FP8: 64) per plane.
+// With ek (the inner-index equilibration), element (i, k) counts as x 2^(esign ek[k]).
+// HBM bounds it (8 bytes read, 14 written per element, the second read from L1 or L2).
+// Measured, both operands of 4096^3: 190 us (3.9 TB/s of those bytes), 344 us with
+// separate exponent launches and a conversion per digit; 512 x 512 x 16384 FP8 153 us
+// against 261 us, 1000 x 1537 x 777 31 us against 63 us.
 template <int S, int FORM>
 __global__ void __launch_bounds__(256)
-slice_fused_kernel(const SliceOp a, const SliceOp b, int nblk_a, int K, int K_pad,
-                   const int* __restrict__ ek) {
+slice_kernel(const SliceOp a, const SliceOp b, int nblk_a, int K, int K_pad,
+             const int* __restrict__ ek, int cl) {
+  namespace cgrp = cooperative_groups;
+  constexpr int kE = Form<FORM>::kElem;
   __shared__ double tile[32][65];
   __shared__ long long red[8][33];
+  __shared__ long long mine[32];
   __shared__ int es[32];
-  const bool on_b = (int)blockIdx.x >= nblk_a;
+  const int rank = blockIdx.x % cl, blk = blockIdx.x / cl;
+  const bool on_b = blk >= nblk_a;
   const SliceOp o = on_b ? b : a;
-  const int i0 = (on_b ? (int)blockIdx.x - nblk_a : (int)blockIdx.x) * 32;
+  const int i0 = (on_b ? blk - nblk_a : blk) * 32;
   const double* Xb = o.X + blockIdx.z * o.strideX;
   const int* ekb = ek ? ek + blockIdx.z * K_pad : nullptr;
   const int tx = threadIdx.x, ty = threadIdx.y;   // 32 x 8
+  const int ntiles = K_pad / 64, per = (ntiles + cl - 1) / cl;
+  const int t_lo = rank * per, t_hi = min(ntiles, t_lo + per);
+  const int k_lo = t_lo * 64, k_hi = min(K, t_hi * 64);
   const unsigned long long kMag = 0x7FFFFFFFFFFFFFFFull;
-  // the row bound as row_exp_kernel forms it: the largest magnitude pattern, or
-  // with the inner-index shifts the largest shifted exponent bound
+  // the row bound: the largest magnitude pattern, or with the inner-index shifts the
+  // largest shifted exponent bound (both reduce with max)
+  const long long none = ekb ? LLONG_MIN : 0;
   auto take = [&](long long& mx, double x, int k) {
     const unsigned long long bits = (unsigned long long)__double_as_longlong(x) & kMag;
     if (!ekb) {
@@ -346,41 +251,106 @@ slice_fused_kernel(const SliceOp a, const SliceOp b, int nblk_a, int K, int K_pa
       mx = e > mx ? e : mx;
     }
   };
-  auto finish = [&](long long v) -> int {
-    if (!ekb) return exp_above((unsigned long long)v);
-    return v == LLONG_MIN ? 0 : (int)v;
-  };
   if (!o.trans) {   // rows contiguous: tx runs along i, k split over ty
     const int i = i0 + tx;
-    long long mx = ekb ? LLONG_MIN : 0;
-    if (i < o.rows)
-      for (int k = ty; k < K; k += 8) take(mx, Xb[i + (int64_t)k * o.ldx], k);
+    long long mx = none;
+    if (i < o.rows) {
+      const double* x = Xb + i;
+      int k = k_lo + ty;
+      for (; k + 56 < k_hi; k += 64) {   // eight loads in flight
+        double v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = x[(int64_t)(k + 8 * u) * o.ldx];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) take(mx, v[u], k + 8 * u);
+      }
+      for (; k < k_hi; k += 8) take(mx, x[(int64_t)k * o.ldx], k);
+    }
     red[ty][tx] = mx;
     __syncthreads();
     if (ty == 0) {
       for (int y = 1; y < 8; ++y) mx = red[y][tx] > mx ? red[y][tx] : mx;
-      es[tx] = finish(mx);
+      mine[tx] = mx;
     }
-  } else {          // K contiguous: one warp per row, lanes along k
-    for (int r = ty; r < 32; r += 8) {
-      const int i = i0 + r;
-      long long mx = ekb ? LLONG_MIN : 0;
-      if (i < o.rows)
-        for (int k = tx; k < K; k += 32) take(mx, Xb[k + (int64_t)i * o.ldx], k);
+  } else {          // K contiguous: one warp per row, lanes along k, four rows at a time
+    long long mx[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) mx[q] = none;
+    for (int k = k_lo + tx; k < k_hi; k += 64) {
+      double v[4][2];
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const int i = i0 + ty + 8 * q;
+          v[q][u] = i < o.rows && k + 32 * u < k_hi ? Xb[k + 32 * u + (int64_t)i * o.ldx] : 0.0;
+        }
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+          if (k + 32 * u < k_hi) take(mx[q], v[q][u], k + 32 * u);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
       for (int s = 16; s > 0; s >>= 1) {
-        const long long t = __shfl_xor_sync(0xffffffffu, mx, s);
-        mx = t > mx ? t : mx;
+        const long long t = __shfl_xor_sync(0xffffffffu, mx[q], s);
+        mx[q] = t > mx[q] ? t : mx[q];
       }
-      if (tx == 0) es[r] = finish(mx);
+      if (tx == 0) mine[ty + 8 * q] = mx[q];
     }
   }
-  __syncthreads();
-  if (ty == 0 && i0 + tx < o.rows_pad) o.e[blockIdx.z * o.rows_pad + i0 + tx] = es[tx];
+  cgrp::cluster_group cluster = cgrp::this_cluster();
+  if (cl > 1) cluster.sync();
+  else __syncthreads();
+  if (ty == 0) {
+    long long mx = mine[tx];
+    for (int q = 0; q < cl; ++q) {
+      if (q == rank) continue;
+      const long long t = cluster.map_shared_rank(mine, q)[tx];
+      mx = t > mx ? t : mx;
+    }
+    es[tx] = !ekb ? exp_above((unsigned long long)mx) : (mx == LLONG_MIN ? 0 : (int)mx);
+    if (rank == 0 && i0 + tx < o.rows_pad) o.e[blockIdx.z * o.rows_pad + i0 + tx] = es[tx];
+  }
+  if (cl > 1) cluster.sync();   // no rank leaves while another reads its maxima
+  else __syncthreads();
   const size_t plane = (size_t)o.rows_pad * K_pad;
-  uint8_t* ob = o.out + (size_t)blockIdx.z * S * plane * Form<FORM>::kElem;
-  for (int k0 = 0; k0 < K_pad; k0 += 64) {
-    slice_tile<S, FORM>(tile, Xb, o.ldx, o.trans, o.rows, K, [&](int r) { return es[r]; }, ob,
-                        o.rows_pad, K_pad, ekb, o.esign, i0, k0);
+  uint8_t* ob = o.out + (size_t)blockIdx.z * S * plane * kE;
+  double v[8];
+  auto load = [&](int t) {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      // not transposed: thread = row tx, k = ty + 8 u; transposed: row ty + 8 (u / 2),
+      // k = tx + 32 (u % 2)
+      const int i = i0 + (o.trans ? ty + 8 * (u >> 1) : tx);
+      const int k = t * 64 + (o.trans ? tx + 32 * (u & 1) : ty + 8 * u);
+      v[u] = i < o.rows && k < K ? (o.trans ? Xb[k + (int64_t)i * o.ldx] : Xb[i + (int64_t)k * o.ldx])
+                                 : 0.0;
+    }
+  };
+  if (t_lo < t_hi) load(t_lo);
+  for (int t = t_lo; t < t_hi; ++t) {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      if (o.trans) tile[ty + 8 * (u >> 1)][tx + 32 * (u & 1)] = v[u];
+      else tile[tx][ty + 8 * u] = v[u];
+    }
+    __syncthreads();
+    if (t + 1 < t_hi) load(t + 1);
+    const int kl = 2 * tx, k = t * 64 + kl;         // this thread's two K entries
+    const int s0 = ekb ? o.esign * ekb[k] : 0, s1 = ekb ? o.esign * ekb[k + 1] : 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int r = ty + 8 * q, i = i0 + r;
+      if (i >= o.rows_pad) continue;
+      // rows beyond the operand are zero: their digits are too
+      uint8_t* w = ob + ((size_t)i * K_pad + k) * kE;
+      slice_pair<S, FORM>(tile[r][kl], tile[r][kl + 1], es[r] - s0, es[r] - s1, [&](int s, unsigned pair) {
+        if (kE == 2) *reinterpret_cast<unsigned*>(w + s * plane * 2) = pair;
+        else *reinterpret_cast<unsigned short*>(w + s * plane) = (unsigned short)pair;
+      });
+    }
     __syncthreads();   // the tile is refilled
   }
 }
@@ -1028,31 +998,6 @@ bool make_map(CUtensorMap* m, const void* base, int64_t rows, int64_t K_pad, int
 
 int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 
-template <int S, int FORM>
-cudaError_t slice_operand(const double* X, int64_t ldx, int64_t strideX, int trans, int rows, int K,
-                          int batch, int* e, uint8_t* out, int rows_pad, int K_pad,
-                          const int* ek, int esign, cudaStream_t st) {
-  {
-    ProfScope ps(kProfSlice, st, 0.0, 8.0 * batch * rows * (double)K);
-    if (!trans) {
-      ps.blocks((const void*)row_exp_kernel, dim3(32, 8), 0, dim3((rows_pad + 31) / 32, 1, batch));
-      row_exp_kernel<<<dim3((rows_pad + 31) / 32, 1, batch), dim3(32, 8), 0, st>>>(
-          X, ldx, strideX, 0, rows, K, e, rows_pad, ek, esign, K_pad);
-    } else {
-      ps.blocks((const void*)row_exp_kernel, dim3(32, 8), 0, dim3((rows_pad + 7) / 8, 1, batch));
-      row_exp_kernel<<<dim3((rows_pad + 7) / 8, 1, batch), dim3(32, 8), 0, st>>>(
-          X, ldx, strideX, 1, rows, K, e, rows_pad, ek, esign, K_pad);
-    }
-  }
-  ProfScope ps(kProfSlice, st, 0.0,
-               (8.0 + (double)Form<FORM>::kElem * S) * batch * rows_pad * (double)K_pad);
-  dim3 grid((unsigned)(K_pad / 64), (unsigned)(rows_pad / 32), batch);
-  ps.blocks((const void*)slice_kernel<S, FORM>, dim3(32, 8), 0, dim3(grid));
-  slice_kernel<S, FORM><<<grid, dim3(32, 8), 0, st>>>(X, ldx, strideX, trans, rows, K, e, out,
-                                                      rows_pad, K_pad, ek, esign);
-  return cudaGetLastError();
-}
-
 constexpr int kSplitSMs = 152;
 
 // CTAs per tile: with too few tiles for the SMs, K is cut over a cluster while
@@ -1111,23 +1056,31 @@ cudaError_t run_split(const GemmArgs& g, SplitWork& w, cudaStream_t st) {
         Xo, swap ? lda : ldb, swap ? sta : stb, swap ? ta : tb, swap ? M : N, K, ek, Kpad);
     if ((err = cudaGetLastError()) != cudaSuccess) return err;
   }
-  if (Kpad <= kFusedSliceK) {
-    // short K runs: both operands' exponents and slices in one launch
+  {
     const SliceOp oa{Xa, lda, sta, ta, M, Mpad, sign_a, ea, sa};
     const SliceOp ob{Xb, ldb, stb, tb, N, Npad, -sign_a, eb, sb};
-    ProfScope ps(kProfSlice, st, 0.0,
-                 (16.0 + (double)Form<FORM>::kElem * S) * nb * (double)(Mpad + Npad) * Kpad);
-    ps.blocks((const void*)slice_fused_kernel<S, FORM>, dim3(32, 8), 0,
-              dim3((unsigned)((Mpad + Npad) / 32), 1, nb));
-    slice_fused_kernel<S, FORM><<<dim3((unsigned)((Mpad + Npad) / 32), 1, nb), dim3(32, 8), 0, st>>>(
-        oa, ob, Mpad / 32, K, Kpad, ek);
-    if ((err = cudaGetLastError()) != cudaSuccess) return err;
-  } else {
-    if ((err = slice_operand<S, FORM>(Xa, lda, sta, ta, M, K, nb, ea, sa, Mpad, Kpad, ek, sign_a,
-                                      st)) != cudaSuccess)
-      return err;
-    if ((err = slice_operand<S, FORM>(Xb, ldb, stb, tb, N, K, nb, eb, sb, Npad, Kpad, ek, -sign_a,
-                                      st)) != cudaSuccess)
+    // CTAs per 32 rows: about four per SM while each keeps a tile of K; one with many
+    // lanes in flight (clusters wait for room: 48 matrices take 117.0 ms with up to
+    // eight, 112.9 with two, 111.8 with one)
+    const int nblk = (Mpad + Npad) / 32, ntiles = Kpad / 64;
+    int cl = 1;
+    while (cl < (w.throughput ? 1 : 8) && (int64_t)nblk * nb * cl < 4 * kSplitSMs && ntiles >= 2 * cl) cl *= 2;
+    ProfScope ps(kProfSlice, st, 0.0, (16.0 + (double)kE * S) * nb * (double)(Mpad + Npad) * Kpad);
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(nblk * cl), 1, nb);
+    cfg.blockDim = dim3(32, 8);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = cl;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = cl > 1 ? 1 : 0;
+    ps.blocks((const void*)slice_kernel<S, FORM>, dim3(32, 8), 0, cfg.gridDim);
+    const int* ekc = ek;
+    if ((err = cudaLaunchKernelEx(&cfg, slice_kernel<S, FORM>, oa, ob, Mpad / 32, K, Kpad, ekc, cl)) !=
+        cudaSuccess)
       return err;
   }
   CUtensorMap mA, mB;
