@@ -189,18 +189,19 @@ size_t layout(void* base, int64_t m, int64_t n, int r, bool svd, PdBufs* b) {
     const int64_t npan = (n + kQrNB - 1) / kQrNB;
     t.qr.strideW = (m + n) * n;
     t.qr.W = q.take<double>(r * t.qr.strideW);
-    const int64_t nblk = (n + kQrBlock - 1) / kQrBlock;
-    t.qr.strideV = (m + kQrBlock) * n;
+    t.qr.sb = qr_super_width(n);
+    const int64_t sb = t.qr.sb, nsup = (n + sb - 1) / sb;
+    t.qr.strideV = (m + sb) * n;
     t.qr.V = q.take<double>(r * t.qr.strideV);
     t.qr.strideT = npan * kQrNB * kQrNB;
     t.qr.T = q.take<double>(r * t.qr.strideT);
-    t.qr.strideTb = nblk * kQrBlock * kQrBlock;
+    t.qr.strideTb = nsup * sb * sb;
     t.qr.Tb = q.take<double>(r * t.qr.strideTb);
-    t.qr.strideG = kQrBlock * kQrBlock;
+    t.qr.strideG = sb * sb;
     t.qr.G = q.take<double>(r * t.qr.strideG);
-    t.qr.strideW1 = kQrBlock * n;
+    t.qr.strideW1 = sb * n;
     t.qr.W1 = q.take<double>(r * t.qr.strideW1);
-    t.qr.strideW2 = kQrBlock * n;
+    t.qr.strideW2 = sb * n;
     t.qr.W2 = q.take<double>(r * t.qr.strideW2);
     c.off = std::max(c.off, q.off);
   }

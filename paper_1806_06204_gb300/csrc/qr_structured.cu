@@ -10,14 +10,20 @@
 // [c0, c0 + m + w), and its compact-WY update (I - V T V^T) touches only that
 // window: every step costs O((m + w) w n) whatever n is.
 //
-// Two levels of blocking.  Panels of NB = 32 columns are factored by one kernel
-// (one CTA, or one 8-CTA cluster, per shift) and applied at once only to the
-// rest of their block of NBb = 128 columns.  The block's reflectors are then
-// merged into one compact-WY factor T_b (from the Gram matrix V_b^T V_b, below)
-// and applied to all later columns with three GEMMs whose inner dimension is the
-// block width: the wide products see the trailing matrix once per 128 columns,
-// not once per 32, and no GEMM dimension is padded up from 32.  The explicit Q
-// applies the same block reflectors in reverse order.
+// Levels of blocking.  Panels of NB = 32 columns are factored by one kernel and applied
+// at once only to the rest of their block of NBb = 128 columns.  The block's reflectors
+// are then merged into one compact-WY factor T_b (from the Gram matrix V_b^T V_b,
+// below) and applied with three GEMMs whose inner dimension is the block width.  On the
+// FP64 pipe the block goes to all later columns.  On the tensor cores a product with an
+// inner dimension of 128 is bound by its outputs (their epilogue and the trailing
+// matrix's traffic) and the trailing matrix is sliced for every one, so blocks are
+// applied within a super-block of 512 columns (from n = 2048), whose merged reflectors
+// go to everything to its right: the trailing matrix is sliced, read and written once
+// per 512 columns.  The explicit Q applies the same (super-)block reflectors in reverse
+// order.  4096^2 at r = 8: 272 -> 242 ms; no gain at 256 columns for n = 512 .. 1024.  The
+// products over a super-block use the 34-pair slices in both 16-bit forms (28 pairs
+// would raise the FP16 form's backward error at 2048^2 from 5.6e-15 to 8.2e-15; so it
+// falls to 3.1e-15); the FP8 form, more accurate than those, keeps 128-column blocks.
 //
 // Q2 (the bottom block of Q) stays exactly upper triangular: the explicit V
 // holds exact zeros outside each reflector's support, so every product that the
@@ -217,9 +223,9 @@ qr_panel_cluster_kernel(double* W, int64_t strideW, int64_t ldw, int64_t m, int6
 }
 
 // T_b of one block: its panel factors on the 32 x 32 diagonal blocks, zero
-// elsewhere (ld NBb).  Grid (ceil(nbb^2 / 256), r).
+// elsewhere (leading dimension ld).  Grid (ceil(nbb^2 / 256), r).
 __global__ void tb_init_kernel(const double* __restrict__ T, int64_t strideT, double* __restrict__ Tb,
-                               int64_t strideTb, int panel0, int nbb) {
+                               int64_t strideTb, int ld, int panel0, int nbb) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= nbb * nbb) return;
   const int i = e % nbb, j = e / nbb;
@@ -227,7 +233,7 @@ __global__ void tb_init_kernel(const double* __restrict__ T, int64_t strideT, do
   if (i / kQrNB == j / kQrNB)
     v = T[blockIdx.y * strideT + (int64_t)(panel0 + i / kQrNB) * kQrNB * kQrNB + (i % kQrNB) +
           (j % kQrNB) * kQrNB];
-  Tb[blockIdx.y * strideTb + i + (int64_t)j * kQrBlock] = v;
+  Tb[blockIdx.y * strideTb + i + (int64_t)j * ld] = v;
 }
 
 // One merge level of the block factor: for each pair of neighbouring diagonal
@@ -237,7 +243,7 @@ __global__ void tb_init_kernel(const double* __restrict__ T, int64_t strideT, do
 // per column j of the right block, per pair and per shift; thread i owns row i.
 __global__ void __launch_bounds__(kQrBlock / 2)
 tb_merge_kernel(const double* __restrict__ G, int64_t strideG, double* __restrict__ Tb,
-                int64_t strideTb, int nbb, int h) {
+                int64_t strideTb, int ld, int nbb, int h) {
   __shared__ double x[kQrBlock / 2];
   const int j = blockIdx.x, i = threadIdx.x;
   const int a = blockIdx.y * 2 * h, b0 = a + h;
@@ -245,7 +251,6 @@ tb_merge_kernel(const double* __restrict__ G, int64_t strideG, double* __restric
   if (w <= 0 || j >= w) return;
   const double* Gs = G + blockIdx.z * strideG;
   double* T = Tb + blockIdx.z * strideTb;
-  constexpr int ld = kQrBlock;
   if (i < h) {
     double t = 0.0;
     for (int k = 0; k <= j; ++k) t = fma(Gs[(a + i) + (int64_t)(b0 + k) * ld], T[(b0 + k) + (int64_t)(b0 + j) * ld], t);
@@ -752,28 +757,68 @@ cudaError_t apply_block(const QrBuffers& b, const double* Vw, int64_t ldv, const
   g.M = w; g.N = (int)ncols; g.K = (int)rows; g.transA = 1; g.transB = 0;
   g.A = Vw; g.lda = ldv; g.strideA = b.strideV;
   g.B = C; g.ldb = ldw; g.strideB = b.strideW;
-  g.Cout = b.W1; g.ldcout = kQrBlock; g.strideCout = b.strideW1;
+  g.Cout = b.W1; g.ldcout = b.sb; g.strideCout = b.strideW1;
   g.batch = r;
   for (int j = 0; j < r; ++j) g.alpha[j] = 1.0;
-  err = w <= kQrNB ? gemm_fine(g, st) : gemm_any(g, st);
+  // over a super-block the later reflectors meet columns that the earlier ones have
+  // not been taken off: the cancellation that follows wants the finer slices
+  err = w <= kQrNB || w > kQrBlock ? gemm_fine(g, st) : gemm_any(g, st);
   if (err != cudaSuccess) return err;
   GemmArgs h = g;
   h.K = w; h.transA = transT;
   h.A = Tw; h.lda = ldt; h.strideA = strideT;
-  h.B = b.W1; h.ldb = kQrBlock; h.strideB = b.strideW1;
-  h.Cout = b.W2; h.strideCout = b.strideW2;
-  if ((err = gemm_any(h, st)) != cudaSuccess) return err;
+  h.B = b.W1; h.ldb = b.sb; h.strideB = b.strideW1;
+  h.Cout = b.W2; h.ldcout = b.sb; h.strideCout = b.strideW2;
+  // the rows of W1 decay like the singular values across the reflectors; over a
+  // super-block one scale per column would cost the small ones their precision
+  h.k_equilibrate = w > kQrBlock;
+  if ((err = w > kQrBlock ? gemm_fine(h, st) : gemm_any(h, st)) != cudaSuccess) return err;
   GemmArgs u = g;
   u.M = (int)rows; u.N = (int)ncols; u.K = w; u.transA = 0; u.transB = 0;
   u.A = Vw; u.lda = ldv; u.strideA = b.strideV;
-  u.B = b.W2; u.ldb = kQrBlock; u.strideB = b.strideW2;
+  u.B = b.W2; u.ldb = b.sb; u.strideB = b.strideW2;
   u.Cin = C; u.ldcin = ldw; u.strideCin = b.strideW; u.beta = 1.0;
   u.Cout = C; u.ldcout = ldw; u.strideCout = b.strideW;
   for (int j = 0; j < r; ++j) u.alpha[j] = -1.0;
   // the rows of W2 follow the trailing matrix, whose size decays across the
   // block's reflectors like the singular values: equilibrate them
   u.k_equilibrate = 1;
-  return gemm_any(u, st);
+  return w > kQrBlock ? gemm_fine(u, st) : gemm_any(u, st);
+}
+
+// The factor of a super-block from its blocks' factors, merged pairwise (128 -> 256 ->
+// 512): T_12 = -T_11 (V_1^T V_2) T_22, V^T V in one product (upper tiles).  The
+// products read T in full: what lies below its diagonal blocks is zero.
+cudaError_t merge_super(const QrBuffers& b, const double* Vs, int64_t ldv, double* Ts, int ldt,
+                        int64_t rows, int sw, int r, cudaStream_t st) {
+  cudaError_t err;
+  GemmArgs g;
+  g.M = g.N = sw; g.K = (int)rows; g.transA = 1;
+  g.A = g.B = Vs; g.lda = g.ldb = ldv; g.strideA = g.strideB = b.strideV;
+  g.Cout = b.G; g.ldcout = ldt; g.strideCout = b.strideG;
+  g.batch = r; g.c_upper = 1;
+  for (int j = 0; j < r; ++j) g.alpha[j] = 1.0;
+  if ((err = gemm_fine(g, st)) != cudaSuccess) return err;
+  for (int h = kQrBlock; h < sw; h *= 2)
+    for (int a = 0; a + h < sw; a += 2 * h) {
+      const int w = sw - a - h < h ? sw - a - h : h;
+      GemmArgs y;   // Y = (V_1^T V_2) T_22, into W2
+      y.M = h; y.N = w; y.K = w;
+      y.A = b.G + a + (int64_t)(a + h) * ldt; y.lda = ldt; y.strideA = b.strideG;
+      y.B = Ts + (a + h) + (int64_t)(a + h) * ldt; y.ldb = ldt; y.strideB = b.strideTb;
+      y.Cout = b.W2; y.ldcout = ldt; y.strideCout = b.strideW2;
+      y.batch = r;
+      for (int j = 0; j < r; ++j) y.alpha[j] = 1.0;
+      if ((err = gemm_fine(y, st)) != cudaSuccess) return err;
+      GemmArgs t = y;   // T_12 = -T_11 Y
+      t.M = h; t.N = w; t.K = h;
+      t.A = Ts + a + (int64_t)a * ldt; t.lda = ldt; t.strideA = b.strideTb;
+      t.B = b.W2; t.ldb = ldt; t.strideB = b.strideW2;
+      t.Cout = Ts + a + (int64_t)(a + h) * ldt; t.ldcout = ldt; t.strideCout = b.strideTb;
+      for (int j = 0; j < r; ++j) t.alpha[j] = -1.0;
+      if ((err = gemm_fine(t, st)) != cudaSuccess) return err;
+    }
+  return cudaSuccess;
 }
 
 }  // namespace
@@ -842,6 +887,8 @@ cudaError_t launch_panel(PanelKind k, const PanelArgs& p, int r, double fl, doub
 
 }  // namespace
 
+int qr_super_width(int64_t n) { return n >= 2048 ? 512 : kQrBlock; }
+
 cudaError_t structured_qr_q(const QrBuffers& b, int64_t m, int64_t n, int r, int* status,
                             cudaStream_t st, bool explicit_q, bool narrow_panels) {
   constexpr int NB = kQrNB, NBb = kQrBlock;
@@ -855,9 +902,13 @@ cudaError_t structured_qr_q(const QrBuffers& b, int64_t m, int64_t n, int r, int
       return cudaErrorInvalidConfiguration;
   }
   const int64_t ldw = m + n;
-  const int64_t ldv = m + NBb;
+  // On the tensor cores the blocks of a super-block are applied to its own columns
+  // one by one and to everything to its right together (see the file's head).
+  const SplitWork* eng = get_split_engine();
+  const int SB = eng && eng->form != kFormFP8 ? b.sb : NBb;
+  const int ldt = SB;
+  const int64_t ldv = m + SB;
   cudaError_t err;
-  const int nblocks = (int)((n + NBb - 1) / NBb);
   // The register panel where there is one; else, with many problems in flight
   // (narrow_panels), the shared-memory panel on the fewest CTAs whose rows fit (one
   // CTA up to m = 736, two up to 1504): the same SMs then serve more panels at once.
@@ -870,15 +921,20 @@ cudaError_t structured_qr_q(const QrBuffers& b, int64_t m, int64_t n, int r, int
   const int64_t rows_cta = cg ? (m + NB + cg - 1) / cg : 0;
   // every V entry outside the rows a panel writes must be an exact zero
   if ((err = cudaMemsetAsync(b.V, 0, sizeof(double) * r * b.strideV, st)) != cudaSuccess) return err;
+  if (SB > NBb &&
+      (err = cudaMemsetAsync(b.Tb, 0, sizeof(double) * r * b.strideTb, st)) != cudaSuccess)
+    return err;
   // ---------------- factorisation (structured GEQRF)
-  for (int blk = 0; blk < nblocks; ++blk) {
-    const int64_t c0b = (int64_t)blk * NBb;
+  for (int64_t c0b = 0; c0b < n; c0b += NBb) {
+    const int64_t s0 = c0b / SB * SB;                              // the super-block
+    const int sw = (int)(n - s0 < SB ? n - s0 : SB);
+    const int off = (int)(c0b - s0);
     const int nbb = (int)(n - c0b < NBb ? n - c0b : NBb);
     for (int p = 0; p * NB < nbb; ++p) {
       const int64_t c0 = c0b + (int64_t)p * NB;
       const int nbp = nbb - p * NB < NB ? nbb - p * NB : NB;
-      // V rows are relative to the block start: this panel's window starts p*NB down
-      double* Vpan = b.V + (int64_t)p * NB;
+      // V rows are relative to the super-block: this panel's window starts there
+      double* Vpan = b.V + off + (int64_t)p * NB;
       const double pf = 3.0 * r * (double)(m + 1) * nbp * nbp, pb = 16.0 * r * (double)(m + NB) * nbp;
       if (reg != kRegNone) {
         const PanelArgs pa{b.W, b.strideW, ldw, m, c0, nbp, Vpan, b.strideV, ldv, b.T, b.strideT, status};
@@ -921,13 +977,14 @@ cudaError_t structured_qr_q(const QrBuffers& b, int64_t m, int64_t n, int r, int
       }
     }
     // ---- the block factor T_b: panel factors on the diagonal, merged pairwise
-    const double* Vb = b.V + c0b * ldv;
-    double* Tb = b.Tb + (int64_t)blk * NBb * NBb;
+    const double* Vb = b.V + off + c0b * ldv;
+    double* Ts = b.Tb + s0 / SB * (int64_t)ldt * ldt;              // the super-block's factor
+    double* Tb = Ts + off + (int64_t)off * ldt;
     {
       ProfScope ps(kProfOther, st);
       ps.blocks((const void*)tb_init_kernel, dim3(256), 0, dim3((nbb * nbb + 255) / 256, r));
       tb_init_kernel<<<dim3((nbb * nbb + 255) / 256, r), 256, 0, st>>>(b.T, b.strideT, Tb,
-                                                                      b.strideTb, (int)(c0b / NB), nbb);
+                                                                      b.strideTb, ldt, (int)(c0b / NB), nbb);
     }
     if ((err = cudaGetLastError()) != cudaSuccess) return err;
     if (nbb > NB) {
@@ -939,7 +996,7 @@ cudaError_t structured_qr_q(const QrBuffers& b, int64_t m, int64_t n, int r, int
       GemmArgs g;
       g.M = g.N = nbb; g.K = (int)(m + nbb); g.transA = 1;
       g.A = g.B = Vb; g.lda = g.ldb = ldv; g.strideA = g.strideB = b.strideV;
-      g.Cout = b.G; g.ldcout = NBb; g.strideCout = b.strideG;
+      g.Cout = b.G; g.ldcout = ldt; g.strideCout = b.strideG;
       g.batch = r; g.c_upper = 1;
       for (int j = 0; j < r; ++j) g.alpha[j] = 1.0;
       if (gemm_fine_splits(g)) {
@@ -951,9 +1008,9 @@ cudaError_t structured_qr_q(const QrBuffers& b, int64_t m, int64_t n, int r, int
           q.M = mt; q.N = nt;
           q.A = Vb + i0 * ldv;
           q.B = Vb + j0 * ldv;
-          q.Cout = b.G + i0 + j0 * NBb;
+          q.Cout = b.G + i0 + j0 * ldt;
           q.inner = inner;
-          q.innerA = q.innerB = 2 * NB * ldv; q.innerC = 2 * NB + 2 * NB * NBb;
+          q.innerA = q.innerB = 2 * NB * ldv; q.innerC = 2 * NB + 2 * NB * ldt;
           return gemm_f64(q, st);
         };
         const int n01 = nbb - NB < NB ? nbb - NB : NB, n23 = nbb - 3 * NB;
@@ -968,27 +1025,37 @@ cudaError_t structured_qr_q(const QrBuffers& b, int64_t m, int64_t n, int r, int
           ProfScope ps(kProfOther, st);
           ps.blocks((const void*)tb_merge_kernel, dim3(NBb / 2), 0, dim3(h, pairs, r));
           tb_merge_kernel<<<dim3(h, pairs, r), NBb / 2, 0, st>>>(b.G, b.strideG, Tb, b.strideTb,
-                                                                 nbb, h);
+                                                                 ldt, nbb, h);
         }
         if ((err = cudaGetLastError()) != cudaSuccess) return err;
       }
     }
-    // ---- all later columns, once per block
-    const int64_t ntr = n - c0b - nbb;
+    // ---- the rest of the super-block's columns, or (its last block) its merged
+    //      factor and all later columns
+    const int64_t nsup = s0 + sw - c0b - nbb;
+    if (nsup > 0) {
+      if ((err = apply_block(b, Vb, ldv, Tb, ldt, b.strideTb, b.W + c0b + (c0b + nbb) * ldw, ldw,
+                             m + nbb, nbb, nsup, r, 1, st)) != cudaSuccess)
+        return err;
+      continue;
+    }
+    const double* Vs = b.V + s0 * ldv;
+    if (sw > NBb && (err = merge_super(b, Vs, ldv, Ts, ldt, m + sw, sw, r, st)) != cudaSuccess)
+      return err;
+    const int64_t ntr = n - s0 - sw;
     if (ntr > 0 &&
-        (err = apply_block(b, Vb, ldv, Tb, NBb, b.strideTb, b.W + c0b + (c0b + nbb) * ldw, ldw,
-                           m + nbb, nbb, ntr, r, 1, st)) != cudaSuccess)
+        (err = apply_block(b, Vs, ldv, Ts, ldt, b.strideTb, b.W + s0 + (s0 + sw) * ldw, ldw,
+                           m + sw, sw, ntr, r, 1, st)) != cudaSuccess)
       return err;
   }
   if (!explicit_q) return cudaSuccess;
   // ---------------- explicit Q (structured ORGQR), overwriting W
   if ((err = init_q_identity(b.W, b.strideW, m, n, r, st)) != cudaSuccess) return err;
-  for (int blk = nblocks - 1; blk >= 0; --blk) {
-    const int64_t c0b = (int64_t)blk * NBb;
-    const int nbb = (int)(n - c0b < NBb ? n - c0b : NBb);
-    if ((err = apply_block(b, b.V + c0b * ldv, ldv, b.Tb + (int64_t)blk * NBb * NBb, NBb,
-                           b.strideTb, b.W + c0b + c0b * ldw, ldw, m + nbb, nbb, n - c0b, r, 0,
-                           st)) != cudaSuccess)
+  for (int64_t s0 = (n - 1) / SB * SB; s0 >= 0; s0 -= SB) {
+    const int sw = (int)(n - s0 < SB ? n - s0 : SB);
+    if ((err = apply_block(b, b.V + s0 * ldv, ldv, b.Tb + s0 / SB * (int64_t)ldt * ldt, ldt,
+                           b.strideTb, b.W + s0 + s0 * ldw, ldw, m + sw, sw, n - s0, r, 0, st)) !=
+        cudaSuccess)
       return err;
   }
   return cudaSuccess;

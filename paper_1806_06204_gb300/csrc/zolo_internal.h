@@ -275,16 +275,20 @@ double alpha_from_sums(const double* sums);
 
 // ------------------------------------------------------------ structured QR
 constexpr int kQrNB = 32;      // panel width (columns factored by one panel kernel)
-constexpr int kQrBlock = 128;  // block width (columns per trailing update / block reflector)
+constexpr int kQrBlock = 128;  // block width (columns a panel's reflectors are applied to at once)
+// Widest super-block of an n-column problem: the columns whose reflectors are applied
+// together to everything to their right.
+int qr_super_width(int64_t n);
 struct QrBuffers {
+  int sb;                         // qr_super_width(n): the strides below hold super-blocks this wide
   double* W;   int64_t strideW;   // stacked (m+n) x n per shift, ld m+n
-  double* V;   int64_t strideV;   // explicit reflectors (m+NBb) x n per shift, ld m+NBb, rows
-                                  // relative to the start of each column's block
+  double* V;   int64_t strideV;   // explicit reflectors (m+sb) x n per shift, ld m+sb, rows
+                                  // relative to the start of each column's super-block
   double* T;   int64_t strideT;   // nb x nb triangular factor per panel
-  double* Tb;  int64_t strideTb;  // NBb x NBb triangular factor per block
-  double* G;   int64_t strideG;   // NBb x NBb Gram V_b^T V_b scratch
-  double* W1;  int64_t strideW1;  // NBb x n scratch
-  double* W2;  int64_t strideW2;  // NBb x n scratch
+  double* Tb;  int64_t strideTb;  // sb x sb triangular factor per super-block
+  double* G;   int64_t strideG;   // sb x sb Gram V^T V scratch
+  double* W1;  int64_t strideW1;  // sb x n scratch
+  double* W2;  int64_t strideW2;  // sb x n scratch
 };
 // Factor [X; sqrt(c_j) I] for j < r and overwrite W_j with the thin Q_j
 // (explicit_q = false: leave R on and above the diagonal of W_j's top block).

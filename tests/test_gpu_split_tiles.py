@@ -74,3 +74,27 @@ def test_split_product_at_the_ends_of_the_range(handle, prec, S, expo):
         ref = np.ldexp(np.ldexp(A, -expo) @ np.ldexp(B, -expo if expo > -1000 else 0),
                        2 * expo if expo > -1000 else expo)
     assert np.array_equal(C, ref)
+
+
+@pytest.mark.parametrize("m,n", [(2048, 2048), (2300, 2177)])
+@pytest.mark.parametrize("prec", [1, 2, 3])
+def test_super_blocks_keep_the_invariants(handle, m, n, prec):
+    # from n = 2048 the 16-bit forms apply 512 columns' reflectors together; 2177 = 4 x 512
+    # + 129 leaves a super-block of a whole and a one-column block
+    import torch
+    zb, h = handle
+    g = torch.Generator(device="cuda").manual_seed(n + prec)
+
+    def haar(rows, cols):
+        return torch.linalg.qr(torch.randn(rows, cols, dtype=torch.float64, device="cuda", generator=g))[0]
+
+    s = torch.logspace(0, -8, n, dtype=torch.float64, device="cuda")
+    U, V = haar(m, n), haar(n, n)
+    A = (V @ (U * s).t()).t()
+    Qp, H, info = zb.zolo_pd(h, A, zb.opts(beta=1e-8, r=2, prec=prec, ns_steps=1))
+    assert info.used_qr[0]
+    bwd = torch.linalg.matrix_norm(A - Qp @ H) / torch.linalg.matrix_norm(A)
+    orth = torch.linalg.matrix_norm(Qp.t() @ Qp - torch.eye(n, dtype=torch.float64, device="cuda")) / n ** 0.5
+    assert float(bwd) <= 1e-13 and float(orth) <= 1e-13
+    # H = V diag(s) V^T to the grade of the iteration (A's own rounding included)
+    assert float(torch.linalg.matrix_norm(H - (V * s) @ V.t()) / torch.linalg.matrix_norm(H)) <= 1e-13
