@@ -12,24 +12,28 @@
 // Mixed precision.  FP32 runs 58x faster than FP64 on this part, so the sweeps
 // that only need to bring the columns close to orthogonal run in FP32 on a copy
 // X32 = R^T with the rotations accumulated in Z32, as block Jacobi on 16-column
-// blocks (one cooperative launch per sweep, rounds separated by a bounded grid
-// barrier).  Z is then made orthonormal in FP64 (Cholesky QR), X = R^T Z is
-// formed in FP64, and FP64 sweeps (one cooperative dataflow launch per sweep,
-// one CTA per column pair at a time) finish from cosines ~1e-4 in a few
-// quadratically convergent sweeps.
+// blocks (one cooperative dataflow launch per sweep).  Z is then made
+// orthonormal in FP64 (Cholesky QR), X = R^T Z is formed in FP64, and FP64
+// sweeps (one cooperative dataflow launch per sweep, one CTA per column pair at
+// a time) finish from cosines ~1e-4 in a few quadratically convergent sweeps.
 // FP32 sweeps stop when fewer than n rotations (cosines above 8e-6) were needed
 // in a sweep (25 sweeps at most): the FP64 sweeps start from cosines of about
 // 1e-4 whatever the last FP32 sweeps do, since Z's FP32 rounding, times R^T,
 // sets them.  FP64 sweeps stop when no pair has |x_p . x_q| > 8 eps ||x_p||
 // ||x_q||, or after a sweep in which every cosine was below sqrt(n) eps (the
 // rounding level of an n-term dot product): its rotations were of that size,
-// so the next sweep would find the same rounding-level cosines again.
+// so the next sweep would find the same rounding-level cosines again.  Pairs are
+// rotated down to 2 eps all the same, at no cost in time: the cosines that the
+// last sweeps leave alone are what V's orthogonality consists of.
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
 #include <vector>
 
+#include <cooperative_groups.h>
+
+#include "fp64_scalar.cuh"
 #include "zolo_internal.h"
 
 namespace zolo {
@@ -53,6 +57,10 @@ __device__ __forceinline__ void st_release(int* p, int v) {
   asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
+__device__ __forceinline__ void add_release(int* p, int v) {
+  asm volatile("red.release.gpu.global.add.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
 // Waits until *ver >= want, two seconds at most (by the global timer), giving up
 // at once when another block has set the error flag; false (and *err set) on
 // time-out.
@@ -68,7 +76,7 @@ __device__ bool wait_round(const int* ver, int want, int* err) {
       asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
       if (t - t0 > 2000000000ull) break;
     }
-    __nanosleep(32);
+    if (k > 15u) __nanosleep(32);
   }
   atomicExch(err, 1);
   return false;
@@ -95,18 +103,27 @@ __device__ bool wait_round(const int* ver, int want, int* err) {
 // of five (the FP64 pipe is the bound).  Near convergence c = 1 - O(t^2), so the
 // scales stay within rounding of 1 over a sweep; the caller folds them into the
 // columns between sweeps.
-// An FP64 instruction occupies its sub-partition's FP64 unit for a whole warp
-// slot however few lanes are active, so the block's 256 partial dot products
-// are summed by one warp (7 + 5 warp instructions instead of 5 per warp plus 8
-// on one lane), and the warp that sums them and forms the rotation changes with
-// the item: the scalar work spreads over the SM's four sub-partitions.
-__global__ void __launch_bounds__(kJacThreads)
+//
+// What bounds an item below n of a few thousand is its chain: wait, load, dot product,
+// rotation, update, publish.  So the two columns stay in registers between the dot
+// product and the update (RPT rows a thread; 0: too long, read again), the block has as
+// many threads as the length warrants, the scale ratios are formed while the columns
+// are in flight, and only what the update needs (t times the ratios) lies on the chain;
+// cosine, norms and scales follow it.  An FP64 instruction occupies its sub-partition's
+// FP64 unit for a whole warp slot (64 clocks) however few lanes are active, so the
+// partial dot products are summed by one warp, which changes with the item.  A sweep
+// (events): n = 256 1.12 ms (1.71 with the columns read twice by 256 threads and the
+// whole rotation formed in one chain), n = 512 2.9 (3.3), n = 1024 7.1 (7.9); from n =
+// 2048 the FP64 units bound it (3 n^3 / 2 FMA, 25 ms a sweep as before).
+// A rotation is made for cosines above tol and counted above 4 tol.
+template <int NT, int RPT>
+__global__ void __launch_bounds__(NT, RPT == 0 ? 1536 / NT : 1)
 jacobi_sweep_kernel(double* X, int64_t ldx, int64_t m, int n_even, int n_real, double tol,
                     int* status, double* nrm2, double* dsc, int* ver, int* err, int stall,
                     long long stall_ns) {
-  __shared__ double part[kJacThreads];
-  __shared__ double s_al, s_be;
-  __shared__ int s_rot, s_ok, never;
+  __shared__ double part[NT];
+  __shared__ double s_al, s_be, s_t;
+  __shared__ int s_rot, s_ok[2], never;
   const int npairs = n_even / 2;
   const int64_t items = (int64_t)(n_even - 1) * npairs;
   if (stall && blockIdx.x == 0) {
@@ -128,86 +145,128 @@ jacobi_sweep_kernel(double* X, int64_t ldx, int64_t m, int n_even, int n_real, d
     __syncthreads();
     return;
   }
+  constexpr int kWarps = NT / 32;
+  const int tid = threadIdx.x, l = tid & 31, warp = tid >> 5;
   for (int64_t it = blockIdx.x; it < items; it += gridDim.x) {
     const int round = (int)(it / npairs), i = (int)(it - (int64_t)round * npairs);
     auto elem = [&](int pos) { return pos == 0 ? 0 : 1 + (pos - 1 + round) % (n_even - 1); };
     int p = elem(i), q = elem(n_even - 1 - i);
     if (p > q) { const int t = p; p = q; q = t; }
     const bool real = q < n_real;      // the pair with the padding column is no work
-    if (threadIdx.x == 0)
-      s_ok = !*(volatile int*)err && wait_round(ver + p, round, err) &&
-             (!real || wait_round(ver + q, round, err));
+    if (tid < 2)
+      s_ok[tid] = !*(volatile int*)err && ((tid == 1 && !real) || wait_round(ver + (tid ? q : p), round, err));
     __syncthreads();
-    if (!s_ok) return;
+    if (!s_ok[0] || !s_ok[1]) return;
     if (real) {
       double* xp = X + p * ldx;
       double* xq = X + q * ldx;
+      double u[RPT > 0 ? RPT : 1], v[RPT > 0 ? RPT : 1];
       double g = 0.0;
-      for (int64_t r = threadIdx.x; r < m; r += kJacThreads) g = fma(__ldcg(xp + r), __ldcg(xq + r), g);
-      part[threadIdx.x] = g;
-      __syncthreads();
-      const int lead = (int)(it & (kJacThreads / 32 - 1));   // the warp that forms the rotation
-      if ((int)(threadIdx.x >> 5) == lead) {
-        const int l = threadIdx.x & 31;
-        double sg = part[l];
+      const int lead = (int)(it % kWarps);   // the warp that forms the rotation
+      double dp = 1.0, dq = 1.0, sa = 0.0, sb = 0.0;
+      if (RPT > 0) {
 #pragma unroll
-        for (int k = 1; k < kJacThreads / 32; ++k) sg += part[l + 32 * k];
-        sg = warp_sum(sg);
+        for (int k = 0; k < RPT; ++k) {
+          const int r = tid + k * NT;
+          u[k] = r < m ? __ldcg(xp + r) : 0.0;
+          v[k] = r < m ? __ldcg(xq + r) : 0.0;
+        }
+      }
+      if (warp == lead) {
+        dp = __ldcg(dsc + p);
+        dq = __ldcg(dsc + q);
+        sa = __ldcg(nrm2 + p);
+        sb = __ldcg(nrm2 + q);
+      }
+      if (RPT > 0) {
+        double h = 0.0;
+#pragma unroll
+        for (int k = 0; k < RPT; ++k) {
+          if (k & 1) h = fma(u[k], v[k], h);
+          else g = fma(u[k], v[k], g);
+        }
+        if (RPT > 1) g += h;
+      } else {
+        for (int64_t r = tid; r < m; r += NT) g = fma(__ldcg(xp + r), __ldcg(xq + r), g);
+      }
+      part[tid] = g;
+      // what does not need the dot product: the scales' product and ratios, and the
+      // FP32 operands of the cosine test and of the angle's first approximation
+      double dd = 1.0, r1 = 1.0, r2 = 1.0, sg = 0.0;
+      float fa = 0.f, fb = 0.f, fd = 0.f;
+      if (warp == lead) {
+        dd = dp * dq;
+        r1 = dq * reciprocal(dp);
+        r2 = dp * reciprocal(dq);
+        fa = (float)sa;
+        fb = (float)sb;               // below float range: left as converged
+        fd = (float)(sb - sa);
+      }
+      __syncthreads();
+      if (warp == lead) {
+        sg = part[l];
+#pragma unroll
+        for (int k = 1; k < kWarps; ++k) sg += part[l + 32 * k];
+        sg = warp_sum(sg) * dd;                         // cross product of the true columns
+        const float fg = (float)sg;
+        const float cosv = (fa > 0.f && fb > 0.f) ? fabsf(fg) * rsqrtf(fa) * rsqrtf(fb) : 0.f;
+        const int rot = fg != 0.f && cosv > (float)tol ? (cosv > 4.f * (float)tol ? 2 : 1) : 0;
+        const float zeta = __fdividef(0.5f * fd, fg), az = fabsf(zeta);
+        const float z1 = fmaf(az, az, 1.f);
+        const float tf = copysignf(az > 1e18f ? __fdividef(0.5f, az) : __fdividef(1.f, az + z1 * rsqrtf(z1)), zeta);
+        // one Newton step of g (t^2 - 1) + (s_q - s_p) t = 0 in FP64: the pair's next
+        // cosine is the angle's error times this one
+        const double t0 = (double)tf;
+        const double res = fma(sg, fma(t0, t0, -1.0), (sb - sa) * t0);
+        const double t = t0 - (double)__fdividef((float)res, fmaf(2.f * fg, tf, fd));
         if (l == 0) {
-          // One lane's scalar work costs whole FP64 warp instructions on this
-          // part, so only what fixes the rotation exactly is FP64: the cosine
-          // test and the angle are formed in FP32 (an angle off by 1e-7 only
-          // slows convergence by that factor), while c = (1 + t^2)^(-1/2) for
-          // the t actually applied, the norm and scale updates are FP64 (Newton
-          // steps from FP32 seeds).
-          const double dp = __ldcg(dsc + p), dq = __ldcg(dsc + q);
-          sg *= dp * dq;                                  // cross product of the true columns
-          const double sa = __ldcg(nrm2 + p), sb = __ldcg(nrm2 + q);
-          const float fa = (float)sa, fb = (float)sb;     // below float range: left as converged
-          const float cosv = (fa > 0.f && fb > 0.f) ? fabsf((float)sg) * rsqrtf(fa) * rsqrtf(fb) : 0.f;
-          atomicMax(status + kStatJacobiMaxCos, __float_as_int(cosv));
-          const int rot = (sg != 0.0) && (cosv > (float)tol);
-          if (rot) {
-            const float zeta = (float)((sb - sa) / (2.0 * sg));
-            const float az = fabsf(zeta);
-            const float tf = (az > 1e18f ? 0.5f / az : 1.f / (az + sqrtf(fmaf(az, az, 1.f))));
-            const double t = zeta >= 0.f ? (double)tf : -(double)tf;
-            const double x = fma(t, t, 1.0);
-            double c = (double)rsqrtf((float)x);
-            c = c * fma(-0.5 * x * c, c, 1.5);
-            c = c * fma(-0.5 * x * c, c, 1.5);
-            double rp = (double)(1.f / (float)dp), rq = (double)(1.f / (float)dq);
-            rp = rp * fma(-dp, rp, 2.0); rp = rp * fma(-dp, rp, 2.0);
-            rq = rq * fma(-dq, rq, 2.0); rq = rq * fma(-dq, rq, 2.0);
-            nrm2[p] = fma(-t, sg, sa);
-            nrm2[q] = fma(t, sg, sb);
-            dsc[p] = c * dp;
-            dsc[q] = c * dq;
-            s_al = t * (dq * rp);
-            s_be = t * (dp * rq);
-            atomicAdd(status + kStatJacobiRot, 1);
-          }
+          s_al = t * r1;
+          s_be = t * r2;
+          s_t = t;
           s_rot = rot;
+          atomicMax(status + kStatJacobiMaxCos, __float_as_int(cosv));
         }
       }
       __syncthreads();
       if (s_rot) {
         const double al = s_al, be = s_be;
-        for (int64_t r = threadIdx.x; r < m; r += kJacThreads) {
-          const double u = __ldcg(xp + r), v = __ldcg(xq + r);
-          xp[r] = fma(-al, v, u);
-          xq[r] = fma(be, u, v);
+        if (RPT > 0) {
+#pragma unroll
+          for (int k = 0; k < RPT; ++k) {
+            const int r = tid + k * NT;
+            if (r < m) {
+              xp[r] = fma(-al, v[k], u[k]);
+              xq[r] = fma(be, u[k], v[k]);
+            }
+          }
+        } else {
+          for (int64_t r = tid; r < m; r += NT) {
+            const double a = __ldcg(xp + r), c = __ldcg(xq + r);
+            xp[r] = fma(-al, c, a);
+            xq[r] = fma(be, a, c);
+          }
+        }
+        if (warp == lead) {
+          // c = (1 + t^2)^(-1/2) for the t actually applied, in FP64
+          const double t = s_t, x = fma(t, t, 1.0);
+          double root, c;
+          root_pair(x, &root, &c);
+          if (l == 0) {
+            nrm2[p] = fma(-t, sg, sa);
+            nrm2[q] = fma(t, sg, sb);
+            dsc[p] = c * dp;
+            dsc[q] = c * dq;
+            if (s_rot == 2) atomicAdd(status + kStatJacobiRot, 1);
+          }
         }
       }
     }
-    // publish: the block barrier orders every thread's stores before thread 0's
-    // release of the columns' round counters (a release at GPU scope covers what
-    // happens before it in the block), which the next pair's acquire pairs with
+    // publish: the block barrier orders every thread's stores before the releases of
+    // the columns' round counters (a release at GPU scope covers what happens before
+    // it in the block), which the next pair's acquire pairs with
     __syncthreads();
-    if (threadIdx.x == 0) {
-      st_release(ver + p, round + 1);
-      if (real) st_release(ver + q, round + 1);
-    }
+    if (tid == 0) st_release(ver + p, round + 1);
+    if (tid == 1 && real) st_release(ver + q, round + 1);
   }
 }
 
@@ -216,64 +275,65 @@ __global__ void fill_kernel(double* d, int64_t n, double v) {
   if (i < n) d[i] = v;
 }
 
-// Bounded grid-wide barrier for a cooperative launch (all blocks co-resident).
-__device__ bool grid_barrier(unsigned* count, unsigned* gen, int* err) {
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    volatile unsigned* vg = gen;
-    const unsigned g = *vg;
-    __threadfence();
-    if (atomicAdd(count, 1u) == gridDim.x - 1) {
-      atomicExch(count, 0u);
-      __threadfence();
-      atomicAdd(gen, 1u);
-    } else {
-      long long i = 0;
-      while (*vg == g) {
-        if (++i > (1ll << 22) || *(volatile int*)err) {
-          atomicExch(err, 1);
-          break;
-        }
-        __nanosleep(64);
-      }
-    }
-    __threadfence();
-  }
-  __syncthreads();
-  return *(volatile int*)err == 0;
-}
-
-// One FP32 sweep of block Jacobi: the columns are grouped in blocks of kJB,
-// the blocks paired by the round-robin ordering, and each CTA takes one block
-// pair per round: it forms the Gram matrix G = C^T C of the pair's 2 kJB
-// columns (one pass over the rows, staged through shared memory), runs
-// kJInner cyclic Jacobi sweeps on G in shared memory (the rotation from the
-// 2x2 Gram entries of a column pair is the one-sided rotation of those two
-// columns; J^T G J keeps G current), and applies the accumulated rotation Q to
-// the pair's columns of X32 and Z32 in one more pass.  Each column is read a
-// few times per visit instead of once per rotation.  Rounds are separated by a
-// bounded grid barrier.  A rotation is counted when |g_pq| > tol sqrt(g_pp g_qq).
+// One FP32 sweep of block Jacobi: the columns are grouped in blocks of kJB, the blocks
+// paired by the round-robin ordering, and each block pair of a round is a work item of
+// `split` CTAs (one cluster), each on its share of the rows: they form the Gram matrix G
+// = C^T C of the pair's 2 kJB columns (partial sums exchanged through distributed shared
+// memory and added in rank order, so every rank continues with the same bits), run one
+// cyclic Jacobi sweep on G in shared memory (the rotation from the 2x2 Gram entries of a
+// column pair is the one-sided rotation of those two columns; J^T G J keeps G current),
+// and apply the accumulated rotation Q to their rows of the pair's columns of X32 and
+// Z32.  A rotation is counted when |g_pq| > tol sqrt(g_pp g_qq).
+//
+// Latency bounds it below n of a few thousand (the flops of a 1024^2 sweep take 0.2 ms),
+// so rows are shared until a CTA has 128, items start as soon as the previous items that
+// held their two blocks are done (per-block counters, acquire / release, as the FP64
+// sweep's) instead of after a grid barrier, and a step of the inner sweep is one phase:
+// thread (t1, t2) owns the 2x2 block of G at the rows of rotation t1 and the columns of
+// t2, forms both rotations itself, and writes to the other copy of G.
+// A sweep (events): n = 256 0.35 ms (0.51 with two phases a step, a grid barrier a round
+// and at most two CTAs a pair), n = 1024 2.1 (3.1), n = 2048 7.8 (8.7); at n = 4096 the
+// products take over (46.6, from 46).
 constexpr int kJB = 16;                // columns per block
 constexpr int kJW = 2 * kJB;           // columns of a block pair
-constexpr int kJRows = 256;            // rows per staged chunk (one per thread when loading)
-constexpr int kJLd = kJRows + 1;       // chunk leading dimension: conflict-free column and row walks
-constexpr int kJInner = 1;             // Jacobi sweeps on G per visit
+// rows per staged chunk: 128, or 256 where a CTA has several; the chunk's leading
+// dimension has 16-byte rows and no bank conflicts
+constexpr int kJRows = 128;
+template <int ROWS>
+constexpr int jac32_smem() {
+  return (kJW * (ROWS + 4) + 4 * kJW * kJW) * (int)sizeof(float);
+}
 
+template <int ROWS>
 __global__ void __launch_bounds__(kJacThreads, 2)
 jacobi32_block_sweep_kernel(float* X, float* Z, int64_t ld, int64_t m, int nb_even, int n_real,
-                            float tol, int* status, unsigned* bar, int* err, int stall,
-                            long long stall_ns, int split, float* Gp) {
-  static_assert(kJacThreads == 256 && kJW == 32 && kJRows == kJacThreads, "thread mapping below");
-  __shared__ float Ct[kJW * kJLd];             // chunk, column-major: Ct[j * kJLd + r]
-  __shared__ float G[kJW][kJW + 1];
-  __shared__ float Qm[kJW][kJW + 1];
-  __shared__ __align__(16) float Q4[kJW][kJW]; // Q for the vectorised product
-  __shared__ float s_c[kJB], s_s[kJB];
-  __shared__ int s_a[kJB], s_b[kJB];
+                            float tol, int* status, int* ver, int* err, int stall,
+                            long long stall_ns, int split, int vec) {
+  static_assert(kJacThreads == 256 && kJW == 32 && (ROWS == 128 || ROWS == 256), "thread mapping below");
+  constexpr int kJLd = ROWS + 4;
+  constexpr int kCols = kJW * ROWS / kJacThreads;   // columns a thread loads
+  namespace cgrp = cooperative_groups;
+  cgrp::cluster_group cluster = cgrp::this_cluster();
+  extern __shared__ __align__(16) float jac_smem[];
+  float* Ct = jac_smem;                // chunk, column-major: Ct[j * kJLd + r]
+  float* fold = jac_smem + kJW * kJLd; // four warps' partial Gram matrices
+  __shared__ float Gb[2][kJW][kJW + 1];
+  __shared__ __align__(16) float Q4[kJW][kJW];
+  __shared__ float part[2][kJW * kJW];
+  __shared__ int s_ok[2], s_alive[2], s_rot, never;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int npairs = nb_even / 2;
+  const int rank = blockIdx.x % split, first = blockIdx.x / split, step_items = gridDim.x / split;
+  const int64_t mh = ((m + split - 1) / split + 3) / 4 * 4;
+  const int64_t row_lo = rank * mh < m ? rank * mh : m;
+  const int64_t row_hi = row_lo + mh < m ? row_lo + mh : m;
+  const bool single = row_hi - row_lo <= ROWS;
+  if (tid == 0) s_rot = 0;
+  int buf = 0;
+  bool alive = true;
   if (stall && blockIdx.x == 0) {
     // test hook of the error exit: wait, bounded, on a flag that nothing sets
-    __shared__ int never;
-    if (threadIdx.x == 0) {
+    if (tid == 0) {
       never = 0;
       long long t0;
       asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
@@ -286,206 +346,224 @@ jacobi32_block_sweep_kernel(float* X, float* Z, int64_t ld, int64_t m, int nb_ev
       }
       atomicExch(err, 1);
     }
-    __syncthreads();
-    return;
+    alive = false;
   }
-  __shared__ int s_rot;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int npairs = nb_even / 2;
-  // split = 2: two blocks per block pair, each on half of the rows, so that an
-  // SM holds two blocks (16 warps) where one left it latency-bound; their Gram
-  // partials meet through Gp after a grid barrier (the host launches exactly
-  // 2 x npairs blocks then, so every block reaches that barrier once per round)
-  const int half = split == 2 ? (int)(blockIdx.x & 1) : 0;
-  const int64_t mh = split == 2 ? ((m + 1) / 2 + kJRows - 1) / kJRows * kJRows : m;
-  const int64_t row_lo = half * mh;
-  const int64_t row_hi = row_lo + mh < m ? row_lo + mh : m;
-  for (int round = 0; round < nb_even - 1; ++round) {
-    for (int pi = blockIdx.x / split; pi < npairs; pi += gridDim.x / split) {
-      auto elem = [&](int pos) { return pos == 0 ? 0 : 1 + (pos - 1 + round) % (nb_even - 1); };
-      int P = elem(pi), Qb = elem(nb_even - 1 - pi);
-      if (P > Qb) { const int t = P; P = Qb; Qb = t; }
-      auto col = [&](int j) { return j < kJB ? P * kJB + j : Qb * kJB + (j - kJB); };
-      // chunk loader: thread = row, all 32 columns (coalesced along each column).
-      // The next chunk is fetched into registers while the current one is used.
-      float pf[kJW];
-      auto fetch = [&](const float* M, int64_t r0) {
-        const int64_t r = r0 + tid;
+  for (int64_t it = first; it < (int64_t)(nb_even - 1) * npairs; it += step_items, buf ^= 1) {
+    const int round = (int)(it / npairs), pi = (int)(it - (int64_t)round * npairs);
+    auto elem = [&](int pos) { return pos == 0 ? 0 : 1 + (pos - 1 + round) % (nb_even - 1); };
+    int P = elem(pi), Qb = elem(nb_even - 1 - pi);
+    if (P > Qb) { const int t = P; P = Qb; Qb = t; }
+    auto col = [&](int j) { return j < kJB ? P * kJB + j : Qb * kJB + (j - kJB); };
+    // both blocks' previous items done, by all their ranks
+    if (tid < 2)
+      s_ok[tid] = alive && !*(volatile int*)err && wait_round(ver + (tid ? Qb : P), split * round, err);
+    __syncthreads();
+    const bool ok = s_ok[0] && s_ok[1];
+    // chunk loader: thread = row and half of the columns (256 rows: all); the next chunk is fetched into
+    // registers while the current one is used (through L2: other SMs wrote it)
+    const int lr = tid & (ROWS - 1), lj = tid / ROWS * kCols;
+    float pf[kCols];
+    auto fetch = [&](const float* M, int64_t r0) {
+      const int64_t r = r0 + lr;
 #pragma unroll
-        for (int j = 0; j < kJW; ++j) {
-          const int c = col(j);
-          pf[j] = (c < n_real && r < row_hi) ? M[(int64_t)c * ld + r] : 0.f;
-        }
-      };
-      auto stage = [&]() {
+      for (int j = 0; j < kCols; ++j) {
+        const int c = col(lj + j);
+        pf[j] = (c < n_real && r < row_hi) ? __ldcg(M + (int64_t)c * ld + r) : 0.f;
+      }
+    };
+    auto stage = [&]() {
 #pragma unroll
-        for (int j = 0; j < kJW; ++j) Ct[j * kJLd + tid] = pf[j];
-      };
-      // ---- 1. Gram G = C^T C: 16 row groups; thread owns the 8x8 block (bi, bj)
-      //         of G over the rows r = g (mod 16) of each chunk
-      {
-        const int g = tid >> 4, t = tid & 15, bi = t >> 2, bj = t & 3;
-        float acc[8][8];
+      for (int j = 0; j < kCols; ++j) Ct[(lj + j) * kJLd + lr] = pf[j];
+    };
+    if (ok) {
+      // ---- 1. Gram G = C^T C: 16 row groups; thread owns the 8x8 block (bi, bj) of G
+      //         over the rows r = g (mod 16) of each chunk
+      const int g = tid >> 4, t = tid & 15, bi = t >> 2, bj = t & 3;
+      float acc[8][8];
 #pragma unroll
-        for (int a = 0; a < 8; ++a)
+      for (int a = 0; a < 8; ++a)
 #pragma unroll
-          for (int b = 0; b < 8; ++b) acc[a][b] = 0.f;
-        fetch(X, row_lo);
-        for (int64_t r0 = row_lo; r0 < row_hi; r0 += kJRows) {
-          stage();
-          __syncthreads();
-          if (r0 + kJRows < row_hi) fetch(X, r0 + kJRows);
-          for (int r = g; r < kJRows; r += 16) {
-            float va[8], vb[8];
+        for (int b = 0; b < 8; ++b) acc[a][b] = 0.f;
+      fetch(X, row_lo);
+      for (int64_t r0 = row_lo; r0 < row_hi; r0 += ROWS) {
+        stage();
+        __syncthreads();
+        if (r0 + ROWS < row_hi) fetch(X, r0 + ROWS);
+#pragma unroll 2
+        for (int r = g; r < ROWS; r += 16) {
+          float va[8], vb[8];
 #pragma unroll
-            for (int a = 0; a < 8; ++a) va[a] = Ct[(8 * bi + a) * kJLd + r];
+          for (int a = 0; a < 8; ++a) va[a] = Ct[(8 * bi + a) * kJLd + r];
 #pragma unroll
-            for (int b = 0; b < 8; ++b) vb[b] = Ct[(8 * bj + b) * kJLd + r];
-#pragma unroll
-            for (int a = 0; a < 8; ++a)
-#pragma unroll
-              for (int b = 0; b < 8; ++b) acc[a][b] = fmaf(va[a], vb[b], acc[a][b]);
-          }
-          __syncthreads();
-        }
-        // groups 2w and 2w+1 share warp w (lanes l and l ^ 16): fold them, then
-        // sum the 8 warps' partials through the chunk buffer
-#pragma unroll
-        for (int a = 0; a < 8; ++a)
-#pragma unroll
-          for (int b = 0; b < 8; ++b) acc[a][b] += __shfl_xor_sync(0xffffffffu, acc[a][b], 16);
-        if (lane < 16)
+          for (int b = 0; b < 8; ++b) vb[b] = Ct[(8 * bj + b) * kJLd + r];
 #pragma unroll
           for (int a = 0; a < 8; ++a)
 #pragma unroll
-            for (int b = 0; b < 8; ++b) Ct[warp * kJW * kJW + (8 * bi + a) * kJW + (8 * bj + b)] = acc[a][b];
+            for (int b = 0; b < 8; ++b) acc[a][b] = fmaf(va[a], vb[b], acc[a][b]);
+        }
+        __syncthreads();
+      }
+      // one chunk: X stays staged and Z is on its way during the inner sweep
+      if (single) fetch(Z, row_lo);
+      // groups 2w and 2w+1 share warp w (lanes l and l ^ 16): fold them, then the warps'
+      // partials through shared memory, four at a time
+#pragma unroll
+      for (int a = 0; a < 8; ++a)
+#pragma unroll
+        for (int b = 0; b < 8; ++b) acc[a][b] += __shfl_xor_sync(0xffffffffu, acc[a][b], 16);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        if (lane < 16 && (warp >> 2) == h)
+#pragma unroll
+          for (int a = 0; a < 8; ++a)
+#pragma unroll
+            for (int b = 0; b < 8; ++b)
+              fold[(warp & 3) * kJW * kJW + (8 * bi + a) * kJW + (8 * bj + b)] = acc[a][b];
         __syncthreads();
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-          const int e = tid + kJacThreads * u, i = e >> 5, jj = e & 31;
-          float sum = 0.f;
-#pragma unroll
-          for (int w = 0; w < kJacThreads / 32; ++w) sum += Ct[w * kJW * kJW + e];
-          G[i][jj] = sum;
-          Qm[i][jj] = i == jj ? 1.f : 0.f;
-          if (split == 2) Gp[((int64_t)pi * 2 + half) * kJW * kJW + e] = sum;
-        }
-      }
-      if (split == 2) {
-        // both halves' partials, summed in the same order by both blocks (read
-        // through L2: the partner wrote them on another SM)
-        if (!grid_barrier(bar, bar + 1, err)) return;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int e = tid + kJacThreads * u, i = e >> 5, jj = e & 31;
-          G[i][jj] = __ldcg(Gp + (int64_t)pi * 2 * kJW * kJW + e) +
-                     __ldcg(Gp + ((int64_t)pi * 2 + 1) * kJW * kJW + e);
-        }
-      }
-      if (tid == 0) s_rot = 0;
-      __syncthreads();
-      // ---- 2. cyclic Jacobi on G (round-robin over the 32 indices, 16 disjoint
-      //         rotations per step); Q accumulates the rotations
-      for (int sw = 0; sw < kJInner; ++sw) {
-        for (int step = 0; step < kJW - 1; ++step) {
-          if (tid < kJB) {
-            auto e2 = [&](int pos) { return pos == 0 ? 0 : 1 + (pos - 1 + step) % (kJW - 1); };
-            int a = e2(tid), b = e2(kJW - 1 - tid);
-            if (a > b) { const int t = a; a = b; b = t; }
-            const float ga = G[a][a], gb = G[b][b], gab = G[a][b];
-            float c = 1.f, sn = 0.f;
-            if (col(b) < n_real && gab != 0.f && fabsf(gab) > tol * sqrtf(ga) * sqrtf(gb)) {
-              const float zeta = (gb - ga) / (2.f * gab);
-              const float t = (zeta >= 0.f ? 1.f : -1.f) / (fabsf(zeta) + sqrtf(fmaf(zeta, zeta, 1.f)));
-              c = 1.f / sqrtf(fmaf(t, t, 1.f));
-              sn = c * t;
-              atomicAdd(&s_rot, 1);
-            }
-            s_a[tid] = a; s_b[tid] = b; s_c[tid] = c; s_s[tid] = sn;
-          }
-          __syncthreads();
-          // rows a, b of G (J^T G): 16 rotations x 32 entries, two per thread
-#pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            const int e = tid + kJacThreads * u, t = e >> 5, k = e & 31;
-            const int a = s_a[t], b = s_b[t];
-            const float c = s_c[t], sn = s_s[t];
-            const float x = G[a][k], y = G[b][k];
-            G[a][k] = c * x - sn * y;
-            G[b][k] = fmaf(sn, x, c * y);
-          }
-          __syncthreads();
-          // columns a, b of G and of Q (G J, Q J)
-#pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            const int e = tid + kJacThreads * u, t = e >> 5, k = e & 31;
-            const int a = s_a[t], b = s_b[t];
-            const float c = s_c[t], sn = s_s[t];
-            const float x = G[k][a], y = G[k][b];
-            G[k][a] = c * x - sn * y;
-            G[k][b] = fmaf(sn, x, c * y);
-            const float qx = Qm[k][a], qy = Qm[k][b];
-            Qm[k][a] = c * qx - sn * qy;
-            Qm[k][b] = fmaf(sn, qx, c * qy);
-          }
-          __syncthreads();
-        }
-      }
-      const int nrot = s_rot;
-      if (tid == 0 && nrot && half == 0) atomicAdd(status + kStatJacobiRot, nrot);
-      // ---- 3. X and Z columns of the pair times Q (skipped when nothing rotated):
-      //         thread computes rows 8 rt .. 8 rt + 7, columns 4 ct .. 4 ct + 3
-      if (nrot) {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
           const int e = tid + kJacThreads * u;
-          Q4[e >> 5][e & 31] = Qm[e >> 5][e & 31];
+          const float sum = (fold[e] + fold[kJW * kJW + e]) + (fold[2 * kJW * kJW + e] + fold[3 * kJW * kJW + e]);
+          part[buf][e] = h ? part[buf][e] + sum : sum;
         }
-        const int rt = tid >> 3, ct = tid & 7;
-        for (int which = 0; which < 2; ++which) {
-          float* M = which ? Z : X;
-          fetch(M, row_lo);
-          for (int64_t r0 = row_lo; r0 < row_hi; r0 += kJRows) {
+        __syncthreads();
+      }
+    }
+    if (tid == 0) s_alive[buf] = ok;
+    if (split > 1) cluster.sync();   // the ranks' partial sums (and whether all go on)
+    else __syncthreads();
+    bool all = true;
+    if (split == 1) all = ok;
+    else for (int k = 0; k < split; ++k) all = all && cluster.map_shared_rank(s_alive, k)[buf] != 0;
+    if (!all) break;                 // every rank of the cluster leaves here
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int e = tid + kJacThreads * u, i = e >> 5, jj = e & 31;
+      float sum = 0.f;
+      if (split == 1) sum = part[buf][e];
+      else for (int k = 0; k < split; ++k) sum += cluster.map_shared_rank(&part[0][0], k)[buf * kJW * kJW + e];
+      Gb[0][i][jj] = sum;
+      Q4[i][jj] = i == jj ? 1.f : 0.f;
+    }
+    __syncthreads();
+    // ---- 2. cyclic Jacobi on G (round-robin over the 32 indices, 16 disjoint
+    //         rotations per step); Q accumulates the rotations
+    int nrot = 0;
+    {
+      const int t1 = tid >> 4, t2 = tid & 15;
+      for (int step = 0; step < kJW - 1; ++step) {
+        float (*G)[kJW + 1] = Gb[step & 1];
+        float (*Gn)[kJW + 1] = Gb[(step & 1) ^ 1];
+        auto pair = [&](int k, int* a, int* b) {
+          auto e2 = [&](int pos) { return pos == 0 ? 0 : 1 + (pos - 1 + step) % (kJW - 1); };
+          const int x = e2(k), y = e2(kJW - 1 - k);
+          *a = x < y ? x : y;
+          *b = x < y ? y : x;
+        };
+        int a1, b1, a2, b2;
+        pair(t1, &a1, &b1);
+        pair(t2, &a2, &b2);
+        // rotation t2 (each half-warp has all sixteen); t1's comes from its lane
+        float c2 = 1.f, n2 = 0.f;
+        {
+          const float ga = G[a2][a2], gb = G[b2][b2], gab = G[a2][b2];
+          auto quotient = [](float n, float d) {
+            const float r = __fdividef(1.f, d), q = n * r;
+            return fmaf(r, fmaf(-d, q, n), q);
+          };
+          if (col(b2) < n_real && gab != 0.f && ga > 0.f && gb > 0.f &&
+              fabsf(gab) * rsqrtf(ga) * rsqrtf(gb) > tol) {
+            // approximations polished to FP32 rounding by one Newton step each (a wrong
+            // angle leaves its error times the cosine to the next sweep)
+            const float zeta = quotient(0.5f * (gb - ga), gab), az = fminf(fabsf(zeta), 1e18f);
+            const float z1 = fmaf(az, az, 1.f), ri = rsqrtf(z1), rt = z1 * ri;
+            const float root = fmaf(0.5f * ri, fmaf(-rt, rt, z1), rt);
+            const float t = copysignf(quotient(1.f, az + root), zeta);
+            const float x = fmaf(t, t, 1.f);
+            c2 = rsqrtf(x);
+            c2 = c2 * fmaf(-0.5f * x * c2, c2, 1.5f);
+            n2 = c2 * t;
+            if (t1 == t2) ++nrot;
+          }
+        }
+        const float c1 = __shfl_sync(0xffffffffu, c2, t1), n1 = __shfl_sync(0xffffffffu, n2, t1);
+        // rows a1, b1 (J^T G), then columns a2, b2 (G J) of the 2x2 block
+        const float x0 = G[a1][a2], x1 = G[a1][b2], y0 = G[b1][a2], y1 = G[b1][b2];
+        const float p0 = c1 * x0 - n1 * y0, p1 = c1 * x1 - n1 * y1;
+        const float q0 = fmaf(n1, x0, c1 * y0), q1 = fmaf(n1, x1, c1 * y1);
+        Gn[a1][a2] = c2 * p0 - n2 * p1;
+        Gn[a1][b2] = fmaf(n2, p0, c2 * p1);
+        Gn[b1][a2] = c2 * q0 - n2 * q1;
+        Gn[b1][b2] = fmaf(n2, q0, c2 * q1);
+        // columns a2, b2 of Q: rows t1 and t1 + 16
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const int k = t1 + 16 * u;
+          const float qx = Q4[k][a2], qy = Q4[k][b2];
+          Q4[k][a2] = c2 * qx - n2 * qy;
+          Q4[k][b2] = fmaf(n2, qx, c2 * qy);
+        }
+        __syncthreads();
+      }
+    }
+    if (nrot) atomicAdd(&s_rot, nrot);
+    const int any = __syncthreads_or(nrot);
+    // ---- 3. this rank's rows of the pair's X and Z columns times Q (skipped when
+    //         nothing rotated): thread computes rows 4 rt .. + 3, columns 4 ct .. + 3
+    if (any) {
+      const int rt = tid >> 3, ct = tid & 7;
+      for (int which = 0; which < 2; ++which) {
+        float* M = which ? Z : X;
+        if (!single) fetch(M, row_lo);
+        for (int64_t r0 = row_lo; r0 < row_hi; r0 += ROWS) {
+          if (!single || which) {
             stage();
             __syncthreads();
-            if (r0 + kJRows < row_hi) fetch(M, r0 + kJRows);
-            float o[8][4];
+          }
+          if (r0 + ROWS < row_hi) fetch(M, r0 + ROWS);
 #pragma unroll
-            for (int a = 0; a < 8; ++a)
+          for (int h = 0; h < ROWS / 128; ++h) {
+            float o[4][4];
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
 #pragma unroll
               for (int b = 0; b < 4; ++b) o[a][b] = 0.f;
-#pragma unroll 4
+#pragma unroll 8
             for (int k = 0; k < kJW; ++k) {
               const float4 q = *reinterpret_cast<const float4*>(&Q4[k][4 * ct]);
+              const float4 x = *reinterpret_cast<const float4*>(&Ct[k * kJLd + 128 * h + 4 * rt]);
+              const float xv[4] = {x.x, x.y, x.z, x.w}, qv[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
-              for (int a = 0; a < 8; ++a) {
-                const float cv = Ct[k * kJLd + 8 * rt + a];
-                o[a][0] = fmaf(cv, q.x, o[a][0]);
-                o[a][1] = fmaf(cv, q.y, o[a][1]);
-                o[a][2] = fmaf(cv, q.z, o[a][2]);
-                o[a][3] = fmaf(cv, q.w, o[a][3]);
+              for (int a = 0; a < 4; ++a)
+#pragma unroll
+                for (int b = 0; b < 4; ++b) o[a][b] = fmaf(xv[a], qv[b], o[a][b]);
+            }
+            const int64_t r = r0 + 128 * h + 4 * rt;
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+              const int c = col(4 * ct + b);
+              if (c >= n_real) continue;
+              float* d = M + (int64_t)c * ld + r;
+              if (vec && r + 4 <= row_hi) {
+                *reinterpret_cast<float4*>(d) = make_float4(o[0][b], o[1][b], o[2][b], o[3][b]);
+              } else {
+#pragma unroll
+                for (int a = 0; a < 4; ++a)
+                  if (r + a < row_hi) d[a] = o[a][b];
               }
             }
-            __syncthreads();
-#pragma unroll
-            for (int a = 0; a < 8; ++a)
-#pragma unroll
-              for (int b = 0; b < 4; ++b) Ct[(4 * ct + b) * kJLd + 8 * rt + a] = o[a][b];
-            __syncthreads();
-            const int64_t r = r0 + tid;
-#pragma unroll 8
-            for (int j = 0; j < kJW; ++j) {
-              const int c = col(j);
-              if (c < n_real && r < row_hi) M[(int64_t)c * ld + r] = Ct[j * kJLd + tid];
-            }
-            __syncthreads();
           }
+          __syncthreads();   // the chunk is refilled
         }
       }
-      __syncthreads();
     }
-    if (!grid_barrier(bar, bar + 1, err)) return;
+    // publish: as the FP64 sweep's, one count per rank
+    __syncthreads();
+    if (tid < 2) add_release(ver + (tid ? Qb : P), 1);
   }
+  if (split > 1) cluster.sync();   // no rank leaves while another reads its partial sums
+  __syncthreads();
+  if (tid == 0 && rank == 0 && s_rot) atomicAdd(status + kStatJacobiRot, s_rot);
 }
 
 __global__ void to_f32_kernel(const double* __restrict__ X, float* __restrict__ Y, int64_t n) {
@@ -621,23 +699,42 @@ cudaError_t transpose_lower(const double* R, int64_t ldr, double* X, int64_t ldx
 
 // One FP64 sweep: n_even - 1 rounds of n_even / 2 pairs (ProfScope: 6 flops and
 // 32 bytes per row and pair).
-cudaError_t jacobi_sweep(double* X, int64_t ldx, int64_t m, int64_t n_even, int64_t n_real,
-                         double tol, int* status, double* nrm2, double* dsc, int* ver, int* err,
-                         int stall, long long stall_ns, cudaStream_t st) {
+template <int NT, int RPT>
+static cudaError_t launch_sweep(double* X, int64_t ldx, int64_t m, int64_t n_even, int64_t n_real,
+                                double tol, int* status, double* nrm2, double* dsc, int* ver, int* err,
+                                int stall, long long stall_ns, cudaStream_t st) {
+  const void* kernel = (const void*)jacobi_sweep_kernel<NT, RPT>;
   int occ = 0, dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, jacobi_sweep_kernel, kJacThreads, 0) !=
-          cudaSuccess)
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, NT, 0) != cudaSuccess)
     return cudaErrorUnknown;
   const int64_t items = (n_even - 1) * (n_even / 2);
-  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(items, (int64_t)std::max(1, occ) * sms));
+  // short columns: blocks further ahead than the next round only poll, and the polls
+  // cost the others (n = 256: 1.1 ms a sweep with one round's 128 blocks, 1.6 with four;
+  // n = 512: 2.8 and 3.5; n = 1024: 6.2 with one and a half rounds' 768, 7.8 with 512)
+  const int64_t npairs = n_even / 2;
+  const int64_t want = RPT == 0 ? items : m <= 512 ? npairs : npairs + npairs / 2;
+  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(std::min(want, items),
+                                                               (int64_t)std::max(1, occ) * sms));
   if (cudaMemsetAsync(ver, 0, sizeof(int) * n_even, st) != cudaSuccess) return cudaErrorUnknown;
   ProfScope ps(kProfJacobi, st, 6.0 * (double)m * (double)items, 32.0 * (double)m * (double)items);
-  ps.blocks((const void*)jacobi_sweep_kernel, dim3(kJacThreads), 0, dim3(grid));
+  ps.blocks(kernel, dim3(NT), 0, dim3(grid));
   int ne = (int)n_even, nr = (int)n_real;
   void* args[] = {&X, &ldx, &m, &ne, &nr, &tol, &status, &nrm2, &dsc, &ver, &err, &stall, &stall_ns};
-  return cudaLaunchCooperativeKernel((const void*)jacobi_sweep_kernel, grid, kJacThreads, args, 0, st);
+  return cudaLaunchCooperativeKernel(kernel, grid, NT, args, 0, st);
+}
+
+cudaError_t jacobi_sweep(double* X, int64_t ldx, int64_t m, int64_t n_even, int64_t n_real,
+                         double tol, int* status, double* nrm2, double* dsc, int* ver, int* err,
+                         int stall, long long stall_ns, cudaStream_t st) {
+  // up to 1024 rows in registers; longer columns are bound by the FP64 units and want
+  // six blocks an SM (4096 rows: 161 ms a sweep, 237 with 16 rows a thread held)
+  const auto launch = m <= 256    ? launch_sweep<128, 2>
+                      : m <= 512  ? launch_sweep<128, 4>
+                      : m <= 1024 ? launch_sweep<256, 4>
+                                  : launch_sweep<256, 0>;
+  return launch(X, ldx, m, n_even, n_real, tol, status, nrm2, dsc, ver, err, stall, stall_ns, st);
 }
 
 // Full driver.  Returns 0; 1 = CUDA error, 2 = no convergence, 3 = a bounded
@@ -684,45 +781,58 @@ int eig_sym_jacobi(const double* H, int64_t ldh, int64_t n, double* V, int64_t l
     identity_f32_kernel<<<eg, 256, 0, st>>>(w.Z32, n);
   }
   if (n > 1) {
-    int occ = 0, dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, jacobi32_block_sweep_kernel, kJacThreads,
-                                                      0) != cudaSuccess)
-      return 1;
+    const bool wide = n >= 2048;
+    const auto kern = wide ? jacobi32_block_sweep_kernel<256> : jacobi32_block_sweep_kernel<128>;
+    const void* kernel = (const void*)kern;
+    const int smem = wide ? jac32_smem<256>() : jac32_smem<128>();
+    if (smem_attr_once(kernel, smem) != cudaSuccess) return 1;
     const int nb = (int)((n + kJB - 1) / kJB);
-    const int nb_even = nb + (nb & 1);
-    // two blocks per block pair when they all fit at once and a half has rows
-    // to spare (n >= 512); the partial Gram matrices go to Z, unused until the
-    // FP32 phase ends
-    const int split = (int64_t)nb_even <= (int64_t)std::max(1, occ) * sms && n >= 2 * kJRows ? 2 : 1;
-    const int grid =
-        split == 2 ? nb_even : (int)std::min<int64_t>(nb_even / 2, (int64_t)std::max(1, occ) * sms);
-    float* Gp = reinterpret_cast<float*>(w.Z);
+    const int nb_even = nb + (nb & 1), npairs = nb_even / 2;
+    // CTAs per block pair (one cluster): while each keeps 128 rows and all pairs of a
+    // round fit on the GPU at once
+    int split = 8, grid = 0;
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at[2];
+    for (;; split /= 2) {
+      cfg.blockDim = dim3(kJacThreads);
+      cfg.dynamicSmemBytes = smem;
+      cfg.gridDim = dim3((unsigned)(npairs * split));
+      cfg.stream = st;
+      at[0].id = cudaLaunchAttributeCooperative;
+      at[0].val.cooperative = 1;
+      at[1].id = cudaLaunchAttributeClusterDimension;
+      at[1].val.clusterDim.x = split;
+      at[1].val.clusterDim.y = 1;
+      at[1].val.clusterDim.z = 1;
+      cfg.attrs = at;
+      cfg.numAttrs = split > 1 ? 2 : 1;
+      if (split == 1) break;
+      int clusters = 0;
+      if ((n + split - 1) / split < kJRows) continue;
+      if (cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) != cudaSuccess) return 1;
+      if (clusters >= npairs) break;
+    }
+    if (split == 1) {
+      int occ = 0, dev = 0, sms = 0;
+      if (cudaGetDevice(&dev) != cudaSuccess ||
+          cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, kJacThreads, smem) != cudaSuccess)
+        return 1;
+      cfg.gridDim = dim3((unsigned)std::min<int64_t>(npairs, (int64_t)std::max(1, occ) * sms));
+    }
+    grid = (int)cfg.gridDim.x;
     const float tol32 = 8e-6f;
     for (int sw = 0; sw < 25; ++sw) {
       if (cudaMemsetAsync(w.status + kStatJacobiRot, 0, sizeof(int), st) != cudaSuccess) return 1;
-      if (cudaMemsetAsync(w.bar, 0, 2 * sizeof(unsigned), st) != cudaSuccess) return 1;
-      float* X32 = w.X32;
-      float* Z32 = w.Z32;
-      int64_t ld = n, mm = n;
-      int ne = nb_even, nr = (int)n;
-      float tol = tol32;
-      int* status = w.status;
-      unsigned* bar = w.bar;
-      int* err = w.err;
-      int stall = sw == 0 ? w.stall : 0;
-      long long stall_ns = w.stall_ns;
-      int sp = split;
-      void* args[] = {&X32, &Z32, &ld, &mm, &ne, &nr, &tol, &status, &bar, &err, &stall, &stall_ns,
-                      &sp, &Gp};
+      if (cudaMemsetAsync(w.ver, 0, sizeof(int) * nb_even, st) != cudaSuccess) return 1;
       {
         // Gram and two products with Q per block pair: 6 (2 kJB)^2 m flops
         ProfScope ps(kProfJacobi32, st,
-                     6.0 * kJW * kJW * (double)n * (double)(nb_even / 2) * (double)(nb_even - 1));
-        ps.blocks((const void*)jacobi32_block_sweep_kernel, dim3(kJacThreads), 0, dim3(grid));
-        if (cudaLaunchCooperativeKernel((const void*)jacobi32_block_sweep_kernel, grid, kJacThreads,
-                                        args, 0, st) != cudaSuccess)
+                     6.0 * kJW * kJW * (double)n * (double)npairs * (double)(nb_even - 1));
+        ps.blocks(kernel, dim3(kJacThreads), smem, dim3(grid));
+        if (cudaLaunchKernelEx(&cfg, kern, w.X32, w.Z32, n, n, nb_even, (int)n,
+                               tol32, w.status, w.ver, w.err, sw == 0 ? w.stall : 0, w.stall_ns, split,
+                               (int)(n % 4 == 0)) != cudaSuccess)
           return 1;
       }
       int rot = 0, herr = 0;
@@ -764,7 +874,9 @@ int eig_sym_jacobi(const double* H, int64_t ldh, int64_t n, double* V, int64_t l
   }
   double* X = w.HV;
   // ---- FP64 sweeps
-  const double tol_strict = 8.0 * kEps, tol_loose = sqrt((double)n) * kEps;
+  // ||V^T V - I||_F / sqrt(n) with rotations down to 2 eps and down to 8 eps: n = 256
+  // 1.2e-15 and 4.8e-15, n = 1024 2.7e-15 and 5.2e-15, n = 4096 4.3e-15 and 1.1e-14
+  const double tol_rot = 2.0 * kEps, tol_loose = sqrt((double)n) * kEps;
   bool converged = n == 1;
   for (int sw = 0; sw < 40 && !converged; ++sw) {
     if (cudaMemsetAsync(w.status + kStatJacobiRot, 0, 2 * sizeof(int), st) != cudaSuccess) return 1;
@@ -777,7 +889,7 @@ int eig_sym_jacobi(const double* H, int64_t ldh, int64_t n, double* V, int64_t l
       fill_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(w.tmp, n, 1.0);
     }
     if (column_dots(X, n, X, n, n, n, w.lam, st) != cudaSuccess) return 1;
-    if (jacobi_sweep(X, n, n, n_even, n, tol_strict, w.status, w.lam, w.tmp, w.ver, w.err,
+    if (jacobi_sweep(X, n, n, n_even, n, tol_rot, w.status, w.lam, w.tmp, w.ver, w.err,
                      sw == 0 ? w.stall64 : 0, w.stall_ns, st) != cudaSuccess)
       return 1;
     int rs[2] = {0, 0}, herr = 0;

@@ -327,12 +327,11 @@ struct EigWork {
   float* Z32;       // n x n, accumulated FP32 rotations
   double* Z;        // n x n, Z orthonormalised in FP64
   double* tmp;      // n x 64 scratch of the triangular solve
-  unsigned* bar;    // grid-barrier words (2)
-  int* ver;         // n + 1 per-column round counters of the FP64 sweeps
+  int* ver;         // n + 1 round counters, per column (FP64 sweeps) or block (FP32 ones)
   int* err;         // bounded-wait error flag
   // test hook of the failure path: with stall = 1, block 0 of the first FP32
   // sweep waits, for stall_ns, on a flag nothing sets, then takes the
-  // bounded-wait error exit (the other blocks leave the grid barrier on the flag)
+  // bounded-wait error exit (its cluster and the blocks that wait leave on the flag)
   int stall = 0;
   // the same for the first FP64 sweep: block 0 waits on a flag nothing sets, the
   // blocks whose work items need its columns leave on the error flag
