@@ -39,7 +39,7 @@
 namespace zolo {
 namespace {
 
-constexpr int kPanelCluster = 8;            // CTAs per shift in the cluster panel
+constexpr int kPanelCluster = 8;            // CTAs per shift in the global-memory panel
 constexpr int64_t kClusterPanelMinRows = 512;
 
 // Reduce-scatter of 32 per-lane partial sums across a warp: on return lane q
@@ -264,209 +264,6 @@ tb_merge_kernel(const double* __restrict__ G, int64_t strideG, double* __restric
   }
 }
 
-// Shared-memory form of the panel factorisation: each of the CG CTAs of a
-// shift (one cluster; CG = 1 is a single CTA) loads its rows of the panel's 32
-// columns into shared memory once, factors them there, and writes W, V and T
-// back at the end.  The per-column steps are those of the cluster kernel above
-// (norm and dot-product partials exchanged through distributed shared memory in
-// rank order, so every CTA forms the same beta, tau and dots); only the panel's
-// storage moves from L2 to shared memory, which removes the L2 round trips of
-// the ~80 accesses per row and column.  The reflector's unit diagonal is kept
-// implicit (the diagonal slot holds beta once it is formed), so no second copy
-// of V is needed.  Rows per CTA: ceil((m + NB) / CG) <= kSmemPanelRows.
-constexpr int kSmemPanelRows = 768;
-
-// A one-CTA "cluster" needs no cluster barrier and no distributed shared memory:
-// the panel kernels of one CTA per shift (the batched call's common case) use a
-// CTA barrier and their own partial sums.
-template <int CG>
-__device__ __forceinline__ void panel_sync(cooperative_groups::cluster_group& cluster) {
-  if constexpr (CG == 1) __syncthreads();
-  else cluster.sync();
-}
-template <int CG>
-__device__ __forceinline__ const double* panel_part(cooperative_groups::cluster_group& cluster,
-                                                    double* p, int rank) {
-  if constexpr (CG == 1) return p;
-  else return cluster.map_shared_rank(p, rank);
-}
-
-template <int NB, int CG>
-__global__ void __cluster_dims__(CG, 1, 1) __launch_bounds__(256)
-qr_panel_smem_kernel(double* W, int64_t strideW, int64_t ldw, int64_t m, int64_t c0, int nbp,
-                     double* V, int64_t strideV, int64_t ldv, double* T, int64_t strideT,
-                     int* status) {
-  namespace cgrp = cooperative_groups;
-  cgrp::cluster_group cluster = cgrp::this_cluster();
-  constexpr int kT = 256, kWarps = kT / 32;
-  extern __shared__ double Ws[];              // NB columns x Rs rows, column-major
-  __shared__ double part[2][NB + 2];          // [0, NB): dots, NB: norm^2, NB+1: alpha
-  __shared__ double red[kWarps][NB + 2];
-  __shared__ double dots[NB];
-  __shared__ double cf[NB];                // -tau dots[q]: the update's coefficients
-  __shared__ double Ts[NB][NB + 1];
-  __shared__ double s_tau, s_scal, s_beta;
-
-  const int rank = (int)cluster.block_rank();
-  const int shift = blockIdx.x / CG;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  double* Wj = W + shift * strideW;
-  double* Vp = V + shift * strideV + c0 * ldv;
-  double* Tp = T + shift * strideT + (c0 / NB) * (int64_t)(NB * NB);
-  const int64_t height = m + NB;
-  const int Rs = (int)((height + CG - 1) / CG);
-  const int64_t lo = c0 + (int64_t)rank * Rs;             // my window rows [lo, hi)
-  const int64_t hi = lo + Rs < c0 + height ? lo + Rs : c0 + height;
-  const int64_t rows_w = ldw;                             // rows that exist in W (m + n)
-  const int nr = hi > lo ? (int)(hi - lo) : 0;
-
-  for (int q = 0; q < NB; ++q)
-    for (int rr = tid; rr < Rs; rr += kT) {
-      const int64_t r = lo + rr;
-      Ws[q * Rs + rr] = (q < nbp && rr < nr && r < rows_w) ? Wj[r + (c0 + q) * ldw] : 0.0;
-    }
-  for (int e = tid; e < NB * (NB + 1); e += kT) (&Ts[0][0])[e] = 0.0;
-  __syncthreads();
-
-  for (int i = 0; i < nbp; ++i) {
-    const int64_t c = c0 + i;
-    const int buf = i & 1;
-    double* col = Ws + i * Rs;
-    const int64_t r0 = lo > c ? lo : c;                  // my part of the support [c, m + c]
-    const int64_t r1 = hi < m + c + 1 ? hi : m + c + 1;
-    // ---- 1. partial norm of the tail (rows > c) and alpha from the owner of row c
-    double ss = 0.0;
-    for (int64_t r = (r0 > c + 1 ? r0 : c + 1) + tid; r < r1; r += kT) {
-      const double v = col[r - lo];
-      ss = fma(v, v, ss);
-    }
-    // the block's partials are summed by warp 0 (kWarps - 1 + 5 FP64 warp
-    // instructions; a butterfly in every warp would take 5 per warp, and an FP64
-    // instruction costs its unit a whole warp slot however few lanes it uses)
-    double* flat = &red[0][0];
-    flat[tid] = ss;
-    __syncthreads();
-    if (warp == 0) {
-      double t = flat[lane];
-#pragma unroll
-      for (int w = 1; w < kWarps; ++w) t += flat[lane + 32 * w];
-      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-      if (lane == 0) {
-        part[buf][NB] = t;
-        part[buf][NB + 1] = (c >= lo && c < hi) ? col[c - lo] : 0.0;
-      }
-    }
-    panel_sync<CG>(cluster);
-    if (tid == 0) {
-      double sum = 0.0, alpha = 0.0;
-      for (int rk = 0; rk < CG; ++rk) {
-        const double* rp = panel_part<CG>(cluster, &part[buf][0], rk);
-        sum += rp[NB];
-        alpha += rp[NB + 1];
-      }
-      double beta, tau, scal;
-      if (sum == 0.0) {
-        beta = alpha; tau = 0.0; scal = 0.0;
-      } else {
-        beta = -copysign(sqrt(fma(alpha, alpha, sum)), alpha);
-        tau = (beta - alpha) / beta;
-        scal = 1.0 / (alpha - beta);
-      }
-      if (rank == 0 && (!isfinite(beta) || !isfinite(tau))) atomicOr(status + kStatNonFinite, 1);
-      s_beta = beta; s_tau = tau; s_scal = scal;
-    }
-    __syncthreads();
-    const double tau = s_tau, scal = s_scal;
-    // ---- 2. my rows of v below the diagonal; the diagonal slot takes beta
-    //         (v's unit diagonal is implicit from here on)
-    for (int64_t r = (r0 > c + 1 ? r0 : c + 1) + tid; r < r1; r += kT) col[r - lo] *= scal;
-    if (tid == 0 && c >= lo && c < hi) col[c - lo] = s_beta;
-    __syncthreads();
-    // ---- 3. dots of v with the other panel columns (the later ones for the
-    //         update, the earlier reflectors for T): warp w takes the four columns
-    //         4w..4w+3 over all my rows, lanes striding the rows, so each dot is
-    //         reduced over 32 lanes (a four-value reduce-scatter, six adds a
-    //         lane) instead of over every thread of the CTA
-    static_assert(NB == 4 * kWarps, "four dot products per warp");
-    {
-      double a4[4] = {0.0, 0.0, 0.0, 0.0};
-      const int q0 = 4 * warp;
-      for (int64_t r = r0 + lane; r < r1; r += 32) {
-        const double v = (r == c) ? 1.0 : col[r - lo];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const int q = q0 + k;
-          if (q < nbp && q != i) {
-            // earlier reflector q: support rows [c0+q, m+c0+q]; r >= c > c0+q
-            const double o = (q > i || r <= m + c0 + q) ? Ws[q * Rs + (r - lo)] : 0.0;
-            a4[k] = fma(v, o, a4[k]);
-          }
-        }
-      }
-      // lanes with bit 16 keep values 2, 3 and send 0, 1 (and the reverse), then
-      // bit 8 halves again; three butterflies finish the remaining value
-      const bool up16 = (lane & 16) != 0, up8 = (lane & 8) != 0;
-      const double k0 = up16 ? a4[2] : a4[0], k1 = up16 ? a4[3] : a4[1];
-      const double s0 = up16 ? a4[0] : a4[2], s1 = up16 ? a4[1] : a4[3];
-      const double b0 = k0 + __shfl_xor_sync(0xffffffffu, s0, 16);
-      const double b1 = k1 + __shfl_xor_sync(0xffffffffu, s1, 16);
-      double t = (up8 ? b1 : b0) + __shfl_xor_sync(0xffffffffu, up8 ? b0 : b1, 8);
-      t += __shfl_xor_sync(0xffffffffu, t, 4);
-      t += __shfl_xor_sync(0xffffffffu, t, 2);
-      t += __shfl_xor_sync(0xffffffffu, t, 1);
-      // lane 8 (2 * up16 + up8) holds column q0 + that index's dot
-      if ((lane & 7) == 0) {
-        const int q = q0 + 2 * (up16 ? 1 : 0) + (up8 ? 1 : 0);
-        part[buf][q] = (q < nbp && q != i) ? t : 0.0;
-      }
-    }
-    panel_sync<CG>(cluster);
-    if (tid < NB) {
-      double t = 0.0;
-      for (int rk = 0; rk < CG; ++rk) t += panel_part<CG>(cluster, &part[buf][0], rk)[tid];
-      dots[tid] = t;
-      cf[tid] = -tau * t;
-    }
-    __syncthreads();
-    // ---- 4. my rows of the later panel columns: W[:, q] -= tau * dots[q] * v
-    //         (the coefficients formed once above: the stores to Ws may alias
-    //         dots for the compiler, so a product written here would be redone
-    //         for every row)
-    for (int64_t r = r0 + tid; r < r1; r += kT) {
-      const double v = (r == c) ? 1.0 : col[r - lo];
-#pragma unroll
-      for (int q = 0; q < NB; ++q) {
-        if (q > i && q < nbp) {
-          double* pq = Ws + q * Rs + (r - lo);
-          *pq = fma(cf[q], v, *pq);
-        }
-      }
-    }
-    // ---- 5. T(0:i, i) = -tau T(0:i, 0:i) V^T v_i (same in every CTA)
-    if (tid < i) {
-      double t = 0.0;
-      for (int pc = tid; pc < i; ++pc) t = fma(Ts[tid][pc], dots[pc], t);
-      Ts[tid][i] = -tau * t;
-    }
-    if (tid == 0) Ts[i][i] = tau;
-    __syncthreads();
-  }
-  // ---- write back: W (R above the diagonal, beta on it, v below), the explicit
-  //      reflectors (unit diagonal, exact zeros outside each support) and T
-  for (int q = 0; q < nbp; ++q) {
-    const int64_t cq = c0 + q;
-    for (int rr = tid; rr < nr; rr += kT) {
-      const int64_t r = lo + rr;
-      const double w = Ws[q * Rs + rr];
-      if (r < rows_w) Wj[r + cq * ldw] = w;
-      Vp[(r - c0) + (int64_t)q * ldv] = (r < cq || r > m + cq) ? 0.0 : (r == cq ? 1.0 : w);
-    }
-  }
-  if (rank == 0)
-    for (int e = tid; e < NB * NB; e += kT) Tp[e] = Ts[e % NB][e / NB];
-  panel_sync<CG>(cluster);   // no CTA leaves while another may still read its partials
-}
-
 // ------------------------------------------------- register-resident panel
 // The panel factorisation with the panel's rows held in registers: lane q of every
 // warp owns column q, a warp owns rows, and the rows are dealt cyclically over NG =
@@ -485,14 +282,15 @@ qr_panel_smem_kernel(double* W, int64_t strideW, int64_t ldw, int64_t m, int64_t
 //     beta = -sign(alpha) sqrt(alpha^2 + s_i),  tau = (beta - alpha) / beta,
 //     scal = 1 / (alpha - beta),   v^T a_q = a_cq + scal s_q,
 // and the update a_q -= tau (v^T a_q) v is -tau scal (v^T a_q) x below the pivot: the
-// reflectors stay unscaled until they are written.  Every warp forms the scalars
-// itself (one FP64 unit each), so a column has one CTA barrier and one cluster barrier.
+// reflectors stay unscaled until they are written.  Four warps, one on each FP64 unit,
+// form the scalars; with eight the others wait for theirs (two warps on a unit took twice
+// as long, 35 us a panel).  The four share the sum over the ranks.
 // The groups' sums are added in a fixed tree (4 groups, then the 8 fours), the same
 // for 8 CTAs x 4 warps x 1 group and for 1 CTA x 8 warps x 4 groups: the one-CTA form
 // of a batch and the cluster form of a single call give the same bits.
-// Measured, 32 columns of 256 / 1024 / 4096 / 8192 rows at r = 3: 98 / 138 / 279 / 436
-// us, against 325 / 285 / 440 / 1480 us of the shared-memory panel below (one CTA
-// under 512 rows, else eight) and the global-memory one; 256 rows on one CTA 264 us.
+// Measured, 32 columns of 256 / 1024 / 4096 / 8192 rows at r = 6: 98 / 125 / 231 / 375
+// us, against 325 / 285 / 440 / 1480 us of a panel in shared memory (one CTA under 512
+// rows, else eight; the global-memory one at 8192); 400 rows on one CTA 231 us.
 template <int N>
 __device__ __forceinline__ double tree_sum(const double (&v)[N]) {
   double t[N];
@@ -514,9 +312,13 @@ qr_panel_reg_kernel(double* W, int64_t strideW, int64_t ldw, int64_t m, int64_t 
   static_assert(NG >= NB, "the diagonal rows are row 0 of their groups");
   namespace cgrp = cooperative_groups;
   cgrp::cluster_group cluster = cgrp::this_cluster();
+  constexpr int LW = 4;                // the warps that form the scalars, one per sub-partition
+  static_assert(WARPS >= LW && (RANKS < LW || RANKS % LW == 0), "equal shares");
   __shared__ double red[2][WARPS][NB];
   __shared__ double part[2][RANKS][NB];
+  __shared__ double quarter[LW][NB];
   __shared__ double piv[2][NB];
+  __shared__ double next[2][NB], next_scalar[2];   // f and cf, beta and scal, for the other warps
   __shared__ double Gs[NB][NB + 1], Ts[NB][NB + 1], Ys[NB][NB + 1];
   __shared__ double taus[NB];
   const int rank = RANKS > 1 ? (int)cluster.block_rank() : 0;
@@ -583,49 +385,80 @@ qr_panel_reg_kernel(double* W, int64_t strideW, int64_t ldw, int64_t m, int64_t 
     }
     red[buf][warp][lane] = tree_sum(acc);
     __syncthreads();
-    double total;
-    {
+    double total = 0.0;
+    if (warp < LW) {
       double w[WARPS];
 #pragma unroll
       for (int q = 0; q < WARPS; ++q) w[q] = red[buf][q][lane];
       total = tree_sum(w);
     }
     if constexpr (RANKS > 1) {
-      for (int q = warp; q < RANKS; q += WARPS)
-        cluster.map_shared_rank(&part[buf][rank][0], q)[lane] = total;
+      constexpr int PER = RANKS < LW ? RANKS : RANKS / LW;
+      if (warp < LW)
+        for (int q = warp; q < RANKS; q += LW)
+          cluster.map_shared_rank(&part[buf][rank][0], q)[lane] = total;
       cluster.sync();
-      double w[RANKS];
+      if (warp < LW) {
+        double w[PER], x[LW];
 #pragma unroll
-      for (int q = 0; q < RANKS; ++q) w[q] = part[buf][q][lane];
-      total = tree_sum(w);
-    }
-    const double pv = piv[buf][lane];
-    const double alpha = __shfl_sync(0xffffffffu, pv, i), ss = __shfl_sync(0xffffffffu, total, i);
-    double tau = 0.0, scal = 0.0;
-    if (ss == 0.0) {
-      beta = alpha;
-    } else {
-      const double n2 = fma(alpha, alpha, ss);
-      double nrm, inv;
-      if (n2 > 1e-280 && n2 < 1e280) {
-        root_pair(n2, &nrm, &inv);
-        beta = -copysign(nrm, alpha);
-        tau = (beta - alpha) * -copysign(inv, alpha);
-        scal = reciprocal(alpha - beta);
-      } else {   // near the ends of the range, or not finite
-        beta = -copysign(sqrt(n2), alpha);
-        tau = (beta - alpha) / beta;
-        scal = 1.0 / (alpha - beta);
+        for (int q = 0; q < PER; ++q) w[q] = part[buf][RANKS < LW ? q : warp * PER + q][lane];
+        total = tree_sum(w);
+        if constexpr (RANKS >= LW) {
+          quarter[warp][lane] = total;
+          asm volatile("bar.sync 1, %0;" ::"n"(LW * 32) : "memory");
+#pragma unroll
+          for (int q = 0; q < LW; ++q) x[q] = quarter[q][lane];
+          total = tree_sum(x);
+        }
       }
     }
-    const double dot = fma(scal, total, pv);   // v^T a_q; unscaled x_q^T v for q < i
-    f = lane > i ? -tau * dot : 0.0;
-    cf = f * scal;
-    if (rank == 0 && warp == 0) {
-      if (lane < i) Gs[lane][i] = scal_q * dot;
-      if (lane == i) {
-        taus[i] = tau;
-        if (!isfinite(beta) || !isfinite(tau)) atomicOr(status + kStatNonFinite, 1);
+    double scal = 0.0;
+    if (warp < LW) {
+      const double pv = piv[buf][lane];
+      const double alpha = __shfl_sync(0xffffffffu, pv, i), ss = __shfl_sync(0xffffffffu, total, i);
+      double tau = 0.0;
+      if (ss == 0.0) {
+        beta = alpha;
+      } else {
+        const double n2 = fma(alpha, alpha, ss);
+        double nrm, inv;
+        if (n2 > 1e-280 && n2 < 1e280) {
+          root_pair(n2, &nrm, &inv);
+          beta = -copysign(nrm, alpha);
+          tau = (beta - alpha) * -copysign(inv, alpha);
+          scal = reciprocal(alpha - beta);
+        } else {   // near the ends of the range, or not finite
+          beta = -copysign(sqrt(n2), alpha);
+          tau = (beta - alpha) / beta;
+          scal = 1.0 / (alpha - beta);
+        }
+      }
+      const double dot = fma(scal, total, pv);   // v^T a_q; unscaled x_q^T v for q < i
+      f = lane > i ? -tau * dot : 0.0;
+      cf = f * scal;
+      if (rank == 0 && warp == 0) {
+        if (lane < i) Gs[lane][i] = scal_q * dot;
+        if (lane == i) {
+          taus[i] = tau;
+          if (!isfinite(beta) || !isfinite(tau)) atomicOr(status + kStatNonFinite, 1);
+        }
+      }
+      if (WARPS > LW && warp == 0) {
+        next[0][lane] = f;
+        next[1][lane] = cf;
+        if (lane == 0) {
+          next_scalar[0] = beta;
+          next_scalar[1] = scal;
+        }
+      }
+    }
+    if constexpr (WARPS > LW) {
+      __syncthreads();
+      if (warp >= LW) {
+        f = next[0][lane];
+        cf = next[1][lane];
+        beta = next_scalar[0];
+        scal = next_scalar[1];
       }
     }
     if (lane == i) scal_q = scal;
@@ -825,42 +658,54 @@ cudaError_t merge_super(const QrBuffers& b, const double* Vs, int64_t ldv, doubl
 
 namespace {
 
-// The register panel that serves m rows, or kRegNone.  Below 512 rows a single call
-// takes a cluster of 8 CTAs and a batch one CTA (the same bits); from there a single
-// call takes 16 CTAs while a thread's rows fit in its registers, and a batch keeps the
-// shared-memory panel on the fewest CTAs.  Seven clusters of 16 find room at once
-// (4096 rows: 279 us up to there, 525 us with eight, in two rounds), so eight shifts
-// take 8 CTAs (399 us).
-enum PanelKind { kRegNone, kReg1x17, kReg8x17, kReg8x33, kReg8w33, kReg8w65, kReg8w97,
-                 kReg16x17, kReg16x33, kReg16w33, kReg16w65, kReg16w97 };
+// The register panel that serves m rows, or kRegNone: kReg<CTAs>x<rows a thread> with four
+// warps a CTA, ...w... with eight.  Below 512 rows a single call takes a cluster of 8 CTAs
+// and a batch one CTA (the same bits).  From there a single call takes 16 CTAs; seven
+// clusters of 16 find room at once and eight of 12, so eight shifts take 12 (4096 rows:
+// 275 us, 403 in two rounds of 16, 397 with the former 8 CTAs; 1024 rows 131 and 178 us).
+// A thread's rows beyond those there are cost a predicate each (4096 rows at r <= 7: 231
+// us with 33, 244 with 65), hence the steps of 16.  With many problems in flight (narrow)
+// the fewest CTAs that hold the rows cost the GPU least: 96 problems of 1024 / 2048 / 4096
+// rows take 0.77 / 1.12 / 2.54 ms, against 0.93 / 1.45 / 3.53 of panels in shared memory
+// (600 rows: 0.51 against 0.47, but 0.28 against 0.47 ms for a few problems alone).
+enum PanelKind { kRegNone, kReg1x17, kReg2x17, kReg4x33, kReg8x17, kReg8x97, kReg8w65, kReg12w17, kReg12w33,
+                 kReg12w49, kReg12w65, kReg12w97, kReg16w17, kReg16w33, kReg16w49, kReg16w65, kReg16w97 };
 PanelKind panel_kind(int64_t m, int r, bool narrow) {
   const int64_t H = m + kQrNB;
   if (m < kClusterPanelMinRows) return narrow ? kReg1x17 : kReg8x17;
-  if (narrow) return kRegNone;
-  if (r > 7) {
-    if (H <= 32 * 33) return kReg8x33;
-    if (H <= 64 * 33) return kReg8w33;
+  if (narrow) {
+    if (H <= 64 * 17) return kReg2x17;
+    if (H <= 64 * 33) return kReg4x33;
+    if (H <= 32 * 97) return kReg8x97;
     if (H <= 64 * 65) return kReg8w65;
-    if (H <= 64 * 97) return kReg8w97;
   }
-  if (H <= 64 * 17) return kReg16x17;
-  if (H <= 64 * 33) return kReg16x33;
+  if (r > 7 || narrow) {
+    if (H <= 96 * 17) return kReg12w17;
+    if (H <= 96 * 33) return kReg12w33;
+    if (H <= 96 * 49) return kReg12w49;
+    if (H <= 96 * 65) return kReg12w65;
+    if (H <= 96 * 97) return kReg12w97;
+  }
+  if (H <= 128 * 17) return kReg16w17;
   if (H <= 128 * 33) return kReg16w33;
+  if (H <= 128 * 49) return kReg16w49;
   if (H <= 128 * 65) return kReg16w65;
   if (H <= 128 * 97) return kReg16w97;
   return kRegNone;
 }
 
-// Clusters of 16 CTAs are beyond the portable size: allowed once per device.
-cudaError_t allow_clusters16() {
+// Clusters of 12 and 16 CTAs are beyond the portable size: allowed once per device.
+cudaError_t allow_wide_clusters() {
   static std::atomic<uint64_t> done{0};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 64 && (done.load() >> dev & 1)) return cudaSuccess;
-  const void* k[] = {(const void*)qr_panel_reg_kernel<16, 4, 1, 17>, (const void*)qr_panel_reg_kernel<16, 4, 1, 33>,
-                     (const void*)qr_panel_reg_kernel<16, 8, 1, 33>, (const void*)qr_panel_reg_kernel<16, 8, 1, 65>,
-                     (const void*)qr_panel_reg_kernel<16, 8, 1, 97>};
+  const void* k[] = {(const void*)qr_panel_reg_kernel<12, 8, 1, 17>, (const void*)qr_panel_reg_kernel<12, 8, 1, 33>,
+                     (const void*)qr_panel_reg_kernel<12, 8, 1, 49>, (const void*)qr_panel_reg_kernel<12, 8, 1, 65>,
+                     (const void*)qr_panel_reg_kernel<12, 8, 1, 97>, (const void*)qr_panel_reg_kernel<16, 8, 1, 17>,
+                     (const void*)qr_panel_reg_kernel<16, 8, 1, 33>, (const void*)qr_panel_reg_kernel<16, 8, 1, 49>,
+                     (const void*)qr_panel_reg_kernel<16, 8, 1, 65>, (const void*)qr_panel_reg_kernel<16, 8, 1, 97>};
   for (const void* f : k)
     if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess)
       return e;
@@ -871,14 +716,19 @@ cudaError_t allow_clusters16() {
 cudaError_t launch_panel(PanelKind k, const PanelArgs& p, int r, double fl, double by, cudaStream_t st) {
   switch (k) {
     case kReg1x17: return launch_panel_reg<1, 8, 4, 17>(p, r, fl, by, st);
+    case kReg2x17: return launch_panel_reg<2, 8, 4, 17>(p, r, fl, by, st);
+    case kReg4x33: return launch_panel_reg<4, 8, 2, 33>(p, r, fl, by, st);
     case kReg8x17: return launch_panel_reg<8, 4, 1, 17>(p, r, fl, by, st);
-    case kReg8x33: return launch_panel_reg<8, 4, 1, 33>(p, r, fl, by, st);
-    case kReg8w33: return launch_panel_reg<8, 8, 1, 33>(p, r, fl, by, st);
+    case kReg8x97: return launch_panel_reg<8, 4, 1, 97>(p, r, fl, by, st);
     case kReg8w65: return launch_panel_reg<8, 8, 1, 65>(p, r, fl, by, st);
-    case kReg8w97: return launch_panel_reg<8, 8, 1, 97>(p, r, fl, by, st);
-    case kReg16x17: return launch_panel_reg<16, 4, 1, 17>(p, r, fl, by, st);
-    case kReg16x33: return launch_panel_reg<16, 4, 1, 33>(p, r, fl, by, st);
+    case kReg12w17: return launch_panel_reg<12, 8, 1, 17>(p, r, fl, by, st);
+    case kReg12w33: return launch_panel_reg<12, 8, 1, 33>(p, r, fl, by, st);
+    case kReg12w49: return launch_panel_reg<12, 8, 1, 49>(p, r, fl, by, st);
+    case kReg12w65: return launch_panel_reg<12, 8, 1, 65>(p, r, fl, by, st);
+    case kReg12w97: return launch_panel_reg<12, 8, 1, 97>(p, r, fl, by, st);
+    case kReg16w17: return launch_panel_reg<16, 8, 1, 17>(p, r, fl, by, st);
     case kReg16w33: return launch_panel_reg<16, 8, 1, 33>(p, r, fl, by, st);
+    case kReg16w49: return launch_panel_reg<16, 8, 1, 49>(p, r, fl, by, st);
     case kReg16w65: return launch_panel_reg<16, 8, 1, 65>(p, r, fl, by, st);
     case kReg16w97: return launch_panel_reg<16, 8, 1, 97>(p, r, fl, by, st);
     default: return cudaErrorInvalidValue;
@@ -892,15 +742,7 @@ int qr_super_width(int64_t n) { return n >= 2048 ? 512 : kQrBlock; }
 cudaError_t structured_qr_q(const QrBuffers& b, int64_t m, int64_t n, int r, int* status,
                             cudaStream_t st, bool explicit_q, bool narrow_panels) {
   constexpr int NB = kQrNB, NBb = kQrBlock;
-  {
-    const int bytes = (int)(sizeof(double) * NB * kSmemPanelRows);
-    if (smem_attr_once((const void*)qr_panel_smem_kernel<NB, 2>, bytes) != cudaSuccess ||
-        smem_attr_once((const void*)qr_panel_smem_kernel<NB, 4>, bytes) != cudaSuccess ||
-        smem_attr_once((const void*)qr_panel_smem_kernel<NB, 1>, bytes) != cudaSuccess ||
-        smem_attr_once((const void*)qr_panel_smem_kernel<NB, kPanelCluster>, bytes) != cudaSuccess ||
-        allow_clusters16() != cudaSuccess)
-      return cudaErrorInvalidConfiguration;
-  }
+  if (allow_wide_clusters() != cudaSuccess) return cudaErrorInvalidConfiguration;
   const int64_t ldw = m + n;
   // On the tensor cores the blocks of a super-block are applied to its own columns
   // one by one and to everything to its right together (see the file's head).
@@ -909,16 +751,8 @@ cudaError_t structured_qr_q(const QrBuffers& b, int64_t m, int64_t n, int r, int
   const int ldt = SB;
   const int64_t ldv = m + SB;
   cudaError_t err;
-  // The register panel where there is one; else, with many problems in flight
-  // (narrow_panels), the shared-memory panel on the fewest CTAs whose rows fit (one
-  // CTA up to m = 736, two up to 1504): the same SMs then serve more panels at once.
-  // cg = 0: the global-memory cluster kernel.
+  // the register panel where there is one, else the global-memory cluster kernel
   const PanelKind reg = panel_kind(m, r, narrow_panels);
-  int cg = 0;
-  if (narrow_panels && reg == kRegNone)
-    for (int c = 1; c <= kPanelCluster; c *= 2)
-      if ((m + NB + c - 1) / c <= kSmemPanelRows) { cg = c; break; }
-  const int64_t rows_cta = cg ? (m + NB + cg - 1) / cg : 0;
   // every V entry outside the rows a panel writes must be an exact zero
   if ((err = cudaMemsetAsync(b.V, 0, sizeof(double) * r * b.strideV, st)) != cudaSuccess) return err;
   if (SB > NBb &&
@@ -941,29 +775,12 @@ cudaError_t structured_qr_q(const QrBuffers& b, int64_t m, int64_t n, int r, int
         if ((err = launch_panel(reg, pa, r, pf, pb, st)) != cudaSuccess) return err;
       } else {
         ProfScope ps(kProfPanel, st, pf, pb);
-        const size_t smem = sizeof(double) * NB * rows_cta;
-        if (cg == 0)
-          ps.blocks((const void*)qr_panel_cluster_kernel<NB, kPanelCluster, 512>, dim3(512), 0,
-                    dim3(r * kPanelCluster));
-        else
-          ps.blocks((const void*)qr_panel_smem_kernel<NB, 1>, dim3(256), smem, dim3(r * cg));
-        if (cg == 1)
-          qr_panel_smem_kernel<NB, 1><<<r, 256, smem, st>>>(
-              b.W, b.strideW, ldw, m, c0, nbp, Vpan, b.strideV, ldv, b.T, b.strideT, status);
-        else if (cg == 2)
-          qr_panel_smem_kernel<NB, 2><<<r * 2, 256, smem, st>>>(
-              b.W, b.strideW, ldw, m, c0, nbp, Vpan, b.strideV, ldv, b.T, b.strideT, status);
-        else if (cg == 4)
-          qr_panel_smem_kernel<NB, 4><<<r * 4, 256, smem, st>>>(
-              b.W, b.strideW, ldw, m, c0, nbp, Vpan, b.strideV, ldv, b.T, b.strideT, status);
-        else if (cg == kPanelCluster)
-          qr_panel_smem_kernel<NB, kPanelCluster><<<r * kPanelCluster, 256, smem, st>>>(
-              b.W, b.strideW, ldw, m, c0, nbp, Vpan, b.strideV, ldv, b.T, b.strideT, status);
-        else
-          // tall panels (m > 8 x 768 rows): 512 threads per CTA halve each thread's
-          // share of the rows on the serial chain of every column
-          qr_panel_cluster_kernel<NB, kPanelCluster, 512><<<r * kPanelCluster, 512, 0, st>>>(
-              b.W, b.strideW, ldw, m, c0, nbp, Vpan, b.strideV, ldv, b.T, b.strideT, status);
+        ps.blocks((const void*)qr_panel_cluster_kernel<NB, kPanelCluster, 512>, dim3(512), 0,
+                  dim3(r * kPanelCluster));
+        // 512 threads per CTA halve each thread's share of the rows on the serial chain
+        // of every column
+        qr_panel_cluster_kernel<NB, kPanelCluster, 512><<<r * kPanelCluster, 512, 0, st>>>(
+            b.W, b.strideW, ldw, m, c0, nbp, Vpan, b.strideV, ldv, b.T, b.strideT, status);
       }
       if ((err = cudaGetLastError()) != cudaSuccess) return err;
       // the rest of this block's columns
