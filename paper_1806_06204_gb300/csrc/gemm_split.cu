@@ -403,18 +403,17 @@ __device__ __forceinline__ Fixed split_fixed(long long iacc, float fm) {
   return r;
 }
 
-// x 2^k rounded to nearest (ties to even), with the sign bit of flip (its high word)
-// toggled; *rare when the result is outside the normal range (its value is then
-// scale_steps').
-__device__ __forceinline__ double fixed_to_double(long long x, int k, unsigned flip, bool* rare) {
-  const double d = (double)x;
+// q times 2^e, rounded to nearest (ties to even), for results in the normal range: e20 is
+// e in the exponent field's place; flip toggles the sign bit (its high word).
+__device__ __forceinline__ double fixed_scaled(const Fixed& q, int e20, unsigned flip) {
+  const double d = (double)q.x;
   const int h = __double2hiint(d);
-  *rare |= h != 0 && (unsigned)(((h >> 20) & 0x7FF) + k - 1) >= 2045u;
-  return __hiloint2double((int)((unsigned)(h + (h != 0 ? k << 20 : 0)) ^ flip), __double2loint(d));
+  return __hiloint2double((int)((unsigned)(h + (h != 0 ? e20 + q.k * (1 << 20) : 0)) ^ flip),
+                          __double2loint(d));
 }
 
-// x 2^k outside the normal range: powers of two applied in steps that are exact
-// until the last one rounds.
+// x 2^k, any range: powers of two applied in steps that are exact until the last one
+// rounds.
 __device__ __forceinline__ double scale_steps(long long x, int k) {
   double d = (double)x;
   for (int i = 0; i < 3 && k != 0; ++i) {
@@ -517,9 +516,8 @@ template <int FORM>
 __device__ __forceinline__ double split_value(const SplitEpi& p, long long iacc, float fm, int ei,
                                               int ej, double al) {
   const Fixed q = split_fixed<Form<FORM>::kLo, true>(iacc, fm);
-  bool rare = false;
-  double v = fixed_to_double(q.x, q.k + ei + ej, 0u, &rare);
-  if (rare) v = scale_steps(q.x, q.k + ei + ej);
+  const int e = ei + ej;
+  double v = e >= -900 && e <= 900 ? fixed_scaled(q, e * (1 << 20), 0u) : scale_steps(q.x, q.k + e);
   if (p.nan_rows && (ei >= 1026 || ej >= 1026)) v = __longlong_as_double(0x7FF8000000000000ll);
   return v * al;
 }
@@ -752,7 +750,7 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     // of 2^-48 has room for 600 chunks of 192, 28 of 4096, at the digit bounds, and
     // gemm_split cuts a longer K into several products)
     constexpr int HALF = BN / (kEpiWarps / 4);     // columns of this warp
-    constexpr int kLd = HALF % 16 == 0 ? 16 : 8;   // columns per TMEM load
+    constexpr bool kWide = F::kLo > 8;             // the float parts may exceed 2^30
     const int q = warp & 3;
     const int half = (warp - 2) >> 2;              // which column slice
     const uint32_t lane_off = (uint32_t)(q * 32) << 16;
@@ -795,111 +793,116 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
           for (int j = 0; j < HALF; ++j, ip += st_i)
             if (j < jn) asm volatile("prefetch.global.L2 [%0];" ::"l"(ip));
         }
+        // the exponents, under the wait for the MMAs (lane l holds column l's)
+        const int ei = p.ea[b * p.Mpad + row];
+        const int ej_lane = __ldg(p.eb + b * p.Npad + col0 + (lane & (HALF - 1)));
         for (int c = 0; c < nchunks && ok; ++c, ++cg) {
 #pragma unroll
           for (int a = 0; a < kAcc; ++a) {
             if (!ok || !(ok = tc::mbar_wait(&lfull[a], cg & 1, err))) break;
             tc::tc_fence_after();
-            const int lv = a + 2;
-#pragma unroll
-            for (int g = 0; g < HALF / kLd; ++g) {
-              float v[kLd];
-              if constexpr (kLd == 16) tc::tmem_ld16(tmem + lane_off + a * BN + half * HALF + g * kLd, v);
-              else tc::tmem_ld8(tmem + lane_off + a * BN + half * HALF + g * kLd, v);
-#pragma unroll
-              for (int i = 0; i < kLd; ++i) {
-                // one 32 x 32 + 64 bit multiply-add per element
-                if (lv <= F::kIntTop) {
-                  const int sh = 48 - F::kBits * lv;
-                  if (sh < 31) iacc[g * kLd + i] += (long long)__float2int_rn(v[i]) * (long long)(1 << (sh < 31 ? sh : 0));
-                  else iacc[g * kLd + i] += (long long)__float2int_rn(v[i]) << sh;
-                } else {
-                  fm[g * kLd + i] += v[i] * __int_as_float((127 + 48 + F::kLo - F::kBits * lv) << 23);
-                }
-              }
-            }
+            uint32_t v[HALF];
+            tc::tmem_ld<HALF>(tmem + lane_off + a * BN + half * HALF, v);
+            tc::tmem_wait<HALF>(v);
+            // the level is free as soon as it is in registers: the next chunk's MMAs wait
+            // for this, not for the conversions
             tc::tc_fence_before();
             __syncwarp();
             if (lane == 0) tc::mbar_arrive(&lempty[a]);
+            const int lv = a + 2;
+#pragma unroll
+            for (int j = 0; j < HALF; ++j) {
+              const float x = __uint_as_float(v[j]);
+              // one 32 x 32 + 64 bit multiply-add per element
+              if (lv <= F::kIntTop) {
+                const int sh = 48 - F::kBits * lv;
+                if (sh < 31) iacc[j] += (long long)__float2int_rn(x) * (long long)(1 << (sh < 31 ? sh : 0));
+                else iacc[j] += (long long)__float2int_rn(x) << sh;
+              } else {
+                fm[j] += x * __int_as_float((127 + 48 + F::kLo - F::kBits * lv) << 23);
+              }
+            }
+          }
+          // 32 chunks keep the float parts below 2^30: what lies above the int64's unit moves
+          if (!kWide && (c & 31) == 31) {
+#pragma unroll
+            for (int j = 0; j < HALF; ++j) {
+              const int f = __float2int_rn(fm[j]);
+              iacc[j] += f >> F::kLo;
+              fm[j] = (float)(f & ((1 << F::kLo) - 1));
+            }
           }
         }
         if (!ok) break;
         if (p.ks > 1) break;      // one entry per tile: joined over the cluster below
-        // end of a batch entry: scale, combine with the addend, write, reset.  The
-        // fast loop's FP64 work is one conversion and the addend's FMA (the sign of
-        // alpha = +-1 is a bit); a result outside the normal range, an Inf or NaN operand or
-        // another alpha sends the warp through the general loop after it.
-        const int ei = p.ea[b * p.Mpad + row];
-        const int* ebb = p.eb + b * p.Npad + col0;
+        // end of a batch entry: scale, combine with the addend, write, reset.  The fast
+        // loop's FP64 work is one conversion and the addend's FMA (the sign of alpha =
+        // +-1 is a bit, the scale an exponent); another alpha, an Inf or NaN operand or
+        // exponents from which a result could leave the normal range take the general
+        // loop instead, decided before the first output: nothing of the sums is kept for
+        // a second look.  4096 x 4096, C += A B, K = 64 / 128: 172 / 183 -> 141 / 148 us;
+        // 8192 x 4096, K = 512: 768 -> 700 us (BF16); 4096^3 2.74 -> 2.67 ms.
         const double al = p.alpha[b], bt = first ? p.beta : 1.0;
-        const unsigned flip = al < 0.0 ? 0x80000000u : 0u;
-        const bool wide = F::kLo > 8 || p.K > 8192;   // |fm| < 2^30 up to there
-        const int nan_at = p.nan_rows ? 1026 : INT_MAX;
-        bool rare = al != 1.0 && al != -1.0;
+        const int emin = __reduce_min_sync(0xffffffffu, ej_lane), emax = __reduce_max_sync(0xffffffffu, ej_lane);
+        const bool slow = __any_sync(0xffffffffu, (al != 1.0 && al != -1.0) || ei + emin < -900 || ei + emax > 900 ||
+                                                      (p.nan_rows && max(ei, emax) >= 1026));
         int64_t st_c = p.swap ? 1 : p.ldc;
         asm volatile("" : "+l"(st_c));
         double* cp = C + (p.swap ? col0 + row * p.ldc : row + col0 * p.ldc);
         const double* ip = ip0;
-        constexpr int kAdd = 8;
-        double add[HALF > kAdd ? HALF : kAdd];
-#pragma unroll
-        for (int j0 = 0; j0 < HALF; j0 += kAdd) {
-          // the addends of eight outputs first (a load after a store to C could alias
-          // it, so a plain loop waits for each)
-          if (addend) {
-#pragma unroll
-            for (int j = j0; j < j0 + kAdd; ++j) {
-              add[j] = j < jn ? *ip : 0.0;
-              ip += st_i;
-            }
-          }
-          double* cq = cp;
-          double v[kAdd];
-#pragma unroll
-          for (int jj = 0; jj < kAdd; ++jj) {
-            const int j = j0 + jj, ej = __ldg(ebb + j);
-            const Fixed q = wide ? split_fixed<F::kLo, true>(iacc[j], fm[j])
-                                 : split_fixed<F::kLo, false>(iacc[j], fm[j]);
-            v[jj] = fixed_to_double(q.x, q.k + ei + ej, flip, &rare);
-            rare |= max(ei, ej) >= nan_at;
-          }
-          if (addend) {
-#pragma unroll
-            for (int jj = 0; jj < kAdd; ++jj) v[jj] = fma(bt, add[j0 + jj], v[jj]);
-          }
-#pragma unroll
-          for (int jj = 0; jj < kAdd; ++jj) {
-            if (j0 + jj < jn) *cq = v[jj];
-            cq += st_c;
-          }
-          if (__any_sync(0xffffffffu, rare)) {
-            cq = cp;
+        if (slow) {
 #pragma unroll 1
-            for (int jj = 0; jj < kAdd; ++jj) {
-              long long xi = 0;
-              float xf = 0.f;
-              double xa = 0.0;
+          for (int j = 0; j < HALF; ++j) {
+            long long xi = 0;
+            float xf = 0.f;
 #pragma unroll
-              for (int u = 0; u < kAdd; ++u)
-                if (u == jj) {
-                  xi = iacc[j0 + u];
-                  xf = fm[j0 + u];
-                  if (addend) xa = add[j0 + u];
-                }
-              if (j0 + jj < jn) {
-                double w = split_value<FORM>(p, xi, xf, ei, __ldg(ebb + j0 + jj), al);
-                if (addend) w = fma(bt, xa, w);
-                *cq = w;
+            for (int u = 0; u < HALF; ++u)
+              if (u == j) {
+                xi = iacc[u];
+                xf = fm[u];
               }
-              cq += st_c;
+            double w = split_value<FORM>(p, xi, xf, ei, __shfl_sync(0xffffffffu, ej_lane, j), al);
+            if (j < jn) {
+              if (addend) w = fma(bt, *ip, w);
+              *cp = w;
+            }
+            ip += st_i;
+            cp += st_c;
+          }
+        } else {
+          const unsigned flip = al < 0.0 ? 0x80000000u : 0u;
+          const int e0 = ei * (1 << 20);
+          const int ejs = ej_lane * (1 << 20);
+          constexpr int kAdd = 4;
+#pragma unroll
+          for (int j0 = 0; j0 < HALF; j0 += kAdd) {
+            // the addends of four outputs first (a load after a store to C could alias
+            // it, so a plain loop waits for each; eight at a time spill the sums)
+            double add[kAdd], v[kAdd];
+            if (addend) {
+#pragma unroll
+              for (int jj = 0; jj < kAdd; ++jj) {
+                add[jj] = j0 + jj < jn ? *ip : 0.0;
+                ip += st_i;
+              }
+            }
+#pragma unroll
+            for (int jj = 0; jj < kAdd; ++jj) {
+              const Fixed q = split_fixed<F::kLo, kWide>(iacc[j0 + jj], fm[j0 + jj]);
+              v[jj] = fixed_scaled(q, e0 + __shfl_sync(0xffffffffu, ejs, j0 + jj), flip);
+            }
+#pragma unroll
+            for (int jj = 0; jj < kAdd; ++jj) {
+              if (addend) v[jj] = fma(bt, add[jj], v[jj]);
+              if (j0 + jj < jn) *cp = v[jj];
+              cp += st_c;
             }
           }
-          cp = cq;
+        }
 #pragma unroll
-          for (int j = j0; j < j0 + kAdd; ++j) {
-            iacc[j] = 0;
-            fm[j] = 0.f;
-          }
+        for (int j = 0; j < HALF; ++j) {
+          iacc[j] = 0;
+          fm[j] = 0.f;
         }
       }
     }
