@@ -141,17 +141,19 @@ __global__ void col_exp_kernel(const double* __restrict__ X, int64_t ldx, int64_
 }
 
 // N = round(x 2^(bS - e)) from the bit pattern (|x| < 2^(e-1), so |N| <= 2^(bS-1));
-// ties round away from zero.
+// ties round away from zero.  The mantissa is raised by 8 bits, so every exponent is one
+// right shift (by 5 at least: a subnormal of a row of subnormals; what is shifted further
+// than 62 is zero).
 template <int BITS>
 __device__ __forceinline__ long long fixed_point(double x, int e) {
-  const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
-  const int ef = (int)(bits >> 52) & 0x7FF;
-  const unsigned long long M = (bits & ((1ull << 52) - 1)) | (ef ? (1ull << 52) : 0ull);
-  const int k = (ef ? ef - 1075 : -1074) - e + BITS;   // |x| = M 2^(k + e - BITS); k <= BITS - 54
-  unsigned long long F;
-  if (k >= 0) F = k < 11 ? M << k : 0;
-  else F = k > -63 ? (M + (1ull << (-k - 1))) >> -k : 0;
-  return (long long)bits < 0 ? -(long long)F : (long long)F;
+  const int hi = __double2hiint(x);
+  const int ef = (hi >> 20) & 0x7FF;
+  const unsigned mh = ((unsigned)hi & 0xFFFFFu) | (ef ? 0x100000u : 0u);
+  const unsigned long long M = ((unsigned long long)mh << 32 | (unsigned)__double2loint(x)) << 8;
+  const int t = min(max(1083 - BITS + e - max(ef, 1), 1), 63);
+  const long long F = (long long)((M + (1ull << (t - 1))) >> t);
+  const long long m = hi >> 31;
+  return (F ^ m) - m;
 }
 
 // The S balanced digits of two neighbouring entries, plane by plane, as one packed
@@ -170,20 +172,29 @@ __device__ __forceinline__ void slice_pair(double x0, double x1, int e0, int e1,
     return t;
   }();
   const long long n0 = fixed_point<B * S>(x0, e0) + bias, n1 = fixed_point<B * S>(x1, e1) + bias;
-  // digit s (1-based, 1 leads) plus half
+  // digit s (1-based, 1 leads) plus half; the fields of the 8-bit digits are bytes
   auto field = [&](long long n, int s) -> unsigned {
     const int sh = B * (S - s);
     return s == 1 ? (unsigned)((int)(n >> sh) + (int)half) : (unsigned)(n >> sh) & ((1u << B) - 1);
   };
+  auto word = [](long long n, int byte) { return (unsigned)(n >> (byte & 4) * 8); };
 #pragma unroll
   for (int s = 1; s <= S; ++s) {
+    const int byte = S - s;
     if (FORM == kFormBF16) {
-      const float f0 = __uint_as_float(0x4B000000u | field(n0, s)) - (8388608.f + (float)half);
-      const float f1 = __uint_as_float(0x4B000000u | field(n1, s)) - (8388608.f + (float)half);
+      auto biased = [&](long long n) -> float {
+        return __uint_as_float(s == 1 ? 0x4B000000u | field(n, s)
+                                      : __byte_perm(word(n, byte), 0x4B000000u, 0x7440 | (byte & 3)));
+      };
+      const float f0 = biased(n0) - (8388608.f + (float)half), f1 = biased(n1) - (8388608.f + (float)half);
       // a digit has at most 8 significant bits: its BF16 is the float's upper half
       put(s - 1, __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632));
     } else {
-      const unsigned t = (field(n0, s) | field(n1, s) << 16) + 0x64006400u;
+      const unsigned t =
+          FORM == kFormFP16 && s > 1
+              ? (__byte_perm(word(n0, byte), word(n1, byte), 0x0400 | (byte & 3) | (byte & 3) << 8) & 0x00FF00FFu) |
+                    0x64006400u
+              : (field(n0, s) | field(n1, s) << 16) + 0x64006400u;
       const __half2 h = __hsub2(*reinterpret_cast<const __half2*>(&t),
                                 __half2half2(__ushort_as_half((unsigned short)(0x6400 + half))));
       if (FORM == kFormFP16) {
@@ -206,152 +217,152 @@ struct SliceOp {
 };
 
 // Row exponents and slices of both operands of a product in one launch.  A cluster of
-// `cl` CTAs takes 32 rows of op(A) (the first nblk_a clusters along x) or of op(B)^T,
+// `cl` CTAs takes 16 rows of op(A) (the first nblk_a clusters along x) or of op(B)^T,
 // blockIdx.z the batch entry; each CTA has its share of the 64-wide tiles of K.  It
+// brings the first `keep` of its tiles to shared memory (every load in flight at once),
 // finds its share's largest magnitudes, the ranks exchange them through distributed
-// shared memory, and then it slices its tiles, the next one loaded while the current
-// one is cut: S planes of rows_pad x K_pad elements, K contiguous, batch entry b at
-// out + b S rows_pad K_pad, plane s at + s rows_pad K_pad elements.  Reads run along
-// X's contiguous dimension, a warp writes a whole 128-byte line (FP8: 64) per plane.
-// With ek (the inner-index equilibration), element (i, k) counts as x 2^(esign ek[k]).
-// HBM bounds it (8 bytes read, 14 written per element, the second read from L1 or L2).
-// Measured, both operands of 4096^3: 190 us (3.9 TB/s of those bytes), 344 us with
-// separate exponent launches and a conversion per digit; 512 x 512 x 16384 FP8 153 us
-// against 261 us, 1000 x 1537 x 777 31 us against 63 us.
+// shared memory, and then it slices the tiles it kept and, beyond those, the others read
+// once more: S planes of rows_pad x K_pad elements, K contiguous, batch entry b at out + b
+// S rows_pad K_pad, plane s at + s rows_pad K_pad elements.  Reads run along X's
+// contiguous dimension, a warp writes a whole 128-byte line (FP8: 64) per plane.  With ek
+// (the inner-index equilibration), element (i, k) counts as x 2^(esign ek[k]).
+// Between HBM (8 bytes read, 14 written per element) and the integer work bound it: the
+// digits of the 8-bit forms are bytes picked by permutes.  Measured, both operands: 4096^3
+// 163 us (4.5 TB/s of those bytes), 196 us with 32 rows a CTA read twice and shifts for
+// digits; 8192 x 4096 x 512 50 -> 35 us, 128 x 512 x 8192 73 -> 43, 1000 x 1537 x 777 27
+// -> 19, 300^3 13.9 -> 9.8, 512 x 512 x 16384 FP8 153 -> 124 us.  Tiles kept: 4 at five
+// CTAs an SM (2: 172 us at 4096^3; 6 at four CTAs 160 us, but 36 and 128 us above).
+constexpr int kSliceRows = 16, kSliceTile = kSliceRows * 65;   // doubles of a tile, rows padded
+constexpr int kSliceKeep = 4;
 template <int S, int FORM>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 5)
 slice_kernel(const SliceOp a, const SliceOp b, int nblk_a, int K, int K_pad,
-             const int* __restrict__ ek, int cl) {
+             const int* __restrict__ ek, int cl, int keep) {
   namespace cgrp = cooperative_groups;
-  constexpr int kE = Form<FORM>::kElem;
-  __shared__ double tile[32][65];
-  __shared__ long long red[8][33];
-  __shared__ long long mine[32];
-  __shared__ int es[32];
+  constexpr int kE = Form<FORM>::kElem, R = kSliceRows;
+  extern __shared__ double xs[];
+  __shared__ int mine[R], es[R];
   const int rank = blockIdx.x % cl, blk = blockIdx.x / cl;
   const bool on_b = blk >= nblk_a;
   const SliceOp o = on_b ? b : a;
-  const int i0 = (on_b ? blk - nblk_a : blk) * 32;
+  const int i0 = (on_b ? blk - nblk_a : blk) * R;
   const double* Xb = o.X + blockIdx.z * o.strideX;
   const int* ekb = ek ? ek + blockIdx.z * K_pad : nullptr;
-  const int tx = threadIdx.x, ty = threadIdx.y;   // 32 x 8
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int ntiles = K_pad / 64, per = (ntiles + cl - 1) / cl;
-  const int t_lo = rank * per, t_hi = min(ntiles, t_lo + per);
-  const int k_lo = t_lo * 64, k_hi = min(K, t_hi * 64);
-  const unsigned long long kMag = 0x7FFFFFFFFFFFFFFFull;
-  // the row bound: the largest magnitude pattern, or with the inner-index shifts the
-  // largest shifted exponent bound (both reduce with max)
-  const long long none = ekb ? LLONG_MIN : 0;
-  auto take = [&](long long& mx, double x, int k) {
-    const unsigned long long bits = (unsigned long long)__double_as_longlong(x) & kMag;
-    if (!ekb) {
-      mx = (long long)bits > mx ? (long long)bits : mx;
-    } else if (bits != 0) {
-      const long long e = exp_above(bits) + o.esign * ekb[k];
-      mx = e > mx ? e : mx;
+  const int t_lo = min(ntiles, rank * per), t_hi = min(ntiles, t_lo + per);
+  const int t_keep = min(t_hi, t_lo + keep);
+  // element u (of 4) of this thread in a tile: along X's contiguous dimension
+  auto row_of = [&](int u) { return o.trans ? (tid >> 6) + 4 * u : tid & (R - 1); };
+  auto col_of = [&](int u) { return o.trans ? tid & 63 : (tid >> 4) + 16 * u; };
+  auto fetch = [&](int t, double* d) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int rr = row_of(u), c = col_of(u), i = i0 + rr, k = t * 64 + c;
+      double* to = d + rr * 65 + c;
+      if (i < o.rows && k < K) {
+        const double* from = Xb + (o.trans ? k + (int64_t)i * o.ldx : i + (int64_t)k * o.ldx);
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(tc::smem_u32(to)), "l"(from) : "memory");
+      } else {
+        *to = 0.0;
+      }
     }
   };
-  if (!o.trans) {   // rows contiguous: tx runs along i, k split over ty
-    const int i = i0 + tx;
-    long long mx = none;
-    if (i < o.rows) {
-      const double* x = Xb + i;
-      int k = k_lo + ty;
-      for (; k + 56 < k_hi; k += 64) {   // eight loads in flight
-        double v[8];
+  for (int t = t_lo; t < t_keep; ++t) fetch(t, xs + (t - t_lo) * kSliceTile);
+  // the row bound: the largest high word (its low bit set for a subnormal below 2^-1042),
+  // or with the inner-index shifts the largest shifted exponent bound
+  const int none = ekb ? INT_MIN : 0;
+  auto take = [&](int& mx, double x, int k) {
+    const int hi = __double2hiint(x) & 0x7FFFFFFF, nz = hi | (__double2loint(x) != 0);
+    if (!ekb) mx = max(mx, nz);
+    else if (nz != 0) mx = max(mx, (nz >> 20 ? (nz >> 20) - 1021 : -1021) + o.esign * ekb[k]);
+  };
+  if (tid < R) mine[tid] = none;
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncthreads();
+  {
+    int mx = none;   // 16 threads per row
+    for (int t = t_lo; t < t_keep; ++t) {
+      const double* d = xs + (t - t_lo) * kSliceTile + (tid >> 4) * 65;
 #pragma unroll
-        for (int u = 0; u < 8; ++u) v[u] = x[(int64_t)(k + 8 * u) * o.ldx];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) take(mx, v[u], k + 8 * u);
+      for (int u = 0; u < 4; ++u) {
+        const int c = (tid & 15) + 16 * u;
+        if (t * 64 + c < K) take(mx, d[c], t * 64 + c);
       }
-      for (; k < k_hi; k += 8) take(mx, x[(int64_t)k * o.ldx], k);
-    }
-    red[ty][tx] = mx;
-    __syncthreads();
-    if (ty == 0) {
-      for (int y = 1; y < 8; ++y) mx = red[y][tx] > mx ? red[y][tx] : mx;
-      mine[tx] = mx;
-    }
-  } else {          // K contiguous: one warp per row, lanes along k, four rows at a time
-    long long mx[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) mx[q] = none;
-    for (int k = k_lo + tx; k < k_hi; k += 64) {
-      double v[4][2];
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          const int i = i0 + ty + 8 * q;
-          v[q][u] = i < o.rows && k + 32 * u < k_hi ? Xb[k + 32 * u + (int64_t)i * o.ldx] : 0.0;
-        }
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-#pragma unroll
-        for (int u = 0; u < 2; ++u)
-          if (k + 32 * u < k_hi) take(mx[q], v[q][u], k + 32 * u);
     }
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      for (int s = 16; s > 0; s >>= 1) {
-        const long long t = __shfl_xor_sync(0xffffffffu, mx[q], s);
-        mx[q] = t > mx[q] ? t : mx[q];
+    for (int h = 8; h > 0; h >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, h));
+    if ((tid & 15) == 0) atomicMax(&mine[tid >> 4], mx);
+  }
+  if (t_keep < t_hi) {
+    int mx[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) mx[u] = none;
+    for (int t = t_keep; t < t_hi; t += 2) {
+      double v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int i = i0 + row_of(u & 3), k = (t + (u >> 2)) * 64 + col_of(u & 3);
+        v[u] = i < o.rows && k < K && t + (u >> 2) < t_hi
+                   ? Xb[o.trans ? k + (int64_t)i * o.ldx : i + (int64_t)k * o.ldx] : 0.0;
       }
-      if (tx == 0) mine[ty + 8 * q] = mx[q];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int k = (t + (u >> 2)) * 64 + col_of(u & 3);
+        if (k < K && t + (u >> 2) < t_hi) take(mx[u & 3], v[u], k);
+      }
+    }
+    if (o.trans) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int w = __reduce_max_sync(0xffffffffu, mx[u]);
+        if (lane == 0) atomicMax(&mine[row_of(u)], w);
+      }
+    } else {
+      atomicMax(&mine[tid & (R - 1)], max(max(mx[0], mx[1]), max(mx[2], mx[3])));
     }
   }
   cgrp::cluster_group cluster = cgrp::this_cluster();
   if (cl > 1) cluster.sync();
   else __syncthreads();
-  if (ty == 0) {
-    long long mx = mine[tx];
-    for (int q = 0; q < cl; ++q) {
-      if (q == rank) continue;
-      const long long t = cluster.map_shared_rank(mine, q)[tx];
-      mx = t > mx ? t : mx;
-    }
-    es[tx] = !ekb ? exp_above((unsigned long long)mx) : (mx == LLONG_MIN ? 0 : (int)mx);
-    if (rank == 0 && i0 + tx < o.rows_pad) o.e[blockIdx.z * o.rows_pad + i0 + tx] = es[tx];
+  if (tid < R) {
+    int mx = mine[tid];
+    for (int q = 0; q < cl; ++q)
+      if (q != rank) mx = max(mx, cluster.map_shared_rank(mine, q)[tid]);
+    es[tid] = ekb ? (mx == INT_MIN ? 0 : mx) : (mx == 0 ? 0 : mx >> 20 ? (mx >> 20) - 1021 : -1021);
+    if (rank == 0 && i0 + tid < o.rows_pad) o.e[blockIdx.z * o.rows_pad + i0 + tid] = es[tid];
   }
   if (cl > 1) cluster.sync();   // no rank leaves while another reads its maxima
   else __syncthreads();
-  const size_t plane = (size_t)o.rows_pad * K_pad;
-  uint8_t* ob = o.out + (size_t)blockIdx.z * S * plane * kE;
-  double v[8];
-  auto load = [&](int t) {
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      // not transposed: thread = row tx, k = ty + 8 u; transposed: row ty + 8 (u / 2),
-      // k = tx + 32 (u % 2)
-      const int i = i0 + (o.trans ? ty + 8 * (u >> 1) : tx);
-      const int k = t * 64 + (o.trans ? tx + 32 * (u & 1) : ty + 8 * u);
-      v[u] = i < o.rows && k < K ? (o.trans ? Xb[k + (int64_t)i * o.ldx] : Xb[i + (int64_t)k * o.ldx])
-                                 : 0.0;
-    }
-  };
-  if (t_lo < t_hi) load(t_lo);
-  for (int t = t_lo; t < t_hi; ++t) {
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      if (o.trans) tile[ty + 8 * (u >> 1)][tx + 32 * (u & 1)] = v[u];
-      else tile[tx][ty + 8 * u] = v[u];
-    }
-    __syncthreads();
-    if (t + 1 < t_hi) load(t + 1);
-    const int kl = 2 * tx, k = t * 64 + kl;         // this thread's two K entries
+  const size_t plane = (size_t)o.rows_pad * K_pad * kE;
+  uint8_t* ob = o.out + (size_t)blockIdx.z * S * plane + (size_t)i0 * K_pad * kE;
+  // rows beyond the operand are zero: their digits are too
+  auto cut = [&](int t, const double* d) {
+    const int k = t * 64 + 2 * lane;                // this thread's two K entries
     const int s0 = ekb ? o.esign * ekb[k] : 0, s1 = ekb ? o.esign * ekb[k + 1] : 0;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int r = ty + 8 * q, i = i0 + r;
-      if (i >= o.rows_pad) continue;
-      // rows beyond the operand are zero: their digits are too
-      uint8_t* w = ob + ((size_t)i * K_pad + k) * kE;
-      slice_pair<S, FORM>(tile[r][kl], tile[r][kl + 1], es[r] - s0, es[r] - s1, [&](int s, unsigned pair) {
-        if (kE == 2) *reinterpret_cast<unsigned*>(w + s * plane * 2) = pair;
-        else *reinterpret_cast<unsigned short*>(w + s * plane) = (unsigned short)pair;
+    for (int q = 0; q < R / 8; ++q) {
+      const int rr = warp + 8 * q;
+      const double* x = d + rr * 65 + 2 * lane;
+      const unsigned at = (unsigned)(rr * K_pad + k) * kE;
+      slice_pair<S, FORM>(x[0], x[1], es[rr] - s0, es[rr] - s1, [&](int s, unsigned pair) {
+        uint8_t* w = ob + s * plane + at;
+        if (kE == 2) *reinterpret_cast<unsigned*>(w) = pair;
+        else *reinterpret_cast<unsigned short*>(w) = (unsigned short)pair;
       });
     }
-    __syncthreads();   // the tile is refilled
+  };
+  for (int t = t_lo; t < t_keep; ++t) cut(t, xs + (t - t_lo) * kSliceTile);
+  if (t_keep < t_hi) {              // the others through two of the tiles' places
+    __syncthreads();
+    fetch(t_keep, xs);
+    for (int t = t_keep; t < t_hi; ++t) {
+      const int slot = (t - t_keep) & 1;
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      __syncthreads();              // tile t is there, the other place is free
+      if (t + 1 < t_hi) fetch(t + 1, xs + (slot ^ 1) * kSliceTile);
+      cut(t, xs + slot * kSliceTile);
+    }
   }
 }
 
@@ -1062,16 +1073,24 @@ cudaError_t run_split(const GemmArgs& g, SplitWork& w, cudaStream_t st) {
   {
     const SliceOp oa{Xa, lda, sta, ta, M, Mpad, sign_a, ea, sa};
     const SliceOp ob{Xb, ldb, stb, tb, N, Npad, -sign_a, eb, sb};
-    // CTAs per 32 rows: about four per SM while each keeps a tile of K; one with many
-    // lanes in flight (clusters wait for room: 48 matrices take 117.0 ms with up to
-    // eight, 112.9 with two, 111.8 with one)
-    const int nblk = (Mpad + Npad) / 32, ntiles = Kpad / 64;
+    // CTAs per 16 rows: about four per SM while each has a tile of K, and as many as keep
+    // their share; one with many lanes in flight (clusters wait for room: 48 matrices took
+    // 117.0 ms with up to eight, 112.9 with two, 111.8 with one)
+    const int nblk = (Mpad + Npad) / kSliceRows, ntiles = Kpad / 64;
     int cl = 1;
-    while (cl < (w.throughput ? 1 : 8) && (int64_t)nblk * nb * cl < 4 * kSplitSMs && ntiles >= 2 * cl) cl *= 2;
+    while (cl < (w.throughput ? 1 : 8) && ntiles >= 2 * cl &&
+           ((int64_t)nblk * nb * cl < 4 * kSplitSMs || ntiles > kSliceKeep * cl))
+      cl *= 2;
+    const int per = (ntiles + cl - 1) / cl, keep = std::min(per, kSliceKeep);
+    const int smem = keep * kSliceTile * (int)sizeof(double);
+    const auto slice = slice_kernel<S, FORM>;
+    if ((err = smem_attr_once((const void*)slice, kSliceKeep * kSliceTile * (int)sizeof(double))) != cudaSuccess)
+      return err;
     ProfScope ps(kProfSlice, st, 0.0, (16.0 + (double)kE * S) * nb * (double)(Mpad + Npad) * Kpad);
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(nblk * cl), 1, nb);
-    cfg.blockDim = dim3(32, 8);
+    cfg.blockDim = dim3(256);
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -1080,9 +1099,9 @@ cudaError_t run_split(const GemmArgs& g, SplitWork& w, cudaStream_t st) {
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = cl > 1 ? 1 : 0;
-    ps.blocks((const void*)slice_kernel<S, FORM>, dim3(32, 8), 0, cfg.gridDim);
+    ps.blocks((const void*)slice, dim3(256), smem, cfg.gridDim);
     const int* ekc = ek;
-    if ((err = cudaLaunchKernelEx(&cfg, slice_kernel<S, FORM>, oa, ob, Mpad / 32, K, Kpad, ekc, cl)) !=
+    if ((err = cudaLaunchKernelEx(&cfg, slice, oa, ob, Mpad / kSliceRows, K, Kpad, ekc, cl, keep)) !=
         cudaSuccess)
       return err;
   }
@@ -1195,6 +1214,7 @@ cudaError_t gemm_split(const GemmArgs& g, SplitWork& w, cudaStream_t st) {
 template <int BN, int S, int FORM>
 static void prepare_form() {
   smem_attr_once((const void*)split_gemm_kernel<BN, S, FORM>, SmemLayout<BN, S, FORM>::kAlloc);
+  smem_attr_once((const void*)slice_kernel<S, FORM>, kSliceKeep * kSliceTile * (int)sizeof(double));
 }
 
 void split_prepare() {
