@@ -448,7 +448,8 @@ struct SplitEpi {
   int batch, reduce, swap;  // swap: the tile computes C^T (rows of the tile are columns of C)
   int c_upper;              // only tiles that touch the upper triangle (square, no swap)
   int b_lower;              // op(B)[k][j] = 0 for k < j: a tile starts at K block n0 / BK (no swap)
-  int ks;                   // CTAs (one cluster) that share a tile's K; 1: none
+  int ks;                   // CTAs (one cluster) that share the K of a tile from full on; 1: none
+  int full;                 // the tiles before it are computed by one CTA each
   int tiles_z, tiles;       // tiles of one batch entry (of the reduced product), in all
   int* err;
   int stall;                // test hook: the MMA issuer first waits on a barrier nothing completes
@@ -533,8 +534,8 @@ __device__ __forceinline__ double split_value(const SplitEpi& p, long long iacc,
   return v * al;
 }
 
-// Persistent: CTA b takes the tiles b, b + gridDim.x, ... (with a K split, cluster
-// b one tile).  Warp 0 streams slice tiles by TMA (two B stages of S tiles, a ring
+// Persistent: CTA b takes the tiles b, b + gridDim.x, ... (with a K split, the last or only
+// tile is its cluster's).  Warp 0 streams slice tiles by TMA (two B stages of S tiles, a ring
 // of A tiles), warp 1 issues the MMAs, sixteen warps drain the level accumulators;
 // the three run ahead of one another across K blocks, chunks and tiles, so a
 // tile's loads, its epilogue and the next tile's MMAs overlap.
@@ -576,13 +577,20 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rank = blockIdx.x % p.ks;
-  const int tile0 = blockIdx.x / p.ks, tile_step = gridDim.x / p.ks;
+  // the tile of this CTA's turn b, b + gridDim.x, ...: whole tiles, then its cluster's shared
+  // one (full is a multiple of the grid where there are any); -1: none is left
+  auto tile_at = [&](int turn) -> int {
+    if (turn < p.full) return turn;
+    if (p.ks == 1 || turn - p.full >= (int)gridDim.x) return -1;
+    const int t = p.full + blockIdx.x / p.ks;
+    return t < p.tiles ? t : -1;
+  };
   const int nkb_all = (p.K + kBK - 1) / kBK;
-  // this rank's K blocks of a tile: [lo, hi), the structurally zero ones skipped
-  auto k_range = [&](int tn, int* lo, int* hi) {
+  // this CTA's K blocks of a tile: [lo, hi), the structurally zero ones skipped
+  auto k_range = [&](int tn, bool split, int* lo, int* hi) {
     *lo = p.b_lower ? tn * BN / kBK : 0;
     *hi = nkb_all;
-    if (p.ks > 1) {
+    if (split) {
       const int per = (nkb_all - *lo + p.ks - 1) / p.ks;
       *lo += rank * per;
       *hi = min(*hi, *lo + per);
@@ -617,11 +625,12 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     int kbg = 0, ia = 0;
     bool ok = true;
     int kbg_armed = 0, ia_armed = 0;   // loads issued (for the error-path drain)
-    for (int idx = tile0; idx < p.tiles && ok; idx += tile_step) {
+    for (int turn = blockIdx.x, idx; ok && (idx = tile_at(turn)) >= 0; turn += gridDim.x) {
+      const bool split = turn >= p.full;
       const TilePos t = split_tile<BN>(p, idx);
       if (!t.valid) continue;
       int kb_lo, kb_hi;
-      k_range(t.tn, &kb_lo, &kb_hi);
+      k_range(t.tn, split, &kb_lo, &kb_hi);
       const int b_first = p.reduce ? 0 : t.z, b_last = p.reduce ? p.batch : t.z + 1;
       for (int b = b_first; b < b_last && ok; ++b) {
         const int arow = b * S * p.Mpad + t.tm * kTileM, brow = b * S * p.Npad + t.tn * BN;
@@ -676,11 +685,12 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
       tc::mbar_stall(never, err, p.stall_ns);
       ok = false;
     }
-    for (int idx = tile0; idx < p.tiles && ok; idx += tile_step) {
+    for (int turn = blockIdx.x, idx; ok && (idx = tile_at(turn)) >= 0; turn += gridDim.x) {
+      const bool split = turn >= p.full;
       const TilePos t = split_tile<BN>(p, idx);
       if (!t.valid) continue;
       int kb_lo, kb_hi;
-      k_range(t.tn, &kb_lo, &kb_hi);
+      k_range(t.tn, split, &kb_lo, &kb_hi);
       const int entries = p.reduce ? p.batch : 1;
       for (int b = 0; b < entries && ok; ++b) {
         for (int kb = kb_lo; kb < kb_hi && ok; ++kb, ++kbg) {
@@ -774,11 +784,12 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
       iacc[j] = 0;
       fm[j] = 0.f;
     }
-    for (int idx = tile0; idx < p.tiles && ok; idx += tile_step) {
+    for (int turn = blockIdx.x, idx; ok && (idx = tile_at(turn)) >= 0; turn += gridDim.x) {
+      const bool split = turn >= p.full;
       const TilePos t = split_tile<BN>(p, idx);
       if (!t.valid) continue;
       int kb_lo, kb_hi;
-      k_range(t.tn, &kb_lo, &kb_hi);
+      k_range(t.tn, split, &kb_lo, &kb_hi);
       const int nchunks = kb_hi > kb_lo ? (kb_hi - kb_lo + kChunkB - 1) / kChunkB : 0;
       const int b_first = p.reduce ? 0 : t.z, b_last = p.reduce ? p.batch : t.z + 1;
       const int row = t.tm * kTileM + q * 32 + lane;   // tile row
@@ -791,7 +802,7 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         // chunks are waited for.  The strides are made opaque here: hoisted out of
         // the loops, the columns' addresses would spill the accumulators.
         const bool first = b == b_first;
-        const bool addend = p.ks == 1 && (!first || (Cin && p.beta != 0.0));
+        const bool addend = !split && (!first || (Cin && p.beta != 0.0));
         const int col0 = n0 + half * HALF;
         const int jn = row < (p.swap ? p.N : p.M) ? (p.swap ? p.M : p.N) - col0 : 0;   // columns left
         const int64_t ldi = first ? p.ldcin : p.ldc;
@@ -845,7 +856,7 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
           }
         }
         if (!ok) break;
-        if (p.ks > 1) break;      // one entry per tile: joined over the cluster below
+        if (split) break;         // the CTA's last tile: joined over the cluster below
         // end of a batch entry: scale, combine with the addend, write, reset.  The fast
         // loop's FP64 work is one conversion and the addend's FMA (the sign of alpha =
         // +-1 is a bit, the scale an exponent); another alpha, an Inf or NaN operand or
@@ -935,8 +946,9 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     cgrp::cluster_group cluster = cgrp::this_cluster();
     __syncthreads();
     cluster.sync();
-    if (warp >= 2 && tile0 < p.tiles) {
-      const TilePos t = split_tile<BN>(p, tile0);
+    const int shared = p.full + blockIdx.x / p.ks;
+    if (warp >= 2 && shared < p.tiles) {
+      const TilePos t = split_tile<BN>(p, shared);
       if (t.valid && !*(volatile int*)err) {
         const int e = threadIdx.x - 64, r = e % kTileM, row = t.tm * kTileM + r;
         const int share = BN / p.ks;
@@ -1124,6 +1136,19 @@ cudaError_t run_split(const GemmArgs& g, SplitWork& w, cudaStream_t st) {
   p.tiles_z = split_tiles_z<BN>(Mpad / kTileM, Npad / BN, p.c_upper);
   p.tiles = p.tiles_z * nz;
   p.ks = split_ks(p.tiles, g.reduce ? nb : 1, Kpad / form_bk<FORM>(), Form<FORM>::kChunkK / form_bk<FORM>());
+  p.full = p.ks > 1 ? 0 : p.tiles;
+  int ctas = p.ks > 1 ? p.tiles * p.ks : std::min(p.tiles, kSplitSMs);
+  // A last wave that fills at most half the SMs has its tiles' K shared by pairs of CTAs:
+  // 4096^3 BF16 (13 waves and 72 tiles) 2656 -> 2591 us, 2000^3 FP16 360 -> 324, 1300 x 1000
+  // x 1000 110 -> 90, x 256 40 -> 38.5 us.  Below four blocks of K the join costs what it
+  // saves; with many lanes in flight other kernels fill the SMs.
+  const int tail = p.tiles % kSplitSMs;
+  if (p.ks == 1 && !g.reduce && !w.throughput && p.tiles > kSplitSMs && tail > 0 && 2 * tail <= kSplitSMs &&
+      Kpad / form_bk<FORM>() >= 4) {
+    p.ks = 2;
+    p.full = p.tiles - tail;
+    ctas = kSplitSMs;
+  }
   p.err = w.err;
   p.stall = w.stall;
   p.stall_ns = w.stall_ns;
@@ -1131,7 +1156,7 @@ cudaError_t run_split(const GemmArgs& g, SplitWork& w, cudaStream_t st) {
   using L = SmemLayout<BN, S, FORM>;
   const auto kernel = split_gemm_kernel<BN, S, FORM>;
   if ((err = smem_attr_once((const void*)kernel, L::kAlloc)) != cudaSuccess) return err;
-  const dim3 grid((unsigned)(p.ks > 1 ? p.tiles * p.ks : std::min(p.tiles, kSplitSMs)));
+  const dim3 grid((unsigned)ctas);
   ProfScope ps(kProfSplitGemm, st, gemm_flops(g), 0.0);
   ps.blocks((const void*)kernel, dim3(kThreads), L::kAlloc, grid);
   if (p.ks == 1) {
