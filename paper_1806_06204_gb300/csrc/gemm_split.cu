@@ -228,10 +228,11 @@ struct SliceOp {
 // (the inner-index equilibration), element (i, k) counts as x 2^(esign ek[k]).
 // Between HBM (8 bytes read, 14 written per element) and the integer work bound it: the
 // digits of the 8-bit forms are bytes picked by permutes.  Measured, both operands: 4096^3
-// 163 us (4.5 TB/s of those bytes), 196 us with 32 rows a CTA read twice and shifts for
-// digits; 8192 x 4096 x 512 50 -> 35 us, 128 x 512 x 8192 73 -> 43, 1000 x 1537 x 777 27
-// -> 19, 300^3 13.9 -> 9.8, 512 x 512 x 16384 FP8 153 -> 124 us.  Tiles kept: 4 at five
-// CTAs an SM (2: 172 us at 4096^3; 6 at four CTAs 160 us, but 36 and 128 us above).
+// 158 us (4.7 TB/s of those bytes), 196 us with 32 rows a CTA read twice and shifts for
+// digits; 8192 x 4096 x 512 50 -> 35 us, 128 x 512 x 8192 73 -> 41, 1000 x 1537 x 777 27
+// -> 18, 300^3 13.9 -> 9.8, 512 x 512 x 16384 FP8 153 -> 120 us.  Tiles kept: 4 at five
+// CTAs an SM (with one tile ahead in place of three: 163 us at 4096^3, 172 with 2 kept, 160
+// with 6 at four CTAs, but 36 and 128 us above).
 constexpr int kSliceRows = 16, kSliceTile = kSliceRows * 65;   // doubles of a tile, rows padded
 constexpr int kSliceKeep = 4;
 template <int S, int FORM>
@@ -353,15 +354,19 @@ slice_kernel(const SliceOp a, const SliceOp b, int nblk_a, int K, int K_pad,
     }
   };
   for (int t = t_lo; t < t_keep; ++t) cut(t, xs + (t - t_lo) * kSliceTile);
-  if (t_keep < t_hi) {              // the others through two of the tiles' places
+  if (t_keep < t_hi) {              // the others through the tiles' places, three ahead
+    static_assert(kSliceKeep == 4, "the places are a ring of four");
     __syncthreads();
-    fetch(t_keep, xs);
+    auto ahead = [&](int t) {
+      if (t < t_hi) fetch(t, xs + ((t - t_keep) & 3) * kSliceTile);
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    for (int u = 0; u < 3; ++u) ahead(t_keep + u);
     for (int t = t_keep; t < t_hi; ++t) {
-      const int slot = (t - t_keep) & 1;
-      asm volatile("cp.async.wait_all;" ::: "memory");
-      __syncthreads();              // tile t is there, the other place is free
-      if (t + 1 < t_hi) fetch(t + 1, xs + (slot ^ 1) * kSliceTile);
-      cut(t, xs + slot * kSliceTile);
+      asm volatile("cp.async.wait_group 2;" ::: "memory");
+      __syncthreads();              // tile t is there, the place of t - 1 is free
+      ahead(t + 3);
+      cut(t, xs + ((t - t_keep) & 3) * kSliceTile);
     }
   }
 }
