@@ -299,8 +299,8 @@ struct GuardScope {
 };
 
 // Slice-plane units for the largest contraction of a decomposition of an
-// m x n matrix (one batch entry, the larger of the BF16 form's nine slices and
-// the FP8 form's eleven, whose K runs are padded to 128).
+// m x n matrix (one batch entry, the larger of the BF16 form's planes and
+// the FP8 form's, whose K runs are padded to 128).
 size_t split_elems_per_entry(int64_t m, int64_t n) {
   const int64_t shapes[][3] = {{kQrNB, n, m + kQrNB}, {m + kQrNB, n, kQrNB}, {m, n, n},
                                {n, n, m}, {m, kCholNB, n}, {m, n, n}};
@@ -1745,6 +1745,8 @@ int zolo_pd_batched(zolo_handle_t h, int count, const double* const* A, const in
       w.stall_ns = h->dbg_ns;
       set_split_engine(is_split(opts[i].prec) ? &w : nullptr);
       TunerScope lane_tuner(sl.tuner.get());
+      // (below 512 rows a batch and a single call give the same bits: the same K splits)
+      CrowdedScope crowded(nslots >= 16 && opts[i].prec == ZOLO_FP64 && m[i] >= 512);
       const int e = pd_enqueue(R, A[i], lda[i], Qp[i], ldq[i], H[i], ldh[i], sch[i], opts[i], alpha[i]);
       set_split_engine(nullptr);
       if (e) return e;

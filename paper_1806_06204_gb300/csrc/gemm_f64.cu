@@ -227,6 +227,12 @@ double gemm_flops(const GemmArgs& g) {
   return per * g.batch * g.inner;
 }
 
+namespace {
+thread_local bool t_gemm_crowded = false;
+}
+CrowdedScope::CrowdedScope(bool on) : prev(t_gemm_crowded) { t_gemm_crowded = on; }
+CrowdedScope::~CrowdedScope() { t_gemm_crowded = prev; }
+
 int gemm_f64_default_variant(const GemmArgs&) { return kGemmVRule; }
 
 // The tile and K split the rule takes: the least estimated time, in clocks, of
@@ -253,7 +259,12 @@ F64Tile gemm_f64_rule(const GemmArgs& g) {
   // with many lanes in flight (the split forms' batch) large clusters wait for
   // room: 48 matrices take 201.5 / 199.2 / 197.2 / 198.1 ms with up to 8 / 4 / 2 / 1
   const bool crowded = get_split_engine() && get_split_engine()->throughput;
-  const int ks_max = g.b_lower || crowded ? 2 : 8;
+  // an FP64 batch's larger matrices fill the FP64 units between them: their products take
+  // the tile that costs the units least, whole (24 matrices of 800^2 .. 1024^2: 955 ms, 975
+  // unsplit by the estimate of a call's own time, 993 by that estimate with K splits, 979
+  // with 64 x 64 tiles throughout)
+  const bool shared = t_gemm_crowded;
+  const int ks_max = shared ? 1 : g.b_lower || crowded ? 2 : 8;
   double best_t = 1e300;
   for (int q = 0; q < nc; ++q) {
     const double tm = (g.M + c[q].bm - 1) / c[q].bm, tn = (g.N + c[q].bn - 1) / c[q].bn;
@@ -272,7 +283,8 @@ F64Tile gemm_f64_rule(const GemmArgs& g) {
       // ends with the longest one alone, and K slices are uneven (1024^3, r = 6
       // reduced: 8.98 / 7.11 / 5.70 ms with 64 / 32 / 16 tiles, 8.45 as 16 cut in two)
       const double uneven = g.b_lower ? (1.0 + 2.0 / per_sm) * (ks > 1 ? 1.5 : 1.0) : 1.0;
-      const double t = std::max(per_sm * kfrac, 1.0) * cta * uneven / eff + (ks > 1 ? 3000.0 + 300.0 * ks : 0.0);
+      double t = std::max(per_sm * kfrac, 1.0) * cta * uneven / eff + (ks > 1 ? 3000.0 + 300.0 * ks : 0.0);
+      if (shared) t = tiles * kfrac * cta / c[q].eff[3] / 152.0;
       if (t < best_t) {
         best_t = t;
         best = {c[q].id, ks};

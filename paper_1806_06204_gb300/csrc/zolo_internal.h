@@ -171,6 +171,13 @@ struct TunerScope {
   explicit TunerScope(GemmTuner* t) : prev(get_gemm_tuner()) { set_gemm_tuner(t); }
   ~TunerScope() { set_gemm_tuner(prev); }
 };
+// FP64 products of this thread run among many others: gemm_f64_rule then counts the time
+// of the FP64 units, not a call's own.
+struct CrowdedScope {
+  bool prev;
+  explicit CrowdedScope(bool on);
+  ~CrowdedScope();
+};
 // algorithmic flops of one call (structural zeros excluded)
 double gemm_flops(const GemmArgs& g);
 
@@ -293,7 +300,7 @@ struct QrBuffers {
 // Factor [X; sqrt(c_j) I] for j < r and overwrite W_j with the thin Q_j
 // (explicit_q = false: leave R on and above the diagonal of W_j's top block).
 // narrow_panels: many problems are in flight on other streams; the panel kernel
-// then takes the fewest CTAs per shift whose rows fit in shared memory.
+// then takes the fewest CTAs per shift whose registers hold the rows.
 cudaError_t structured_qr_q(const QrBuffers& b, int64_t m, int64_t n, int r, int* status,
                             cudaStream_t st, bool explicit_q = true, bool narrow_panels = false);
 // Inverses of the NB x NB diagonal blocks of an upper-triangular R (ld n) in the
