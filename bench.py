@@ -4,7 +4,7 @@
 Default workload: the batch of 512 square matrices (n uniform in {64,...,1024},
 kappa log-uniform in [1e2, 1e12], r per matrix from kappa) through one
 zolo_pd_batched call per step.  The split-precision form (the iterations'
-products on the BF16 tensor cores as nine Ozaki slices) is the timed headline
+products on the BF16 tensor cores as Ozaki digit slices) is the timed headline
 (`value`, matrices/s); the plain FP64 form runs on the same matrices in the same
 process (`fp64`, `fp64_value`), and `split_over_fp64` is their ratio.  Every
 result's backward error and orthogonality are checked against 1e-13 (exit code
@@ -358,9 +358,9 @@ def split_prec(zb, slices):
 # state); bench.py scales it by the bytes its own launches state.  Set to None
 # when the kernel changes.
 TRAFFIC_PER_STATED_BYTE = {
-    # qr_panel_smem_kernel, 12 launches at n = 960, r = 5: 1.313 MB read, 0
+    # qr_panel_reg_kernel, 9 launches at n = 960, r = 5: 1.364 MB read, 0
     # written, of 2.54 MB stated (profiles/traffic_batch4_split.md)
-    "qr_panel": 0.517,
+    "qr_panel": 0.537,
 }
 
 

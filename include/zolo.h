@@ -41,7 +41,7 @@ enum {
   ZOLO_ENOMEM = 5,     /* workspace too small / device allocation failed        */
   ZOLO_EEIG = 6,       /* the Jacobi eigensolver did not converge               */
   ZOLO_ETIMEOUT = 7,   /* a bounded device wait expired (split GEMM pipeline,
-                          Jacobi grid barrier or column-pair wait)              */
+                          Jacobi block-pair or column-pair wait)                */
   ZOLO_EIO = 8,        /* a tuning-cache file could not be written or read      */
   ZOLO_EINVAL = 9,     /* a tuning-cache file is malformed or from another GPU  */
   ZOLO_ECOMM = 10,     /* the caller's sum over ranks (zolo_pd_sharded) failed  */
