@@ -162,8 +162,7 @@ gemm_f64_kernel(const GemmArgs g, int ks) {
       for (int i = 0; i < TM; ++i) put(tr + i * RT, tc + j * CT, acc[i][j]);
     return;
   }
-  // every rank has read its operands before any rank writes C (the barrier), so
-  // a product whose one row tile covers M may be formed in place
+  // every rank of this tile has read its operands before any rank writes C (the barrier)
   namespace cgrp = cooperative_groups;
   cgrp::cluster_group cluster = cgrp::this_cluster();
 #pragma unroll
@@ -251,7 +250,9 @@ F64Tile gemm_f64_rule(const GemmArgs& g) {
                              {2, 16, 16, {0.54, 0.78, 0.86, 0.93}}};
   static const Cand inplace[] = {{3, 64, 16, {0.73, 0.92, 0.96, 0.97}},
                                  {0, 64, 64, {0.95, 0.99, 1.0, 1.0}}};
-  // C over A or B: only tiles that hold all of a column's rows (M <= 64)
+  // C in the address range of A or B: tiles that are right in place where elements are
+  // shared (if none is, gemm_f64_variant forms the product beside C), and tall ones where
+  // none are (the Cholesky updates)
   const bool alias = gemm_output_aliases_input(g);
   const Cand* c = alias ? inplace : all;
   const int nc = alias ? 2 : 3;
@@ -269,6 +270,7 @@ F64Tile gemm_f64_rule(const GemmArgs& g) {
   for (int q = 0; q < nc; ++q) {
     const double tm = (g.M + c[q].bm - 1) / c[q].bm, tn = (g.N + c[q].bn - 1) / c[q].bn;
     if (tm > 65535.0) continue;   // grid.y
+    if (alias && !gemm_tile_in_place(g, c[q].bm, c[q].bn)) continue;
     double tiles = tm * tn * (g.reduce ? 1 : g.batch * g.inner);
     if (g.c_upper) tiles *= 0.5 * (1.0 + 1.0 / tn);
     const double kfrac = g.b_lower ? 0.5 * (1.0 + (double)c[q].bn / std::max(g.K, c[q].bn)) : 1.0;
@@ -303,6 +305,33 @@ cudaError_t gemm_f64_tile(const GemmArgs& g, F64Tile t, cudaStream_t st) {
   }
 }
 
+namespace {
+
+// The product into a scratch, then copied over C: for an output that shares elements
+// with an input and a tile that would write what another tile has yet to read.
+cudaError_t gemm_f64_beside(const GemmArgs& g, int variant, cudaStream_t st) {
+  const int nz = g.reduce ? 1 : g.batch * g.inner;
+  double* tmp = nullptr;
+  cudaError_t e = cudaMallocAsync((void**)&tmp, sizeof(double) * (size_t)nz * g.M * (size_t)g.N, st);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return e;
+  }
+  GemmArgs h = g;
+  h.Cout = tmp;
+  h.ldcout = g.M;
+  h.innerC = (int64_t)g.M * g.N;
+  h.strideCout = h.innerC * g.inner;
+  e = gemm_f64_variant(h, variant, st);
+  for (int z = 0; z < nz && e == cudaSuccess; ++z)
+    e = copy_matrix(tmp + z * h.innerC, g.M,
+                    g.Cout + (z / g.inner) * g.strideCout + (z % g.inner) * g.innerC, g.ldcout, g.M, g.N, st);
+  const cudaError_t f = cudaFreeAsync(tmp, st);
+  return e != cudaSuccess ? e : f;
+}
+
+}  // namespace
+
 cudaError_t gemm_f64_variant(const GemmArgs& g, int variant, cudaStream_t st) {
   if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return cudaSuccess;
   if (g.batch > kGemmMaxBatch) return cudaErrorInvalidValue;
@@ -315,13 +344,20 @@ cudaError_t gemm_f64_variant(const GemmArgs& g, int variant, cudaStream_t st) {
     gemm_beta_only<<<grid, 256, 0, st>>>(g);
     return cudaGetLastError();
   }
+  static const int kTile[4][2] = {{64, 64}, {32, 32}, {16, 16}, {64, 16}};   // by F64Tile::tile
+  const bool wide = variant == kGemmV32x128 || variant == kGemmV32x64;
+  const bool split_k = variant == kGemmVSplitK2 || variant == kGemmVSplitK4 || variant == kGemmVSplitK8;
+  const F64Tile t = wide || split_k ? F64Tile{0, 1} : gemm_f64_rule(g);
+  const int bm = wide ? 32 : kTile[t.tile][0];
+  const int bn = variant == kGemmV32x128 ? 128 : wide ? 64 : kTile[t.tile][1];
+  if (!gemm_tile_in_place(g, bm, bn)) return gemm_f64_beside(g, variant, st);
   switch (variant) {
     case kGemmV32x128: return launch<32, 128, 4, 4>(g, 1, st);
     case kGemmV32x64: return launch<32, 64, 4, 4>(g, 1, st);
     case kGemmVSplitK2: return launch<64, 64, 4, 4>(g, 2, st);
     case kGemmVSplitK4: return launch<64, 64, 4, 4>(g, 4, st);
     case kGemmVSplitK8: return launch<64, 64, 4, 4>(g, 8, st);
-    default: return gemm_f64_tile(g, gemm_f64_rule(g), st);
+    default: return gemm_f64_tile(g, t, st);
   }
 }
 

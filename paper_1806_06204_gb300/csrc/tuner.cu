@@ -74,9 +74,8 @@ bool ensure_scratch(GemmTuner& t, size_t elems, cudaStream_t st) {
 // the split path untimed, and one estimated 4x slower on it is not timed
 // there; a shape whose built-in kernel takes over 50 ms keeps it.  When the
 // output overlaps A or B (a product computed in place, as the Cholesky panel
-// update is) the only candidates are the built-in tile, which the call site is
-// written for, and the variants that read all of A and B before writing C
-// (split-K, split).
+// update is) the wide tiles are not candidates; what does run there is made safe by
+// gemm_f64_variant, or (the split path) has sliced A and B before it writes C.
 int tune(GemmTuner& t, const GemmArgs& g, SplitWork* split, cudaStream_t st) {
   const size_t out = (size_t)(g.reduce ? 1 : g.batch * g.inner) * (size_t)g.M * (size_t)g.N;
   std::vector<int> cand = {kGemmVRule, kGemmV32x128, kGemmV32x64};
@@ -176,6 +175,55 @@ bool gemm_output_aliases_input(const GemmArgs& g) {
   return overlap(c, a) || overlap(c, b);
 }
 
+namespace {
+
+// Whether C's elements are among those of an operand of rows x cols: entry against entry,
+// since the entries of a batch interleave; two views with one leading dimension share
+// nothing where their rows are apart (a Cholesky update's operands lie above its output).
+bool shares_elements(const GemmArgs& g, const double* p, int64_t ld, int64_t rows, int64_t cols,
+                     int64_t stride, int64_t inner_stride) {
+  const int nc = g.reduce ? 1 : g.batch;
+  if (!overlap(extent(g.Cout, g.ldcout, g.M, g.N, g.strideCout, nc, g.innerC, g.inner),
+               extent(p, ld, rows, cols, stride, g.batch, inner_stride, g.inner)))
+    return false;
+  for (int x = 0; x < nc * g.inner; ++x)
+    for (int y = 0; y < g.batch * g.inner; ++y) {
+      const double* c = g.Cout + x / g.inner * g.strideCout + x % g.inner * g.innerC;
+      const double* q = p + y / g.inner * stride + y % g.inner * inner_stride;
+      if (!overlap(extent(c, g.ldcout, g.M, g.N, 0, 1, 0, 1), extent(q, ld, rows, cols, 0, 1, 0, 1)))
+        continue;
+      if (ld != g.ldcout) return true;
+      const int64_t d = ((c - q) % ld + ld) % ld;   // C's first row in the operand's columns
+      if (d < rows || d + g.M > ld) return true;
+    }
+  return false;
+}
+
+}  // namespace
+
+// A tile reads the rows of op(A) and the columns of op(B) that its outputs lie in, by all
+// ranks of a K split before any of them writes; nothing orders two tiles.  So C may lie
+// over A, entry for entry, where a tile holds all columns, over B where it holds all rows,
+// and anywhere where it is the only tile.
+bool gemm_tile_in_place(const GemmArgs& g, int bm, int bn) {
+  const bool on_a = shares_elements(g, g.A, g.lda, g.transA ? g.K : g.M, g.transA ? g.M : g.K,
+                                    g.strideA, g.innerA);
+  const bool on_b = shares_elements(g, g.B, g.ldb, g.transB ? g.N : g.K, g.transB ? g.K : g.N,
+                                    g.strideB, g.innerB);
+  if (!on_a && !on_b) return true;
+  const int planes = g.reduce ? 1 : g.batch * g.inner;
+  if (planes == 1 && g.M <= bm && g.N <= bn) return true;
+  // the same place in every entry, and the entries apart
+  auto same = [&](const double* p, int64_t ld, int64_t stride, int64_t rows, int64_t cols) {
+    return p == g.Cout && ld == g.ldcout && g.inner == 1 &&
+           (g.batch == 1 || (!g.reduce && stride == g.strideCout && stride >= (cols - 1) * ld + rows));
+  };
+  const int64_t wide = std::max(g.N, g.K), tall = std::max(g.M, g.K);
+  if (on_a && (g.transA || g.N > bn || !same(g.A, g.lda, g.strideA, g.M, wide))) return false;
+  if (on_b && (g.transB || g.M > bm || !same(g.B, g.ldb, g.strideB, tall, g.N))) return false;
+  return true;
+}
+
 std::array<int, 7> gemm_key(const GemmArgs& g, int split_slices) {
   const int flags = (g.transA ? 1 : 0) | (g.transB ? 2 : 0) | (g.reduce ? 4 : 0) |
                     (g.b_lower ? 8 : 0) | (g.c_upper ? 16 : 0) |
@@ -190,7 +238,8 @@ bool gemm_variant_allowed(const std::array<int, 7>& key, int v) {
   if (v == kGemmVSplit) return key[5] != 0;
   if (!split_k && !tiles) return false;
   if (!(key[4] & 128) || split_k) return true;
-  // in place: only the built-in rule (which then takes a tile of 64 rows)
+  // in place: the built-in rule (which then takes a tile that is right there) or split K;
+  // either forms the product beside C where no tile is (gemm_f64_variant)
   return v == kGemmVRule || (key[0] <= 32 && v == kGemmV32x128);
 }
 

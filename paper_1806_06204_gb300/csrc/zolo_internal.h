@@ -158,8 +158,10 @@ struct GemmTuner {
   ~GemmTuner();
 };
 std::array<int, 7> gemm_key(const GemmArgs& g, int split_slices);
-// C's elements overlap those of A or B (flag 128 of the key)
+// C lies in the address range of A or B (flag 128 of the key)
 bool gemm_output_aliases_input(const GemmArgs& g);
+// whether tiles of bm x bn leave C right when it shares elements with A or B
+bool gemm_tile_in_place(const GemmArgs& g, int bm, int bn);
 // whether kernel v may serve a key (tile variants other than the built-in one
 // are barred for in-place products: their CTAs would overwrite rows of B that
 // other CTAs still read)
