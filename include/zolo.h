@@ -271,6 +271,12 @@ int zolo_pd_batched(zolo_handle_t handle, int count, const double* const* A, con
    and replays.  Returns 0, -1 (NULL handle) or -2 (enable not 0/1). */
 int zolo_batch_graphs(zolo_handle_t handle, int enable);
 
+/* Graphs zolo_pd_batched has recorded on this handle so far: a call that replays
+   one leaves the count as it was; one whose pointers, sizes or options differ, or
+   for which the handle's buffers have moved since, adds one.  -1 for a NULL
+   handle. */
+int64_t zolo_batch_graphs_recorded(zolo_handle_t handle);
+
 /* As zolo_pd / zolo_svd, but every matrix pointer is a HOST pointer: the call
    copies A to the device, computes, and copies the results back (pageable or
    pinned host memory; pinned is faster).  Device buffers come from the

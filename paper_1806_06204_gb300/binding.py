@@ -103,6 +103,8 @@ def _load():
     lib.zolo_debug_guards.restype = I
     lib.zolo_batch_graphs.argtypes = [P, I]
     lib.zolo_batch_graphs.restype = I
+    lib.zolo_batch_graphs_recorded.argtypes = [P]
+    lib.zolo_batch_graphs_recorded.restype = I64
     lib.zolo_debug_stall.argtypes = [P, I, I64]
     lib.zolo_debug_stall.restype = I
     lib.zolo_autotune.argtypes = [P, I]
@@ -129,7 +131,8 @@ EXPORTED = ["zolo_opts_default", "zolo_create", "zolo_destroy", "zolo_coefficien
             "zolo_dgemm", "zolo_dgemm_noalloc", "zolo_pd_batched", "zolo_tuned_r",
             "zolo_tune_save", "zolo_tune_load", "zolo_autotune",
             "zolo_workspace_bytes", "zolo_debug_stall", "zolo_shift_range",
-            "zolo_pd_sharded", "zolo_pd_async", "zolo_batch_graphs", "zolo_debug_guards"]
+            "zolo_pd_sharded", "zolo_pd_async", "zolo_batch_graphs",
+            "zolo_batch_graphs_recorded", "zolo_debug_guards"]
 
 
 def kernel_launches() -> int:
@@ -246,6 +249,11 @@ def batch_graphs(handle, enable: bool) -> None:
     e = LIB.zolo_batch_graphs(handle.ptr, int(enable))
     if e:
         raise ZoloError(e, "zolo_batch_graphs")
+
+
+def batch_graphs_recorded(handle) -> int:
+    """Graphs zolo_pd_batched has recorded on this handle so far."""
+    return int(LIB.zolo_batch_graphs_recorded(handle.ptr))
 
 
 def debug_stall(handle, where: int, ns: int = 0) -> None:

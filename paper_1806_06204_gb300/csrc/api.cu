@@ -85,6 +85,7 @@ struct zolo_handle_s {
   double* hrec = nullptr;        // pinned host mirror of brec
   size_t hrec_count = 0;
   std::vector<BatchGraph> graphs;
+  uint64_t graphs_recorded = 0;
   void* ws = nullptr;
   size_t ws_bytes = 0;
   void* io = nullptr;
@@ -1698,7 +1699,14 @@ int zolo_pd_batched(zolo_handle_t h, int count, const double* const* A, const in
   key.push_back((uint64_t)count);
   key.push_back((uint64_t)(uintptr_t)h->brec);
   key.push_back(h->tuner.gen);   // graphs recorded with older kernel choices are not replayed
-  for (int k = 0; k < nslots; ++k) key.push_back((uint64_t)(uintptr_t)h->slots[k].ws);
+  // every buffer the recorded kernels hold: the split ones grow apart from the workspace
+  for (int k = 0; k < nslots; ++k) {
+    const BatchSlot& sl = h->slots[k];
+    key.push_back((uint64_t)(uintptr_t)sl.ws);
+    key.push_back(any_split ? (uint64_t)(uintptr_t)sl.slices : 0);
+    key.push_back(any_split ? (uint64_t)(uintptr_t)sl.exps : 0);
+    key.push_back(any_split ? (uint64_t)(uintptr_t)sl.err : 0);
+  }
   for (int i = 0; i < count; ++i) {
     const uint64_t f[] = {(uint64_t)(uintptr_t)A[i], (uint64_t)m[i], (uint64_t)n[i],
                           (uint64_t)lda[i], (uint64_t)(uintptr_t)Qp[i], (uint64_t)ldq[i],
@@ -1782,6 +1790,7 @@ int zolo_pd_batched(zolo_handle_t h, int count, const double* const* A, const in
         // the capture itself ran no kernel: take the recorded ones back off the counter
         add_launches(-(int64_t)graph_launches);
         h->graphs.push_back({key, exec, graph_launches});
+        ++h->graphs_recorded;
         if (h->graphs.size() > 8) {
           cudaGraphExecDestroy(h->graphs.front().exec);
           h->graphs.erase(h->graphs.begin());
@@ -1866,6 +1875,10 @@ int zolo_batch_graphs(zolo_handle_t h, int enable) {
   if (enable != 0 && enable != 1) return -2;
   h->batch_graphs = enable != 0;
   return 0;
+}
+
+int64_t zolo_batch_graphs_recorded(zolo_handle_t h) {
+  return h ? (int64_t)h->graphs_recorded : -1;
 }
 
 int zolo_debug_stall(zolo_handle_t h, int where, int64_t ns) {
