@@ -381,8 +381,10 @@ slice_kernel(const SliceOp a, const SliceOp b, int nblk_a, int K, int K_pad,
 
 // An output's value from its level sums, iacc in units of 2^-48 and fm in units of
 // 2^-(48 + LO), as x 2^k with |x| < 2^63: the LO bits below iacc's unit are kept while
-// they fit; where x has 53 bits and more without them, they only decide the rounding
-// (the last bit is set when any of them is).  WIDE: fm may exceed 2^30.
+// they fit.  The FP8 form's 17 do not above 2^45: there x takes nine of them (or none,
+// above 2^54) and has 55 bits and more, two below the last of FP64's 53, so the lowest
+// one may stand for all that is cut (set when any of it is) and x's own rounding to FP64
+// is the only one.  WIDE: fm may exceed 2^30.
 struct Fixed {
   long long x;
   int k;
@@ -394,6 +396,7 @@ __device__ __forceinline__ bool beyond(long long hi) {
 }
 template <int LO, bool WIDE>
 __device__ __forceinline__ Fixed split_fixed(long long iacc, float fm) {
+  constexpr int kLow = LO > 8 ? 9 : 8;   // low bits kept below 2^54
   long long hi;
   int lo;
   if (WIDE) {
@@ -412,10 +415,10 @@ __device__ __forceinline__ Fixed split_fixed(long long iacc, float fm) {
     r.k = -48 - LO;
     return r;
   }
-  if (LO > 8) lo = (lo >> (LO - 8)) | ((lo & ((1 << (LO - 8)) - 1)) != 0);
+  if (LO > 8) lo = (lo >> (LO - kLow)) | ((lo & ((1 << (LO - kLow)) - 1)) != 0);
   const bool big = beyond<54>(hi);
-  r.x = big ? (hi | (lo != 0)) : ((hi << 8) | lo);
-  r.k = big ? -48 : -56;
+  r.x = big ? (hi | (lo != 0)) : ((hi << kLow) | lo);
+  r.k = big ? -48 : -48 - kLow;
   return r;
 }
 
