@@ -19,7 +19,11 @@
 // FP32 sweeps stop when fewer than n rotations (cosines above 8e-6) were needed
 // in a sweep (25 sweeps at most): the FP64 sweeps start from cosines of about
 // 1e-4 whatever the last FP32 sweeps do, since Z's FP32 rounding, times R^T,
-// sets them.  FP64 sweeps stop when no pair has |x_p . x_q| > 8 eps ||x_p||
+// sets them.  The FP32 sweeps' Gram entries and the FP64 sweeps' FP32 cosines and angles
+// are of the size of H's eigenvalues, so X is R^T times a power of two that puts the
+// largest diagonal entry of H in [2^90, 2^92): their range then holds eigenvalues down to
+// 1e-50 of the largest, whatever the matrix's own scale (V and the Rayleigh quotients do
+// not see it).  FP64 sweeps stop when no pair has |x_p . x_q| > 8 eps ||x_p||
 // ||x_q||, or after a sweep in which every cosine was below sqrt(n) eps (the
 // rounding level of an n-term dot product): its rotations were of that size,
 // so the next sweep would find the same rounding-level cosines again.  Pairs are
@@ -210,7 +214,8 @@ jacobi_sweep_kernel(double* X, int64_t ldx, int64_t m, int n_even, int n_real, d
         sg = warp_sum(sg) * dd;                         // cross product of the true columns
         const float fg = (float)sg;
         const float cosv = (fa > 0.f && fb > 0.f) ? fabsf(fg) * rsqrtf(fa) * rsqrtf(fb) : 0.f;
-        const int rot = fg != 0.f && cosv > (float)tol ? (cosv > 4.f * (float)tol ? 2 : 1) : 0;
+        // (a cross product below FLT_MIN: left as converged)
+        const int rot = fabsf(fg) >= 0x1p-126f && cosv > (float)tol ? (cosv > 4.f * (float)tol ? 2 : 1) : 0;
         const float zeta = __fdividef(0.5f * fd, fg), az = fabsf(zeta);
         const float z1 = fmaf(az, az, 1.f);
         const float tf = copysignf(az > 1e18f ? __fdividef(0.5f, az) : __fdividef(1.f, az + z1 * rsqrtf(z1)), zeta);
@@ -471,7 +476,7 @@ jacobi32_block_sweep_kernel(float* X, float* Z, int64_t ld, int64_t m, int nb_ev
             const float r = __fdividef(1.f, d), q = n * r;
             return fmaf(r, fmaf(-d, q, n), q);
           };
-          if (col(b2) < n_real && gab != 0.f && ga > 0.f && gb > 0.f &&
+          if (col(b2) < n_real && fabsf(gab) >= 0x1p-126f && ga > 0.f && gb > 0.f &&
               fabsf(gab) * rsqrtf(ga) * rsqrtf(gb) > tol) {
             // approximations polished to FP32 rounding by one Newton step each (a wrong
             // angle leaves its error times the cosine to the next sweep)
@@ -638,12 +643,28 @@ __global__ void gather_columns_kernel(const double* __restrict__ X, int64_t ldx,
     y[r] = f * x[r];
 }
 
+// *scale = 2^k with 4^k times the largest diagonal entry of H in [2^90, 2^92) (1 where that
+// entry is not a positive number).  One block.
+__global__ void eig_scale_kernel(const double* __restrict__ H, int64_t ldh, int64_t n, double* scale) {
+  __shared__ double red[kJacThreads / 32];
+  double mx = 0.0;
+  for (int64_t i = threadIdx.x; i < n; i += kJacThreads) mx = fmax(mx, H[i + i * ldh]);
+  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int k = 0; k < kJacThreads / 32; ++k) mx = fmax(mx, red[k]);
+    *scale = mx > 0.0 && isfinite(mx) ? ldexp(1.0, (91 - ilogb(mx)) >> 1) : 1.0;
+  }
+}
+
+// X = scale R^T, the strictly upper part zero.
 __global__ void transpose_lower_kernel(const double* __restrict__ R, int64_t ldr, double* __restrict__ X,
-                                       int64_t ldx, int64_t n) {
+                                       int64_t ldx, int64_t n, const double* __restrict__ scale) {
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n * n;
        e += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = e % n, j = e / n;
-    X[i + j * ldx] = i >= j ? R[j + i * ldr] : 0.0;
+    X[i + j * ldx] = i >= j ? *scale * R[j + i * ldr] : 0.0;
   }
 }
 
@@ -688,12 +709,12 @@ cudaError_t gather_columns(const double* X, int64_t ldx, double* Y, int64_t ldy,
 }
 
 cudaError_t transpose_lower(const double* R, int64_t ldr, double* X, int64_t ldx, int64_t n,
-                            cudaStream_t st) {
+                            const double* scale, cudaStream_t st) {
   const int64_t b = std::min<int64_t>((n * n + 255) / 256, 4096);
   ProfScope ps(kProfOther, st);
   ps.blocks((const void*)transpose_lower_kernel, dim3(256), 0,
             dim3((unsigned)std::max<int64_t>(b, 1)));
-  transpose_lower_kernel<<<(unsigned)std::max<int64_t>(b, 1), 256, 0, st>>>(R, ldr, X, ldx, n);
+  transpose_lower_kernel<<<(unsigned)std::max<int64_t>(b, 1), 256, 0, st>>>(R, ldr, X, ldx, n, scale);
   return cudaGetLastError();
 }
 
@@ -769,7 +790,13 @@ int eig_sym_jacobi(const double* H, int64_t ldh, int64_t n, double* V, int64_t l
   int total_sweeps = 0;
   // ---- FP32 phase on X32 = R^T, rotations accumulated in Z32
   if (cudaMemsetAsync(w.err, 0, sizeof(int), st) != cudaSuccess) return 1;
-  if (transpose_lower(w.R, n, w.X, n, n, st) != cudaSuccess) return 1;
+  double* scale = w.lam;   // free until the FP64 sweeps
+  {
+    ProfScope ps(kProfOther, st);
+    ps.blocks((const void*)eig_scale_kernel, dim3(kJacThreads), 0, dim3(1));
+    eig_scale_kernel<<<1, kJacThreads, 0, st>>>(H, ldh, n, scale);
+  }
+  if (transpose_lower(w.R, n, w.X, n, n, scale, st) != cudaSuccess) return 1;
   {
     ProfScope ps(kProfOther, st);
     ps.blocks((const void*)to_f32_kernel, dim3(256), 0, dim3(eg));
@@ -863,8 +890,8 @@ int eig_sym_jacobi(const double* H, int64_t ldh, int64_t n, double* V, int64_t l
     if (cholesky_upper_batched(cz, n, 1, w.status, st) != cudaSuccess) return 1;
     if (trsm_right_upper_batched(w.Z, n, cz, w.X, 0, w.tmp, 0, n, n, 1, st) != cudaSuccess) return 1;
   }
-  // ---- X = R^T Z in FP64 (w.Z <- R^T, w.HV <- R^T Z)
-  if (transpose_lower(w.R, n, w.Z, n, n, st) != cudaSuccess) return 1;
+  // ---- X = R^T Z in FP64 (w.Z <- R^T, scaled as before, w.HV <- R^T Z)
+  if (transpose_lower(w.R, n, w.Z, n, n, scale, st) != cudaSuccess) return 1;
   {
     GemmArgs g;
     g.M = g.N = g.K = (int)n;

@@ -361,8 +361,9 @@ cudaError_t column_dots(const double* A, int64_t lda, const double* B, int64_t l
                         int64_t n, double* out, cudaStream_t st);
 cudaError_t gather_columns(const double* X, int64_t ldx, double* Y, int64_t ldy, int64_t m,
                            int64_t n, const int* perm, const double* sign, cudaStream_t st);
+// X = *scale R^T (lower triangular, zero above)
 cudaError_t transpose_lower(const double* R, int64_t ldr, double* X, int64_t ldx, int64_t n,
-                            cudaStream_t st);
+                            const double* scale, cudaStream_t st);
 // One FP64 sweep of the one-sided Jacobi rounds (a cooperative launch; ver holds
 // n_even round counters, err the bounded waits' flag).
 cudaError_t jacobi_sweep(double* X, int64_t ldx, int64_t m, int64_t n_even, int64_t n_real,
