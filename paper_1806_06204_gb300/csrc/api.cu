@@ -301,10 +301,14 @@ struct GuardScope {
 
 // Slice-plane units for the largest contraction of a decomposition of an
 // m x n matrix (one batch entry, the larger of the BF16 form's planes and
-// the FP8 form's, whose K runs are padded to 128).
+// the FP8 form's, whose K runs are padded to 128): the panels' products, those of a
+// block or super-block of w columns (V^T C and V^T V over its row window, V W), and the
+// products of the iterations with n and m.
 size_t split_elems_per_entry(int64_t m, int64_t n) {
+  const int64_t w = std::min<int64_t>(n, kQrBlock), sw = std::min<int64_t>(n, qr_super_width(n));
   const int64_t shapes[][3] = {{kQrNB, n, m + kQrNB}, {m + kQrNB, n, kQrNB}, {m, n, n},
-                               {n, n, m}, {m, kCholNB, n}, {m, n, n}};
+                               {n, n, m}, {m, kCholNB, n}, {w, n, m + w}, {w, w, m + w},
+                               {m + w, n, w}, {sw, n, m + sw}, {sw, sw, m + sw}, {m + sw, n, sw}};
   size_t mx = 0;
   for (auto& sh : shapes)
     mx = std::max({mx, split_slice_elems(sh[0], sh[1], sh[2], 1, 9, kFormBF16),
