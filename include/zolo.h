@@ -364,7 +364,8 @@ int zolo_dgemm_noalloc(int transA, int transB, int64_t m, int64_t n, int64_t k, 
 
    zolo_tune_save / zolo_tune_load write and read both caches as text: a first
    line "zolo-tune 2 <device name>", then "r m n prec decade r" lines and
-   "g M N K batch flags slices kernel" lines; loading a file written on a
+   "g M N K batch flags slices kernel" lines ("gi ... slices inner kernel" where a
+   batch entry holds several products); loading a file written on a
    device of another name, or any malformed line, returns ZOLO_EINVAL and
    keeps the caches as they were.  Both return 0, -1/-2 for a NULL argument,
    or ZOLO_EIO when the file cannot be written or read. */

@@ -1919,9 +1919,14 @@ int zolo_tune_save(zolo_handle_t h, const char* path) {
     ok = ok && std::fprintf(f, "r %lld %lld %lld %lld %d\n", (long long)kv.first[0],
                             (long long)kv.first[1], (long long)kv.first[2], (long long)kv.first[3],
                             kv.second) > 0;
-  for (const auto& kv : h->tuner.choice)
-    ok = ok && std::fprintf(f, "g %d %d %d %d %d %d %d\n", kv.first[0], kv.first[1], kv.first[2],
-                            kv.first[3], kv.first[4], kv.first[5], kv.second) > 0;
+  for (const auto& kv : h->tuner.choice) {
+    // products within a batch entry: a line of their own kind, with their count
+    const bool inner = kv.first[6] > 1;
+    ok = ok && std::fprintf(f, "%s %d %d %d %d %d %d ", inner ? "gi" : "g", kv.first[0], kv.first[1],
+                            kv.first[2], kv.first[3], kv.first[4], kv.first[5]) > 0;
+    if (inner) ok = ok && std::fprintf(f, "%d ", kv.first[6]) > 0;
+    ok = ok && std::fprintf(f, "%d\n", kv.second) > 0;
+  }
   ok = (std::fclose(f) == 0) && ok;
   return ok ? 0 : ZOLO_EIO;
 }
@@ -1955,16 +1960,17 @@ int zolo_tune_load(zolo_handle_t h, const char* path) {
         rc = ZOLO_EINVAL;
       else
         got_r[{a, b, c, d}] = r;
-    } else if (std::strcmp(tag, "g") == 0) {
-      int k[6], v;
-      if (std::fscanf(f, "%d %d %d %d %d %d %d", &k[0], &k[1], &k[2], &k[3], &k[4], &k[5], &v) !=
-              7 ||
-          k[0] < 1 || k[1] < 1 || k[2] < 1 || k[3] < 1 || k[3] > kGemmMaxBatch || k[4] < 0 ||
+    } else if (std::strcmp(tag, "g") == 0 || std::strcmp(tag, "gi") == 0) {
+      int k[6], inner = 1, v;
+      bool ok = std::fscanf(f, "%d %d %d %d %d %d", &k[0], &k[1], &k[2], &k[3], &k[4], &k[5]) == 6;
+      if (tag[1]) ok = ok && std::fscanf(f, "%d", &inner) == 1 && inner > 1 && inner <= INT_MAX / kGemmMaxBatch;
+      ok = ok && std::fscanf(f, "%d", &v) == 1;
+      if (!ok || k[0] < 1 || k[1] < 1 || k[2] < 1 || k[3] < 1 || k[3] > kGemmMaxBatch || k[4] < 0 ||
           k[4] > 255 || (k[5] != 0 && k[5] != 8 && k[5] != 9 && k[5] != 108 && k[5] != 211) ||
-          !gemm_variant_allowed({k[0], k[1], k[2], k[3], k[4], k[5], 0}, v))
+          !gemm_variant_allowed({k[0], k[1], k[2], k[3], k[4], k[5], inner}, v))
         rc = ZOLO_EINVAL;
       else
-        got_g[{k[0], k[1], k[2], k[3], k[4], k[5], 0}] = v;
+        got_g[{k[0], k[1], k[2], k[3], k[4], k[5], inner}] = v;
     } else {
       rc = ZOLO_EINVAL;
     }

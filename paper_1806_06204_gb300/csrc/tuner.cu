@@ -229,7 +229,7 @@ std::array<int, 7> gemm_key(const GemmArgs& g, int split_slices) {
                     (g.b_lower ? 8 : 0) | (g.c_upper ? 16 : 0) |
                     (g.Cin && g.beta != 0.0 ? 32 : 0) | (g.k_equilibrate ? 64 : 0) |
                     (gemm_output_aliases_input(g) ? 128 : 0);
-  return {g.M, g.N, g.K, g.batch, flags, split_slices, 0};
+  return {g.M, g.N, g.K, g.batch, flags, split_slices, g.inner};
 }
 
 bool gemm_variant_allowed(const std::array<int, 7>& key, int v) {

@@ -142,7 +142,7 @@ cudaError_t gemm_f64_tile(const GemmArgs& g, F64Tile t, cudaStream_t st);
 cudaError_t gemm_f64(const GemmArgs& g, cudaStream_t st);
 
 // Measured kernel choice per contraction shape (sizes, batch, transposes,
-// structure flags, slice count): the cache of a handle, made current for the
+// structure flags, slice count, products within an entry): the cache of a handle, made current for the
 // calls of one API entry point by TunerScope.  With `tuning` set, a shape met
 // for the first time is run with every candidate variant into a scratch output
 // (the real output untouched) and timed with CUDA events; the fastest is kept.
