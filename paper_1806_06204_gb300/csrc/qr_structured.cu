@@ -425,7 +425,7 @@ qr_panel_reg_kernel(double* W, int64_t strideW, int64_t ldw, int64_t m, int64_t 
         if (n2 > 1e-280 && n2 < 1e280) {
           root_pair(n2, &nrm, &inv);
           beta = -copysign(nrm, alpha);
-          tau = (beta - alpha) * -copysign(inv, alpha);
+          tau = fma(fabs(alpha), inv, 1.0);   // (beta - alpha) / beta with beta = -sign(alpha) nrm
           scal = reciprocal(alpha - beta);
         } else {   // near the ends of the range, or not finite
           beta = -copysign(sqrt(n2), alpha);
