@@ -1,6 +1,6 @@
 // Split-precision FP64 GEMM on the tensor cores (tcgen05 + TMEM + TMA), the Ozaki
 // scheme: every FP64 operand row (of op(A)) / column (of op(B)) is scaled by a
-// power of two 2^e so that its entries lie in (-1/2, 1/2), rounded to the
+// power of two 2^e so that its entries lie in [-1/2, 1/2], rounded to the
 // fixed-point integer N = round(x 2^(bS - e)) and written in S balanced base-2^b
 // digits,
 //     x 2^-e = sum_{s=1..S} d_s 2^{-bs} (+ rounding below 2^{-bS-1}),
@@ -81,9 +81,8 @@ constexpr int kThreads = 64 + 32 * kEpiWarps;   // warp 0 TMA, warp 1 MMA, the r
 // Row i of op(X) (rows x K):  trans = 0: X[i + k ldx] (rows contiguous),
 //                             trans = 1: X[k + i ldx] (row contiguous along k).
 
-// e_i with max_k |op(X)_ik| < 2^(e_i - 1) (0 for a zero row).  Integer
-// arithmetic on the FP64 bit patterns (|x| orders like its magnitude bits); no
-// FP64 pipe work.
+// e with |x| < 2^(e - 1) (0 for a zero).  Integer arithmetic on the FP64 bit patterns
+// (|x| orders like its magnitude bits); no FP64 pipe work.
 __device__ __forceinline__ int exp_above(unsigned long long mag) {
   if (mag == 0) return 0;
   const int ef = (int)(mag >> 52);
@@ -140,7 +139,16 @@ __global__ void col_exp_kernel(const double* __restrict__ X, int64_t ldx, int64_
   }
 }
 
-// N = round(x 2^(bS - e)) from the bit pattern (|x| < 2^(e-1), so |N| <= 2^(bS-1));
+// e with |x| <= 2^(e - 1) from the high word of |x|, its low bit set where the low word is
+// not zero (one where that is a subnormal below 2^-1042).  A power of two is its own bound:
+// the leading digit takes +-2^(b-1), and a column of reflectors, whose largest entry is the 1
+// of its diagonal, keeps one more bit of the others.
+__device__ __forceinline__ int exp_bound(int nz) {
+  const int b = nz >= 0x7FF00000 ? nz : nz - 1;   // Inf and NaN: 1026
+  return b >> 20 ? (b >> 20) - 1021 : -1021;
+}
+
+// N = round(x 2^(bS - e)) from the bit pattern (|x| <= 2^(e-1), so |N| <= 2^(bS-1));
 // ties round away from zero.  The mantissa is raised by 8 bits, so every exponent is one
 // right shift (by 5 at least: a subnormal of a row of subnormals; what is shifted further
 // than 62 is zero).
@@ -276,7 +284,7 @@ slice_kernel(const SliceOp a, const SliceOp b, int nblk_a, int K, int K_pad,
   auto take = [&](int& mx, double x, int k) {
     const int hi = __double2hiint(x) & 0x7FFFFFFF, nz = hi | (__double2loint(x) != 0);
     if (!ekb) mx = max(mx, nz);
-    else if (nz != 0) mx = max(mx, (nz >> 20 ? (nz >> 20) - 1021 : -1021) + o.esign * ekb[k]);
+    else if (nz != 0) mx = max(mx, exp_bound(nz) + o.esign * ekb[k]);
   };
   if (tid < R) mine[tid] = none;
   asm volatile("cp.async.wait_all;" ::: "memory");
@@ -330,7 +338,7 @@ slice_kernel(const SliceOp a, const SliceOp b, int nblk_a, int K, int K_pad,
     int mx = mine[tid];
     for (int q = 0; q < cl; ++q)
       if (q != rank) mx = max(mx, cluster.map_shared_rank(mine, q)[tid]);
-    es[tid] = ekb ? (mx == INT_MIN ? 0 : mx) : (mx == 0 ? 0 : mx >> 20 ? (mx >> 20) - 1021 : -1021);
+    es[tid] = ekb ? (mx == INT_MIN ? 0 : mx) : (mx == 0 ? 0 : exp_bound(mx));
     if (rank == 0 && i0 + tid < o.rows_pad) o.e[blockIdx.z * o.rows_pad + i0 + tid] = es[tid];
   }
   if (cl > 1) cluster.sync();   // no rank leaves while another reads its maxima
