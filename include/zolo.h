@@ -169,7 +169,8 @@ int zolo_schedule(double ell0, int r, int max_iter, double* ells, int* used_qr, 
    matrix keeps in its handle (host computation, no GPU work): the workspace
    for r shifts (r <= 0: for up to 8) plus, for a split precision, the slice
    planes and exponents, as the call allocates them (the planes are capped at
-   16 GB; a smaller allocation is tried when that fails).  Not counted: the
+   16 GB; a smaller allocation is tried when that fails, and for the 16-bit forms
+   from n = 2048 a workspace for blocks of 128 columns in place of 512).  Not counted: the
    host entry points' staging copies of A and the results, and the tuner's
    scratch (zolo_autotune).  Returns 0 and writes *bytes, or -i for an illegal
    argument i (m < n, n < 1, r outside -1..8, prec, svd not 0/1, NULL). */

@@ -165,9 +165,15 @@ struct PdBufs {
   EigWork eig;
 };
 
-// Workspace layout for (m, n, r).  The QR, Cholesky and eigensolver regions
-// are never live at the same time and share one union region.
-size_t layout(void* base, int64_t m, int64_t n, int r, bool svd, PdBufs* b) {
+// Columns of the widest super-block a call of this precision applies at once: the FP64 and
+// FP8 forms work on blocks alone and hold no buffers for more.
+int64_t super_width(int64_t n, int prec) {
+  return prec == ZOLO_SPLIT_BF16 || prec == ZOLO_SPLIT_FP16 ? qr_super_width(n) : kQrBlock;
+}
+
+// Workspace layout for (m, n, r) and super-blocks of sb columns.  The QR, Cholesky and
+// eigensolver regions are never live at the same time and share one union region.
+size_t layout(void* base, int64_t m, int64_t n, int r, bool svd, int64_t sb, PdBufs* b) {
   if (base && t_guard_on) t_guards.clear();
   Carve c(base);
   PdBufs t{};
@@ -190,8 +196,8 @@ size_t layout(void* base, int64_t m, int64_t n, int r, bool svd, PdBufs* b) {
     const int64_t npan = (n + kQrNB - 1) / kQrNB;
     t.qr.strideW = (m + n) * n;
     t.qr.W = q.take<double>(r * t.qr.strideW);
-    t.qr.sb = qr_super_width(n);
-    const int64_t sb = t.qr.sb, nsup = (n + sb - 1) / sb;
+    t.qr.sb = (int)sb;
+    const int64_t nsup = (n + sb - 1) / sb;
     t.qr.strideV = (m + sb) * n;
     t.qr.V = q.take<double>(r * t.qr.strideV);
     t.qr.strideT = npan * kQrNB * kQrNB;
@@ -256,6 +262,18 @@ int ensure_ws(zolo_handle_t h, size_t bytes) {
   }
   h->ws_bytes = bytes;
   return 0;
+}
+
+// A call's buffers in the handle's workspace, grown to hold them.  Where the memory for
+// super-blocks cannot be had, or a workspace that must not move (fixed) does not hold them,
+// those of blocks alone.
+int place(zolo_handle_t h, int64_t m, int64_t n, int r, bool svd, int prec, bool fixed, PdBufs* b) {
+  for (int64_t sb = super_width(n, prec);; sb = kQrBlock) {
+    const size_t bytes = layout(nullptr, m, n, r, svd, sb, b);
+    int e = fixed && sb != kQrBlock && h->ws_bytes < bytes ? ZOLO_ENOMEM : ensure_ws(h, bytes);
+    if (e == 0) layout(h->ws, m, n, r, svd, sb, b);
+    if (e == 0 || sb == kQrBlock) return e;
+  }
 }
 
 // Fill the listed guard zones of the workspace and clear the flag (guard mode).
@@ -744,7 +762,7 @@ int tune_r(zolo_handle_t h, const double* A, int64_t m, int64_t n, int64_t lda, 
   }
   {
     PdBufs tb;
-    if (int e = ensure_ws(h, layout(nullptr, m, n, kMaxR, svd, &tb))) return e;
+    if (int e = place(h, m, n, kMaxR, svd, o.prec, svd, &tb)) return e;
     if (is_split(o.prec)) {
       SplitScope pre;
       if (int e = pre.begin(h, m, n, kMaxR, st, o.prec)) return e;
@@ -804,9 +822,7 @@ int pd_core(zolo_handle_t h, const double* A, int64_t m, int64_t n, int64_t lda,
   int r_sched = o.r;
   if (alpha <= 0.0) {
     PdBufs tmpb;
-    const size_t bytes = layout(nullptr, m, n, 1, svd, &tmpb);
-    if (int e = ensure_ws(h, bytes)) return e;
-    layout(h->ws, m, n, 1, svd, &tmpb);
+    if (int e = place(h, m, n, 1, svd, ZOLO_FP64, svd, &tmpb)) return e;
     // row partial sums in X (m * ceil(n / 256) <= m n), column sums in Xn
     CK(alpha_bound_sums(A, lda, m, n, tmpb.X, tmpb.Xn, tmpb.partials, tmpb.norms, st));
     double sums[3];
@@ -818,9 +834,7 @@ int pd_core(zolo_handle_t h, const double* A, int64_t m, int64_t n, int64_t lda,
   double beta = o.beta;
   if (!(beta > 0.0)) {
     PdBufs eb;
-    const size_t bytes1 = layout(nullptr, m, n, 1, svd, &eb);
-    if (int e = ensure_ws(h, bytes1)) return e;
-    layout(h->ws, m, n, 1, svd, &eb);
+    if (int e = place(h, m, n, 1, svd, ZOLO_FP64, svd, &eb)) return e;
     if (int e = estimate_beta(A, lda, m, n, alpha, eb, st, &beta)) return e;
   }
   const double ell0 = std::min(1.0, beta / alpha);
@@ -834,9 +848,7 @@ int pd_core(zolo_handle_t h, const double* A, int64_t m, int64_t n, int64_t lda,
   Run R{m, n, r, {}, st};
   R.inv_chol = use_inverse_form(o.chol_form, m, n, r);
   info->chol_form = R.inv_chol ? 2 : 1;
-  const size_t bytes = layout(nullptr, m, n, r, svd, &R.b);
-  if (int e = ensure_ws(h, bytes)) return e;
-  layout(h->ws, m, n, r, svd, &R.b);
+  if (int e = place(h, m, n, r, svd, o.prec, svd, &R.b)) return e;
   if (out_bufs) *out_bufs = R.b;
   const PdBufs& b = R.b;
   if (int e = guards_arm(h, st)) return e;
@@ -1144,7 +1156,7 @@ int zolo_workspace_bytes(int64_t m, int64_t n, int r, int prec, int svd, uint64_
   if (!bytes) return -6;
   const int rr = r > 0 ? r : kMaxR;   // r chosen by the call: at most 8 shifts
   PdBufs b;
-  uint64_t total = layout(nullptr, m, n, rr, svd != 0, &b);
+  uint64_t total = layout(nullptr, m, n, rr, svd != 0, super_width(n, prec), &b);
   if (is_split(prec)) {
     // as SplitScope::begin asks for: slice planes (BF16), exponents (int), error flag
     const size_t per = split_elems_per_entry(m, n);
@@ -1229,8 +1241,7 @@ int zolo_pd_async(zolo_handle_t h, const double* A, int64_t m, int64_t n, int64_
   if (build_schedule(ell0, o.r, o.max_iter, &sch) != 0) return -10;
   Run R{m, n, sch.r, {}, st};
   R.inv_chol = use_inverse_form(o.chol_form, m, n, sch.r);
-  if (int e = ensure_ws(h, layout(nullptr, m, n, sch.r, false, &R.b))) return info->status = e;
-  layout(h->ws, m, n, sch.r, false, &R.b);
+  if (int e = place(h, m, n, sch.r, false, o.prec, false, &R.b)) return info->status = e;
   SplitScope split;
   if (is_split(o.prec))
     if (int e = split.begin(h, m, n, sch.r, st, o.prec)) return info->status = e;
@@ -1329,9 +1340,7 @@ int zolo_svd(zolo_handle_t h, const double* A, int64_t m, int64_t n, int64_t lda
   int e = 0;
   const int r_size = opts->r <= 0 ? kMaxR : opts->r;
   {
-    const size_t bytes = layout(nullptr, m, n, r_size, true, &b);
-    if ((e = ensure_ws(h, bytes)) != 0) return info->status = e;
-    layout(h->ws, m, n, r_size, true, &b);
+    if ((e = place(h, m, n, r_size, true, opts->prec, false, &b)) != 0) return info->status = e;
   }
   double* Qp = b.Qp_int;
   double* Hm = b.H_int;
@@ -1577,11 +1586,10 @@ int zolo_pd_batched(zolo_handle_t h, int count, const double* const* A, const in
       beta[i] = opts[i].beta;
       if (!(beta[i] > 0.0)) {
         PdBufs eb;
-        if (int e = ensure_ws(h, layout(nullptr, m[i], n[i], 1, false, &eb))) {
+        if (int e = place(h, m[i], n[i], 1, false, ZOLO_FP64, false, &eb)) {
           info[i].status = e;
           return e;
         }
-        layout(h->ws, m[i], n[i], 1, false, &eb);
         if (int e = estimate_beta(A[i], lda[i], m[i], n[i], alpha[i], eb, st, &beta[i])) {
           info[i].status = e;
           return e;
@@ -1615,7 +1623,17 @@ int zolo_pd_batched(zolo_handle_t h, int count, const double* const* A, const in
   if ((int)h->slots.size() < nslots) h->slots.resize(nslots);
   if (!h->fork && cudaEventCreateWithFlags(&h->fork, cudaEventDisableTiming) != cudaSuccess)
     return ZOLO_ECUDA;
-  const size_t ws_bytes = layout(nullptr, mmax, nmax, rmax, false, nullptr);
+  // super-blocks where some matrix takes them and every lane can hold them
+  bool wide = false;
+  for (int i = 0; i < count; ++i) wide |= super_width(n[i], opts[i].prec) > kQrBlock;
+  auto width = [&](int i) { return wide ? super_width(n[i], opts[i].prec) : (int64_t)kQrBlock; };
+  auto lane_bytes = [&] {
+    return layout(nullptr, mmax, nmax, rmax, false, wide ? qr_super_width(nmax) : kQrBlock, nullptr);
+  };
+  size_t ws_bytes = lane_bytes();
+  for (int k = 0; wide && k < nslots; ++k)
+    if (grow(&h->slots[k].ws, &h->slots[k].ws_bytes, ws_bytes) != 0) wide = false;
+  ws_bytes = lane_bytes();
   for (int k = 0; k < nslots; ++k) {
     BatchSlot& sl = h->slots[k];
     if (!sl.st && cudaStreamCreateWithFlags(&sl.st, cudaStreamNonBlocking) != cudaSuccess)
@@ -1670,7 +1688,7 @@ int zolo_pd_batched(zolo_handle_t h, int count, const double* const* A, const in
       Run R{m[i], n[i], sch[i].r, {}, st};
       R.inv_chol = inv;
       R.narrow_panels = true;
-      layout(sl.ws, m[i], n[i], sch[i].r, false, &R.b);
+      layout(sl.ws, m[i], n[i], sch[i].r, false, width(i), &R.b);
       SplitWork w{sl.slices, sl.slice_elems, sl.exps, sl.exp_elems, sl.err, 9};
       w.slices_s = split_slices(opts[i].prec);
       w.form = split_form(opts[i].prec);
@@ -1701,6 +1719,7 @@ int zolo_pd_batched(zolo_handle_t h, int count, const double* const* A, const in
   std::vector<uint64_t> key;
   key.reserve(8 + 12 * (size_t)count);
   key.push_back((uint64_t)count);
+  key.push_back((uint64_t)wide);
   key.push_back((uint64_t)(uintptr_t)h->brec);
   key.push_back(h->tuner.gen);   // graphs recorded with older kernel choices are not replayed
   // every buffer the recorded kernels hold: the split ones grow apart from the workspace
@@ -1745,7 +1764,7 @@ int zolo_pd_batched(zolo_handle_t h, int count, const double* const* A, const in
       Run R{m[i], n[i], sch[i].r, {}, sl.st};
       R.inv_chol = use_inverse_form(opts[i].chol_form, m[i], n[i], sch[i].r);
       R.narrow_panels = true;
-      layout(sl.ws, m[i], n[i], sch[i].r, false, &R.b);
+      layout(sl.ws, m[i], n[i], sch[i].r, false, width(i), &R.b);
       double* rec = h->brec + (size_t)i * kRecDoubles;
       R.b.status = reinterpret_cast<int*>(rec);
       R.b.norms = rec + 4;

@@ -285,11 +285,11 @@ double alpha_from_sums(const double* sums);
 // ------------------------------------------------------------ structured QR
 constexpr int kQrNB = 32;      // panel width (columns factored by one panel kernel)
 constexpr int kQrBlock = 128;  // block width (columns a panel's reflectors are applied to at once)
-// Widest super-block of an n-column problem: the columns whose reflectors are applied
-// together to everything to their right.
+// Widest super-block of an n-column problem on the 16-bit split forms: the columns whose
+// reflectors are applied together to everything to their right.
 int qr_super_width(int64_t n);
 struct QrBuffers {
-  int sb;                         // qr_super_width(n): the strides below hold super-blocks this wide
+  int sb;                         // qr_super_width(n) or kQrBlock: the strides below hold super-blocks this wide
   double* W;   int64_t strideW;   // stacked (m+n) x n per shift, ld m+n
   double* V;   int64_t strideV;   // explicit reflectors (m+sb) x n per shift, ld m+sb, rows
                                   // relative to the start of each column's super-block
