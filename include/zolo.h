@@ -407,6 +407,13 @@ int zolo_tune_load(zolo_handle_t handle, const char* path);
    0, -1 (NULL handle) or -2 (enable not 0/1). */
 int zolo_debug_guards(zolo_handle_t handle, int enable);
 
+/* zolo_debug_max_cluster(h, ctas): zolo_pd, zolo_svd and zolo_pd_sharded calls on h
+   factor their QR panels on thread-block clusters of at most `ctas` CTAs (8, 12 or 16),
+   as they do where the GPU, or the partition of it, has no room for larger ones
+   (no counterpart in the paper; for tests).  0: the largest the device has room
+   for.  Returns 0, -1 (NULL handle) or -2 (ctas). */
+int zolo_debug_max_cluster(zolo_handle_t handle, int ctas);
+
 #define ZOLO_STALL_SPLIT_GEMM 1
 #define ZOLO_STALL_JACOBI32 2
 #define ZOLO_STALL_JACOBI64 3

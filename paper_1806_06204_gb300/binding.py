@@ -101,6 +101,8 @@ def _load():
     lib.zolo_pd_sharded.restype = I
     lib.zolo_debug_guards.argtypes = [P, I]
     lib.zolo_debug_guards.restype = I
+    lib.zolo_debug_max_cluster.argtypes = [P, I]
+    lib.zolo_debug_max_cluster.restype = I
     lib.zolo_batch_graphs.argtypes = [P, I]
     lib.zolo_batch_graphs.restype = I
     lib.zolo_batch_graphs_recorded.argtypes = [P]
@@ -132,7 +134,7 @@ EXPORTED = ["zolo_opts_default", "zolo_create", "zolo_destroy", "zolo_coefficien
             "zolo_tune_save", "zolo_tune_load", "zolo_autotune",
             "zolo_workspace_bytes", "zolo_debug_stall", "zolo_shift_range",
             "zolo_pd_sharded", "zolo_pd_async", "zolo_batch_graphs",
-            "zolo_batch_graphs_recorded", "zolo_debug_guards"]
+            "zolo_batch_graphs_recorded", "zolo_debug_guards", "zolo_debug_max_cluster"]
 
 
 def kernel_launches() -> int:
@@ -242,6 +244,13 @@ def debug_guards(handle, enable: bool) -> None:
     e = LIB.zolo_debug_guards(handle.ptr, int(enable))
     if e:
         raise ZoloError(e, "zolo_debug_guards")
+
+
+def debug_max_cluster(handle, ctas: int) -> None:
+    """QR panels of this handle's calls on clusters of at most 8, 12 or 16 CTAs (0: the device's most)."""
+    e = LIB.zolo_debug_max_cluster(handle.ptr, int(ctas))
+    if e:
+        raise ZoloError(e, "zolo_debug_max_cluster")
 
 
 def batch_graphs(handle, enable: bool) -> None:

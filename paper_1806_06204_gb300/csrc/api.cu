@@ -109,6 +109,7 @@ struct zolo_handle_s {
   int async_next = 0;
   bool batch_graphs = true;                // zolo_pd_batched records and replays a graph
   bool guards = false;                     // zolo_debug_guards
+  int max_cluster = 0;                     // zolo_debug_max_cluster
   int* guard_flag = nullptr;               // set by the guard check
 };
 
@@ -1188,6 +1189,7 @@ int zolo_pd(zolo_handle_t h, const double* A, int64_t m, int64_t n, int64_t lda,
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   TunerScope ts(&h->tuner);
   GuardScope guard(h->guards);
+  PanelClusterScope panels(h->max_cluster);
   PhaseClock pc;
   pc.start(h, st);
   cudaEventRecord(h->e0, st);
@@ -1300,6 +1302,7 @@ int zolo_pd_sharded(zolo_handle_t h, const double* A, int64_t m, int64_t n, int6
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   TunerScope ts(&h->tuner);
   GuardScope guard(h->guards);
+  PanelClusterScope panels(h->max_cluster);
   ShardCtx sh;
   sh.rank = rank;
   sh.nranks = nranks;
@@ -1332,6 +1335,7 @@ int zolo_svd(zolo_handle_t h, const double* A, int64_t m, int64_t n, int64_t lda
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   TunerScope ts(&h->tuner);
   GuardScope guard(h->guards);
+  PanelClusterScope panels(h->max_cluster);
   cudaEventRecord(h->e0, st);
   // Qp and H go to internal buffers carved ahead of the union region; their
   // offsets do not depend on r, and sizing with r = 8 when r is chosen by the
@@ -1715,6 +1719,7 @@ int zolo_pd_batched(zolo_handle_t h, int count, const double* const* A, const in
   if (!h->joined && cudaEventCreateWithFlags(&h->joined, cudaEventDisableTiming) != cudaSuccess)
     return ZOLO_ECUDA;
   if (any_split) split_prepare();
+  qr_prepare();
   // ---- the batch as one graph: key = every pointer, size and option of the call
   std::vector<uint64_t> key;
   key.reserve(8 + 12 * (size_t)count);
@@ -1890,6 +1895,13 @@ int zolo_debug_guards(zolo_handle_t h, int enable) {
   if (!h) return -1;
   if (enable != 0 && enable != 1) return -2;
   h->guards = enable != 0;
+  return 0;
+}
+
+int zolo_debug_max_cluster(zolo_handle_t h, int ctas) {
+  if (!h) return -1;
+  if (ctas != 0 && ctas != 8 && ctas != 12 && ctas != 16) return -2;
+  h->max_cluster = ctas;
   return 0;
 }
 

@@ -30,6 +30,7 @@
 // structure makes zero is an exact zero in floating point too.
 #include <cooperative_groups.h>
 
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 
@@ -673,47 +674,81 @@ namespace {
 // (600 rows: 0.51 against 0.47, but 0.28 against 0.47 ms for a few problems alone).
 enum PanelKind { kRegNone, kReg1x17, kReg2x17, kReg4x33, kReg8x17, kReg8x97, kReg8w65, kReg12w17, kReg12w33,
                  kReg12w49, kReg12w65, kReg12w97, kReg16w17, kReg16w33, kReg16w49, kReg16w65, kReg16w97 };
-PanelKind panel_kind(int64_t m, int r, bool narrow) {
+// Clusters of 12 and 16 CTAs are beyond the portable size of 8 and a partition of the GPU
+// may have no room for them: `most` is the largest there is, and without 12 the clusters of
+// 8 serve what they hold.
+PanelKind panel_kind(int64_t m, int r, bool narrow, int most) {
   const int64_t H = m + kQrNB;
   if (m < kClusterPanelMinRows) return narrow ? kReg1x17 : kReg8x17;
-  if (narrow) {
-    if (H <= 64 * 17) return kReg2x17;
-    if (H <= 64 * 33) return kReg4x33;
+  if (narrow || most < 12) {
+    if (narrow && H <= 64 * 17) return kReg2x17;
+    if (narrow && H <= 64 * 33) return kReg4x33;
     if (H <= 32 * 97) return kReg8x97;
     if (H <= 64 * 65) return kReg8w65;
   }
-  if (r > 7 || narrow) {
+  if (most >= 12 && (r > 7 || narrow || most < 16)) {
     if (H <= 96 * 17) return kReg12w17;
     if (H <= 96 * 33) return kReg12w33;
     if (H <= 96 * 49) return kReg12w49;
     if (H <= 96 * 65) return kReg12w65;
     if (H <= 96 * 97) return kReg12w97;
   }
-  if (H <= 128 * 17) return kReg16w17;
-  if (H <= 128 * 33) return kReg16w33;
-  if (H <= 128 * 49) return kReg16w49;
-  if (H <= 128 * 65) return kReg16w65;
-  if (H <= 128 * 97) return kReg16w97;
+  if (most >= 16) {
+    if (H <= 128 * 17) return kReg16w17;
+    if (H <= 128 * 33) return kReg16w33;
+    if (H <= 128 * 49) return kReg16w49;
+    if (H <= 128 * 65) return kReg16w65;
+    if (H <= 128 * 97) return kReg16w97;
+  }
   return kRegNone;
 }
 
-// Clusters of 12 and 16 CTAs are beyond the portable size: allowed once per device.
-cudaError_t allow_wide_clusters() {
-  static std::atomic<uint64_t> done{0};
+// Allows the kernel its cluster; whether there is room for one (an error of the query: no,
+// and *asked stays false).
+template <int RANKS, int KMAX>
+bool allow_cluster(bool* asked) {
+  const auto kernel = qr_panel_reg_kernel<RANKS, 8, 1, KMAX>;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(RANKS);
+  cfg.blockDim = dim3(256);
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = RANKS;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  int clusters = 0;
+  if (cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
+          cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    *asked = false;
+  }
+  return clusters > 0;
+}
+template <int RANKS>
+bool allow_clusters(bool* asked) {
+  return allow_cluster<RANKS, 17>(asked) && allow_cluster<RANKS, 33>(asked) && allow_cluster<RANKS, 49>(asked) &&
+         allow_cluster<RANKS, 65>(asked) && allow_cluster<RANKS, 97>(asked);
+}
+
+thread_local int t_cluster_limit = 16;
+
+// The largest of 16, 12 and 8 CTAs whose panel kernels the current device has room for,
+// asked once per device.
+int largest_cluster() {
+  static std::atomic<uint64_t> done{0}, has12{0}, has16{0};
   int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev < 64 && (done.load() >> dev & 1)) return cudaSuccess;
-  const void* k[] = {(const void*)qr_panel_reg_kernel<12, 8, 1, 17>, (const void*)qr_panel_reg_kernel<12, 8, 1, 33>,
-                     (const void*)qr_panel_reg_kernel<12, 8, 1, 49>, (const void*)qr_panel_reg_kernel<12, 8, 1, 65>,
-                     (const void*)qr_panel_reg_kernel<12, 8, 1, 97>, (const void*)qr_panel_reg_kernel<16, 8, 1, 17>,
-                     (const void*)qr_panel_reg_kernel<16, 8, 1, 33>, (const void*)qr_panel_reg_kernel<16, 8, 1, 49>,
-                     (const void*)qr_panel_reg_kernel<16, 8, 1, 65>, (const void*)qr_panel_reg_kernel<16, 8, 1, 97>};
-  for (const void* f : k)
-    if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess)
-      return e;
-  if (dev < 64) done.fetch_or(1ull << dev);
-  return cudaSuccess;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev >= 64) return 8;
+  const uint64_t bit = 1ull << dev;
+  if (!(done.load() & bit)) {
+    bool asked = true;
+    if (allow_clusters<12>(&asked)) has12.fetch_or(bit);
+    if (allow_clusters<16>(&asked)) has16.fetch_or(bit);
+    if (asked) done.fetch_or(bit);
+  }
+  return std::min(t_cluster_limit, has16.load() & bit ? 16 : has12.load() & bit ? 12 : 8);
 }
 
 cudaError_t launch_panel(PanelKind k, const PanelArgs& p, int r, double fl, double by, cudaStream_t st) {
@@ -740,12 +775,18 @@ cudaError_t launch_panel(PanelKind k, const PanelArgs& p, int r, double fl, doub
 
 }  // namespace
 
+void qr_prepare() { largest_cluster(); }
+
+PanelClusterScope::PanelClusterScope(int limit) : prev(t_cluster_limit) {
+  if (limit > 0) t_cluster_limit = limit;
+}
+PanelClusterScope::~PanelClusterScope() { t_cluster_limit = prev; }
+
 int qr_super_width(int64_t n) { return n >= 2048 ? 512 : kQrBlock; }
 
 cudaError_t structured_qr_q(const QrBuffers& b, int64_t m, int64_t n, int r, int* status,
                             cudaStream_t st, bool explicit_q, bool narrow_panels) {
   constexpr int NB = kQrNB, NBb = kQrBlock;
-  if (allow_wide_clusters() != cudaSuccess) return cudaErrorInvalidConfiguration;
   const int64_t ldw = m + n;
   // On the tensor cores the blocks of a super-block are applied to its own columns
   // one by one and to everything to its right together (see the file's head).
@@ -755,7 +796,7 @@ cudaError_t structured_qr_q(const QrBuffers& b, int64_t m, int64_t n, int r, int
   const int64_t ldv = m + SB;
   cudaError_t err;
   // the register panel where there is one, else the global-memory cluster kernel
-  const PanelKind reg = panel_kind(m, r, narrow_panels);
+  const PanelKind reg = panel_kind(m, r, narrow_panels, largest_cluster());
   // every V entry outside the rows a panel writes must be an exact zero
   if ((err = cudaMemsetAsync(b.V, 0, sizeof(double) * r * b.strideV, st)) != cudaSuccess) return err;
   if (SB > NBb &&

@@ -305,6 +305,14 @@ struct QrBuffers {
 // then takes the fewest CTAs per shift whose registers hold the rows.
 cudaError_t structured_qr_q(const QrBuffers& b, int64_t m, int64_t n, int r, int* status,
                             cudaStream_t st, bool explicit_q = true, bool narrow_panels = false);
+// Asks the current device for its cluster sizes (before a stream capture).
+void qr_prepare();
+// This thread's panels take clusters of `limit` CTAs at most (8, 12 or 16; 0: as they are).
+struct PanelClusterScope {
+  int prev;
+  explicit PanelClusterScope(int limit);
+  ~PanelClusterScope();
+};
 // Inverses of the NB x NB diagonal blocks of an upper-triangular R (ld n) in the
 // layout cholesky_upper_batched leaves in Rinv; a zero pivot sets status.
 cudaError_t tri_inv_diag_blocks(const double* R, int64_t n, double* Rinv, int* status,
