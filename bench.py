@@ -340,7 +340,8 @@ FP64_DFMA_MEASURED_TFLOPS = 1.20
 # 76.  The FP8 products run at twice the 16-bit rate (nominal 4.5 against 2.25
 # PFLOP/s), so their peak is the measured BF16 peak times 2.
 SPLIT_PAIRS_OF = {"bf16": 34, "fp16": 28, "fp8": 76}
-SPLIT_PAIRS = 53   # roofline()'s default: nine six-bit slices
+SPLIT_PAIRS = 53   # roofline()'s default where no form is named (nine six-bit digits, which no form
+                   # here uses; every call below passes its form's SPLIT_PAIRS_OF)
 SLICE_PEAK_RATIO = {"bf16": 1.0, "fp16": 1.0, "fp8": 2.0}
 SLICE_DTYPE = {"bf16": "bf16x7-slices->f64", "fp16": "fp16x7-slices->f64",
                "fp8": "e4m3x11-slices->f64"}

@@ -254,9 +254,12 @@ int zolo_pd_sharded(zolo_handle_t handle, const double* A, int64_t m, int64_t n,
    the whole batch is recorded as one CUDA graph and the graph is replayed when
    the same batch (pointers, sizes, options) is decomposed again.  A Cholesky
    breakdown found at the end is redone for that matrix on the single-matrix
-   path.  Each matrix's result equals zolo_pd's to rounding (bit for bit below
-   512 rows: with many problems in flight the batched call factors a taller
-   QR panel on fewer CTAs, which sums its column norms in another order).
+   path.  Each matrix's result equals zolo_pd's to rounding (in ZOLO_FP64 bit for bit
+   below 512 rows; with many problems in flight the batched call factors a taller QR
+   panel on fewer CTAs, which sums its column norms in another order, a batch of 16
+   matrices or more takes other tiles and no K splits for a taller matrix's FP64 products,
+   so those bits depend on whether there are that many, and the split forms choose between
+   the tensor cores and FP64 by the batch's throughput).
    opts[i].posteriori must be 0.  Returns the first non-zero status
    (info[i].status per matrix); -i codes refer to the arguments as in zolo_pd
    with the offending matrix's info[].status set. */
@@ -296,7 +299,11 @@ int zolo_svd_host(zolo_handle_t handle, const double* A, int64_t m, int64_t n, i
    seven 8-bit ones) on the tensor cores, ZOLO_SPLIT_FP16 (`slices` 0 or 8: the
    accuracy of eight seven-bit slices, held as seven 8-bit ones) or ZOLO_SPLIT_FP8
    (`slices` 0 or 11: eleven five-bit slices).  On the split path an Inf or NaN in a row of
-   op(A) or a column of op(B) makes that row or column of the product NaN.
+   op(A) or a column of op(B) makes that row or column of the product NaN.  C may
+   share elements with A or B (k <= 114688 on the split path): the product is that of
+   the operands as they were; in ZOLO_FP64, where no tile holds all that its outputs
+   cover (C over A with n > 64, over B with m > 64, or displaced), it is formed in a
+   stream-ordered allocation and copied.
    Not in the paper as
    an interface; it exposes the building block for testing and reuse.
    Synchronises the stream before returning. */
@@ -348,7 +355,8 @@ int zolo_dgemm_noalloc(int transA, int transB, int64_t m, int64_t n, int64_t k, 
    for that shape; the call's own outputs are written once, by the kept
    kernel.  To bound the cost of measuring, a shape whose built-in kernel takes
    over 50 ms keeps it, and the split path (or FP64) is not timed where the
-   cost model puts it 4x behind the other.  zolo_autotune(h, 0) stops measuring; choices already made stay in
+   cost model puts it 4x behind the other; the products that set the QR's T factors on
+   the 16-bit forms follow the cost model alone.  zolo_autotune(h, 0) stops measuring; choices already made stay in
    use.  Without choices the built-in rules apply (the split path where its
    cost model predicts a gain, else the FP64 tile and K split of least estimated
    time).

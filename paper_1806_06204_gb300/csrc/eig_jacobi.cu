@@ -117,8 +117,8 @@ __device__ bool wait_round(const int* ver, int want, int* err) {
 // FP64 unit for a whole warp slot (64 clocks) however few lanes are active, so the
 // partial dot products are summed by one warp, which changes with the item.  A sweep
 // (events): n = 256 1.12 ms (1.71 with the columns read twice by 256 threads and the
-// whole rotation formed in one chain), n = 512 2.9 (3.3), n = 1024 7.1 (7.9); from n =
-// 2048 the FP64 units bound it (3 n^3 / 2 FMA, 25 ms a sweep as before).
+// whole rotation formed in one chain), n = 512 2.9 (3.3), n = 1024 7.0 (7.3); from n =
+// 2048 the FP64 units bound it (3 n^3 / 2 FMA: 25.5 ms a sweep, 167 at 4096; 24.9 and 164).
 // A rotation is made for cosines above tol and counted above 4 tol.
 template <int NT, int RPT>
 __global__ void __launch_bounds__(NT, RPT == 0 ? 1536 / NT : 1)
@@ -297,8 +297,8 @@ __global__ void fill_kernel(double* d, int64_t n, double v) {
 // thread (t1, t2) owns the 2x2 block of G at the rows of rotation t1 and the columns of
 // t2, forms both rotations itself, and writes to the other copy of G.
 // A sweep (events): n = 256 0.35 ms (0.51 with two phases a step, a grid barrier a round
-// and at most two CTAs a pair), n = 1024 2.1 (3.1), n = 2048 7.8 (8.7); at n = 4096 the
-// products take over (46.6, from 46).
+// and at most two CTAs a pair), n = 1024 2.1 (3.0), n = 2048 7.9 (8.9); from n = 3000 the
+// products take over (26.6 and 25.4 ms, n = 4096 45.9 and 42.9).
 constexpr int kJB = 16;                // columns per block
 constexpr int kJW = 2 * kJB;           // columns of a block pair
 // rows per staged chunk: 128, or 256 where a CTA has several; the chunk's leading

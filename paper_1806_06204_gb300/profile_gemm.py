@@ -11,8 +11,8 @@ measures the candidates (zolo_autotune) and F is written with the choice.  Print
 call, FP64-equivalent TFLOP/s (2MNK per call), and for the split path the BF16
 tensor TFLOP/s actually issued (34, 28 or 76 slice-pair products; FP8 at twice
 the rate).  Also the launch
-target for kernel profilers: each call is one row-exponent + slicing pass per
-operand and one GEMM kernel (split), or one GEMM kernel (FP64).
+target for kernel profilers: each call is one slicing launch (both operands' row
+exponents and digits) and one GEMM kernel (split), or one GEMM kernel (FP64).
 """
 import argparse
 import json
@@ -62,7 +62,7 @@ def main():
     if args.tune_cache:
         zb.autotune(h, False)
         zb.tune_save(h, args.tune_cache)
-        names = {0: "64x64", 1: "32x128", 2: "32x64", 3: "64x64 split-K 2", 4: "64x64 split-K 4",
+        names = {0: "built-in rule", 1: "32x128", 2: "32x64", 3: "64x64 split-K 2", 4: "64x64 split-K 4",
                  5: "64x64 split-K 8", 8: "split"}
         for line in open(args.tune_cache).read().splitlines():
             f = line.split()

@@ -83,6 +83,19 @@ def test_c_shifted_against_a(zb, handle, first):
     assert np.array_equal(out[:, :first], P[:, :first])
 
 
+@pytest.mark.parametrize("prec", [1, 2, 3])
+@pytest.mark.parametrize("m,n", [(1000, 64), (300, 300), (60, 500)])
+def test_split_products_in_place_have_the_bits_of_others(zb, handle, prec, m, n):
+    # the split path slices both operands before it writes C
+    rng = np.random.default_rng(m + n)
+    A, B, L = dev(rng.standard_normal((m, n))), dev(rng.standard_normal((n, n))), dev(rng.standard_normal((m, m)))
+    right, left = (zb.zolo_dgemm(handle, A, B, prec=prec).cpu().numpy(), zb.zolo_dgemm(handle, L, A, prec=prec).cpu().numpy())
+    C, D = A.t().clone().t(), A.t().clone().t()
+    zb.zolo_dgemm(handle, C, B, C, prec=prec)
+    zb.zolo_dgemm(handle, L, D, D, prec=prec)
+    assert np.array_equal(C.cpu().numpy(), right) and np.array_equal(D.cpu().numpy(), left)
+
+
 @pytest.mark.parametrize("v", [0, 3, 4])
 @pytest.mark.parametrize("m,n", [(1000, 64), (150, 150), (64, 300)])
 def test_forced_kernels_in_place(zb, tmp_path, v, m, n):
