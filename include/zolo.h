@@ -395,8 +395,8 @@ int zolo_tune_load(zolo_handle_t handle, const char* path);
        product (opts.prec = ZOLO_SPLIT_BF16, FP16 or FP8, zolo_dgemm's split path),
        on an mbarrier no thread or copy arrives at;
      ZOLO_STALL_JACOBI32: block 0 of the first FP32 sweep of zolo_svd's
-       eigensolver, on a flag no thread sets (the other blocks leave the grid
-       barrier when they see the error flag);
+       eigensolver, on a flag no thread sets (its cluster and the blocks that wait
+       for its columns leave when they see the error flag);
      ZOLO_STALL_JACOBI64: block 0 of the first FP64 sweep, on a flag no thread
        sets, before its first column pair (the blocks whose pairs wait for that
        pair's columns leave when they see the error flag).

@@ -1725,6 +1725,8 @@ int zolo_pd_batched(zolo_handle_t h, int count, const double* const* A, const in
   key.reserve(8 + 12 * (size_t)count);
   key.push_back((uint64_t)count);
   key.push_back((uint64_t)wide);
+  key.push_back((uint64_t)h->dbg_stall);   // zolo_debug_stall is a parameter of the recorded kernels
+  key.push_back((uint64_t)h->dbg_ns);
   key.push_back((uint64_t)(uintptr_t)h->brec);
   key.push_back(h->tuner.gen);   // graphs recorded with older kernel choices are not replayed
   // every buffer the recorded kernels hold: the split ones grow apart from the workspace

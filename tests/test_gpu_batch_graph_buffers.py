@@ -61,3 +61,16 @@ def test_graph_recorded_anew_after_the_split_buffers_grew(zb, prec):
         assert zb.batch_graphs_recorded(h) == 4
     finally:
         h.close()
+
+
+def test_graph_recorded_with_the_stall_hook_on_is_not_replayed_with_it_off(zb):
+    h = zb.Handle(0)
+    try:
+        b = Batch(zb, 96, 2, zb.ZOLO_SPLIT_BF16, 40)
+        zb.debug_stall(h, zb.ZOLO_STALL_SPLIT_GEMM, 100_000)
+        _, _, infos, st = zb.zolo_pd_batched(h, b.As, b.os, Qps=b.Qs, Hs=b.Hs, check=False)
+        assert st == 7 and all(i.status == 7 for i in infos)   # ZOLO_ETIMEOUT
+        zb.debug_stall(h, 0, 0)
+        b.run(zb, h)
+    finally:
+        h.close()
